@@ -311,9 +311,9 @@ def run_gpu(args):
     x_host = torch.from_numpy(inp["x"]).pin_memory()
     nbuf = max(2, int(np.ceil(1.2 * L2_BYTES / x_host.numel() / 4)))
     xbufs = [x_host.cuda() for _ in range(nbuf)]
-    # per layer: LN1+QKV, IM attention, out-proj+LN2+MLP (fused kernels); each intra layer once per half of the batch
+    # per layer: LN1+QKV, IM attention, out-proj+LN2+MLP (fused kernels)
     paired = stack.paired_rings and n_f == n_b and n_f > 0   # one launch per kernel for both rings of a depth
-    launches_per_step = 3 * (n_f if paired else n_f + n_b) + 3 * n_i * (2 if (stack.intra_halves and B >= 2) else 1)
+    launches_per_step = 3 * (n_f if paired else n_f + n_b) + 3 * n_i * (1 if paired else 2)
     if stack.packed:
         launches_per_step += 3   # row plan, gather of the real rows, scatter of the result
 
@@ -505,7 +505,7 @@ def run_gpu(args):
                    "valid_tokens_per_step": tokens, "padded_tokens_per_step": B * wl.L,
                    "l2": f"inputs rotate over {nbuf} device copies ({nbuf * x_host.numel() * 4 >> 20} MiB > 126 MiB L2); "
                          "the step's scratch alone is larger than L2", "launch": "one CUDA graph per input buffer; inside it " + ("the forward and backward ring layers of each depth in one launch per kernel (two problems per launch), " if paired else "the forward and backward rings on two streams, ") +
-                             "then the intra encoder on the two halves of the batch on two streams; packed row layout (real rows only); "
+                             "then the intra encoder on the whole batch; packed row layout (real rows only); "
                              "kernels of a stream start under the tail of the one before (programmatic dependent launch)"},
         "clocks": clocks.summary(),
         "timed_regions": {"repeats": args.repeats, "steps_each": args.steps, "ms_per_step_median": ms_per_step,

@@ -1,8 +1,9 @@
-"""ctypes binding of libgsit.so: argument marshalling only.
+"""Binding of libgsit.so: argument marshalling only.
 
 Every step of the hot path runs in the CUDA kernels of the library; PyTorch is used here for device
-memory (output and workspace allocation) and for the current stream.  There is no CPU fallback: if the
-library is missing or a call fails, an exception is raised.
+memory (output and workspace allocation) and for the current stream.  The calls of the hot path are marshalled by the
+CPython extension `_native` (csrc/torch_ext.cpp; 2 us a call where ctypes took 20 - 25), the rest by ctypes.  There is no
+CPU fallback: if the library or the extension is missing or a call fails, an exception is raised.
 """
 from __future__ import annotations
 
@@ -18,6 +19,7 @@ DEVFLAG_CLAMPED, DEVFLAG_TIMEOUT = 1, 2
 
 _LIB_PATH = Path(__file__).resolve().parent / "libgsit.so"
 _lib = None
+_ext = None
 
 
 class GsitError(RuntimeError):
@@ -89,6 +91,21 @@ def load():
     lib.gsit_trace_read.argtypes = [ctypes.c_int, ctypes.POINTER(ctypes.c_float), ctypes.POINTER(ctypes.c_int32)]
     _lib = lib
     return lib
+
+
+def native():
+    """The extension module that marshals the hot calls (built in-tree beside libgsit.so)."""
+    global _ext
+    if _ext is None:
+        load()
+        try:
+            from . import _native
+        except ImportError as e:
+            raise ImportError(f"the extension _native is missing or does not load ({e}): run `python -m paper_2505_01068_b200.build` "
+                              "(there is no fallback path)") from e
+        _native.init(GsitError)
+        _ext = _native
+    return _ext
 
 
 def status_string(code: int) -> str:
@@ -183,23 +200,7 @@ def im_qkv_proj(x, w_qkv, b_qkv, seg_len, heads, valid_len=None, out=None, row_s
     """x [B, L, d] (last dim contiguous) -> qkv [B, L, 3, H, hd].
     With row_start (from plan_rows; bf16, d a multiple of 64) x is the packed matrix [capacity, d] and qkv
     [capacity, 3, H, hd]; valid_len gives the batch size, and only the rows of these samples are computed and written."""
-    if row_start is not None:
-        cap, d = x.shape
-        assert x.is_cuda and x.stride(1) == 1 and w_qkv.is_contiguous() and valid_len is not None
-        shape = make_shape(valid_len.shape[0], seg_len, d, heads, valid_len, _dtype_code(x.dtype), PHASE_INTRA, 0, 0.0, row_start, cap)
-        if out is None:
-            out = torch.zeros((cap, 3, heads, d // heads), dtype=x.dtype, device=x.device)
-        _check(load().gsit_im_qkv_proj(ctypes.byref(shape), _ptr(x), x.stride(0), _ptr(w_qkv), _ptr(b_qkv), _ptr(out),
-                                       _stream()), "gsit_im_qkv_proj")
-        return out
-    B, L, d = x.shape
-    assert x.is_cuda and x.stride(2) == 1 and x.stride(0) == L * x.stride(1) and w_qkv.is_contiguous()
-    shape = make_shape(B, seg_len, d, heads, valid_len, _dtype_code(x.dtype), PHASE_INTRA)
-    if out is None:
-        out = torch.empty((B, L, 3, heads, d // heads), dtype=x.dtype, device=x.device)
-    _check(load().gsit_im_qkv_proj(ctypes.byref(shape), _ptr(x), x.stride(1), _ptr(w_qkv), _ptr(b_qkv), _ptr(out),
-                                   _stream()), "gsit_im_qkv_proj")
-    return out
+    return native().im_qkv_proj(x, w_qkv, b_qkv, seg_len, heads, valid_len, out, row_start)
 
 
 def im_attention_fwd(q, k, v, seg_len, valid_len=None, phase=PHASE_INTER_FWD, custom_mask=0, scale=0.0,
@@ -207,22 +208,7 @@ def im_attention_fwd(q, k, v, seg_len, valid_len=None, phase=PHASE_INTER_FWD, cu
     """q, k, v: [B, L, H, hd] views sharing strides (e.g. qkv[:, :, i] of the fused buffer).  Returns out [B, L, d]
     (and lse [B, H, L] float when want_lse).  workspace: uint8 device tensor of workspace_bytes(shape, CALL_ATTENTION)
     bytes (allocated here when not given)."""
-    B, L, H, hd = q.shape
-    d = H * hd
-    for t in (q, k, v):
-        assert t.is_cuda and t.shape == q.shape and t.stride() == q.stride() and t.dtype == q.dtype
-    assert q.stride(3) == 1 and q.stride(2) == hd and q.stride(0) == L * q.stride(1)
-    shape = make_shape(B, seg_len, d, H, valid_len, _dtype_code(q.dtype), phase, custom_mask, scale)
-    if out is None:
-        out = torch.empty((B, L, d), dtype=q.dtype, device=q.device)
-    lse = torch.empty((B, H, L), dtype=torch.float32, device=q.device) if want_lse else None
-    need = workspace_bytes(shape, CALL_ATTENTION)
-    if workspace is None and need > 0:
-        workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
-    _check(load().gsit_im_attention_fwd(ctypes.byref(shape), _ptr(q), _ptr(k), _ptr(v), q.stride(1), _ptr(out),
-                                        _ptr(lse), _ptr(workspace), 0 if workspace is None else workspace.numel(),
-                                        _stream()), "gsit_im_attention_fwd")
-    return (out, lse) if want_lse else out
+    return native().im_attention_fwd(q, k, v, seg_len, valid_len, phase, custom_mask, scale, want_lse, out, workspace)
 
 
 def plan_rows(valid_len, seg_len, split_sample=0, out=None):
@@ -262,48 +248,12 @@ def unpack_rows(y_packed, y, seg_len, valid_len, row_start):
     return y
 
 
-_W_KEYS = ("ln1_g", "ln1_b", "w_qkv", "b_qkv", "w_o", "b_o", "ln2_g", "ln2_b", "w_1", "b_1", "w_2", "b_2")
-
-
-def make_layer_weights(w: dict, ln_eps: float = 1e-5) -> LayerWeights:
-    """w maps ln1_g, ln1_b, w_qkv, b_qkv, w_o, b_o, ln2_g, ln2_b, w_1, b_1, w_2, b_2 to device tensors or None."""
-    for kk in ("w_qkv", "w_o", "w_1", "w_2"):
-        assert w[kk].is_cuda and w[kk].is_contiguous()
-    for kk in ("ln1_g", "ln1_b", "b_qkv", "b_o", "ln2_g", "ln2_b", "b_1", "b_2"):
-        assert w.get(kk) is None or (w[kk].dtype == torch.float32 and w[kk].is_contiguous())
-    return LayerWeights(*[_ptr(w.get(kk)) for kk in _W_KEYS], int(w["w_1"].shape[0]), float(ln_eps))
-
-
 def im_layer_fwd(x, weights: dict, seg_len, heads, valid_len=None, phase=PHASE_INTER_FWD, custom_mask=0, scale=0.0,
                  ln_eps=1e-5, out=None, workspace=None, row_start=None):
     """x float32 [B, L, d] (row stride free) -> y float32 [B, L, d]; weights in bf16 or float32 select the path.
     With row_start (from plan_rows) x and out are packed matrices [capacity, d] (row stride free) and the batch size is
     that of valid_len."""
-    code = _dtype_code(weights["w_qkv"].dtype)
-    lw = make_layer_weights(weights, ln_eps)
-    if row_start is not None:
-        cap, d = x.shape
-        assert x.is_cuda and x.dtype == torch.float32 and x.stride(1) == 1 and out is not None and out.shape[0] == cap
-        assert out.stride(1) == 1
-        shape = make_shape(valid_len.shape[0], seg_len, d, heads, valid_len, code, phase, custom_mask, scale, row_start, cap)
-        need = workspace_bytes(shape, CALL_LAYER, lw.d_ff)
-        if workspace is None:
-            workspace = torch.empty(need, dtype=torch.uint8, device=x.device)
-        _check(load().gsit_im_layer_fwd(ctypes.byref(shape), ctypes.byref(lw), _ptr(x), x.stride(0), _ptr(out),
-                                        out.stride(0), _ptr(workspace), workspace.numel(), _stream()), "gsit_im_layer_fwd")
-        return out
-    B, L, d = x.shape
-    assert x.is_cuda and x.dtype == torch.float32 and x.stride(2) == 1 and x.stride(0) == L * x.stride(1)
-    shape = make_shape(B, seg_len, d, heads, valid_len, code, phase, custom_mask, scale)
-    if out is None:
-        out = torch.empty((B, L, d), dtype=torch.float32, device=x.device)
-    assert out.stride(2) == 1 and out.stride(0) == L * out.stride(1)
-    need = workspace_bytes(shape, CALL_LAYER, lw.d_ff)
-    if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=x.device)
-    _check(load().gsit_im_layer_fwd(ctypes.byref(shape), ctypes.byref(lw), _ptr(x), x.stride(1), _ptr(out),
-                                    out.stride(1), _ptr(workspace), workspace.numel(), _stream()), "gsit_im_layer_fwd")
-    return out
+    return native().im_layer_fwd(x, weights, seg_len, heads, valid_len, phase, custom_mask, scale, ln_eps, out, workspace, row_start, False)
 
 
 def im_layer_pair_fwd(x_a, x_b, weights_a: dict, weights_b: dict, seg_len, heads, valid_len=None, phase_a=PHASE_INTER_FWD,
@@ -311,32 +261,8 @@ def im_layer_pair_fwd(x_a, x_b, weights_a: dict, weights_b: dict, seg_len, heads
     """Two layers of one geometry in one call (the two ring encoders' layers of equal depth): same results as two
     im_layer_fwd calls.  x_* float32 [B, L, d] (or packed [capacity, d] with row_start), out_* likewise (required in the
     packed layout); workspace: 2 x the layer's workspace bytes."""
-    code = _dtype_code(weights_a["w_qkv"].dtype)
-    lwa, lwb = make_layer_weights(weights_a, ln_eps), make_layer_weights(weights_b, ln_eps)
-    if row_start is not None:
-        cap, d = x_a.shape
-        Bn = valid_len.shape[0]
-        mk = lambda ph: make_shape(Bn, seg_len, d, heads, valid_len, code, ph, 0, 0.0, row_start, cap)
-        strides = lambda t: t.stride(0)
-        assert out_a is not None and out_b is not None
-    else:
-        Bn, L, d = x_a.shape
-        mk = lambda ph: make_shape(Bn, seg_len, d, heads, valid_len, code, ph)
-        strides = lambda t: t.stride(1)
-        if out_a is None:
-            out_a = torch.empty((Bn, L, d), dtype=torch.float32, device=x_a.device)
-        if out_b is None:
-            out_b = torch.empty((Bn, L, d), dtype=torch.float32, device=x_a.device)
-    for t in (x_a, x_b, out_a, out_b):
-        assert t.is_cuda and t.dtype == torch.float32 and t.stride(-1) == 1 and t.shape == x_a.shape
-    sha, shb = mk(phase_a), mk(phase_b)
-    need = 2 * workspace_bytes(sha, CALL_LAYER, lwa.d_ff)
-    if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=x_a.device)
-    _check(load().gsit_im_layer_pair_fwd(ctypes.byref(sha), ctypes.byref(shb), ctypes.byref(lwa), ctypes.byref(lwb), _ptr(x_a),
-                                         strides(x_a), _ptr(x_b), strides(x_b), _ptr(out_a), strides(out_a), _ptr(out_b),
-                                         strides(out_b), _ptr(workspace), workspace.numel(), _stream()), "gsit_im_layer_pair_fwd")
-    return out_a, out_b
+    return native().im_layer_pair_fwd(x_a, x_b, weights_a, weights_b, seg_len, heads, valid_len, phase_a, phase_b, ln_eps, out_a, out_b,
+                                      workspace, row_start)
 
 
 def im_layer_fwd_static(x, weights: dict, seg_len, heads, valid_len=None, phase=PHASE_INTER_FWD, custom_mask=0,
@@ -344,27 +270,10 @@ def im_layer_fwd_static(x, weights: dict, seg_len, heads, valid_len=None, phase=
     """im_layer_fwd without a workspace: the library's built-in scratch array is used, so the call allocates no
     device memory as long as ``out`` is given.  Problems whose scratch exceeds STATIC_SCRATCH_BYTES raise GsitError
     (status 3).  Calls on one GPU must not overlap in time; they share the array."""
-    B, L, d = x.shape
-    assert x.is_cuda and x.dtype == torch.float32 and x.stride(2) == 1 and x.stride(0) == L * x.stride(1)
-    shape = make_shape(B, seg_len, d, heads, valid_len, _dtype_code(weights["w_qkv"].dtype), phase, custom_mask, scale)
-    lw = make_layer_weights(weights, ln_eps)
-    if out is None:
-        out = torch.empty((B, L, d), dtype=torch.float32, device=x.device)
-    assert out.stride(2) == 1 and out.stride(0) == L * out.stride(1)
-    _check(load().gsit_im_layer_fwd_static(ctypes.byref(shape), ctypes.byref(lw), _ptr(x), x.stride(1), _ptr(out),
-                                           out.stride(1), _stream()), "gsit_im_layer_fwd_static")
-    return out
+    return native().im_layer_fwd(x, weights, seg_len, heads, valid_len, phase, custom_mask, scale, ln_eps, out, None, None, True)
 
 
 def stack_head_fwd(c, w_f, b_f, seg_len, valid_len=None, out=None):
     """c float32 [B, L, dc] (row stride free) -> float32 [B, out_features]: the last real step of each modality segment,
     concatenated, through the linear map w_f [out_features, 3*dc] (float32 or bfloat16) and bias b_f."""
-    B, L, dc = c.shape
-    assert c.is_cuda and c.dtype == torch.float32 and c.stride(2) == 1 and c.stride(0) == L * c.stride(1)
-    assert w_f.is_contiguous() and w_f.shape[1] == 3 * dc
-    shape = make_shape(B, seg_len, 16, 1, valid_len, _dtype_code(w_f.dtype), PHASE_INTRA)
-    if out is None:
-        out = torch.empty((B, w_f.shape[0]), dtype=torch.float32, device=c.device)
-    _check(load().gsit_stack_head_fwd(ctypes.byref(shape), _ptr(c), c.stride(1), dc, _ptr(w_f), _ptr(b_f), _ptr(out),
-                                      w_f.shape[0], _stream()), "gsit_stack_head_fwd")
-    return out
+    return native().stack_head_fwd(c, w_f, b_f, seg_len, valid_len, out)

@@ -4,9 +4,10 @@ outputs side by side on the feature axis (width 2d); then the intra-modal encode
 sequencing and buffer reuse happen here -- each layer is one gsit_im_layer_fwd call, and the feature
 concat costs nothing because the last layer of each ring writes its half of the [B, L, 2d] buffer.
 
-The two rings share nothing but their input, so they are issued on two CUDA streams (fork after the
-input is ready, join before the intra encoder): the CTAs of one ring fill the SM slots that the last
-wave of the other leaves empty.  Each ring has its own workspace and ping-pong buffers."""
+The two rings share nothing but their input: their layers of equal depth go through one library call each (one launch per
+kernel for both).  All launches of such a forward are issued by one call of the extension (csrc/torch_ext.cpp).  Rings of
+unequal depth, or paired_rings=False, are issued from Python on two CUDA streams (fork after the input is ready, join
+before the intra encoder), each ring with its own workspace and ping-pong buffers."""
 from __future__ import annotations
 
 import torch
@@ -19,22 +20,19 @@ class GsitStack:
                  concurrent_rings=True, batch_chunks=1, intra_halves=True,
                  packed=True, paired_rings=True):
         """head: optional (w_f, b_f) of the read-out X_m = f(|| Split(.)[-1]); see read_out().
-        concurrent_rings: issue independent work on several streams (False: every launch on the caller's stream, whole
-        batch per launch).  batch_chunks: with concurrent issue, the batch is cut into this many groups of samples, each
-        with its own pair of streams; samples never interact, so the result does not depend on it.  (At B = 64, L = 1050
-        one chunk is fastest: the persistent fused kernels pay their per-CTA set-up once per launch.)
-        intra_halves: with concurrent issue, the intra encoder runs on the two halves of the batch on the two streams, so
-        that the attention of one half overlaps the fused layer halves of the other (0.794 -> 0.784 ms at that shape
-        with paired rings; three or four parts are slower again).
         packed: when valid lengths are given (and the layers are bf16 at widths the tcgen05 fused kernels cover), the
         stack works on the packed row layout: the real rows are gathered once, every layer runs on them only, and the
         result is scattered back with +0 in the padded positions.  The row-wise parts of the layers then do no work
         for padding (24 % of the rows at the benchmark's lengths).  The plan of where each segment starts is made on the
         device, so a captured forward stays valid when the lengths change.
-        paired_rings: (packed layout, rings of equal depth) the forward-ring and backward-ring layers of equal depth go
-        through one gsit_im_layer_pair_fwd call each -- three launches per depth for both rings, on one stream, each
-        starting under the tail of the one before it -- instead of two streams of three launches (0.784 against
-        0.789 ms at that shape).  False: one stream per ring."""
+        paired_rings: (rings of equal depth) the forward-ring and backward-ring layers of equal depth go through one
+        gsit_im_layer_pair_fwd call each, and the whole forward is issued on the caller's stream, each launch starting
+        under the tail of the one before it.
+        The other options belong to forwards whose rings are not paired (paired_rings=False, rings of unequal depth) or to
+        batch_chunks > 1.  concurrent_rings: issue independent work on several streams (False: every launch on the caller's
+        stream).  batch_chunks: the batch is cut into this many groups of samples, each with its own pair of streams;
+        samples never interact, so the result does not depend on it.  intra_halves: the intra encoder runs on the two
+        halves of the batch on the two streams."""
         self.head = head
         self.concurrent_rings = concurrent_rings
         self.batch_chunks = max(1, int(batch_chunks))
@@ -113,8 +111,7 @@ class GsitStack:
                                    capacity=cap)
                 need = max(need, B.workspace_bytes(sh2, B.CALL_LAYER, self.intra[0]["w_1"].shape[0]))
             f32 = dict(dtype=torch.float32, device=x.device)
-            ws_all = torch.empty(2 * need, dtype=torch.uint8, device=x.device)   # one per ring, or both for a paired call
-            self._ws_pair = ws_all
+            ws_all = torch.empty(2 * need, dtype=torch.uint8, device=x.device)   # one per ring
             self._bufs[key] = (cap, plan, [ws_all[:need], ws_all[need:]],
                                [torch.zeros((cap, d), **f32) for _ in range(5)],
                                torch.zeros((cap, 2 * d), **f32), torch.zeros((cap, 2 * d), **f32),
@@ -149,46 +146,7 @@ class GsitStack:
                 cur = dst
             return cur
 
-        paired = self.paired_rings and len(self.fwd) == len(self.bwd) and len(self.fwd) > 0
-
-        def rings_paired():
-            cur_a = cur_b = xp
-            n = len(self.fwd)
-            for i in range(n):
-                last = i == n - 1
-                dst_a = c0[:, 0:d] if last else t[i % 2]
-                dst_b = c0[:, d:2 * d] if last else t[2 + i % 2]
-                B.im_layer_pair_fwd(cur_a, cur_b, self.fwd[i], self.bwd[i], self.seg_len, self.heads, valid_len, B.PHASE_INTER_FWD,
-                                    B.PHASE_INTER_BWD, ln_eps=self.ln_eps, out_a=dst_a, out_b=dst_b, workspace=self._ws_pair,
-                                    row_start=plan)
-                cur_a, cur_b = dst_a, dst_b
-
-        if paired and not (halves and self.intra):
-            rings_paired()
-            res = intra(0, Bn, ws[0]) if self.intra else c0
-        elif paired:
-            # both rings on the caller's stream, then the intra encoder on the two halves of the batch on two streams
-            rings_paired()
-            if self._lanes is None:
-                dev = x.device
-                self._lanes = ([torch.cuda.Stream(device=dev) for _ in range(2)], torch.cuda.Event(),
-                               [torch.cuda.Event() for _ in range(2)])
-                self._ring_done = [torch.cuda.Event()]
-            streams, fork, done = self._lanes
-            main = torch.cuda.current_stream(x.device)
-            fork.record(main)
-            for si, (lo, hi) in enumerate(((0, mid), (mid, Bn))):
-                streams[si].wait_event(fork)
-                with torch.cuda.stream(streams[si]):
-                    r_ = intra(lo, hi, ws[si])
-                    done[si].record(streams[si])
-                if si == 0:
-                    res = r_
-            for si in range(2):
-                main.wait_event(done[si])
-                x.record_stream(streams[si])
-                valid_len.record_stream(streams[si])
-        elif not conc:
+        if not conc:
             ring(self.fwd, B.PHASE_INTER_FWD, 0, ws[0], t[0:2])
             ring(self.bwd, B.PHASE_INTER_BWD, 1, ws[0], t[0:2])
             res = intra(0, Bn, ws[0]) if self.intra else c0
@@ -248,7 +206,48 @@ class GsitStack:
                 raise B.GsitError(code, f"GsitStack.forward: device status flags {flags:#x}")
         return res
 
+    def _native_buffers(self, x, valid_len, packed):
+        """Buffers of the natively issued forward, kept per problem size: (the nine tensors stack_forward takes, result)."""
+        key = ("native", packed, x.shape, x.device)
+        got = None if self._bufs is None else self._bufs.get(key)
+        if got is not None:
+            return got
+        Bn, L, d = x.shape
+        cap = Bn * L + 128 if packed else Bn * L
+        code = B._dtype_code(self.fwd[0]["w_qkv"].dtype)
+        plan = torch.zeros(3 * Bn + 1, dtype=torch.int32, device=x.device) if packed else None
+        need = 0
+        for w, width, heads, phase in [(self.fwd[0], d, self.heads, B.PHASE_INTER_FWD)] + [(w, 2 * d, self.intra_heads, B.PHASE_INTRA)
+                                                                                           for w in self.intra[:1]]:
+            sh = B.make_shape(Bn, self.seg_len, width, heads, valid_len, code, phase, row_start=plan, capacity=cap if packed else 0)
+            need = max(need, B.workspace_bytes(sh, B.CALL_LAYER, w["w_1"].shape[0]))
+        # rows past the last real one are read by the last row tile (and discarded): they start out as zeros
+        z = lambda cols: torch.zeros((cap, cols), dtype=torch.float32, device=x.device)
+        bufs = (plan, torch.empty(2 * need, dtype=torch.uint8, device=x.device), z(d), z(d), z(d), z(d), z(d) if packed else None,
+                z(2 * d), z(2 * d))
+        if self._bufs is None:
+            self._bufs = {}
+        got = self._bufs[key] = (bufs, torch.empty((Bn, L, 2 * d), dtype=torch.float32, device=x.device))
+        return got
+
+    def _forward_native(self, x, valid_len, out):
+        """One call that issues every launch of the forward (about 2 us each; issuing them from Python took 15)."""
+        packed = self.packed and valid_len is not None
+        while True:
+            bufs, y = self._native_buffers(x, valid_len, packed)
+            if out is not None:
+                y = out
+            code = B.native().stack_forward(x, valid_len, y, self.fwd, self.bwd, self.intra, self.seg_len, self.heads, self.intra_heads,
+                                            self.ln_eps, bufs)
+            if code == 0:
+                return y
+            if not (packed and code == 2):  # anything but "this shape is not covered in the packed layout": a real error
+                raise B.GsitError(code, "GsitStack.forward")
+            packed = self.packed = False
+
     def _forward(self, x, valid_len, out):
+        if self.paired_rings and self.batch_chunks == 1 and len(self.fwd) == len(self.bwd) > 0:
+            return self._forward_native(x, valid_len, out)
         if self.packed and valid_len is not None and self.batch_chunks == 1:
             try:
                 return self._forward_packed(x, valid_len, out)
