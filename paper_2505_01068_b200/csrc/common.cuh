@@ -153,6 +153,13 @@ struct LinearArgs {
   int mask_rows;    // zero the padded rows of C (uses geometry)
 };
 cudaError_t launch_linear_f32(const Geometry& g, const LinearArgs& a, cudaStream_t st);
+// The two halves of a float layer, fused (linear_f32.cu): d <= 128.
+bool fused_layer_f32_supported(const Geometry& g, int d_ff);
+cudaError_t launch_ln_qkv_f32(const Geometry& g, const float* x, int64_t ldx, const float* gamma, const float* beta, float eps,
+                              const float* w_qkv, const float* b_qkv, float* qkv, cudaStream_t st);
+cudaError_t launch_proj_mlp_f32(const Geometry& g, const float* att, const float* x, int64_t ldx, const float* w_o, const float* b_o,
+                                const float* gamma, const float* beta, float eps, const float* w_1, const float* b_1, const float* w_2,
+                                const float* b_2, int d_ff, float* y, int64_t ldy, cudaStream_t st);
 // bf16 linear layer on tcgen05 tensor cores with TMEM accumulators (gemm_tc.cu): K a multiple of 64, N a multiple of 8
 bool linear_tc_supported(const LinearArgs& a);
 cudaError_t launch_linear_tc_bf16(const Geometry& g, const LinearArgs& a, cudaStream_t st);

@@ -304,6 +304,20 @@ gsit_status gsit_im_layer_fwd(const gsit_shape* shape, const gsit_layer_weights*
                                           static_cast<const __nv_bfloat16*>(w->w_1), w->b_1,
                                           static_cast<const __nv_bfloat16*>(w->w_2), w->b_2, w->d_ff, y, y_row_stride, cs));
   }
+  if (!bf && fused_layer_f32_supported(g, w->d_ff)) {  // the same three launches for float operands
+    auto f32 = [](const void* p) { return static_cast<const float*>(p); };
+    float *fq = static_cast<float*>(qkv), *fa = static_cast<float*>(att);
+    {
+      TraceScope t(GSIT_KERNEL_LINEAR, cs);
+      st = from_cuda(launch_ln_qkv_f32(g, x, x_row_stride, w->ln1_gamma, w->ln1_beta, eps, f32(w->w_qkv), w->b_qkv, fq, cs));
+      if (st != GSIT_OK) return st;
+    }
+    if ((st = run_attention(g, dtype, fq, fq + d, fq + 2 * d, 3 * (int64_t)d, fa, nullptr, pick_scale(shape, g), nullptr, cs)) != GSIT_OK)
+      return st;
+    TraceScope t(GSIT_KERNEL_LINEAR, cs);
+    return from_cuda(launch_proj_mlp_f32(g, fa, x, x_row_stride, f32(w->w_o), w->b_o, w->ln2_gamma, w->ln2_beta, eps, f32(w->w_1), w->b_1,
+                                         f32(w->w_2), w->b_2, w->d_ff, y, y_row_stride, cs));
+  }
   // h = LN1(x)
   if ((st = run_layernorm(g, x, x_row_stride, w->ln1_gamma, w->ln1_beta, eps, h, bf, cs)) != GSIT_OK) return st;
   // qkv = h W_qkv^T + b_qkv   (shared projection of the whole concatenated sequence)

@@ -1,59 +1,11 @@
 // Linear layers and LayerNorm around the IM attention: C = act(A W^T + bias) (+ residual).
 //   - bf16: cp.async-pipelined mma.sync.m16n8k16 tiles, float accumulate, fused bias / ReLU / residual /
 //     padded-row zeroing epilogue, bf16 or float output.
-//   - f32:  shared-memory tiled FMA kernel with the same epilogue (the 1e-4 parity path).
+// (float operands: linear_f32.cu)
 #include "common.cuh"
 
 namespace gsit {
 namespace {
-
-// ------------------------------------------------------------------------------------------------ f32
-constexpr int FT = 64, FK = 16;  // 64x64 tile, 16-deep slices, 256 threads of 4x4 outputs
-
-__global__ void __launch_bounds__(256) linear_f32_kernel(Geometry g, LinearArgs a) {
-  __shared__ float As[FK][FT + 1], Ws[FK][FT + 1];
-  const float* A = static_cast<const float*>(a.A);
-  const float* W = static_cast<const float*>(a.W);
-  float* C = static_cast<float*>(a.C);
-  const int m0 = blockIdx.y * FT, n0 = blockIdx.x * FT;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < a.K; k0 += FK) {
-    for (int idx = threadIdx.x; idx < FT * FK; idx += 256) {
-      const int r = idx / FK, kk = idx % FK;
-      const int m = m0 + r, n = n0 + r, k = k0 + kk;
-      As[kk][r] = (m < a.M && k < a.K) ? A[(int64_t)m * a.lda + k] : 0.f;
-      Ws[kk][r] = (n < a.N && k < a.K) ? W[(int64_t)n * a.K + k] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < FK; ++kk) {
-      float av[4], wv[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) { av[i] = As[kk][ty * 4 + i]; wv[i] = Ws[kk][tx * 4 + i]; }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], wv[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
-    if (m >= a.M) continue;
-    const bool real = !a.mask_rows || row_is_real(g, m);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n >= a.N) continue;
-      float v = acc[i][j] + (a.bias ? a.bias[n] : 0.f);
-      if (a.relu) v = fmaxf(v, 0.f);
-      if (a.residual) v += a.residual[(int64_t)m * a.ldr + n];
-      C[(int64_t)m * a.ldc + n] = real ? v : 0.f;
-    }
-  }
-}
 
 // ------------------------------------------------------------------------------------------------ bf16
 constexpr int BM = 128, BK = 32, GSTAGES = 3;
@@ -203,13 +155,6 @@ __global__ void __launch_bounds__(256) layernorm_kernel(Geometry g, const float*
 }
 
 }  // namespace
-
-cudaError_t launch_linear_f32(const Geometry& g, const LinearArgs& a, cudaStream_t st) {
-  const dim3 grid((a.N + FT - 1) / FT, (a.M + FT - 1) / FT);
-  if (grid.y > 65535) return cudaErrorNotSupported;
-  linear_f32_kernel<<<grid, 256, 0, st>>>(g, a);
-  return cudaGetLastError();
-}
 
 extern int g_attn_variant;  // kernel selection (attn_bf16.cu): GSIT_ATTN_LEGACY keeps every bf16 kernel on the mma.sync path
 

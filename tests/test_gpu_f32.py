@@ -1,0 +1,84 @@
+"""Float kernels at the sizes where their tiles end: head widths around the slices of a row, key counts around the key tiles,
+batches that use one, two and four key splits, and layer widths around the 32-feature slices of the fused halves."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads as wk
+from gpu_util import check_close, pad_mask, to_dev, to_np64, weights_to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def g():
+    import paper_2505_01068_b200 as lib
+    lib.load()
+    return lib
+
+
+@pytest.mark.parametrize("H,hd", [(2, 1), (3, 5), (2, 8), (1, 12), (2, 16), (1, 24), (2, 32), (1, 40), (1, 64), (1, 100), (1, 128), (1, 200), (1, 256)])
+def test_attention_every_head_width(g, H, hd):
+    rng = np.random.default_rng(hd)
+    seg = (9, 129, 66)
+    valid = np.array([[9, 129, 66], [1, 64, 65], [8, 0, 17]], dtype=np.int32)
+    q, k, v = wk.draw_qkv(rng, 3, sum(seg), H, hd, "f32")
+    pm = pad_mask(seg, valid, 3)
+    dev = [to_dev(np.where(pm[:, :, None, None], np.nan, t).astype(np.float32)) for t in (q, k, v)]
+    for phase, mask in ((g.PHASE_INTER_FWD, 0), (g.PHASE_INTRA, 0), (g.PHASE_CUSTOM, 0x1FF), (g.PHASE_CUSTOM, 0b000100011)):
+        out, lse = g.im_attention_fwd(*dev, seg, torch.from_numpy(valid).cuda(), phase, mask, want_lse=True)
+        ref, ref_lse = oracle.im_attention_dense(q, k, v, seg, valid, phase, custom_mask=mask, want_lse=True)
+        check_close(to_np64(out), ref, "f32", pm, f"hd {hd} phase {phase}")
+        a, b = to_np64(lse), np.asarray(ref_lse)
+        assert np.array_equal(np.isneginf(a), np.isneginf(b)) and np.abs(a[np.isfinite(b)] - b[np.isfinite(b)]).max() <= 1e-4
+
+
+@pytest.mark.parametrize("B", [1, 24, 96])
+def test_attention_key_splits(g, B):
+    rng = np.random.default_rng(B)
+    seg = (5, 130, 257)
+    q, k, v = wk.draw_qkv(rng, B, sum(seg), 4, 8, "f32")
+    q *= 6.0   # the running maximum moves
+    valid = np.stack([rng.integers(0, n + 1, size=B) for n in seg], axis=1).astype(np.int32)
+    out = g.im_attention_fwd(*[to_dev(t) for t in (q, k, v)], seg, torch.from_numpy(valid).cuda(), g.PHASE_INTER_BWD)
+    ref = oracle.im_attention_dense(q, k, v, seg, valid, g.PHASE_INTER_BWD)
+    check_close(to_np64(out), ref, "f32", pad_mask(seg, valid, B), f"B {B}")
+
+
+@pytest.mark.parametrize("d,heads,d_ff,seg,B", [(32, 4, 128, (8, 12, 10), 2), (36, 3, 100, (64, 64, 0), 1), (64, 8, 256, (50, 75, 100), 3),
+                                                (96, 4, 200, (1, 63, 1), 2), (128, 2, 512, (33, 64, 31), 2), (4, 1, 4, (3, 2, 1), 1),
+                                                (160, 4, 320, (33, 64, 31), 2), (30, 3, 62, (33, 64, 31), 1), (64, 8, 256, (50, 375, 500), 40)])
+def test_layer_widths(g, d, heads, d_ff, seg, B):
+    """d <= 128 with whole 16-byte rows takes the fused halves, the others (160; 30 and 62) the separate kernels."""
+    rng = np.random.default_rng(d + d_ff)
+    L = sum(seg)
+    x = rng.standard_normal((B, L, d), dtype=np.float32)
+    w = wk.draw_layer_weights(rng, d, d_ff, "f32", affine=True)
+    valid = np.stack([rng.integers(0, n + 1, size=B) for n in seg], axis=1).astype(np.int32)
+    pm = pad_mask(seg, valid, B)
+    xd = to_dev(np.where(pm[:, :, None], np.nan, x).astype(np.float32))
+    if d % 4:   # rows of whole 16-byte pieces are required: give the rows a stride of 32
+        wide = torch.full((B, L, 32), float("nan"), device="cuda")
+        wide[:, :, :d] = xd
+        y = torch.full((B, L, 32), float("nan"), device="cuda")
+        g.im_layer_fwd(wide[:, :, :d], weights_to_dev(w, "f32"), seg, heads, torch.from_numpy(valid).cuda(), g.PHASE_INTER_FWD, out=y[:, :, :d])
+        y = y[:, :, :d]
+    else:
+        y = g.im_layer_fwd(xd, weights_to_dev(w, "f32"), seg, heads, torch.from_numpy(valid).cuda(), g.PHASE_INTER_FWD)
+    n = min(B, 4)
+    ref = oracle.im_layer_fwd(x[-n:], w, seg, heads, valid[-n:], g.PHASE_INTER_FWD)
+    check_close(to_np64(y)[-n:], ref, "f32", pm[-n:], f"d {d}")
+    assert bool((y[torch.from_numpy(pm).cuda()] == 0).all())
+
+
+@pytest.mark.parametrize("d,heads", [(30, 5), (64, 8), (129, 3)])
+def test_projection_odd_widths(g, d, heads):
+    rng = np.random.default_rng(d)
+    seg, valid = (7, 70, 52), np.array([[7, 70, 52], [3, 0, 51]], dtype=np.int32)
+    x, w = rng.standard_normal((2, sum(seg), d), dtype=np.float32), wk.xavier_uniform(rng, 3 * d, d)
+    b = rng.standard_normal(3 * d).astype(np.float32)
+    qkv = g.im_qkv_proj(to_dev(x), to_dev(w), to_dev(b), seg, heads, torch.from_numpy(valid).cuda())
+    ref = x.astype(np.float64) @ w.T.astype(np.float64) + b
+    ref[pad_mask(seg, valid, 2)] = 0
+    check_close(to_np64(qkv).reshape(ref.shape), ref, "f32", pad_mask(seg, valid, 2), f"d {d}")
