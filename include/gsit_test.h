@@ -15,12 +15,12 @@ extern "C" {
 
 /* Kernel selection (process-wide host state; 0 restores the defaults).  Every choice computes the same result up to
  * floating-point summation order.
- *   GSIT_ATTN_DEFAULT   head_dim 64, 32, 16: tcgen05 / tensor-memory attention; head_dim 8: mma.sync attention;
+ *   GSIT_ATTN_DEFAULT   head_dim 64, 32, 16: tcgen05 / tensor-memory attention for all but small problems, mma.sync attention
+ *                       for those and at head_dim 8;
  *                       layer at d_model 64 / 128: fused tcgen05 halves; linear layers: tcgen05 GEMM where it applies
- *   1 .. 7              the mma.sync attention with its n-th alternative tile configuration (where the shape has one)
  *   GSIT_ATTN_UNFUSED   the layer as separate LayerNorm / linear / attention kernels (padded layout only)
  *   GSIT_ATTN_LEGACY    the mma.sync family everywhere: attention, fused layer halves, linear layers (padded layout only)
- *   GSIT_ATTN_TMEM      the tensor-memory attention also at head_dim 8 */
+ *   GSIT_ATTN_TMEM      the tensor-memory attention at every head_dim and size it covers */
 typedef enum { GSIT_ATTN_DEFAULT = 0, GSIT_ATTN_UNFUSED = 8, GSIT_ATTN_LEGACY = 9, GSIT_ATTN_TMEM = 10 } gsit_kernel_choice;
 gsit_status gsit_tune_attention(int choice);
 

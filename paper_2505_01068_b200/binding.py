@@ -166,7 +166,7 @@ def last_device_status() -> tuple[int, int]:
 
 
 def tune_attention(variant: int):
-    """Test / measurement hook: selects a kernel family (ATTN_* above, or 1..7 for alternative mma.sync tile shapes)."""
+    """Test / measurement hook: selects a kernel family (ATTN_* above)."""
     _check(load().gsit_tune_attention(int(variant)), "gsit_tune_attention")
 
 

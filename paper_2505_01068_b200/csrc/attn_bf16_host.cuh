@@ -48,7 +48,7 @@ cudaError_t launch_one(const Geometry& g, const AttnOperands* ops, int n, int64_
 
 }  // namespace
 
-int g_attn_variant = 0;  // gsit_kernel_choice, or 1..7 = alternative tile configurations of the mma.sync attention
+int g_attn_variant = 0;  // gsit_kernel_choice
 
 cudaError_t launch_attn_bf16_n(const Geometry& g, const AttnOperands* ops, int n, int64_t row_stride, float scale, int* next_item,
                                cudaStream_t st, bool counter_cleared) {
@@ -56,35 +56,83 @@ cudaError_t launch_attn_bf16_n(const Geometry& g, const AttnOperands* ops, int n
   if (g.batch > 65535 || g.d % 16 != 0) return cudaErrorNotSupported;
   const int cw = (g.d % 64 == 0) ? 64 : (g.d % 32 == 0) ? 32 : 16;
   const int var = g_attn_variant;
-  // head_dim 64 is a dense contraction: tcgen05 / TMEM kernel (GSIT_ATTN_LEGACY keeps the mma.sync kernel for comparison)
-  if (g.hd == 64 && var != GSIT_ATTN_LEGACY) {
+  int n_sm = 0;
+  cudaError_t e = sm_count_and_smem_once(nullptr, 0, &n_sm);
+  if (e != cudaSuccess) return e;
+  auto tiles = [&](int rows) {  // query tiles of one head of one problem
+    int64_t t = 0;
+    for (int s = 0; s < 3; ++s) t += (g.seg_len[s] + rows - 1) / rows;
+    return t * g.batch;
+  };
+  // Which kernel, decided for each problem by itself, so that a launch for two problems gives the bits of two launches.
+  // The tensor-memory kernels take long to set up and to hand over a work item, the mma.sync kernel takes longer per score: what
+  // counts is the number of units (128 query rows x 64 keys of one head) that the padded lengths amount to.
+  //   head_dim 16: they meet at about 110 units per SM (32 samples of (50, 500, 500), 8 heads, intra: both 46 us; one sample: 8
+  //   against 16 us; 64 samples: 83 against 77).  head_dim 32: at about 55 (16 samples, 8 heads: 34 us).
+  //   head_dim 64 is a dense contraction; there only a few short walks (at most two key tiles per row) are over sooner in the
+  //   mma.sync kernel (32 x (50, 50, 50), 2 heads: 4.8 against 6.1 us; 128 samples: 14.8 against 11.5).
+  //   head_dim 8: the tensor-memory kernel is slower throughout (55 against 44 us at 64 x (50, 500, 500)): a tcgen05 hand-over
+  //   per 64 keys of one head costs more than the 8192 exponentials it feeds.
+  auto tensor_memory = [&](uint32_t allowed) {
+    if (var == GSIT_ATTN_LEGACY || (g.hd != 64 && !attn_tcs_supported(g))) return false;
+    if (var == GSIT_ATTN_TMEM) return true;
+    if (g.hd == 8) return false;
+    int64_t units = 0;
+    int longest = 0;  // most key tiles that a row walks
+    for (int s = 0; s < 3; ++s) {
+      int kt = 0;
+      for (int r = 0; r < 3; ++r)
+        if ((allowed >> (3 * s + r)) & 1u) kt += (g.seg_len[r] + KT - 1) / KT;
+      units += (int64_t)((g.seg_len[s] + 127) / 128) * kt;
+      if (kt > longest) longest = kt;
+    }
+    units *= (int64_t)g.batch * g.heads;
+    if (g.hd == 64) return longest > 2 || units > 2LL * n_sm;
+    return units > (g.hd == 16 ? 110LL : 55LL) * n_sm;
+  };
+  const bool tm = tensor_memory(ops[0].allowed);
+  if (n == 2 && tm != tensor_memory(ops[1].allowed)) {
+    for (int i = 0; i < n; ++i)
+      if ((e = launch_attn_bf16_n(g, ops + i, 1, row_stride, scale, nullptr, st)) != cudaSuccess) return e;
+    return cudaSuccess;
+  }
+  if (tm && g.hd == 64) {
     for (int i = 0; i < n; ++i) {  // one launch per problem
       Geometry gi = g;
       gi.allowed = ops[i].allowed;
-      cudaError_t e = launch_attn_tc_hd64(gi, ops[i].q, ops[i].k, ops[i].v, row_stride, ops[i].out, ops[i].lse, scale, st);
+      e = launch_attn_tc_hd64(gi, ops[i].q, ops[i].k, ops[i].v, row_stride, ops[i].out, ops[i].lse, scale, st);
       if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
   }
-  // head_dim 16 / 32: thread-per-row softmax on tensor-memory tiles.  At head_dim 8 that kernel measures slower than the
-  // mma.sync kernel below (61 against 46 us at the MOSEI cross shape: a tcgen05 hand-over per 64 keys of one head costs
-  // more than the 8192 exponentials it feeds), so there it is selected by the knob only.
-  if (attn_tcs_supported(g) && (var == GSIT_ATTN_TMEM || (var == 0 && g.hd >= 16)))
-    return launch_attn_tcs(g, ops, n, row_stride, scale, next_item, st, counter_cleared);
-#define GSIT_CASE(VAR_, HD_, CW_, R_, KS_, MB_)         \
-  if (g.hd == HD_ && cw == CW_ && (var == VAR_ || VAR_ == 0)) \
-    return launch_one<Cfg<HD_, CW_, R_, KS_, MB_>>(g, ops, n, row_stride, scale, st);
-  // alternatives first (selected only by the knob), then the defaults (VAR_ == 0 matches any knob value)
-  GSIT_CASE(1, 8, 64, 4, 64, 2) GSIT_CASE(2, 8, 64, 4, 32, 2) GSIT_CASE(3, 8, 64, 2, 64, 2)
-  GSIT_CASE(4, 8, 64, 2, 32, 3) GSIT_CASE(5, 8, 64, 2, 64, 3) GSIT_CASE(6, 8, 64, 1, 64, 3)
-  GSIT_CASE(7, 8, 64, 1, 32, 4)
-  GSIT_CASE(1, 16, 64, 2, 64, 2) GSIT_CASE(2, 16, 64, 2, 32, 2) GSIT_CASE(3, 16, 64, 1, 64, 2)
-  GSIT_CASE(4, 16, 64, 1, 32, 3)
-  GSIT_CASE(0, 8, 64, 4, 64, 2) GSIT_CASE(0, 16, 64, 2, 64, 2) GSIT_CASE(0, 32, 64, 1, 32, 2)
-  GSIT_CASE(0, 64, 64, 1, 32, 2)
-  GSIT_CASE(0, 8, 32, 2, 64, 2) GSIT_CASE(0, 16, 32, 1, 64, 2) GSIT_CASE(0, 32, 32, 1, 32, 2)
-  GSIT_CASE(0, 8, 16, 1, 64, 2) GSIT_CASE(0, 16, 16, 1, 64, 2)
-#undef GSIT_CASE
+  if (tm) return launch_attn_tcs(g, ops, n, row_stride, scale, next_item, st, counter_cleared);
+  // mma.sync tiles.  Rows per warp: more of them reuse the key fragments, fewer give more CTAs and shorter walks; a row's result
+  // does not depend on it (the keys per step are the same), so the number of problems may count here.
+#define GSIT_LAUNCH(HD_, CW_, R_, KS_, MB_) return launch_one<Cfg<HD_, CW_, R_, KS_, MB_>>(g, ops, n, row_stride, scale, st)
+  const int64_t slices = (int64_t)n * (g.d / cw);
+  if (g.hd == 8 && cw == 64) {
+    // 16 us with 64 rows per CTA, 10 with 32, 8 with 16 for one sample of (50, 500, 500); from three CTAs per SM on 64 is best
+    const int64_t ctas = tiles(64) * slices;
+    if (2 * ctas <= 3LL * n_sm) GSIT_LAUNCH(8, 64, 1, 64, 3);
+    if (ctas <= 3LL * n_sm) GSIT_LAUNCH(8, 64, 2, 64, 2);
+    GSIT_LAUNCH(8, 64, 4, 64, 2);
+  }
+  if (g.hd == 8 && cw == 32) {
+    if (tiles(64) * slices <= n_sm) GSIT_LAUNCH(8, 32, 1, 64, 3);
+    GSIT_LAUNCH(8, 32, 2, 64, 2);
+  }
+  if (g.hd == 8) GSIT_LAUNCH(8, 16, 1, 64, 2);
+  if (g.hd == 16 && cw == 64) {
+    // one sample of (50, 500, 500): 8 us with 16 rows per warp, 11 with 32; 8 samples: 18 and 17
+    if (2 * tiles(128) * ((g.heads + 1) / 2) * n <= 3LL * n_sm) GSIT_LAUNCH(16, 64, 1, 64, 2);
+    GSIT_LAUNCH(16, 64, 2, 64, 2);
+  }
+  if (g.hd == 16 && cw == 32) GSIT_LAUNCH(16, 32, 1, 64, 2);
+  if (g.hd == 16) GSIT_LAUNCH(16, 16, 1, 64, 2);
+  if (g.hd == 32 && cw == 64) GSIT_LAUNCH(32, 64, 1, 32, 2);
+  if (g.hd == 32) GSIT_LAUNCH(32, 32, 1, 32, 2);
+  if (g.hd == 64) GSIT_LAUNCH(64, 64, 1, 32, 2);
+#undef GSIT_LAUNCH
   return cudaErrorNotSupported;
 }
 

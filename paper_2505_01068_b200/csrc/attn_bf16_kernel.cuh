@@ -17,11 +17,6 @@ struct AttnProblem {
   int seg_order;
 };
 
-#ifndef GSIT_MS_POLY
-#define GSIT_MS_POLY 0
-#endif
-constexpr unsigned MS_POLY = GSIT_MS_POLY;  // bit i: score n-tile i of a step takes the polynomial 2^x
-
 template <typename C>
 __global__ void __launch_bounds__(NTHREADS, C::MINB)
 attn_bf16_kernel(const __grid_constant__ AttnProblem prob0, const __grid_constant__ AttnProblem prob1, const Geometry g0,
@@ -91,9 +86,9 @@ attn_bf16_kernel(const __grid_constant__ AttnProblem prob0, const __grid_constan
     krem = kn - t * KT;
     yrow = ((r == 0) ? kbase0 : (r == 1) ? kbase1 : kbase2) + t * KT;
   };
-  auto issue = [&](int i) {  // one thread: TMA loads of key tile i into its stage
+  auto issue = [&](int i) {  // one thread: TMA loads of key tile i (of tile i - T in a second walk) into its stage
     int krem, yrow;
-    locate(i, krem, yrow);
+    locate(i >= T ? i - T : i, krem, yrow);
     const int st = i % STAGES;
     mbar_expect_tx(bar_full + 8 * st, 2 * C::KV_BYTES);
     tma_load_2d(sK + st * C::KV_BYTES, &tmK, xcol, yrow, bar_full + 8 * st);
@@ -101,14 +96,18 @@ attn_bf16_kernel(const __grid_constant__ AttnProblem prob0, const __grid_constan
   };
 
   float O[R][NTO][4];
-  float m[R][2], l[R][4];  // l: accumulator tile of P 1 (elements 0 and 2 are the sums of rows g and g + 8)
+  float m[R][2], l[R][4];  // m: reference of rows g and g + 8, in base-2 score units; l: accumulator tile of P 1 (elements 0 and
+                           // 2 are the sums of those rows)
+  auto reset = [&]() {
 #pragma unroll
-  for (int r_ = 0; r_ < R; ++r_) {
-    m[r_][0] = m[r_][1] = -INFINITY;
-    l[r_][0] = l[r_][1] = l[r_][2] = l[r_][3] = 0.f;
+    for (int r_ = 0; r_ < R; ++r_) {
+      m[r_][0] = m[r_][1] = -INFINITY;
+      l[r_][0] = l[r_][1] = l[r_][2] = l[r_][3] = 0.f;
 #pragma unroll
-    for (int n = 0; n < NTO; ++n) O[r_][n][0] = O[r_][n][1] = O[r_][n][2] = O[r_][n][3] = 0.f;
-  }
+      for (int n = 0; n < NTO; ++n) O[r_][n][0] = O[r_][n][1] = O[r_][n][2] = O[r_][n][3] = 0.f;
+    }
+  };
+  reset();
 
   if (T > 0) {
     if (tid == 0) {
@@ -153,7 +152,15 @@ attn_bf16_kernel(const __grid_constant__ AttnProblem prob0, const __grid_constan
     // the instantiation then covers only the first NTV score n-tiles (8 keys each, NTV even: whole 16-key groups of
     // P V), so that a tile with few real keys costs proportionally less, and only its last two n-tiles are masked
     // element by element.  Everything stays straight-line code inside an instantiation.
-    auto process = [&](auto ragged_tag, auto ntv_tag, const uint32_t sKs, const uint32_t sVs, const int krem) {
+    //
+    // Reference of the exponentials.  A softmax does not depend on what is subtracted from the scores as long as nothing
+    // overflows, and float (and bf16 weights, which share its exponents) has room for 2^127: the reference of a row is the
+    // maximum of its FIRST key step and stays (SAFE = false).  The weight of that maximum is 1, so the row sum cannot
+    // underflow; a later score would have to exceed the reference by 2^90 to endanger it, and the end of the walk checks for
+    // that: then the CTA walks its keys again with the running maximum (SAFE = true).  The running maximum cost 60 of the
+    // 207 instructions per 16 x 64 scores and put its shuffles and the rescale between Q K^T and the exponentials.
+    auto process = [&](auto safe_tag, auto ragged_tag, auto ntv_tag, const uint32_t sKs, const uint32_t sVs, const int krem, const bool first_tile) {
+      constexpr bool SAFE = decltype(safe_tag)::value;
       constexpr bool RAGGED = decltype(ragged_tag)::value;
       constexpr int NTV = decltype(ntv_tag)::value;  // n-tiles computed (== NT for a full tile)
       static_assert(NTV % 2 == 0 && NTV >= 2 && NTV <= NT && (KT == KSTEP || !RAGGED || NTV == NT), "n-tile count");
@@ -252,55 +259,56 @@ attn_bf16_kernel(const __grid_constant__ AttnProblem prob0, const __grid_constan
               if (c0 + n * 8 + 1 >= krem) S[n][1] = S[n][3] = -INFINITY;
             }
           }
-          // ---- online softmax (base 2, scale folded into sl2); pairwise trees keep dependency chains short ----
-          float t0[NTV], t1[NTV];
+          // ---- reference of the row (base 2, scale folded into sl2); pairwise trees keep dependency chains short ----
+          float al0 = 1.f, al1 = 1.f;
+          if (SAFE || (first_tile && kb == 0)) {
+            float t0[NTV], t1[NTV];
 #pragma unroll
-          for (int n = 0; n < NTV; ++n) { t0[n] = fmaxf(S[n][0], S[n][1]); t1[n] = fmaxf(S[n][2], S[n][3]); }
+            for (int n = 0; n < NTV; ++n) { t0[n] = fmaxf(S[n][0], S[n][1]); t1[n] = fmaxf(S[n][2], S[n][3]); }
 #pragma unroll
-          for (int cnt = NTV; cnt > 1; cnt = (cnt + 1) / 2)  // pairwise tree over any count
+            for (int cnt = NTV; cnt > 1; cnt = (cnt + 1) / 2)  // pairwise tree over any count
 #pragma unroll
-            for (int n = 0; n < cnt / 2; ++n) {
-              t0[n] = fmaxf(t0[n], t0[n + (cnt + 1) / 2]);
-              t1[n] = fmaxf(t1[n], t1[n + (cnt + 1) / 2]);
+              for (int n = 0; n < cnt / 2; ++n) {
+                t0[n] = fmaxf(t0[n], t0[n + (cnt + 1) / 2]);
+                t1[n] = fmaxf(t1[n], t1[n + (cnt + 1) / 2]);
+              }
+            float mx0 = t0[0], mx1 = t1[0];
+            mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1));
+            mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
+            mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2)) * sl2;
+            mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2)) * sl2;
+            // every key tile that is walked holds at least one real key, so the new maximum is finite (only the old one can
+            // be -inf, on the first tile, where the factor below becomes exp2(-inf) = 0)
+            const float mn0 = fmaxf(m[r_][0], mx0), mn1 = fmaxf(m[r_][1], mx1);
+            if constexpr (SAFE) {
+              al0 = ex2(m[r_][0] - mn0);
+              al1 = ex2(m[r_][1] - mn1);
             }
-          float mx0 = t0[0], mx1 = t1[0];
-          mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1));
-          mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
-          mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
-          mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
-          const float mn0 = fmaxf(m[r_][0], mx0), mn1 = fmaxf(m[r_][1], mx1);
-          // every key tile that is walked holds at least one real key, so the new maximum is finite (only the old one can
-          // be -inf, on the first tile, where the factor below becomes exp2(-inf) = 0)
-          const float ms0 = mn0 * sl2, ms1 = mn1 * sl2;
-          const float al0 = ex2(fmaf(m[r_][0], sl2, -ms0)), al1 = ex2(fmaf(m[r_][1], sl2, -ms1));
-          m[r_][0] = mn0;
-          m[r_][1] = mn1;
-          // One packed FMA forms s * sl2 - m * sl2 for a pair of scores (both <= 0); each gets its own f32 ex2 (the
+            m[r_][0] = mn0;
+            m[r_][1] = mn1;
+          }
+          // One packed FMA forms s * sl2 - m * sl2 for a pair of scores; each gets its own f32 ex2 (the
           // packed bf16 form of ex2 issues two special-function operations as well, plus unpacking), and the pair is
           // rounded once into the bf16x2 layout of the A operand of P V.  The row sum is taken by the tensor core from
           // those same bf16 weights (a column of ones appended to V), so numerator and denominator of the softmax see
           // identical values.
-          const float2 sl2v = make_float2(sl2, sl2), nm0 = make_float2(-ms0, -ms0), nm1 = make_float2(-ms1, -ms1);
+          const float2 sl2v = make_float2(sl2, sl2), nm0 = make_float2(-m[r_][0], -m[r_][0]), nm1 = make_float2(-m[r_][1], -m[r_][1]);
           uint32_t P[NTV][2];
 #pragma unroll
           for (int n = 0; n < NTV; ++n) {
             const float2 x0 = __ffma2_rn(make_float2(S[n][0], S[n][1]), sl2v, nm0);
             const float2 x1 = __ffma2_rn(make_float2(S[n][2], S[n][3]), sl2v, nm1);
-            if ((MS_POLY >> (n & 7)) & 1) {
-              const float2 p0 = ptx::ex2_poly2(x0), p1 = ptx::ex2_poly2(x1);
-              P[n][0] = __byte_perm(__float_as_uint(p0.x), __float_as_uint(p0.y), 0x7632);
-              P[n][1] = __byte_perm(__float_as_uint(p1.x), __float_as_uint(p1.y), 0x7632);
-            } else {
-              P[n][0] = __byte_perm(__float_as_uint(ex2(x0.x)), __float_as_uint(ex2(x0.y)), 0x7632);
-              P[n][1] = __byte_perm(__float_as_uint(ex2(x1.x)), __float_as_uint(ex2(x1.y)), 0x7632);
-            }
+            P[n][0] = __byte_perm(__float_as_uint(ex2(x0.x)), __float_as_uint(ex2(x0.y)), 0x7632);
+            P[n][1] = __byte_perm(__float_as_uint(ex2(x1.x)), __float_as_uint(ex2(x1.y)), 0x7632);
           }
-          l[r_][0] *= al0;
-          l[r_][2] *= al1;
+          if constexpr (SAFE) {
+            l[r_][0] *= al0;
+            l[r_][2] *= al1;
 #pragma unroll
-          for (int n = 0; n < NTO; ++n) {
-            O[r_][n][0] *= al0; O[r_][n][1] *= al0;
-            O[r_][n][2] *= al1; O[r_][n][3] *= al1;
+            for (int n = 0; n < NTO; ++n) {
+              O[r_][n][0] *= al0; O[r_][n][1] *= al0;
+              O[r_][n][2] *= al1; O[r_][n][3] *= al1;
+            }
           }
           // ---- O += P V and l += P 1, the weights being the A operand ----
 #pragma unroll
@@ -323,36 +331,61 @@ attn_bf16_kernel(const __grid_constant__ AttnProblem prob0, const __grid_constan
       }    // steps
     };
 
-    for (int i = 0; i < T; ++i) {
-      const int st = i % STAGES;
-      if (tid == 0) {
-        // request further key tiles whose stage every warp has released; never block unless tile i itself is missing
-        while (next_issue < T) {
-          const uint32_t eb = bar_empty + 8 * (next_issue % STAGES);
-          const uint32_t par = ((next_issue / STAGES) - 1) & 1;
-          if (next_issue <= i) mbar_wait(g, eb, par);
-          else if (!mbar_test(eb, par)) break;
-          issue(next_issue);
-          ++next_issue;
+    auto walk = [&](auto safe_tag, const int from) {  // tiles from .. from + T - 1 of the stage sequence
+      const int end = from + T;
+      for (int i = from; i < end; ++i) {
+        const int st = i % STAGES;
+        if (tid == 0) {
+          // request further key tiles whose stage every warp has released; never block unless tile i itself is missing
+          while (next_issue < end) {
+            const uint32_t eb = bar_empty + 8 * (next_issue % STAGES);
+            const uint32_t par = ((next_issue / STAGES) - 1) & 1;
+            if (next_issue >= STAGES) {
+              if (next_issue <= i) mbar_wait(g, eb, par);
+              else if (!mbar_test(eb, par)) break;
+            }
+            issue(next_issue);
+            ++next_issue;
+          }
         }
+        __syncwarp();
+        mbar_wait(g, bar_full + 8 * st, (i / STAGES) & 1);
+        int krem, yrow;
+        locate(i - from, krem, yrow);
+        const bool first = i == from;
+        const uint32_t sKs = sK + st * C::KV_BYTES, sVs = sV + st * C::KV_BYTES;
+        if (krem >= KT) {
+          process(safe_tag, BoolTag<false>{}, IntTag<NT>{}, sKs, sVs, KT, first);
+        } else if constexpr (KT == KSTEP && NT == 8) {  // as many 16-key groups as hold real keys
+          if (krem <= 16) process(safe_tag, BoolTag<true>{}, IntTag<2>{}, sKs, sVs, krem, first);
+          else if (krem <= 32) process(safe_tag, BoolTag<true>{}, IntTag<4>{}, sKs, sVs, krem, first);
+          else if (krem <= 48) process(safe_tag, BoolTag<true>{}, IntTag<6>{}, sKs, sVs, krem, first);
+          else process(safe_tag, BoolTag<true>{}, IntTag<8>{}, sKs, sVs, krem, first);
+        } else {
+          process(safe_tag, BoolTag<true>{}, IntTag<NT>{}, sKs, sVs, krem, first);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_empty + 8 * st);  // this warp is done with the stage
       }
-      __syncwarp();
-      mbar_wait(g, bar_full + 8 * st, (i / STAGES) & 1);
-      int krem, yrow;
-      locate(i, krem, yrow);
-      const uint32_t sKs = sK + st * C::KV_BYTES, sVs = sV + st * C::KV_BYTES;
-      if (krem >= KT) {
-        process(BoolTag<false>{}, IntTag<NT>{}, sKs, sVs, KT);
-      } else if constexpr (KT == KSTEP && NT == 8) {  // as many 16-key groups as hold real keys
-        if (krem <= 16) process(BoolTag<true>{}, IntTag<2>{}, sKs, sVs, krem);
-        else if (krem <= 32) process(BoolTag<true>{}, IntTag<4>{}, sKs, sVs, krem);
-        else if (krem <= 48) process(BoolTag<true>{}, IntTag<6>{}, sKs, sVs, krem);
-        else process(BoolTag<true>{}, IntTag<8>{}, sKs, sVs, krem);
-      } else {
-        process(BoolTag<true>{}, IntTag<NT>{}, sKs, sVs, krem);
+    };
+    walk(BoolTag<false>{}, 0);
+    bool fits = true;  // did every row stay in range of its reference?
+#pragma unroll
+    for (int r_ = 0; r_ < R; ++r_) {
+      if ((sg * R + r_) * 16 >= q_real) continue;
+      const int row = (sg * R + r_) * 16 + (lane >> 2);
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        if (row + 8 * half >= q_real) continue;  // rows past the last real one hold anything
+        float top = 0.f;
+#pragma unroll
+        for (int n = 0; n < NTO; ++n) top = fmaxf(top, fmaxf(fabsf(O[r_][n][2 * half]), fabsf(O[r_][n][2 * half + 1])));
+        fits = fits && top < 1.2e27f && l[r_][2 * half] < 1.2e27f;  // 2^90; a NaN sum does not fit either
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar_empty + 8 * st);  // this warp is done with the stage
+    }
+    if (!__syncthreads_and(fits)) {
+      reset();
+      walk(BoolTag<true>{}, T);
     }
 
     // ---- normalise and stage the tile in shared memory.  A warp overwrites only the Q bytes it alone read. ----
@@ -375,8 +408,8 @@ attn_bf16_kernel(const __grid_constant__ AttnProblem prob0, const __grid_constan
         const int head = cs * G + head_in_slice;
         float* lp = lse + ((int64_t)b * g.heads + head) * g.L + g.seg_off[s] + q0;
         const float ln2 = 0.6931471805599453f;
-        if (rowA < q_real) lp[rowA] = l0 > 0.f ? (m[r_][0] * sl2 + log2f(l0)) * ln2 : -INFINITY;
-        if (rowB < q_real) lp[rowB] = l1 > 0.f ? (m[r_][1] * sl2 + log2f(l1)) * ln2 : -INFINITY;
+        if (rowA < q_real) lp[rowA] = l0 > 0.f ? (m[r_][0] + log2f(l0)) * ln2 : -INFINITY;
+        if (rowB < q_real) lp[rowB] = l1 > 0.f ? (m[r_][1] + log2f(l1)) * ln2 : -INFINITY;
       }
     }
     __syncthreads();

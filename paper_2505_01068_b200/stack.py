@@ -31,7 +31,8 @@ class GsitStack:
         The other options belong to forwards whose rings are not paired (paired_rings=False, rings of unequal depth) or to
         batch_chunks > 1.  concurrent_rings: issue independent work on several streams (False: every launch on the caller's
         stream).  batch_chunks: the batch is cut into this many groups of samples, each with its own pair of streams;
-        samples never interact, so the result does not depend on it.  intra_halves: the intra encoder runs on the two
+        samples never interact, so it changes the result by rounding at most
+        (where a group's size selects another attention kernel).  intra_halves: the intra encoder runs on the two
         halves of the batch on the two streams."""
         self.head = head
         self.concurrent_rings = concurrent_rings

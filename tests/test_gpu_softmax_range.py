@@ -1,0 +1,50 @@
+"""Scores that outgrow the reference a row took from its first key tile: every bf16 kernel must then fall back to a new reference."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads as wk
+from gpu_util import to_dev, to_np64
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def g():
+    import paper_2505_01068_b200 as lib
+    lib.load()
+    return lib
+
+
+@pytest.mark.parametrize("choice", ["ATTN_DEFAULT", "ATTN_TMEM", "ATTN_LEGACY"])
+@pytest.mark.parametrize("H,hd", [(8, 8), (4, 8), (2, 8), (4, 16), (2, 32), (2, 64)])
+@pytest.mark.parametrize("size", [1.0, 30.0, 400.0])
+def test_growing_scores(g, choice, H, hd, size):
+    """Keys grow along the sequence (in one head only in some samples), so the maximum moves far past the first tile's; the last
+    size leaves differences of thousands between neighbouring scores."""
+    rng = np.random.default_rng(hd + H)
+    seg, B = (40, 330, 200), 3
+    q, k, v = wk.draw_qkv(rng, B, sum(seg), H, hd, "bf16")
+    ramp = np.ones((B, sum(seg), H, 1), np.float32)
+    ramp[0] *= (np.arange(sum(seg)) / sum(seg) * size)[:, None, None]
+    ramp[1, 250:260, H - 1] = size
+    ramp[2, 333:, 0] = size
+    k = wk.storage_round(k * ramp, "bf16")
+    valid = np.array([[40, 330, 200], [17, 301, 129], [40, 320, 65]], dtype=np.int32)
+    vl = torch.from_numpy(valid).cuda()
+    dev = [to_dev(t, "bf16") for t in (q, k, v)]
+    g.tune_attention(getattr(g, choice))
+    try:
+        for phase in (g.PHASE_INTER_FWD, g.PHASE_INTRA):
+            out, lse = g.im_attention_fwd(*dev, seg, vl, phase, want_lse=True)
+            ref, ref_lse = oracle.im_attention_dense(q, k, v, seg, valid, phase, want_lse=True)
+            err = np.abs(to_np64(out) - ref)
+            assert err.max() <= 4e-2 and err.mean() <= 2e-3, (phase, err.max(), err.mean())  # one weight of 1 leaves V whole: |V| reaches 4
+            fin = np.isfinite(ref_lse)
+            a = to_np64(lse)
+            assert np.array_equal(np.isfinite(a), fin)
+            assert (np.abs(a[fin] - ref_lse[fin]) <= 1.2e-2 + 1e-5 * np.abs(ref_lse[fin])).all()
+    finally:
+        g.tune_attention(g.ATTN_DEFAULT)
+    assert g.last_device_status() == (0, 0)
