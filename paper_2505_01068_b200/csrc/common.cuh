@@ -202,6 +202,12 @@ struct FusedHalfArgs {
 cudaError_t launch_ln_qkv_tc_pair(const Geometry& g, const FusedHalfArgs (&h)[2], float eps, int* zero_word, cudaStream_t st);
 cudaError_t launch_proj_mlp_tc_pair(const Geometry& g, const FusedHalfArgs (&h)[2], float eps, int d_ff, cudaStream_t st);
 
+// Both halves on small row tiles and mma.sync (d_model 32, 64, 128; fused_rows.cu), for one or two problems of one geometry.
+bool fused_rows_supported(const Geometry& g, int d_ff);
+bool fused_rows_preferred(const Geometry& g);
+cudaError_t launch_ln_qkv_rows(const Geometry& g, const FusedHalfArgs* h, int n, float eps, int* zero_word, cudaStream_t st);
+cudaError_t launch_proj_mlp_rows(const Geometry& g, const FusedHalfArgs* h, int n, float eps, int d_ff, cudaStream_t st);
+
 // ... and at d_model 128 (d_ff <= 512), with the MLP weights streamed in chunks (fused_layer_tc128.cu)
 bool fused_layer_tc128_supported(const Geometry& g, int d_ff);
 cudaError_t launch_ln_qkv_tc128(const Geometry& g, const float* x, int64_t ldx, const float* gamma, const float* beta, float eps,

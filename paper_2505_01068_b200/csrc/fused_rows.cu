@@ -1,0 +1,382 @@
+// The two fused halves of a bf16 layer on small row tiles and mma.sync, for d_model 32, 64 and 128:
+//   ln_qkv_rows     qkv = LN1(x) W_qkv^T + b_qkv
+//   proj_mlp_rows   y1 = x + att W_o^T + b_o;  y = y1 + relu(LN2(y1) W_1^T + b_1) W_2^T + b_2
+//
+// A CTA of eight warps takes 16 R rows through the whole half.  What bounds the halves at these widths is not arithmetic but
+// latency: the chain load - LayerNorm - product - product - product - store of a tile, and how many tiles are in flight to
+// cover it.  So tiles are small and many, nothing is handed from role to role, and the weights take the shortest way there
+// is: each lane loads its B fragments straight from global memory as 16-byte pieces (all CTAs read the same few tens of
+// kilobytes: they stay in L1), no shared-memory staging, no barrier per weight chunk.  For that the k index of a product is
+// permuted, the same way in both operands: lane t of a quad holds k = 32 i + 8 t .. + 7 of its rows, which serve two
+// m16n8k16 steps.  The A operand lies in shared memory as bf16 rows in 16-byte pieces, swizzled so that the fragment reads
+// (16 bytes per lane) and the writes from accumulators (4 bytes per lane) are both free of bank conflicts.
+// Row statistics of LN2 are merged over the warps with the pairwise update of Chan, Golub and LeVeque.
+// A row's result does not depend on R, on the tile it falls into or on the layout.
+#include "common.cuh"
+#include "ptx.cuh"
+
+namespace gsit {
+namespace {
+
+constexpr int THREADS = 256, WARPS = 8, ROWS_MAX_FF = 512;
+
+__device__ __forceinline__ void mma(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// Byte offset of 16-byte piece c of row r in a tile of K bf16 columns.
+template <int K>
+__device__ __forceinline__ uint32_t piece(int r, int c) {
+  if constexpr (K == 32) return (uint32_t)(r * 64 + ((c ^ ((r >> 1) & 3)) << 4));
+  else return (uint32_t)(r * (K * 2) + ((c ^ (((r & 1) << 2) | ((r >> 1) & 3))) << 4));
+}
+__device__ __forceinline__ uint4 lds16(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts4(uint32_t a, uint32_t v) { asm volatile("st.shared.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+__device__ __forceinline__ void sts8(uint32_t a, uint32_t v, uint32_t w) { asm volatile("st.shared.v2.b32 [%0], {%1,%2};" ::"r"(a), "r"(v), "r"(w) : "memory"); }
+
+// Two k-steps (32 k's): rows of the slab at `lo` (row g) and `hi` (row g + 8), weights w of one n-tile.
+__device__ __forceinline__ void step(float (&c)[4], const uint4& lo, const uint4& hi, const uint4& w) {
+  mma(c, lo.x, hi.x, lo.y, hi.y, w.x, w.y);
+  mma(c, lo.z, hi.z, lo.w, hi.w, w.z, w.w);
+}
+__device__ __forceinline__ uint4 ldw(const __nv_bfloat16* p) { return __ldg(reinterpret_cast<const uint4*>(p)); }
+
+// Rows of this CTA: m0 .. m0 + 16 R - 1, those at or past `end` are not its own.
+struct Rows { int m0, end; };
+template <int BM>
+__device__ __forceinline__ Rows rows_of(const Geometry& g) {
+  const int lo = rows_begin(g);
+  return Rows{lo + (int)blockIdx.x * BM, rows_end(g)};
+}
+__device__ __forceinline__ bool is_real(const Geometry& g, int m, int end) {
+  if (m >= end) return false;
+  if (g.row_start != nullptr) return true;  // packed layout: every row is
+  const int b = m / g.L, p = m - b * g.L, s = segment_of(g, p);
+  return p - g.seg_off[s] < valid_rows(g, b, s);
+}
+
+struct Pair { FusedHalfArgs a[2]; };
+
+// ------------------------------------------------------------------------------------------------ LN1 + QKV
+template <int D, int R>
+__global__ void __launch_bounds__(THREADS)
+ln_qkv_rows_kernel(const Geometry g, const __grid_constant__ Pair pair, const float eps, int* __restrict__ zero_word) {
+  constexpr int BM = 16 * R, V = D / 32;            // rows of a tile; float4s per thread of a row (eight threads)
+  constexpr int GROUPS = 3 * D / 16, UNITS = GROUPS * R;
+  __shared__ __align__(128) uint8_t sH[BM * D * 2];
+  const FusedHalfArgs& a = pair.a[blockIdx.y];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gr = lane >> 2, t = lane & 3;
+  const uint32_t h = smem_u32(sH);
+  ptx::grid_dep_wait();
+  ptx::grid_dep_launch();
+  if (zero_word != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *zero_word = 0;
+  const Rows rows = rows_of<BM>(g);
+  if (rows.m0 >= rows.end) return;
+  // LayerNorm, eight threads per row, 32 rows at a time
+  bool any = false;
+#pragma unroll
+  for (int pass = 0; pass < (BM + 31) / 32; ++pass) {
+    const int r = pass * 32 + (tid >> 3), m = rows.m0 + r;
+    const bool real = r < BM && is_real(g, m, rows.end);
+    any |= real;
+    float4 v[V];
+    float s = 0.f;
+#pragma unroll
+    for (int c = 0; c < V; ++c) v[c] = real ? *reinterpret_cast<const float4*>(a.x + (int64_t)m * a.ldx + 4 * ((tid & 7) + 8 * c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int c = 0; c < V; ++c) s += (v[c].x + v[c].y) + (v[c].z + v[c].w);
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const float mean = s * (1.f / D);
+    float q = 0.f;
+#pragma unroll
+    for (int c = 0; c < V; ++c) {
+      v[c].x -= mean; v[c].y -= mean; v[c].z -= mean; v[c].w -= mean;
+      q += fmaf(v[c].x, v[c].x, v[c].y * v[c].y) + fmaf(v[c].z, v[c].z, v[c].w * v[c].w);
+    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    const float rstd = rsqrtf(q * (1.f / D) + eps);
+    if (r < BM) {
+#pragma unroll
+      for (int c = 0; c < V; ++c) {
+        const int e = 4 * ((tid & 7) + 8 * c);
+        const float4 ga = a.ln1_gamma != nullptr ? make_float4(a.ln1_gamma[e], a.ln1_gamma[e + 1], a.ln1_gamma[e + 2], a.ln1_gamma[e + 3]) : make_float4(1.f, 1.f, 1.f, 1.f);
+        const float4 be = a.ln1_beta != nullptr ? make_float4(a.ln1_beta[e], a.ln1_beta[e + 1], a.ln1_beta[e + 2], a.ln1_beta[e + 3]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const uint32_t lo = ptx::pack_bf16(fmaf(v[c].x * rstd, ga.x, be.x), fmaf(v[c].y * rstd, ga.y, be.y));
+        const uint32_t hi = ptx::pack_bf16(fmaf(v[c].z * rstd, ga.z, be.z), fmaf(v[c].w * rstd, ga.w, be.w));
+        sts8(h + piece<D>(r, e >> 3) + (e & 4) * 2, real ? lo : 0u, real ? hi : 0u);
+      }
+    }
+  }
+  const bool work = __syncthreads_or(any) != 0;
+  // units of 16 columns x one slab of 16 rows.  The two n-tiles of a unit take their columns interleaved, so that a lane ends up
+  // with four consecutive ones: 8-byte stores, 32-byte sectors written whole.
+#pragma unroll
+  for (int u = warp; u < UNITS; u += WARPS) {
+    const int grp = u % GROUPS, slab = u / GROUPS, n0 = grp * 16;
+    float c[2][4] = {};
+    if (work) {
+      uint4 w[2][D / 32];
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int k = 0; k < D / 32; ++k) w[j][k] = ldw(a.w_qkv + (int64_t)(n0 + 4 * (gr >> 1) + (gr & 1) + 2 * j) * D + 32 * k + 8 * t);
+#pragma unroll
+      for (int k = 0; k < D / 32; ++k) {
+        const uint4 lo = lds16(h + piece<D>(slab * 16 + gr, 4 * k + t)), hi = lds16(h + piece<D>(slab * 16 + gr + 8, 4 * k + t));
+        step(c[0], lo, hi, w[0][k]);
+        step(c[1], lo, hi, w[1][k]);
+      }
+    }
+    float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (a.b_qkv != nullptr) {
+      const float* p = a.b_qkv + n0 + 4 * t;
+      b = make_float4(p[0], p[1], p[2], p[3]);
+    }
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      const int m = rows.m0 + slab * 16 + gr + 8 * half;
+      if (m >= rows.end) continue;
+      const bool real = work && is_real(g, m, rows.end);
+      const uint32_t lo = ptx::pack_bf16(c[0][2 * half] + b.x, c[0][2 * half + 1] + b.y), hi = ptx::pack_bf16(c[1][2 * half] + b.z, c[1][2 * half + 1] + b.w);
+      *reinterpret_cast<uint2*>(a.qkv + (int64_t)m * (3 * D) + n0 + 4 * t) = real ? make_uint2(lo, hi) : make_uint2(0u, 0u);
+    }
+  }
+}
+
+// ------------------------------------------------------------------------------------------------ out-projection + LN2 + MLP
+template <int D, int R>
+__global__ void __launch_bounds__(THREADS, R <= 2 && D <= 64 ? 2 : 1)
+proj_mlp_rows_kernel(const Geometry g, const __grid_constant__ Pair pair, const float eps, const int d_ff) {
+  constexpr int BM = 16 * R, KD = D / 32;
+  constexpr int WN = D / 8 < WARPS ? D / 8 : WARPS, WM = WARPS / WN;   // warps along the D output columns, along the slabs
+  constexpr int NT = D / 8 / WN, SW = R / WM;                          // n-tiles and slabs of a warp in the D-wide products
+  static_assert(R % WM == 0, "slabs");
+  extern __shared__ __align__(128) uint8_t sm[];
+  __shared__ float2 stat[BM][WN];
+  const FusedHalfArgs& a = pair.a[blockIdx.y];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gr = lane >> 2, t = lane & 3;
+  const int wn = warp % WN, wm = warp / WN;
+  const uint32_t sH = smem_u32(sm), sF = sH + BM * D * 2;
+  const int fpitch = d_ff * 2;
+  auto fpiece = [&](int r, int c) { return sF + (uint32_t)(r * fpitch + ((c ^ (((r & 1) << 2) | ((r >> 1) & 3))) << 4)); };
+  uint4 wo[NT][KD];
+#pragma unroll
+  for (int j = 0; j < NT; ++j)
+#pragma unroll
+    for (int k = 0; k < KD; ++k) wo[j][k] = ldw(a.w_o + (int64_t)((wn * NT + j) * 8 + gr) * D + 32 * k + 8 * t);
+  ptx::grid_dep_wait();
+  ptx::grid_dep_launch();
+  const Rows rows = rows_of<BM>(g);
+  if (rows.m0 >= rows.end) return;
+  bool real[SW][2];
+  bool any = false;
+#pragma unroll
+  for (int s = 0; s < SW; ++s)
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      real[s][half] = is_real(g, rows.m0 + (wm * SW + s) * 16 + gr + 8 * half, rows.end);
+      any |= real[s][half];
+    }
+  if (g.row_start == nullptr && !__syncthreads_or(any)) {  // padding only
+    for (int i = tid; i < BM * (D / 4); i += THREADS) {
+      const int m = rows.m0 + i / (D / 4);
+      if (m < rows.end) *reinterpret_cast<float4*>(a.y + (int64_t)m * a.ldy + 4 * (i % (D / 4))) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    return;
+  }
+
+  // ---- y1 = x + att W_o^T + b_o, in registers; the attention rows are fragments as they lie in memory ----
+  float y1[SW][NT][4];
+  const uint4 zero = make_uint4(0, 0, 0, 0);
+#pragma unroll
+  for (int s = 0; s < SW; ++s) {
+    const int64_t m = rows.m0 + (wm * SW + s) * 16 + gr;
+    uint4 lo[KD], hi[KD];
+    float2 x[NT][2];
+#pragma unroll
+    for (int k = 0; k < KD; ++k) {
+      lo[k] = real[s][0] ? *reinterpret_cast<const uint4*>(a.att + m * D + 32 * k + 8 * t) : zero;
+      hi[k] = real[s][1] ? *reinterpret_cast<const uint4*>(a.att + (m + 8) * D + 32 * k + 8 * t) : zero;
+    }
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+      for (int half = 0; half < 2; ++half)
+        x[j][half] = real[s][half] ? *reinterpret_cast<const float2*>(a.x + (m + 8 * half) * a.ldx + (wn * NT + j) * 8 + 2 * t) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < NT; ++j) {
+      float c[4] = {};
+#pragma unroll
+      for (int k = 0; k < KD; ++k) step(c, lo[k], hi[k], wo[j][k]);
+      const int n = (wn * NT + j) * 8 + 2 * t;
+      const float b0 = a.b_o != nullptr ? a.b_o[n] : 0.f, b1 = a.b_o != nullptr ? a.b_o[n + 1] : 0.f;
+      y1[s][j][0] = c[0] + b0 + x[j][0].x; y1[s][j][1] = c[1] + b1 + x[j][0].y;
+      y1[s][j][2] = c[2] + b0 + x[j][1].x; y1[s][j][3] = c[3] + b1 + x[j][1].y;
+    }
+    // statistics of this warp's 8 NT columns of the two rows
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      float sum = 0.f, q = 0.f;
+#pragma unroll
+      for (int j = 0; j < NT; ++j) sum += y1[s][j][2 * half] + y1[s][j][2 * half + 1];
+      sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+      sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+      const float mean = sum * (1.f / (8 * NT));
+#pragma unroll
+      for (int j = 0; j < NT; ++j) {
+        const float d0 = y1[s][j][2 * half] - mean, d1 = y1[s][j][2 * half + 1] - mean;
+        q += fmaf(d0, d0, d1 * d1);
+      }
+      q += __shfl_xor_sync(0xffffffffu, q, 1);
+      q += __shfl_xor_sync(0xffffffffu, q, 2);
+      if (t == 0) stat[(wm * SW + s) * 16 + gr + 8 * half][wn] = make_float2(mean, q);
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int s = 0; s < SW; ++s)
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      const int r = (wm * SW + s) * 16 + gr + 8 * half;
+      float mean = 0.f, q = 0.f;
+#pragma unroll
+      for (int i = 0; i < WN; ++i) { mean += stat[r][i].x; q += stat[r][i].y; }
+      mean *= 1.f / WN;
+      float dev = 0.f;
+#pragma unroll
+      for (int i = 0; i < WN; ++i) { const float d = stat[r][i].x - mean; dev = fmaf(d, d, dev); }
+      const float rstd = rsqrtf(fmaf(dev, 8.f * NT, q) * (1.f / D) + eps);
+#pragma unroll
+      for (int j = 0; j < NT; ++j) {
+        const int n = (wn * NT + j) * 8 + 2 * t;
+        const float g0 = a.ln2_gamma != nullptr ? a.ln2_gamma[n] : 1.f, g1 = a.ln2_gamma != nullptr ? a.ln2_gamma[n + 1] : 1.f;
+        const float e0 = a.ln2_beta != nullptr ? a.ln2_beta[n] : 0.f, e1 = a.ln2_beta != nullptr ? a.ln2_beta[n + 1] : 0.f;
+        const uint32_t v = ptx::pack_bf16(fmaf((y1[s][j][2 * half] - mean) * rstd, g0, e0), fmaf((y1[s][j][2 * half + 1] - mean) * rstd, g1, e1));
+        sts4(sH + piece<D>(r, wn * NT + j) + 4 * t, real[s][half] ? v : 0u);
+      }
+    }
+  __syncthreads();
+
+  // ---- hidden units: every warp takes its n-tiles for all slabs, with the rows' fragments in registers ----
+  {
+    uint4 lo[R][KD], hi[R][KD];
+#pragma unroll
+    for (int s = 0; s < R; ++s)
+#pragma unroll
+      for (int k = 0; k < KD; ++k) {
+        lo[s][k] = lds16(sH + piece<D>(s * 16 + gr, 4 * k + t));
+        hi[s][k] = lds16(sH + piece<D>(s * 16 + gr + 8, 4 * k + t));
+      }
+    const int tiles = d_ff / 8;
+    uint4 w[KD];
+#pragma unroll
+    for (int k = 0; k < KD; ++k) w[k] = ldw(a.w_1 + (int64_t)(warp * 8 + gr) * D + 32 * k + 8 * t);
+#pragma unroll 2
+    for (int nt = warp; nt < tiles; nt += WARPS) {
+      uint4 next[KD];
+      const int ahead = nt + WARPS < tiles ? nt + WARPS : nt;
+#pragma unroll
+      for (int k = 0; k < KD; ++k) next[k] = ldw(a.w_1 + (int64_t)(ahead * 8 + gr) * D + 32 * k + 8 * t);
+      const int n = nt * 8 + 2 * t;
+      const float b0 = a.b_1 != nullptr ? a.b_1[n] : 0.f, b1 = a.b_1 != nullptr ? a.b_1[n + 1] : 0.f;
+#pragma unroll
+      for (int s = 0; s < R; ++s) {
+        float c[4] = {b0, b1, b0, b1};
+#pragma unroll
+        for (int k = 0; k < KD; ++k) step(c, lo[s][k], hi[s][k], w[k]);
+        sts4(fpiece(s * 16 + gr, nt) + 4 * t, ptx::pack_bf16_relu(c[0], c[1]));
+        sts4(fpiece(s * 16 + gr + 8, nt) + 4 * t, ptx::pack_bf16_relu(c[2], c[3]));
+      }
+#pragma unroll
+      for (int k = 0; k < KD; ++k) w[k] = next[k];
+    }
+  }
+  const __nv_bfloat16* w2[NT];
+#pragma unroll
+  for (int j = 0; j < NT; ++j) w2[j] = a.w_2 + (int64_t)((wn * NT + j) * 8 + gr) * d_ff + 8 * t;
+  __syncthreads();
+
+  // ---- y = y1 + f W_2^T + b_2 ----
+  float acc[SW][NT][4] = {};
+#pragma unroll 4
+  for (int k = 0; k < d_ff / 32; ++k) {
+    uint4 w[NT];
+#pragma unroll
+    for (int j = 0; j < NT; ++j) w[j] = ldw(w2[j] + 32 * k);
+#pragma unroll
+    for (int s = 0; s < SW; ++s) {
+      const int r = (wm * SW + s) * 16 + gr;
+      const uint4 lo = lds16(fpiece(r, 4 * k + t)), hi = lds16(fpiece(r + 8, 4 * k + t));
+#pragma unroll
+      for (int j = 0; j < NT; ++j) step(acc[s][j], lo, hi, w[j]);
+    }
+  }
+#pragma unroll
+  for (int s = 0; s < SW; ++s)
+#pragma unroll
+    for (int j = 0; j < NT; ++j) {
+      const int n = (wn * NT + j) * 8 + 2 * t;
+      const float b0 = a.b_2 != nullptr ? a.b_2[n] : 0.f, b1 = a.b_2 != nullptr ? a.b_2[n + 1] : 0.f;
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        const int64_t m = rows.m0 + (wm * SW + s) * 16 + gr + 8 * half;
+        if (m >= rows.end) continue;
+        const float v0 = y1[s][j][2 * half] + (acc[s][j][2 * half] + b0), v1 = y1[s][j][2 * half + 1] + (acc[s][j][2 * half + 1] + b1);
+        *reinterpret_cast<float2*>(a.y + m * a.ldy + n) = real[s][half] ? make_float2(v0, v1) : make_float2(0.f, 0.f);
+      }
+    }
+}
+
+template <int D, int R>
+cudaError_t launch_ln_qkv(const Geometry& g, const Pair& p, int n, float eps, int* zero_word, cudaStream_t st) {
+  const int64_t tiles = (matrix_rows(g) + 16 * R - 1) / (16 * R);
+  return launch_overlapped(ln_qkv_rows_kernel<D, R>, dim3((unsigned)tiles, n), dim3(THREADS), 0, st, g, p, eps, zero_word);
+}
+template <int D, int R>
+cudaError_t launch_proj_mlp(const Geometry& g, const Pair& p, int n, float eps, int d_ff, cudaStream_t st) {
+  constexpr int BM = 16 * R;
+  const int64_t tiles = (matrix_rows(g) + BM - 1) / BM;
+  cudaError_t e = sm_count_and_smem_once(reinterpret_cast<const void*>(proj_mlp_rows_kernel<D, R>), BM * (D + ROWS_MAX_FF) * 2, nullptr);
+  if (e != cudaSuccess) return e;
+  return launch_overlapped(proj_mlp_rows_kernel<D, R>, dim3((unsigned)tiles, n), dim3(THREADS), BM * (D + d_ff) * 2, st, g, p, eps, d_ff);
+}
+
+}  // namespace
+
+bool fused_rows_supported(const Geometry& g, int d_ff) {
+  return (g.d == 32 || g.d == 64 || g.d == 128) && d_ff % 64 == 0 && d_ff <= ROWS_MAX_FF;
+}
+// Where these kernels are the better ones: always at width 32 (which no tcgen05 half covers); at 64 and 128 as long as a launch is
+// about the latency of a tile.  One layer without open blocks: d 64 14.3 (tcgen05) -> 9.3 us at 1050 rows, 14.4 -> 10.6 at 2100,
+// 14.7 -> 13.0 at 4200, 16.3 -> 16.2 at 8400, 33 -> 70 at 67200; d 128 23.8 -> 14.7, 23.9 -> 17.6, 24.2 -> 21.9, 24.6 -> 30.
+bool fused_rows_preferred(const Geometry& g) { return g.d == 32 || (int64_t)g.batch * g.L <= 6400; }
+
+// n problems (1 or 2) of one geometry in one launch each.  Rows per tile: 16 for the shortest chain while there are few tiles,
+// more where the weight reads of many tiles (through L1) become what counts.
+cudaError_t launch_ln_qkv_rows(const Geometry& g, const FusedHalfArgs* h, int n, float eps, int* zero_word, cudaStream_t st) {
+  Pair p;
+  p.a[0] = h[0];
+  p.a[1] = h[n - 1];
+  const int64_t rows = (int64_t)g.batch * g.L * n;
+  if (g.d == 32) return rows > 48000 ? launch_ln_qkv<32, 4>(g, p, n, eps, zero_word, st) : launch_ln_qkv<32, 2>(g, p, n, eps, zero_word, st);
+  if (g.d == 64) return launch_ln_qkv<64, 1>(g, p, n, eps, zero_word, st);
+  return launch_ln_qkv<128, 1>(g, p, n, eps, zero_word, st);
+}
+cudaError_t launch_proj_mlp_rows(const Geometry& g, const FusedHalfArgs* h, int n, float eps, int d_ff, cudaStream_t st) {
+  Pair p;
+  p.a[0] = h[0];
+  p.a[1] = h[n - 1];
+  const int64_t rows = (int64_t)g.batch * g.L * n;
+  if (g.d == 32) return rows > 12000 ? launch_proj_mlp<32, 4>(g, p, n, eps, d_ff, st) : launch_proj_mlp<32, 2>(g, p, n, eps, d_ff, st);
+  if (g.d == 64) return rows > 5000 ? launch_proj_mlp<64, 2>(g, p, n, eps, d_ff, st) : launch_proj_mlp<64, 1>(g, p, n, eps, d_ff, st);
+  return rows > 1600 ? launch_proj_mlp<128, 2>(g, p, n, eps, d_ff, st) : launch_proj_mlp<128, 1>(g, p, n, eps, d_ff, st);
+}
+
+}  // namespace gsit

@@ -184,6 +184,25 @@ __global__ void expire_wait_kernel(unsigned int* status) {
   __syncthreads();
 }
 
+// Which kernels run the two halves of a bf16 layer around the attention.
+enum Halves { HALVES_NONE = 0, HALVES_ROWS, HALVES_TC, HALVES_TC128, HALVES_LEGACY };
+Halves pick_halves(const Geometry& g, int d_ff) {
+  const bool packed = g.row_start != nullptr;
+  if (!packed && g_attn_variant == GSIT_ATTN_UNFUSED) return HALVES_NONE;
+  if (!packed && g_attn_variant == GSIT_ATTN_LEGACY) return fused_layer_supported(g, d_ff) ? HALVES_LEGACY : HALVES_NONE;
+  if (fused_rows_supported(g, d_ff) && fused_rows_preferred(g)) return HALVES_ROWS;
+  if (fused_layer_tc_supported(g, d_ff)) return HALVES_TC;
+  if (fused_layer_tc128_supported(g, d_ff)) return HALVES_TC128;
+  if (!packed && fused_layer_supported(g, d_ff)) return HALVES_LEGACY;
+  return HALVES_NONE;
+}
+
+FusedHalfArgs half_args(const gsit_layer_weights* w, const float* x, int64_t ldx, __nv_bfloat16* qkv, __nv_bfloat16* att, float* y, int64_t ldy) {
+  auto b = [](const void* p) { return static_cast<const __nv_bfloat16*>(p); };
+  return FusedHalfArgs{x, ldx, w->ln1_gamma, w->ln1_beta, b(w->w_qkv), w->b_qkv, qkv, att, b(w->w_o), w->b_o, w->ln2_gamma, w->ln2_beta,
+                       b(w->w_1), w->b_1, b(w->w_2), w->b_2, y, ldy};
+}
+
 float pick_scale(const gsit_shape* s, const Geometry& g) {
   return (s->scale > 0.f) ? s->scale : 1.0f / sqrtf((float)g.hd);
 }
@@ -262,47 +281,30 @@ gsit_status gsit_im_layer_fwd(const gsit_shape* shape, const gsit_layer_weights*
   const int bf = (dtype == GSIT_BF16);
   const int es = bf ? 2 : 4;
   const int M = g.batch * g.L, d = g.d;
-  if (g.row_start != nullptr &&
-      !(bf && g.hd <= 32 && (fused_layer_tc_supported(g, w->d_ff) || fused_layer_tc128_supported(g, w->d_ff))))
-    return GSIT_ERR_UNSUPPORTED;  // the packed layout is implemented by the tcgen05 fused halves and the mma.sync attention
+  const Halves halves = bf ? pick_halves(g, w->d_ff) : HALVES_NONE;
+  if (g.row_start != nullptr && (halves == HALVES_NONE || g.hd > 32))
+    return GSIT_ERR_UNSUPPORTED;  // the packed layout is implemented by the fused halves and the mma.sync / tensor-memory attention
 
-  if (bf && fused_layer_supported(g, w->d_ff) && (g_attn_variant != GSIT_ATTN_UNFUSED || g.row_start != nullptr)) {
+  if (halves != HALVES_NONE) {
     // three launches: LN1 + shared projection, IM attention, out-projection + residual + LN2 + MLP + residual
-    // d_model 64 and 128 run both halves on tcgen05 (GSIT_ATTN_LEGACY keeps the mma.sync kernels)
-    const bool tc = fused_layer_tc_supported(g, w->d_ff) && (g_attn_variant != GSIT_ATTN_LEGACY || g.row_start != nullptr);
-    const bool tc128 = fused_layer_tc128_supported(g, w->d_ff) && (g_attn_variant != GSIT_ATTN_LEGACY || g.row_start != nullptr);
+    const FusedHalfArgs h = half_args(w, x, x_row_stride, static_cast<__nv_bfloat16*>(qkv), static_cast<__nv_bfloat16*>(att), y, y_row_stride);
+    int* counter = reinterpret_cast<int*>(ws + sc.sched);
     {
       TraceScope t(GSIT_KERNEL_LINEAR, cs);
-      st = from_cuda(tc ? launch_ln_qkv_tc(g, x, x_row_stride, w->ln1_gamma, w->ln1_beta, eps,
-                                           static_cast<const __nv_bfloat16*>(w->w_qkv), w->b_qkv,
-                                           static_cast<__nv_bfloat16*>(qkv), reinterpret_cast<int*>(ws + sc.sched), cs)
-                     : tc128 ? launch_ln_qkv_tc128(g, x, x_row_stride, w->ln1_gamma, w->ln1_beta, eps,
-                                                   static_cast<const __nv_bfloat16*>(w->w_qkv), w->b_qkv,
-                                                   static_cast<__nv_bfloat16*>(qkv), reinterpret_cast<int*>(ws + sc.sched), cs)
-                        : launch_ln_qkv_bf16(g, x, x_row_stride, w->ln1_gamma, w->ln1_beta, eps,
-                                             static_cast<const __nv_bfloat16*>(w->w_qkv), w->b_qkv,
-                                             static_cast<__nv_bfloat16*>(qkv), cs));
+      st = from_cuda(halves == HALVES_ROWS    ? launch_ln_qkv_rows(g, &h, 1, eps, counter, cs)
+                     : halves == HALVES_TC    ? launch_ln_qkv_tc(g, x, x_row_stride, h.ln1_gamma, h.ln1_beta, eps, h.w_qkv, h.b_qkv, h.qkv, counter, cs)
+                     : halves == HALVES_TC128 ? launch_ln_qkv_tc128(g, x, x_row_stride, h.ln1_gamma, h.ln1_beta, eps, h.w_qkv, h.b_qkv, h.qkv, counter, cs)
+                                              : launch_ln_qkv_bf16(g, x, x_row_stride, h.ln1_gamma, h.ln1_beta, eps, h.w_qkv, h.b_qkv, h.qkv, cs));
     }
     if (st != GSIT_OK) return st;
-    const uint8_t* qb = static_cast<const uint8_t*>(qkv);
-    // the tcgen05 first halves clear the attention kernel's work counter, so no memset separates the three kernels
-    if ((st = run_attention(g, dtype, qb, qb + (size_t)d * es, qb + (size_t)2 * d * es, 3 * (int64_t)d, att, nullptr,
-                            pick_scale(shape, g), ws + sc.sched, cs, tc || tc128)) != GSIT_OK) return st;
+    // the first halves clear the attention kernel's work counter (but the legacy one), so no memset separates the three kernels
+    if ((st = run_attention(g, dtype, h.qkv, h.qkv + d, h.qkv + 2 * d, 3 * (int64_t)d, att, nullptr, pick_scale(shape, g), counter, cs,
+                            halves != HALVES_LEGACY)) != GSIT_OK) return st;
     TraceScope t(GSIT_KERNEL_LINEAR, cs);
-    if (tc)
-      return from_cuda(launch_proj_mlp_tc(g, static_cast<const __nv_bfloat16*>(att), x, x_row_stride,
-                                          static_cast<const __nv_bfloat16*>(w->w_o), w->b_o, w->ln2_gamma, w->ln2_beta, eps,
-                                          static_cast<const __nv_bfloat16*>(w->w_1), w->b_1,
-                                          static_cast<const __nv_bfloat16*>(w->w_2), w->b_2, w->d_ff, y, y_row_stride, cs));
-    if (tc128)
-      return from_cuda(launch_proj_mlp_tc128(g, static_cast<const __nv_bfloat16*>(att), x, x_row_stride,
-                                             static_cast<const __nv_bfloat16*>(w->w_o), w->b_o, w->ln2_gamma, w->ln2_beta, eps,
-                                             static_cast<const __nv_bfloat16*>(w->w_1), w->b_1,
-                                             static_cast<const __nv_bfloat16*>(w->w_2), w->b_2, w->d_ff, y, y_row_stride, cs));
-    return from_cuda(launch_proj_mlp_bf16(g, static_cast<const __nv_bfloat16*>(att), x, x_row_stride,
-                                          static_cast<const __nv_bfloat16*>(w->w_o), w->b_o, w->ln2_gamma, w->ln2_beta, eps,
-                                          static_cast<const __nv_bfloat16*>(w->w_1), w->b_1,
-                                          static_cast<const __nv_bfloat16*>(w->w_2), w->b_2, w->d_ff, y, y_row_stride, cs));
+    if (halves == HALVES_ROWS) return from_cuda(launch_proj_mlp_rows(g, &h, 1, eps, w->d_ff, cs));
+    auto second = halves == HALVES_TC ? launch_proj_mlp_tc : halves == HALVES_TC128 ? launch_proj_mlp_tc128 : launch_proj_mlp_bf16;
+    return from_cuda(second(g, h.att, x, x_row_stride, h.w_o, h.b_o, h.ln2_gamma, h.ln2_beta, eps, h.w_1, h.b_1, h.w_2, h.b_2, w->d_ff, y,
+                            y_row_stride, cs));
   }
   if (!bf && fused_layer_f32_supported(g, w->d_ff)) {  // the same three launches for float operands
     auto f32 = [](const void* p) { return static_cast<const float*>(p); };
@@ -368,8 +370,8 @@ gsit_status gsit_im_layer_pair_fwd(const gsit_shape* shape_a, const gsit_shape* 
   if (!workspace || workspace_bytes < 2 * sc.total || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return GSIT_ERR_WORKSPACE;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   const float eps_a = (w_a->ln_eps > 0.f) ? w_a->ln_eps : 1e-5f, eps_b = (w_b->ln_eps > 0.f) ? w_b->ln_eps : 1e-5f;
-  const bool one_launch = shape_a->dtype == GSIT_BF16 && fused_layer_tc_supported(ga, w_a->d_ff) && eps_a == eps_b &&
-                          ga.hd <= 32 && g_attn_variant != GSIT_ATTN_UNFUSED && g_attn_variant != GSIT_ATTN_LEGACY;
+  const Halves halves = shape_a->dtype == GSIT_BF16 ? pick_halves(ga, w_a->d_ff) : HALVES_NONE;
+  const bool one_launch = (halves == HALVES_ROWS || halves == HALVES_TC) && eps_a == eps_b && ga.hd <= 32;
   if (!one_launch) {  // shapes the paired kernels do not cover: the two layers one after the other, same results
     st = gsit_im_layer_fwd(shape_a, w_a, x_a, x_a_row_stride, y_a, y_a_row_stride, ws, sc.total, stream);
     if (st != GSIT_OK) return st;
@@ -395,15 +397,14 @@ gsit_status gsit_im_layer_pair_fwd(const gsit_shape* shape_a, const gsit_shape* 
     uint8_t* wsi = ws + i * sc.total;
     __nv_bfloat16* qkv = reinterpret_cast<__nv_bfloat16*>(wsi + sc.qkv);
     __nv_bfloat16* att = reinterpret_cast<__nv_bfloat16*>(wsi + sc.att);
-    h[i] = FusedHalfArgs{x[i], ldx[i], w[i]->ln1_gamma, w[i]->ln1_beta, static_cast<const __nv_bfloat16*>(w[i]->w_qkv), w[i]->b_qkv,
-                         qkv, att, static_cast<const __nv_bfloat16*>(w[i]->w_o), w[i]->b_o, w[i]->ln2_gamma, w[i]->ln2_beta,
-                         static_cast<const __nv_bfloat16*>(w[i]->w_1), w[i]->b_1, static_cast<const __nv_bfloat16*>(w[i]->w_2),
-                         w[i]->b_2, y[i], ldy[i]};
+    h[i] = half_args(w[i], x[i], ldx[i], qkv, att, y[i], ldy[i]);
     ops[i] = AttnOperands{qkv, qkv + ga.d, qkv + 2 * ga.d, att, nullptr, allowed[i]};
   }
   {
     TraceScope t(GSIT_KERNEL_LINEAR, cs);
-    if ((st = from_cuda(launch_ln_qkv_tc_pair(ga, h, eps_a, reinterpret_cast<int*>(ws + sc.sched), cs))) != GSIT_OK) return st;
+    int* counter = reinterpret_cast<int*>(ws + sc.sched);
+    st = from_cuda(halves == HALVES_ROWS ? launch_ln_qkv_rows(ga, h, 2, eps_a, counter, cs) : launch_ln_qkv_tc_pair(ga, h, eps_a, counter, cs));
+    if (st != GSIT_OK) return st;
   }
   {
     TraceScope t(GSIT_KERNEL_ATTENTION, cs);
@@ -412,7 +413,7 @@ gsit_status gsit_im_layer_pair_fwd(const gsit_shape* shape_a, const gsit_shape* 
       return st;
   }
   TraceScope t(GSIT_KERNEL_LINEAR, cs);
-  return from_cuda(launch_proj_mlp_tc_pair(ga, h, eps_a, w_a->d_ff, cs));
+  return from_cuda(halves == HALVES_ROWS ? launch_proj_mlp_rows(ga, h, 2, eps_a, w_a->d_ff, cs) : launch_proj_mlp_tc_pair(ga, h, eps_a, w_a->d_ff, cs));
 }
 
 gsit_status gsit_plan_rows(const gsit_shape* shape, int32_t split_sample, int32_t* row_start, gsit_stream stream) {

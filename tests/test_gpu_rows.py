@@ -1,0 +1,63 @@
+"""The fused layer halves on small row tiles: every width, tiles of 16, 32 and 64 rows (chosen by the row count), row counts that end
+inside a tile, tiles of padding only, strided rows, the packed layout and the pair call."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads as wk
+from gpu_util import check_close, pad_mask, to_dev, to_np64, weights_to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def g():
+    import paper_2505_01068_b200 as lib
+    lib.load()
+    return lib
+
+
+@pytest.mark.parametrize("d,heads,d_ff,seg,B", [(32, 4, 128, (5, 11, 2), 1), (32, 2, 64, (50, 130, 77), 5), (32, 1, 512, (50, 300, 270), 25),
+                                                (32, 4, 128, (50, 300, 270), 80), (64, 8, 256, (3, 0, 4), 1), (64, 4, 192, (50, 130, 77), 3),
+                                                (64, 2, 512, (50, 300, 270), 9), (128, 8, 512, (7, 1, 1), 1), (128, 4, 320, (50, 130, 77), 6),
+                                                (128, 8, 512, (50, 300, 270), 2)])
+def test_layer_on_row_tiles(g, d, heads, d_ff, seg, B):
+    rng = np.random.default_rng(d + d_ff + B)
+    L = sum(seg)
+    x = rng.standard_normal((B, L, d), dtype=np.float32)
+    w = wk.draw_layer_weights(rng, d, d_ff, "bf16", affine=True)
+    wd = weights_to_dev(w, "bf16")
+    valid = np.stack([rng.integers(0, n + 1, size=B) for n in seg], axis=1).astype(np.int32)
+    valid[B // 2] = 0
+    pm = pad_mask(seg, valid, B)
+    vl = torch.from_numpy(valid).cuda()
+    wide = torch.full((B, L, 2 * d), float("nan"), device="cuda")
+    wide[:, :, d:] = to_dev(np.where(pm[:, :, None], np.nan, x).astype(np.float32))
+    out = torch.full((B, L, 2 * d), 7.0, device="cuda")
+    g.im_layer_fwd(wide[:, :, d:], wd, seg, heads, vl, g.PHASE_INTER_BWD, out=out[:, :, :d])
+    assert bool((out[:, :, d:] == 7.0).all())
+    y = out[:, :, :d]
+    assert bool((y[torch.from_numpy(pm).cuda()] == 0).all())
+    for b in {0, B - 1}:
+        ref = oracle.im_layer_fwd(x[b:b + 1], w, seg, heads, valid[b:b + 1], g.PHASE_INTER_BWD)
+        check_close(to_np64(y[b:b + 1]), ref, "bf16", pm[b:b + 1], f"sample {b}")
+    # packed rows: the same bits in every real row, nothing written past them
+    cap = B * L + 128
+    plan = g.plan_rows(vl, seg)
+    xp = torch.full((cap, d), float("nan"), device="cuda")
+    g.pack_rows(wide[:, :, d:].contiguous(), xp, seg, vl, plan)
+    yp = torch.full((cap, d), 7.0, device="cuda")
+    g.im_layer_fwd(xp, wd, seg, heads, vl, g.PHASE_INTER_BWD, out=yp, row_start=plan)
+    used = int(plan[-1])
+    assert bool((yp[used:] == 7.0).all())
+    back = torch.empty((B, L, d), device="cuda")
+    g.unpack_rows(yp, back, seg, vl, plan)
+    assert torch.equal(back, y.contiguous())
+    # the pair call gives the bits of two calls
+    w2 = weights_to_dev(wk.draw_layer_weights(rng, d, d_ff, "bf16", affine=True), "bf16")
+    xc = wide[:, :, d:].contiguous()
+    ya, yb = g.im_layer_pair_fwd(xc, xc, wd, w2, seg, heads, vl, g.PHASE_INTER_BWD, g.PHASE_INTER_FWD)
+    assert torch.equal(ya, y.contiguous())
+    assert torch.equal(yb, g.im_layer_fwd(xc, w2, seg, heads, vl, g.PHASE_INTER_FWD))
+    assert g.last_device_status() == (0, 0)
