@@ -198,9 +198,6 @@ ln_qkv_tc_kernel(const __grid_constant__ LnQkvArgs arg0, const __grid_constant__
 #pragma unroll
         for (int e = 0; e < TD; ++e) v[e] = 0.f;
       }
-      fence_reads_before_release();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bars + B_XFREE);
       if (i > 0) {  // the previous tile's stores must have finished reading the staging rows (the normalised rows overlay them)
         if (tid == 64) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         t_bar_rows();
@@ -208,7 +205,10 @@ ln_qkv_tc_kernel(const __grid_constant__ LnQkvArgs arg0, const __grid_constant__
       layernorm_row_to_tile(v, real, s_gamma, s_beta, eps, base + OFF_H, r);
       fence_async_smem();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bars + B_HREADY);
+      if (lane == 0) {
+        mbar_arrive(bars + B_HREADY);
+        mbar_arrive(bars + B_XFREE);  // the row has been used, not only loaded
+      }
       const bool real_next = row_real32(g, row_base + (t + ctas) * TM + r, rows);  // overlaps the MMA
 
       mbar_wait(wc, bars + B_ACCFULL, i & 1);  // the MMA has also finished reading the normalised rows
@@ -427,9 +427,6 @@ proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_consta
 #pragma unroll
         for (int e = 0; e < 32; ++e) v_[e] = 0.f;
       }
-      fence_reads_before_release();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bars + B_XFREE);
       mbar_wait(wc, bars + B_ACC1, i_ & 1);
       tc_fence_after();
       {
@@ -452,7 +449,10 @@ proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_consta
       fence_async_smem();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bars + B_HREADY);
+      if (lane == 0) {
+        mbar_arrive(bars + B_HREADY);
+        mbar_arrive(bars + B_XFREE);  // the row has been used, not only loaded
+      }
     };
     int i = 0;
     bool real = row_real32(g, row_base + cta * TM + r, rows);

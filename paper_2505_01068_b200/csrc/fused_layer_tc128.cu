@@ -142,9 +142,6 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
 #pragma unroll
         for (int e = 0; e < 64; ++e) v[e] = 0.f;
       }
-      fence_reads_before_release();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bars + B_XFREE);
       if (i > 0 && tid == 64) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
       // the barrier inside: the previous tile's stores have finished reading the staging rows the normalised rows overlay
       float mean, rstd;
@@ -152,7 +149,10 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
       normalise_to_tile<64>(v, mean, rstd, real, s_gamma, s_beta, 64 * hf, base + OFF_H + hf * XBOX, r, 0);
       fence_async_smem();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bars + B_HREADY);
+      if (lane == 0) {
+        mbar_arrive(bars + B_HREADY);
+        mbar_arrive(bars + B_XFREE);  // the row has been used, not only loaded
+      }
       const bool real_next = row_real32(g, row_base + (t + (int)gridDim.x) * TM + r, rows);  // overlaps the MMA
 
       mbar_wait(wc, bars + B_ACCFULL, i & 1);  // the MMA has also finished reading the normalised rows
@@ -429,9 +429,6 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
 #pragma unroll
         for (int e = 0; e < 64; ++e) v[e] = 0.f;
       }
-      fence_reads_before_release();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bars + B_XFREE);
       mbar_wait(wc, bars + B_ACC1, i & 1);
       tc_fence_after();
 #pragma unroll
@@ -456,7 +453,10 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
       fence_async_smem();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bars + B_HREADY);
+      if (lane == 0) {
+        mbar_arrive(bars + B_HREADY);
+        mbar_arrive(bars + B_XFREE);  // the row has been used, not only loaded
+      }
       const bool real_next = row_real32(g, row_base + (t + (int)gridDim.x) * TM + r, rows);
       // ---- hidden chunks: f = relu(h W_1c^T + b_1c) -> A operand of the second product (32 of the 64 units each) ----
 #pragma unroll 1

@@ -136,10 +136,12 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 
 // True in exactly one lane of a converged warp.  Whole warps run the producer / issuer loops so that addresses,
 // descriptors and barrier phases stay warp-uniform; only the asynchronous instruction itself is issued by one lane.
-// Between reading a shared-memory buffer into registers and releasing that buffer for an asynchronous refill.  The
-// loaded values need not be used before the release, and nothing else keeps the loads from being performed after it (the
-// release is one lane's mbarrier arrive behind a warp barrier); measured: without this fence the last 16-byte load of a
-// row was served from the refilled buffer in about 3 % of repeated full-batch runs of the pipelined out-projection + MLP.
+// Between reading a shared-memory buffer into registers and releasing that buffer for a refill, where the values are not
+// used before the release: nothing else keeps the loads from being performed after it (the release is one lane's mbarrier
+// arrive behind a warp barrier).  It is not enough for a buffer that the asynchronous proxy (a TMA load) refills at once:
+// the out-projection + MLP kernel, whose x rows used to be released this way, still took the last 16-byte load of a few
+// rows from the refilled buffer in about 1 of 12000 full-batch runs (3 % without the fence).  Such buffers are released
+// after the loaded values have been used in arithmetic.
 __device__ __forceinline__ void fence_reads_before_release() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
 
 // Programmatic dependent launch.  A kernel launched with the "programmatic stream serialization" attribute may start
