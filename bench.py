@@ -315,7 +315,7 @@ def run_gpu(args):
     paired = stack.paired_rings and n_f == n_b and n_f > 0   # one launch per kernel for both rings of a depth
     launches_per_step = 3 * (n_f if paired else n_f + n_b) + 3 * n_i * (1 if paired else 2)
     if stack.packed:
-        launches_per_step += 3   # row plan, gather of the real rows, scatter of the result
+        launches_per_step += 2   # row plan and gather of the real rows, scatter of the result
 
     for i in range(max(1, min(args.warmup, 2))):           # eager warm-up (module load, attributes, buffers)
         stack.forward(xbufs[i % nbuf], vl)

@@ -154,7 +154,7 @@ gsit_status gsit_im_layer_pair_fwd(const gsit_shape* shape_a, const gsit_shape* 
                                    int64_t x_b_row_stride, float* y_a, int64_t y_a_row_stride, float* y_b, int64_t y_b_row_stride,
                                    void* workspace, size_t workspace_bytes, gsit_stream stream);
 
-/* Packed row layout, the three helpers (Section "Inner Decomposition for Efficiency": padded positions take no part in
+/* Packed row layout, the helpers (Section "Inner Decomposition for Efficiency": padded positions take no part in
  * the computation; here they take no memory either).  All run on the device, asynchronously on `stream`, and need no
  * host knowledge of the lengths, so a captured sequence of calls stays valid when valid_len changes.
  *
@@ -165,11 +165,14 @@ gsit_status gsit_im_layer_pair_fwd(const gsit_shape* shape_a, const gsit_shape* 
  *   shape: batch, seg_len, valid_len (required) are read.  row_start: DEVICE int32 [3 B + 1].
  * gsit_pack_rows: x_packed[row_start[3 b + s] + i, :] = x[b, seg_off[s] + i, :] for i < valid_len[b][s].
  * gsit_unpack_rows: the inverse; padded positions of y are written as +0.
+ * gsit_plan_pack_rows: gsit_plan_rows without a split and gsit_pack_rows in one launch.
  *   x / y float [B, L, cols] with the given row strides (elements); the packed matrices are float [capacity, cols].
  * A capacity of B * L + 128 rows always suffices. */
 gsit_status gsit_plan_rows(const gsit_shape* shape, int32_t split_sample, int32_t* row_start, gsit_stream stream);
 gsit_status gsit_pack_rows(const gsit_shape* shape, const float* x, int64_t x_row_stride, float* x_packed,
                            int64_t packed_row_stride, int32_t cols, gsit_stream stream);
+gsit_status gsit_plan_pack_rows(const gsit_shape* shape, int32_t* row_start, const float* x, int64_t x_row_stride, float* x_packed,
+                                int64_t packed_row_stride, int32_t cols, gsit_stream stream);
 gsit_status gsit_unpack_rows(const gsit_shape* shape, const float* y_packed, int64_t packed_row_stride, float* y,
                              int64_t y_row_stride, int32_t cols, gsit_stream stream);
 

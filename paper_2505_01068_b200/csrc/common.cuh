@@ -227,6 +227,9 @@ cudaError_t launch_stack_head(const Geometry& g, int dtype, const float* c, int6
 
 // packed row layout (rows.cu)
 cudaError_t launch_plan_rows(const Geometry& g, int split_sample, int32_t* row_start, cudaStream_t st);
+bool plan_pack_supported(const Geometry& g);
+cudaError_t launch_plan_pack(const Geometry& g, int32_t* row_start, const float* src, int64_t src_stride, float* dst, int64_t dst_stride, int cols,
+                             cudaStream_t st);
 cudaError_t launch_move_rows(const Geometry& g, bool pack, const float* src, int64_t src_stride, float* dst, int64_t dst_stride,
                              int cols, cudaStream_t st);
 

@@ -448,6 +448,25 @@ gsit_status gsit_pack_rows(const gsit_shape* shape, const float* x, int64_t x_ro
   return move_rows(shape, true, x, x_row_stride, x_packed, packed_row_stride, cols, stream);
 }
 
+gsit_status gsit_plan_pack_rows(const gsit_shape* shape, int32_t* row_start, const float* x, int64_t x_row_stride, float* x_packed,
+                                int64_t packed_row_stride, int32_t cols, gsit_stream stream) {
+  if (shape == nullptr || row_start == nullptr || shape->valid_len == nullptr || !x || !x_packed) return GSIT_ERR_INVALID_ARG;
+  if (cols < 4 || cols % 4 != 0 || x_row_stride < cols || packed_row_stride < cols || x_row_stride % 4 != 0 || packed_row_stride % 4 != 0)
+    return GSIT_ERR_INVALID_ARG;
+  if (!aligned16(x) || !aligned16(x_packed)) return GSIT_ERR_INVALID_ARG;
+  gsit_shape sh = *shape;
+  sh.d_model = 16; sh.heads = 1; sh.phase = GSIT_PHASE_INTRA; sh.dtype = GSIT_F32; sh.row_start = nullptr; sh.packed_capacity = 0;
+  Geometry g;
+  gsit_status st = make_geometry(&sh, &g);
+  if (st != GSIT_OK) return st;
+  if (from_cuda(status_ptr(&g.status)) != GSIT_OK) return GSIT_ERR_CUDA;
+  cudaStream_t cs = static_cast<cudaStream_t>(stream);
+  if (plan_pack_supported(g)) return from_cuda(launch_plan_pack(g, row_start, x, x_row_stride, x_packed, packed_row_stride, cols, cs));
+  if ((st = from_cuda(launch_plan_rows(g, 0, row_start, cs))) != GSIT_OK) return st;
+  g.row_start = row_start;
+  return from_cuda(launch_move_rows(g, true, x, x_row_stride, x_packed, packed_row_stride, cols, cs));
+}
+
 gsit_status gsit_unpack_rows(const gsit_shape* shape, const float* y_packed, int64_t packed_row_stride, float* y,
                              int64_t y_row_stride, int32_t cols, gsit_stream stream) {
   return move_rows(shape, false, y_packed, packed_row_stride, y, y_row_stride, cols, stream);

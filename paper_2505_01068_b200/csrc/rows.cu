@@ -86,7 +86,72 @@ __global__ void __launch_bounds__(256) move_rows_kernel(const Geometry g, const 
     if (out[u] != nullptr) *out[u] = v[u];
 }
 
+// Plan and gather in one launch: every CTA scans the valid lengths itself (3 B integers, a microsecond) instead of waiting for a
+// kernel that does nothing else, and CTA 0 writes the plan down for the kernels that follow.
+constexpr int PLAN_MAX = 3072;  // entries (samples x segments) a CTA can hold
+__global__ void __launch_bounds__(256) plan_pack_kernel(const Geometry g, int32_t* __restrict__ row_start, const float* __restrict__ src,
+                                                        const int64_t src_stride, float* __restrict__ dst, const int64_t dst_stride, const int cpr,
+                                                        const unsigned total, const unsigned quarter) {
+  __shared__ int starts[PLAN_MAX + 1];
+  __shared__ int warp_sum[8];
+  ptx::grid_dep_wait();
+  ptx::grid_dep_launch();
+  const int n = 3 * g.batch, tid = threadIdx.x, lane = tid & 31;
+  const int per = (n + 255) / 256, lo = min(n, tid * per), hi = min(n, lo + per);
+  int sum = 0;
+  for (int e = lo; e < hi; ++e) {
+    starts[e] = sum;                      // within this thread's entries
+    sum += valid_rows(g, e / 3, e % 3);
+  }
+  int inc = sum;                          // inclusive scan over the warp, then over the warps
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += v;
+  }
+  if (lane == 31) warp_sum[tid >> 5] = inc;
+  __syncthreads();
+  int before = inc - sum;
+  for (int w = 0; w < (tid >> 5); ++w) before += warp_sum[w];
+  for (int e = lo; e < hi; ++e) starts[e] += before;
+  if (tid == 255) starts[n] = before + sum;
+  __syncthreads();
+  if (blockIdx.x == 0)
+    for (int e = tid; e <= n; e += 256) row_start[e] = starts[e];
+  const unsigned idx0 = blockIdx.x * 256u + tid;
+  if (idx0 >= quarter) return;
+  float4 v[MOVE_UNROLL];
+  float4* out[MOVE_UNROLL];
+#pragma unroll
+  for (int u = 0; u < MOVE_UNROLL; ++u) {
+    const unsigned idx = idx0 + (unsigned)u * quarter;
+    out[u] = nullptr;
+    v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (idx >= total) continue;
+    const unsigned w = idx / (unsigned)cpr, c = idx - w * (unsigned)cpr;  // padded-layout row, chunk in the row
+    const int b = (int)(w / (unsigned)g.L), p = (int)(w - (unsigned)b * (unsigned)g.L);
+    const int s = segment_of(g, p), i = p - g.seg_off[s], at = starts[3 * b + s];
+    if (i >= starts[3 * b + s + 1] - at) continue;
+    out[u] = reinterpret_cast<float4*>(dst + (int64_t)(at + i) * dst_stride) + c;
+    v[u] = __ldg(reinterpret_cast<const float4*>(src + (int64_t)w * src_stride) + c);
+  }
+#pragma unroll
+  for (int u = 0; u < MOVE_UNROLL; ++u)
+    if (out[u] != nullptr) *out[u] = v[u];
+}
+
 }  // namespace
+
+bool plan_pack_supported(const Geometry& g) { return 3 * g.batch <= PLAN_MAX; }
+
+cudaError_t launch_plan_pack(const Geometry& g, int32_t* row_start, const float* src, int64_t src_stride, float* dst, int64_t dst_stride, int cols,
+                             cudaStream_t st) {
+  const int cpr = cols / 4;
+  const int64_t total = (int64_t)g.batch * g.L * cpr;
+  if (total > 0xffffffffLL || !plan_pack_supported(g)) return cudaErrorNotSupported;
+  const unsigned quarter = (unsigned)((total + MOVE_UNROLL - 1) / MOVE_UNROLL);
+  return launch_overlapped(plan_pack_kernel, dim3((quarter + 255u) / 256u), dim3(256), 0, st, g, row_start, src, src_stride, dst, dst_stride, cpr,
+                           (unsigned)total, quarter);
+}
 
 cudaError_t launch_plan_rows(const Geometry& g, int split_sample, int32_t* row_start, cudaStream_t st) {
   plan_rows_kernel<<<1, 1024, 0, st>>>(g, split_sample, row_start);

@@ -404,9 +404,8 @@ PyObject* stack_forward(PyObject* const* a) {
     gsit_status st = GSIT_OK;
     if (plan != nullptr) {
       float* xp = f(b[6]);
-      st = gsit_plan_rows(&ring_shape, 0, static_cast<int32_t*>(plan->data_ptr()), cs);
+      st = gsit_plan_pack_rows(&ring_shape, static_cast<int32_t*>(plan->data_ptr()), x_in, ldx, xp, d, (int32_t)d, cs);
       if (st != GSIT_OK) return st;
-      if ((st = gsit_pack_rows(&ring_shape, x_in, ldx, xp, d, (int32_t)d, cs)) != GSIT_OK) return st;
       x_in = xp;
       ldx = d;
     }
