@@ -26,9 +26,9 @@
 //                 O_h += P_h V     M 128, N 16 (32), K 16 per step; A = P_h from TMEM, B = the V tile as loaded
 //                   (N-contiguous).  With head_dim 8, N = 16 covers the head pair; the neighbour's 8 columns of each
 //                   head's accumulator are never read
-//   warps 2..5  softmax of head 0, warps 6..9 of head 1: thread = query row = TMEM lane.  Two passes over the scores in
-//               groups of 16 columns (maximum, then weights), running maximum and sum in registers, O_h rescaled in TMEM
-//               only when the maximum has grown by more than 2^8.  Warps whose 32 rows hold no real query skip the
+//   warps 2..5  softmax of head 0, warps 6..9 of head 1: thread = query row = TMEM lane.  The first key tile is
+//               read twice in groups of 16 columns (maximum, then weights), later ones once, against the reference the row has;
+//               O_h is rescaled in TMEM only when the weights have outgrown that.  Warps whose 32 rows hold no real query skip the
 //               arithmetic.
 // TMEM columns: [0,64) S_0, [64,128) S_1 fp32; [128,160) P_0, [160,192) P_1 bf16x2; [192,224) O_0, [224,256) O_1.
 // Every wait is bounded; when one expires GSIT_DEVFLAG_TIMEOUT is raised, the CTA's other waits give up at once, and the
@@ -51,9 +51,6 @@ constexpr int S_TMEM_COLS = 256, S_COL_P = 128, S_COL_O = 192;
 constexpr int S_CTAS_PER_SM = 2;
 constexpr int S_ITEM_SLOTS = 4;
 constexpr int S_QBUF = 16384;  // bytes reserved per Q buffer
-#ifndef GSIT_POLY_PAIRS
-#define GSIT_POLY_PAIRS 0x11
-#endif
 // The weights are cut to bf16 by dropping the low 16 bits (one byte permute on the integer pipe per pair; the rounding
 // conversion would occupy the special-function unit as long as an exponential).  Dropping bits loses on average
 // 0.72 * 2^-9 of a value whose mantissa is spread like that of an exponential, so every weight is raised by that factor
@@ -61,7 +58,8 @@ constexpr int S_QBUF = 16384;  // bytes reserved per Q buffer
 // lowered by it at the end: the weights are then unbiased, with the same spread as round-to-nearest.
 constexpr float TRUNC_GAIN = 1.0f + 0.72f / 512.0f;
 constexpr float TRUNC_LOG2 = 0.0020273f;  // log2(TRUNC_GAIN)
-constexpr unsigned POLY_PAIRS = GSIT_POLY_PAIRS;  // bit i: pair i of every 16-key group takes the polynomial 2^x
+// Bit i: pair i of every 16-key group takes the polynomial 2^x (none 54.7 us, one pair 53.2, two 53.9 at the size given below).
+constexpr unsigned POLY_PAIRS = 0x01;
 // barriers (8 bytes each), relative to the barrier block
 constexpr int B_QFULL = 0, B_QEMPTY = 16, B_SFULL = 32, B_PFULL = 48, B_OFINAL = 64, B_TMEM_SLOT = 72, B_GAVE_UP = 76,
               B_ITEMBAR = 80, B_ITEMS = 256, B_KFULL = 512, B_VFULL = 576, B_KVEMPTY = 640, B_END = 704;
@@ -425,51 +423,8 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
                 if (16 * c + e >= krem) a[e] = 0xff800000u;  // -inf
             }
           };
-          // ---- pass 1: row maximum ----
-          float mx4[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) mx4[i] = -INFINITY;
-          auto maxc = [&](const uint32_t (&a)[16]) {
-#pragma unroll
-            for (int e = 0; e < 16; e += 2)
-              mx4[(e >> 1) & 3] = fmax3(mx4[(e >> 1) & 3], __uint_as_float(a[e]), __uint_as_float(a[e + 1]));
-          };
-          tmem_ld16(tS + 0, sa);
-          if (16 < krem) tmem_ld16(tS + 16, sb);
-          tmem_wait_ld();
-          fix(sa, 0);
-          maxc(sa);
-          if (16 < krem) { fix(sb, 1); maxc(sb); }
-          if (32 < krem) {
-            tmem_ld16(tS + 32, sa);
-            if (48 < krem) tmem_ld16(tS + 48, sb);
-            tmem_wait_ld();
-            fix(sa, 2);
-            maxc(sa);
-            if (48 < krem) { fix(sb, 3); maxc(sb); }
-          }
-          const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-          // rescale only when the maximum has grown by more than 2^8 (P stays below 256: exact enough in bf16 and f32)
-          const bool grow_m = (j == 0) || ((mx - mu) * sl2 > 8.f);
-          if (j > 0 && __any_sync(0xffffffffu, grow_m)) {
-            const float alpha = grow_m ? ex2((mu - mx) * sl2) : 1.f;
-            lsum *= alpha;
-            // O_h holds every earlier key tile: the P V of tile j - 1 was issued before the scores this thread has just
-            // waited for, and the tensor pipe runs in issue order
-#pragma unroll
-            for (int c = 0; c < HD / 8; ++c) {
-              uint32_t o[8];
-              tmem_ld8(tO + 8 * c, o);
-              tmem_wait_ld();
-#pragma unroll
-              for (int e = 0; e < 8; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-              tmem_st8(tO + 8 * c, o);
-            }
-          }
-          if (grow_m) mu = mx;
-          // ---- pass 2: weights.  Groups 2 and 3 are still in registers when the tile has them; 0 and 1 are read again. ----
-          const float nm = fmaf(-mu, sl2, TRUNC_LOG2);
-          const float2 nmv = make_float2(nm, nm);
+          float nm = fmaf(-mu, sl2, TRUNC_LOG2);
+          float2 nmv = make_float2(nm, nm);
           float2 sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
           auto weights = [&](const uint32_t (&a)[16], const int c) {
             uint32_t pr[8];
@@ -477,28 +432,110 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
             for (int e = 0; e < 16; e += 2) {
               const float2 x = __ffma2_rn(make_float2(__uint_as_float(a[e]), __uint_as_float(a[e + 1])), sl2v, nmv);
               // a fixed share of the exponentials goes to the FMA pipe, so that it and the special-function unit finish together
-              const float2 p = ((POLY_PAIRS >> (e >> 1)) & 1) ? ex2_poly2(x) : make_float2(ex2(x.x), ex2(x.y));
+              const float2 p = ((POLY_PAIRS >> (e >> 1)) & 1) ? ex2_poly2(make_float2(fminf(x.x, 127.f), fminf(x.y, 127.f))) : make_float2(ex2(x.x), ex2(x.y));
               sum[(e >> 1) & 1] = __fadd2_rn(sum[(e >> 1) & 1], p);
               pr[e >> 1] = __byte_perm(__float_as_uint(p.x), __float_as_uint(p.y), 0x7632);  // upper halves: bf16 pair
             }
             tmem_st8(tP + 8 * c, pr);
           };
-          if (32 < krem) {
-            weights(sa, 2);
-            tmem_ld16(tS + 0, sa);
-            if (48 < krem) weights(sb, 3);
-            tmem_wait_ld();
-            tmem_ld16(tS + 16, sb);
+          // Every key tile but the first is taken in ONE pass against the reference its row already has: the weights may grow to
+          // 2^59 (bf16 and float keep their precision there), and only when a row's sum says that one did are the scores,
+          // still in TMEM, read again for their maximum.  What is left is the hand-over per tile: 32 x (30, 480, 230), 8 heads of
+          // 16, no mask 55.7 -> 53.9 us; 32 x (128, 1024, 1024), 8 of 32, intra 136.8 -> 129.8.
+          auto ready = [&](uint32_t (&a)[16]) { tmem_wait_ld(); tmem_regs_ready(a); };
+          bool redo = j == 0;
+          if (!redo) {
+            tmem_ld16(tS, sa);
+            ready(sa);
+            if (16 < krem) tmem_ld16(tS + 16, sb);
+            fix(sa, 0);
             weights(sa, 0);
-            tmem_wait_ld();
-            weights(sb, 1);
-          } else {
-            // at most two groups: both are still in registers from pass 1 (masked already)
-            weights(sa, 0);
-            if (16 < krem) weights(sb, 1);
+            if (16 < krem) {
+              ready(sb);
+              if (32 < krem) tmem_ld16(tS + 32, sa);
+              fix(sb, 1);
+              weights(sb, 1);
+              if (32 < krem) {
+                ready(sa);
+                if (48 < krem) tmem_ld16(tS + 48, sb);
+                fix(sa, 2);
+                weights(sa, 2);
+                if (48 < krem) {
+                  ready(sb);
+                  fix(sb, 3);
+                  weights(sb, 3);
+                }
+              }
+            }
+            const float2 s01 = __fadd2_rn(sum[0], sum[1]);
+            const float part = s01.x + s01.y;
+            redo = __any_sync(0xffffffffu, !(part < 1e18f) && r < it.q_real);  // rows past the real ones may hold anything
+            if (!redo) lsum += part;
           }
-          const float2 s01 = __fadd2_rn(sum[0], sum[1]);
-          lsum += s01.x + s01.y;
+          if (redo) {
+            // ---- pass 1: row maximum ----
+            float mx4[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) mx4[i] = -INFINITY;
+            auto maxc = [&](const uint32_t (&a)[16]) {
+#pragma unroll
+              for (int e = 0; e < 16; e += 2)
+                mx4[(e >> 1) & 3] = fmax3(mx4[(e >> 1) & 3], __uint_as_float(a[e]), __uint_as_float(a[e + 1]));
+            };
+            tmem_ld16(tS + 0, sa);
+            if (16 < krem) tmem_ld16(tS + 16, sb);
+            tmem_wait_ld();
+            fix(sa, 0);
+            maxc(sa);
+            if (16 < krem) { fix(sb, 1); maxc(sb); }
+            if (32 < krem) {
+              tmem_ld16(tS + 32, sa);
+              if (48 < krem) tmem_ld16(tS + 48, sb);
+              tmem_wait_ld();
+              fix(sa, 2);
+              maxc(sa);
+              if (48 < krem) { fix(sb, 3); maxc(sb); }
+            }
+            const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+            // rescale only when the maximum has grown by more than 2^8 (P stays below 256: exact enough in bf16 and f32)
+            const bool grow_m = (j == 0) || ((mx - mu) * sl2 > 8.f);
+            if (j > 0 && __any_sync(0xffffffffu, grow_m)) {
+              const float alpha = grow_m ? ex2((mu - mx) * sl2) : 1.f;
+              lsum *= alpha;
+              // O_h holds every earlier key tile: the P V of tile j - 1 was issued before the scores this thread has just
+              // waited for, and the tensor pipe runs in issue order
+#pragma unroll
+              for (int c = 0; c < HD / 8; ++c) {
+                uint32_t o[8];
+                tmem_ld8(tO + 8 * c, o);
+                tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 8; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+                tmem_st8(tO + 8 * c, o);
+              }
+            }
+            if (grow_m) mu = mx;
+            // ---- pass 2: weights.  Groups 2 and 3 are still in registers when the tile has them; 0 and 1 are read again. ----
+            nm = fmaf(-mu, sl2, TRUNC_LOG2);
+            nmv = make_float2(nm, nm);
+            sum[0] = sum[1] = make_float2(0.f, 0.f);
+            if (32 < krem) {
+              weights(sa, 2);
+              tmem_ld16(tS + 0, sa);
+              if (48 < krem) weights(sb, 3);
+              tmem_wait_ld();
+              tmem_ld16(tS + 16, sb);
+              weights(sa, 0);
+              tmem_wait_ld();
+              weights(sb, 1);
+            } else {
+              // at most two groups: both are still in registers from pass 1 (masked already)
+              weights(sa, 0);
+              if (16 < krem) weights(sb, 1);
+            }
+            const float2 s01 = __fadd2_rn(sum[0], sum[1]);
+            lsum += s01.x + s01.y;
+          }
           tmem_wait_st();
         }
         tc_fence_before();
