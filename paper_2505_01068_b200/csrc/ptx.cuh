@@ -134,8 +134,6 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* tm, uint32_t src
 }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// True in exactly one lane of a converged warp.  Whole warps run the producer / issuer loops so that addresses,
-// descriptors and barrier phases stay warp-uniform; only the asynchronous instruction itself is issued by one lane.
 // Between reading a shared-memory buffer into registers and releasing that buffer for a refill, where the values are not
 // used before the release: nothing else keeps the loads from being performed after it (the release is one lane's mbarrier
 // arrive behind a warp barrier).  It is not enough for a buffer that the asynchronous proxy (a TMA load) refills at once:
@@ -153,6 +151,8 @@ __device__ __forceinline__ void fence_reads_before_release() { asm volatile("fen
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// True in exactly one lane of a converged warp.  Whole warps run the producer / issuer loops so that addresses,
+// descriptors and barrier phases stay warp-uniform; only the asynchronous instruction itself is issued by one lane.
 __device__ __forceinline__ bool elect_one() {
   uint32_t pred;
   asm volatile(
