@@ -285,14 +285,27 @@ cudaError_t launch(const Geometry& g, const float* q, const float* k, const floa
     for (int s = 0; s < 3; ++s) n += (g.seg_len[s] + rows - 1) / rows;
     return n;
   };
-  if (g.heads > 65535 || g.batch > 65535) return cudaErrorNotSupported;
   // At most 128 rows per CTA, so that a segment's last tile wastes little (256: 92 us instead of 81 at the size above; 64: 88),
   // and the keys split further over the warps of a CTA while there are fewer than four CTAs (16 warps) per SM.
   int splits = T == 1 ? 2 : 1;
   while (splits < 4 && tiles(splits) * g.heads * g.batch < 4LL * n_sm) splits *= 2;
-  const dim3 grid((unsigned)tiles(splits), g.heads, g.batch);
-  return launch_overlapped(kernel, grid, dim3(F32_WARPS * 32), smem, st, g, q, k, v, row_stride, out, lse, scale * 1.4426950408889634f,
-                           splits);
+  if (tiles(splits) > 0x7fffffffLL) return cudaErrorNotSupported;
+  // Heads and samples lie along y and z, which hold 65535 blocks each; more of them take further launches.  (All three folded into
+  // x costs the kernel ten registers and with them a CTA per SM: 173 -> 179 us for a layer at the size above.)
+  constexpr int MOST = 65535;
+  for (int b0 = 0; b0 < g.batch; b0 += MOST)
+    for (int h0 = 0; h0 < g.heads; h0 += MOST) {
+      Geometry gs = g;
+      gs.batch = g.batch - b0 < MOST ? g.batch - b0 : MOST;
+      if (g.valid_len != nullptr) gs.valid_len = g.valid_len + 3 * (int64_t)b0;
+      const int heads = g.heads - h0 < MOST ? g.heads - h0 : MOST;
+      const int64_t in = (int64_t)b0 * g.L * row_stride + (int64_t)h0 * g.hd, to = (int64_t)b0 * g.L * g.d + (int64_t)h0 * g.hd;
+      float* lse_s = lse != nullptr ? lse + ((int64_t)b0 * g.heads + h0) * g.L : nullptr;
+      e = launch_overlapped(kernel, dim3((unsigned)tiles(splits), heads, gs.batch), dim3(F32_WARPS * 32), smem, st, gs, q + in, k + in, v + in,
+                            row_stride, out + to, lse_s, scale * 1.4426950408889634f, splits);
+      if (e != cudaSuccess) return e;
+    }
+  return cudaSuccess;
 }
 
 }  // namespace

@@ -46,6 +46,27 @@ def test_attention_key_splits(g, B):
     check_close(to_np64(out), ref, "f32", pad_mask(seg, valid, B), f"B {B}")
 
 
+@pytest.mark.parametrize("B,H", [(65535, 2), (65536, 2), (131072, 2), (2, 65537)])
+def test_batches_and_heads_beyond_one_grid_dimension(g, B, H):
+    """A grid's y and z hold 65535 blocks each; attention and layer take larger batches, and attention more heads."""
+    rng = np.random.default_rng(B)
+    seg, hd = (1, 2, 1), 4
+    q, k, v = wk.draw_qkv(rng, B, sum(seg), H, hd, "f32")
+    valid = rng.integers(0, 3, size=(B, 3)).astype(np.int32).clip(None, seg).astype(np.int32)
+    vl = torch.from_numpy(valid).cuda()
+    out, lse = g.im_attention_fwd(*[to_dev(t) for t in (q, k, v)], seg, vl, g.PHASE_CUSTOM, 0x1FF, want_lse=True)
+    ref, ref_lse = oracle.im_attention_dense(q, k, v, seg, valid, g.PHASE_CUSTOM, custom_mask=0x1FF, want_lse=True)
+    check_close(to_np64(out), ref, "f32", pad_mask(seg, valid, B), f"B {B}")
+    a, b = to_np64(lse), np.asarray(ref_lse)
+    assert np.array_equal(np.isneginf(a), np.isneginf(b)) and np.abs(a[np.isfinite(b)] - b[np.isfinite(b)]).max() <= 1e-4
+    if H > 2:
+        return
+    x = rng.standard_normal((B, sum(seg), H * hd), dtype=np.float32)
+    w = wk.draw_layer_weights(rng, H * hd, 16, "f32", affine=True)
+    y = to_np64(g.im_layer_fwd(to_dev(x), weights_to_dev(w, "f32"), seg, H, vl, g.PHASE_INTRA)[-70:])
+    check_close(y, oracle.im_layer_fwd(x[-70:], w, seg, H, valid[-70:], g.PHASE_INTRA), "f32", pad_mask(seg, valid[-70:], 70), f"layer B {B}")
+
+
 @pytest.mark.parametrize("d,heads,d_ff,seg,B", [(32, 4, 128, (8, 12, 10), 2), (36, 3, 100, (64, 64, 0), 1), (64, 8, 256, (50, 75, 100), 3),
                                                 (96, 4, 200, (1, 63, 1), 2), (128, 2, 512, (33, 64, 31), 2), (4, 1, 4, (3, 2, 1), 1),
                                                 (160, 4, 320, (33, 64, 31), 2), (30, 3, 62, (33, 64, 31), 1), (64, 8, 256, (50, 375, 500), 40)])
