@@ -12,6 +12,7 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <deque>
 #include <exception>
 #include <vector>
 
@@ -144,21 +145,38 @@ struct NoGil {  // a launch may block when the stream's queue is full: other Pyt
 enum WKey { LN1_G, LN1_B, W_QKV, B_QKV, W_O, B_O, LN2_G, LN2_B, W_1, B_1, W_2, B_2, N_WKEYS };
 const char* const W_NAMES[N_WKEYS] = {"ln1_g", "ln1_b", "w_qkv", "b_qkv", "w_o", "b_o", "ln2_g", "ln2_b", "w_1", "b_1", "w_2", "b_2"};
 PyObject* g_wkeys[N_WKEYS];
+PyObject* g_get;
 
-gsit_layer_weights layer_weights(PyObject* dict, double eps, int32_t* dtype) {
-  if (!PyDict_Check(dict)) fail(PyExc_TypeError, "layer weights: a dict of tensors");
+// Owned references to the tensors of a layer's weights, kept until the call has been issued.  A plain dict is read directly; any
+// other mapping (nn.ParameterDict, a subclass with its own look-up) as w[key] for the matrices and w.get(key) for the rest.
+struct WeightRefs {
+  PyObject* o[N_WKEYS] = {};
+  WeightRefs() = default;
+  WeightRefs(const WeightRefs&) = delete;
+  ~WeightRefs() {
+    for (PyObject* p : o) Py_XDECREF(p);
+  }
+};
+bool is_matrix(int key) { return key == W_QKV || key == W_O || key == W_1 || key == W_2; }
+void read_weights(PyObject* map, WeightRefs& r) {
+  const bool dict = PyDict_CheckExact(map);
+  for (const bool matrices : {true, false})
+    for (int i = 0; i < N_WKEYS; ++i) {
+      if (is_matrix(i) != matrices) continue;
+      if (dict) r.o[i] = Py_XNewRef(PyDict_GetItemWithError(map, g_wkeys[i]));
+      else r.o[i] = matrices ? PyObject_GetItem(map, g_wkeys[i]) : PyObject_CallMethodOneArg(map, g_get, g_wkeys[i]);
+      if (r.o[i] == nullptr && matrices && !PyErr_Occurred()) PyErr_SetObject(PyExc_KeyError, g_wkeys[i]);
+      if (r.o[i] == nullptr && PyErr_Occurred()) throw PyFail{};
+    }
+}
+
+gsit_layer_weights layer_weights(PyObject* map, double eps, int32_t* dtype, WeightRefs& refs) {
+  read_weights(map, refs);
   const void* p[N_WKEYS];
   gsit_layer_weights w = {};
   for (int i = 0; i < N_WKEYS; ++i) {
-    PyObject* o = PyDict_GetItemWithError(dict, g_wkeys[i]);
-    if (o == nullptr && PyErr_Occurred()) throw PyFail{};
-    const bool matrix = (i == W_QKV || i == W_O || i == W_1 || i == W_2);
-    if (o == nullptr && matrix) {
-      PyErr_SetObject(PyExc_KeyError, g_wkeys[i]);
-      throw PyFail{};
-    }
-    const at::Tensor* t = opt_tensor(o);
-    if (matrix) {
+    const at::Tensor* t = opt_tensor(refs.o[i]);
+    if (is_matrix(i)) {
       require(t != nullptr && t->is_cuda() && t->is_contiguous(), "layer weights: contiguous device matrices");
       if (i == W_QKV) *dtype = dtype_code(*t);
       if (i == W_1) w.d_ff = (int32_t)t->size(0);
@@ -255,7 +273,8 @@ PyObject* im_layer_fwd(PyObject* const* a) {
   const at::Tensor *valid = opt_tensor(a[4]), *out = opt_tensor(a[9]), *ws = opt_tensor(a[10]), *row_start = opt_tensor(a[11]);
   const bool use_static = as_bool(a[12]);
   int32_t dtype = GSIT_F32;
-  const gsit_layer_weights w = layer_weights(a[1], as_float(a[8]), &dtype);
+  WeightRefs refs;
+  const gsit_layer_weights w = layer_weights(a[1], as_float(a[8]), &dtype, refs);
   require(x.is_cuda() && x.scalar_type() == at::kFloat && x.stride(-1) == 1, "x: float32 on the device, features contiguous");
   const int64_t heads = as_int(a[3]);
   at::Tensor made, made_ws;
@@ -325,7 +344,8 @@ PyObject* im_layer_pair_fwd(PyObject* const* a) {
   const at::Tensor &xa = tensor(a[0]), &xb = tensor(a[1]);
   const at::Tensor *valid = opt_tensor(a[6]), *oa = opt_tensor(a[10]), *ob = opt_tensor(a[11]), *ws = opt_tensor(a[12]), *row_start = opt_tensor(a[13]);
   int32_t dtype = GSIT_F32, other = GSIT_F32;
-  const gsit_layer_weights wa = layer_weights(a[2], as_float(a[9]), &dtype), wb = layer_weights(a[3], as_float(a[9]), &other);
+  WeightRefs refs_a, refs_b;
+  const gsit_layer_weights wa = layer_weights(a[2], as_float(a[9]), &dtype, refs_a), wb = layer_weights(a[3], as_float(a[9]), &other, refs_b);
   at::Tensor made[2], made_ws;
   const bool packed = row_start != nullptr;
   if (packed) require(xa.dim() == 2 && valid != nullptr && oa != nullptr && ob != nullptr, "packed rows: x and out [capacity, d], with valid_len");
@@ -361,11 +381,11 @@ PyObject* im_layer_pair_fwd(PyObject* const* a) {
 
 // ---- the fusion stack: every launch of one forward issued from here ----
 
-std::vector<gsit_layer_weights> all_layers(PyObject* list, double eps, int32_t* dtype) {
-  require(PyList_Check(list), "layers: a list of weight dicts");
+std::vector<gsit_layer_weights> all_layers(PyObject* list, double eps, int32_t* dtype, std::deque<WeightRefs>& refs) {
+  require(PyList_Check(list), "layers: a list of weight mappings");
   std::vector<gsit_layer_weights> w;
   w.reserve(PyList_GET_SIZE(list));
-  for (Py_ssize_t i = 0; i < PyList_GET_SIZE(list); ++i) w.push_back(layer_weights(PyList_GET_ITEM(list, i), eps, dtype));
+  for (Py_ssize_t i = 0; i < PyList_GET_SIZE(list); ++i) w.push_back(layer_weights(PyList_GET_ITEM(list, i), eps, dtype, refs.emplace_back()));
   return w;
 }
 
@@ -383,7 +403,9 @@ PyObject* stack_forward(PyObject* const* a) {
           "x: float32 [B, L, d] on the device with a uniform row stride");
   const double eps = as_float(a[9]);
   int32_t dtype = GSIT_F32;
-  const std::vector<gsit_layer_weights> intra = all_layers(a[5], eps, &dtype), fwd = all_layers(a[3], eps, &dtype), bwd = all_layers(a[4], eps, &dtype);
+  std::deque<WeightRefs> refs;
+  const std::vector<gsit_layer_weights> intra = all_layers(a[5], eps, &dtype, refs), fwd = all_layers(a[3], eps, &dtype, refs),
+                                        bwd = all_layers(a[4], eps, &dtype, refs);
   require(fwd.size() == bwd.size() && !fwd.empty(), "rings of equal depth");
   require(PyTuple_Check(a[10]) && PyTuple_GET_SIZE(a[10]) == 9, "buffers: nine tensors");
   const at::Tensor* b[9];
@@ -487,5 +509,6 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nu
 
 PyMODINIT_FUNC PyInit__native() {
   for (int i = 0; i < N_WKEYS; ++i) g_wkeys[i] = PyUnicode_InternFromString(W_NAMES[i]);
+  g_get = PyUnicode_InternFromString("get");
   return PyModule_Create(&module);
 }

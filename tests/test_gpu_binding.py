@@ -1,6 +1,12 @@
-"""What the native argument marshalling passes on: torch's own exception types."""
+"""What the native argument marshalling passes on and accepts: torch's own exception types, weights in any mapping."""
+import collections
+
+import numpy as np
 import pytest
 import torch
+
+import workloads as wk
+from gpu_util import weights_to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -27,3 +33,30 @@ def test_failed_allocation_raises_torch_out_of_memory_error(g):
     finally:
         torch.cuda.set_per_process_memory_fraction(1.0)
     assert bool((half == 0).all()) and g.last_device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_weights_in_any_mapping(g, dtype):
+    """An nn.ParameterDict without the optional vectors, an OrderedDict, and a mapping that makes its tensors when asked."""
+    rng = np.random.default_rng(0)
+    seg, d = (5, 40, 21), 64
+    w = {k: t for k, t in weights_to_dev(wk.draw_layer_weights(rng, d, 4 * d, dtype), dtype).items() if t is not None}
+    x = torch.randn((2, sum(seg), d), device="cuda")
+    call = lambda m: g.im_layer_fwd(x, m, seg, 8)
+
+    class Made(collections.abc.Mapping):
+        __len__, __iter__ = (lambda self: len(w)), (lambda self: iter(w))
+        __getitem__ = lambda self, k: w[k].clone()
+
+    ref = call(w)
+    assert torch.equal(ref, call(torch.nn.ParameterDict({k: torch.nn.Parameter(t, requires_grad=False) for k, t in w.items()})))
+    assert torch.equal(ref, call(collections.OrderedDict(w)))
+    for _ in range(3):
+        assert torch.equal(ref, call(Made()))
+    ya, yb = g.im_layer_pair_fwd(x, x, Made(), torch.nn.ParameterDict(w), seg, 8, None, g.PHASE_INTER_FWD, g.PHASE_INTER_FWD)
+    assert torch.equal(ya, ref) and torch.equal(yb, ref)
+    for m in (dict, collections.OrderedDict):
+        with pytest.raises(KeyError):
+            call(m({k: t for k, t in w.items() if k != "w_o"}))
+    with pytest.raises(TypeError):
+        call([w])
