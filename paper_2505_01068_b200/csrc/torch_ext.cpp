@@ -14,7 +14,6 @@
 
 #include <deque>
 #include <exception>
-#include <vector>
 
 #include "gsit.h"
 
@@ -179,6 +178,7 @@ gsit_layer_weights layer_weights(PyObject* map, double eps, int32_t* dtype, Weig
     if (is_matrix(i)) {
       require(t != nullptr && t->is_cuda() && t->is_contiguous(), "layer weights: contiguous device matrices");
       if (i == W_QKV) *dtype = dtype_code(*t);
+      require(dtype_code(*t) == *dtype, "layer weights: matrices of one type");
       if (i == W_1) w.d_ff = (int32_t)t->size(0);
     } else if (t != nullptr) {
       require(t->scalar_type() == at::kFloat && t->is_contiguous(), "layer weights: contiguous float32 vectors");
@@ -346,6 +346,7 @@ PyObject* im_layer_pair_fwd(PyObject* const* a) {
   int32_t dtype = GSIT_F32, other = GSIT_F32;
   WeightRefs refs_a, refs_b;
   const gsit_layer_weights wa = layer_weights(a[2], as_float(a[9]), &dtype, refs_a), wb = layer_weights(a[3], as_float(a[9]), &other, refs_b);
+  require(dtype == other, "both layers' weights of one type");
   at::Tensor made[2], made_ws;
   const bool packed = row_start != nullptr;
   if (packed) require(xa.dim() == 2 && valid != nullptr && oa != nullptr && ob != nullptr, "packed rows: x and out [capacity, d], with valid_len");
@@ -381,12 +382,19 @@ PyObject* im_layer_pair_fwd(PyObject* const* a) {
 
 // ---- the fusion stack: every launch of one forward issued from here ----
 
-std::vector<gsit_layer_weights> all_layers(PyObject* list, double eps, int32_t* dtype, std::deque<WeightRefs>& refs) {
+struct Layer {
+  WeightRefs refs;
+  int32_t dtype = GSIT_F32;
+  gsit_layer_weights w;
+};
+std::deque<Layer> all_layers(PyObject* list, double eps) {
   require(PyList_Check(list), "layers: a list of weight mappings");
-  std::vector<gsit_layer_weights> w;
-  w.reserve(PyList_GET_SIZE(list));
-  for (Py_ssize_t i = 0; i < PyList_GET_SIZE(list); ++i) w.push_back(layer_weights(PyList_GET_ITEM(list, i), eps, dtype, refs.emplace_back()));
-  return w;
+  std::deque<Layer> layers;
+  for (Py_ssize_t i = 0; i < PyList_GET_SIZE(list); ++i) {
+    Layer& l = layers.emplace_back();
+    l.w = layer_weights(PyList_GET_ITEM(list, i), eps, &l.dtype, l.refs);
+  }
+  return layers;
 }
 
 // x, valid_len, y, fwd, bwd, intra, seg_len, heads, intra_heads, ln_eps, buffers
@@ -402,20 +410,17 @@ PyObject* stack_forward(PyObject* const* a) {
   require(x.is_cuda() && x.scalar_type() == at::kFloat && x.dim() == 3 && x.stride(2) == 1 && x.stride(0) == x.size(1) * x.stride(1),
           "x: float32 [B, L, d] on the device with a uniform row stride");
   const double eps = as_float(a[9]);
-  int32_t dtype = GSIT_F32;
-  std::deque<WeightRefs> refs;
-  const std::vector<gsit_layer_weights> intra = all_layers(a[5], eps, &dtype, refs), fwd = all_layers(a[3], eps, &dtype, refs),
-                                        bwd = all_layers(a[4], eps, &dtype, refs);
+  const std::deque<Layer> intra = all_layers(a[5], eps), fwd = all_layers(a[3], eps), bwd = all_layers(a[4], eps);
   require(fwd.size() == bwd.size() && !fwd.empty(), "rings of equal depth");
   require(PyTuple_Check(a[10]) && PyTuple_GET_SIZE(a[10]) == 9, "buffers: nine tensors");
   const at::Tensor* b[9];
   for (int i = 0; i < 9; ++i) b[i] = opt_tensor(PyTuple_GET_ITEM(a[10], i));
   const at::Tensor* plan = b[0];
   const int64_t B = x.size(0), d = x.size(2), cap = plan != nullptr ? b[6]->size(0) : 0;
-  const gsit_shape ring_shape = make_shape(B, a[6], d, as_int(a[7]), valid, dtype, GSIT_PHASE_INTER_FWD, 0, 0.0, plan, cap);
-  const gsit_shape intra_shape = make_shape(B, a[6], 2 * d, as_int(a[8]), valid, dtype, GSIT_PHASE_INTRA, 0, 0.0, plan, cap);
+  const gsit_shape ring_shape = make_shape(B, a[6], d, as_int(a[7]), valid, fwd[0].dtype, GSIT_PHASE_INTER_FWD, 0, 0.0, plan, cap);
+  const gsit_shape intra_shape = make_shape(B, a[6], 2 * d, as_int(a[8]), valid, fwd[0].dtype, GSIT_PHASE_INTRA, 0, 0.0, plan, cap);
   uint8_t* ws = static_cast<uint8_t*>(b[1]->data_ptr());
-  const size_t ws_n = (size_t)b[1]->numel();
+  const size_t ws_n = (size_t)b[1]->numel(), ws_half = ws_n / 2;
   auto f = [](const at::Tensor* t) { return static_cast<float*>(t->data_ptr()); };
   float *ping_a[2] = {f(b[2]), f(b[3])}, *ping_b[2] = {f(b[4]), f(b[5])}, *wide[2] = {f(b[7]), f(b[8])};
   float* out = f(&y);
@@ -442,14 +447,24 @@ PyObject* stack_forward(PyObject* const* a) {
       const bool last = i + 1 == fwd.size();
       float *dst_a = last ? c : ping_a[i & 1], *dst_b = last ? c + d : ping_b[i & 1];
       const int64_t ldy = last ? 2 * d : d;
-      st = gsit_im_layer_pair_fwd(&sa, &sb, &fwd[i], &bwd[i], cur_a, ld, cur_b, ld, dst_a, ldy, dst_b, ldy, ws, ws_n, cs);
+      // every layer in the type of its own weights; a pair of one type goes through one call
+      sa.dtype = fwd[i].dtype;
+      sb.dtype = bwd[i].dtype;
+      if (sa.dtype == sb.dtype && fwd[i].w.d_ff == bwd[i].w.d_ff) {
+        st = gsit_im_layer_pair_fwd(&sa, &sb, &fwd[i].w, &bwd[i].w, cur_a, ld, cur_b, ld, dst_a, ldy, dst_b, ldy, ws, ws_n, cs);
+      } else {
+        st = gsit_im_layer_fwd(&sa, &fwd[i].w, cur_a, ld, dst_a, ldy, ws, ws_half, cs);
+        if (st == GSIT_OK) st = gsit_im_layer_fwd(&sb, &bwd[i].w, cur_b, ld, dst_b, ldy, ws + ws_half, ws_half, cs);
+      }
       if (st != GSIT_OK) return st;
       cur_a = dst_a; cur_b = dst_b; ld = ldy;
     }
     int in_wide = 0;
     for (size_t i = 0; i < intra.size(); ++i) {
       float* dst = (i + 1 == intra.size() && plan == nullptr) ? out : wide[in_wide ^ 1];
-      st = gsit_im_layer_fwd(&intra_shape, &intra[i], wide[in_wide], 2 * d, dst, 2 * d, ws, ws_n, cs);
+      gsit_shape si = intra_shape;
+      si.dtype = intra[i].dtype;
+      st = gsit_im_layer_fwd(&si, &intra[i].w, wide[in_wide], 2 * d, dst, 2 * d, ws, ws_n, cs);
       if (st != GSIT_OK) return st;
       in_wide ^= 1;
     }

@@ -56,6 +56,16 @@ class GsitStack:
             lo = hi
         return out
 
+    def _workspace_need(self, Bn, d, valid_len, plan=None, capacity=0):
+        """Bytes that the most demanding layer of the stack asks for (layers may differ in type and MLP width)."""
+        need = 0
+        for layers, width, heads, phase in ((self.fwd, d, self.heads, B.PHASE_INTER_FWD), (self.bwd, d, self.heads, B.PHASE_INTER_BWD),
+                                            (self.intra, 2 * d, self.intra_heads, B.PHASE_INTRA)):
+            for code, d_ff in {(B._dtype_code(w["w_qkv"].dtype), int(w["w_1"].shape[0])) for w in layers}:
+                sh = B.make_shape(Bn, self.seg_len, width, heads, valid_len, code, phase, row_start=plan, capacity=capacity)
+                need = max(need, B.workspace_bytes(sh, B.CALL_LAYER, d_ff))
+        return need
+
     def _buffers(self, x, valid_len):
         Bn, L, d = x.shape
         chunks = self._chunks(Bn)
@@ -63,16 +73,9 @@ class GsitStack:
         if self._bufs is None:
             self._bufs = {}
         if key not in self._bufs:
-            code = B._dtype_code(self.fwd[0]["w_qkv"].dtype)
             ws = []
             for sl in chunks:  # two workspaces per chunk of the batch: one per ring (the intra encoder reuses the first)
-                n = sl.stop - sl.start
-                vl = None if valid_len is None else valid_len[sl]
-                sh1 = B.make_shape(n, self.seg_len, d, self.heads, vl, code, B.PHASE_INTER_FWD)
-                need = B.workspace_bytes(sh1, B.CALL_LAYER, self.fwd[0]["w_1"].shape[0])
-                if self.intra:
-                    sh2 = B.make_shape(n, self.seg_len, 2 * d, self.intra_heads, vl, code, B.PHASE_INTRA)
-                    need = max(need, B.workspace_bytes(sh2, B.CALL_LAYER, self.intra[0]["w_1"].shape[0]))
+                need = self._workspace_need(sl.stop - sl.start, d, None if valid_len is None else valid_len[sl])
                 ws.append([torch.empty(need, dtype=torch.uint8, device=x.device) for _ in range(2)])
             f32 = dict(dtype=torch.float32, device=x.device)
             self._bufs[key] = (ws, [torch.empty((Bn, L, d), **f32) for _ in range(4)],
@@ -103,14 +106,8 @@ class GsitStack:
             self._bufs = {}
         if key not in self._bufs:
             cap = Bn * L + 128  # always enough: the real rows plus the alignment of the second half's first row
-            code = B._dtype_code(self.fwd[0]["w_qkv"].dtype)
             plan = torch.zeros(3 * Bn + 1, dtype=torch.int32, device=x.device)
-            sh1 = B.make_shape(Bn, self.seg_len, d, self.heads, valid_len, code, B.PHASE_INTER_FWD, row_start=plan, capacity=cap)
-            need = B.workspace_bytes(sh1, B.CALL_LAYER, self.fwd[0]["w_1"].shape[0])
-            if self.intra:
-                sh2 = B.make_shape(Bn, self.seg_len, 2 * d, self.intra_heads, valid_len, code, B.PHASE_INTRA, row_start=plan,
-                                   capacity=cap)
-                need = max(need, B.workspace_bytes(sh2, B.CALL_LAYER, self.intra[0]["w_1"].shape[0]))
+            need = self._workspace_need(Bn, d, valid_len, plan, cap)
             f32 = dict(dtype=torch.float32, device=x.device)
             ws_all = torch.empty(2 * need, dtype=torch.uint8, device=x.device)   # one per ring
             self._bufs[key] = (cap, plan, [ws_all[:need], ws_all[need:]],
@@ -215,13 +212,8 @@ class GsitStack:
             return got
         Bn, L, d = x.shape
         cap = Bn * L + 128 if packed else Bn * L
-        code = B._dtype_code(self.fwd[0]["w_qkv"].dtype)
         plan = torch.zeros(3 * Bn + 1, dtype=torch.int32, device=x.device) if packed else None
-        need = 0
-        for w, width, heads, phase in [(self.fwd[0], d, self.heads, B.PHASE_INTER_FWD)] + [(w, 2 * d, self.intra_heads, B.PHASE_INTRA)
-                                                                                           for w in self.intra[:1]]:
-            sh = B.make_shape(Bn, self.seg_len, width, heads, valid_len, code, phase, row_start=plan, capacity=cap if packed else 0)
-            need = max(need, B.workspace_bytes(sh, B.CALL_LAYER, w["w_1"].shape[0]))
+        need = self._workspace_need(Bn, d, valid_len, plan, cap if packed else 0)
         # rows past the last real one are read by the last row tile (and discarded): they start out as zeros
         z = lambda cols: torch.zeros((cap, cols), dtype=torch.float32, device=x.device)
         bufs = (plan, torch.empty(2 * need, dtype=torch.uint8, device=x.device), z(d), z(d), z(d), z(d), z(d) if packed else None,

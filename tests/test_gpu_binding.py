@@ -1,4 +1,4 @@
-"""What the native argument marshalling passes on and accepts: torch's own exception types, weights in any mapping."""
+"""What the native argument marshalling passes on and accepts: torch's own exception types, weights in any mapping, a type per layer."""
 import collections
 
 import numpy as np
@@ -60,3 +60,39 @@ def test_weights_in_any_mapping(g, dtype):
             call(m({k: t for k, t in w.items() if k != "w_o"}))
     with pytest.raises(TypeError):
         call([w])
+
+
+@pytest.mark.parametrize("types", [("f32", "f32", "bf16"), ("bf16", "bf16", "f32"), ("bf16", "f32", "bf16"), ("f32", "bf16", "f32")])
+@pytest.mark.parametrize("padded", [False, True])
+def test_stack_runs_every_layer_in_the_type_of_its_weights(g, types, padded):
+    """Rings and intra encoder of different types, and MLP widths that differ from layer to layer: the bits of the layers called
+    one by one, whichever way the stack issues them."""
+    rng = np.random.default_rng(1)
+    seg, d, B, H, IH = (5, 70, 33), 32, 3, 4, 4
+    layers = lambda width, t, ffs: [weights_to_dev(wk.draw_layer_weights(rng, width, f, t, affine=True), t) for f in ffs]
+    fwd, bwd, intra = layers(d, types[0], (64, 128)), layers(d, types[1], (64, 192)), layers(2 * d, types[2], (128, 256))
+    x = torch.randn((B, sum(seg), d), device="cuda")
+    vl = torch.tensor([[5, 70, 33], [2, 41, 0], [1, 64, 17]], dtype=torch.int32, device="cuda") if padded else None
+
+    def chain(cur, ws, heads, phase):
+        for w in ws:
+            cur = g.im_layer_fwd(cur, w, seg, heads, vl, phase)
+        return cur
+
+    want = chain(torch.cat([chain(x, fwd, H, g.PHASE_INTER_FWD), chain(x, bwd, H, g.PHASE_INTER_BWD)], dim=2), intra, IH, g.PHASE_INTRA)
+    for kw in (dict(), dict(packed=False), dict(paired_rings=False), dict(paired_rings=False, concurrent_rings=False)):
+        got = g.GsitStack(fwd, bwd, intra, seg, H, IH, **kw).forward(x, vl).clone()
+        torch.cuda.synchronize()
+        assert torch.equal(got, want), kw
+    assert g.last_device_status() == (0, 0)
+
+
+def test_weights_of_two_types_in_one_layer_are_refused(g):
+    """The type of w_qkv is the type every matrix of the call is read in."""
+    seg, d = (5, 9, 3), 32
+    w = [weights_to_dev(wk.draw_layer_weights(np.random.default_rng(2), d, 64, "bf16"), t) for t in ("bf16", "f32")]
+    x = torch.randn((1, sum(seg), d), device="cuda")
+    with pytest.raises(AssertionError):
+        g.im_layer_fwd(x, dict(w[1], w_2=w[0]["w_2"]), seg, 4)
+    with pytest.raises(AssertionError):
+        g.im_layer_pair_fwd(x, x, w[0], w[1], seg, 4)
