@@ -43,6 +43,11 @@ gsit_status gsit_trace_reset(void);
  * gsit_last_device_status() answers GSIT_ERR_TIMEOUT once and clears the flag.  Asynchronous on `stream`. */
 gsit_status gsit_test_expire_wait(gsit_stream stream);
 
+/* Copies `bytes` (a multiple of 16; both DEVICE pointers 16-byte aligned) from src to dst in a one-CTA kernel that allows
+ * the kernel after it in the stream to start at once and writes only some delay_us (at most 1000) microseconds later: a
+ * predecessor whose writes a call of this library must wait for before it reads anything.  Asynchronous on `stream`. */
+gsit_status gsit_test_late_write(void* dst, const void* src, size_t bytes, int32_t delay_us, gsit_stream stream);
+
 #ifdef __cplusplus
 }
 #endif

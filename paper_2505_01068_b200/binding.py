@@ -43,7 +43,7 @@ class LayerWeights(ctypes.Structure):
 
 EXPORTS = ("gsit_im_qkv_proj", "gsit_im_attention_fwd", "gsit_im_layer_fwd", "gsit_workspace_bytes",
            "gsit_last_device_status", "gsit_status_string", "gsit_version", "gsit_trace_enable", "gsit_trace_read",
-           "gsit_trace_launches", "gsit_trace_reset", "gsit_tune_attention", "gsit_test_expire_wait", "gsit_im_layer_fwd_static",
+           "gsit_trace_launches", "gsit_trace_reset", "gsit_tune_attention", "gsit_test_expire_wait", "gsit_test_late_write", "gsit_im_layer_fwd_static",
            "gsit_stack_head_fwd", "gsit_im_layer_pair_fwd",
            "gsit_plan_rows", "gsit_pack_rows", "gsit_unpack_rows", "gsit_plan_pack_rows")
 STATIC_SCRATCH_BYTES = 4 << 20
@@ -175,6 +175,16 @@ def expire_wait_selftest():
     lib = load()
     lib.gsit_test_expire_wait.argtypes = [ctypes.c_void_p]
     _check(lib.gsit_test_expire_wait(_stream()), "gsit_test_expire_wait")
+
+
+def late_write(dst, src, delay_us: int = 100):
+    """Test hook: dst <- src (equal sizes, multiples of 16 bytes) by a kernel that its successor need not wait to see the end
+    of (see include/gsit_test.h)."""
+    n = src.numel() * src.element_size()
+    assert dst.is_cuda and src.is_cuda and dst.is_contiguous() and src.is_contiguous() and dst.numel() * dst.element_size() == n
+    lib = load()
+    lib.gsit_test_late_write.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_int32, ctypes.c_void_p]
+    _check(lib.gsit_test_late_write(_ptr(dst), _ptr(src), n, int(delay_us), _stream()), "gsit_test_late_write")
 
 
 def trace_enable(on: bool):

@@ -116,9 +116,6 @@ ln_qkv_tc_kernel(const __grid_constant__ LnQkvArgs arg0, const __grid_constant__
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   float* prm = reinterpret_cast<float*>(base_ptr + OFF_P);
-  stage_vector(prm, gamma, TD, 1.f, tid, T_THREADS);
-  stage_vector(prm + TD, beta, TD, 0.f, tid, T_THREADS);
-  stage_vector(prm + 2 * TD, bias, NQ, 0.f, tid, T_THREADS);
   if (tid == 0) {
     asm volatile("st.shared.u32 [%0], %1;" ::"r"(bars + SLOT + 4), "r"(0u) : "memory");
     mbar_init(bars + B_W, 1);
@@ -139,14 +136,7 @@ ln_qkv_tc_kernel(const __grid_constant__ LnQkvArgs arg0, const __grid_constant__
   tc_fence_after();
   uint32_t tmem;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(bars + SLOT) : "memory");
-  if (warp == 0) {  // the weights do not depend on the kernel before this one
-    if (elect_one()) {
-      mbar_expect_tx(bars + B_W, NQ * 128);
-      tma_load_2d(base + OFF_W, &tmW, 0, 0, bars + B_W);
-    }
-    __syncwarp();
-  }
-  grid_dep_wait();
+  grid_dep_wait();  // the weights, too, are read behind it: this kernel may be the first of a call, right after the one that wrote them
   grid_dep_launch();
   const int row_base = rows_begin(g), rows = rows_end(g);  // this problem's rows of the activation matrices
   const int ntiles = (rows - row_base + TM - 1) / TM;
@@ -161,13 +151,17 @@ ln_qkv_tc_kernel(const __grid_constant__ LnQkvArgs arg0, const __grid_constant__
         mbar_expect_tx(bars + B_XFULL, 2 * XBOX);
         tma_load_2d(base + OFF_X, &tmX, 0, row_base + t * TM, bars + B_XFULL);
         tma_load_2d(base + OFF_X + XBOX, &tmX, 32, row_base + t * TM, bars + B_XFULL);
+        if (i == 0) {  // the weights once, behind the rows, which are needed first
+          mbar_expect_tx(bars + B_W, NQ * 128);
+          tma_load_2d(base + OFF_W, &tmW, 0, 0, bars + B_W);
+        }
       }
       __syncwarp();
     }
   } else if (warp == 1) {
     // ================================ MMA issuer ================================
     constexpr uint32_t IDESC = idesc_bf16(NQ, false);
-    mbar_wait(wc, bars + B_W, 0);
+    if (cta < ntiles) mbar_wait(wc, bars + B_W, 0);
     int i = 0;
     for (int t = cta; t < ntiles; t += ctas, ++i) {
       mbar_wait(wc, bars + B_HREADY, i & 1);
@@ -186,6 +180,8 @@ ln_qkv_tc_kernel(const __grid_constant__ LnQkvArgs arg0, const __grid_constant__
     const int r = ((warp & 3) << 5) + lane;
     const uint32_t tl = tmem + ((uint32_t)((warp & 3) << 5) << 16);
     const uint32_t s_gamma = base + OFF_P, s_beta = s_gamma + TD * 4, s_bias = s_beta + TD * 4;
+    stage_parameters<TD, NQ, 128>(prm, gamma, beta, bias, tid - 64);  // while the first rows are on their way
+    t_bar_rows();
     int i = 0;
     bool real = row_real32(g, row_base + cta * TM + r, rows);
     for (int t = cta; t < ntiles; t += ctas, ++i) {
@@ -328,7 +324,7 @@ proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_consta
   tc_fence_after();
   uint32_t tmem;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(bars + SLOT) : "memory");
-  if (warp == 0) {  // the weights do not depend on the kernel before this one
+  if (warp == 0) {  // before the wait: the attention before this kernel has waited for whatever wrote the weights
     if (elect_one()) {
       mbar_expect_tx(bars + B_W, (uint32_t)(TD * 128 + d_ff * 128 + nh * TD * 128));
       tma_load_2d(base + OFF_WO, &tmWo, 0, 0, bars + B_W);

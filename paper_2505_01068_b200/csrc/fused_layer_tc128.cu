@@ -53,9 +53,6 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   float* prm = reinterpret_cast<float*>(base_ptr + OFF_P);
-  stage_vector(prm, gamma, D2, 1.f, tid, T_THREADS8);
-  stage_vector(prm + D2, beta, D2, 0.f, tid, T_THREADS8);
-  stage_vector(prm + 2 * D2, bias, NQ, 0.f, tid, T_THREADS8);
   if (tid == 0) {
     asm volatile("st.shared.u32 [%0], %1;" ::"r"(bars + SLOT + 4), "r"(0u) : "memory");
     mbar_init(bars + B_W, 1);
@@ -76,16 +73,7 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
   tc_fence_after();
   uint32_t tmem;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(bars + SLOT) : "memory");
-  if (warp == 0) {  // the weights do not depend on the kernel before this one
-    if (elect_one()) {
-      mbar_expect_tx(bars + B_W, 2 * NQ * 128);
-      for (int kb = 0; kb < 2; ++kb)
-        for (int j = 0; j < 3; ++j)  // boxes of 128 weight rows
-          tma_load_2d(base + OFF_W + kb * NQ * 128 + j * XBOX, &tmW, 64 * kb, 128 * j, bars + B_W);
-    }
-    __syncwarp();
-  }
-  grid_dep_wait();
+  grid_dep_wait();  // the weights, too, are read behind it: this kernel may be the first of a call, right after the one that wrote them
   grid_dep_launch();
   const int row_base = rows_begin(g), rows = rows_end(g);  // this problem's rows of the activation matrices
   const int ntiles = (rows - row_base + TM - 1) / TM;
@@ -99,13 +87,19 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
       if (elect_one()) {
         mbar_expect_tx(bars + B_XFULL, 4 * XBOX);
         for (int j = 0; j < 4; ++j) tma_load_2d(base + OFF_X + j * XBOX, &tmX, 32 * j, row_base + t * TM, bars + B_XFULL);
+        if (i == 0) {  // the weights once, behind the rows, which are needed first
+          mbar_expect_tx(bars + B_W, 2 * NQ * 128);
+          for (int kb = 0; kb < 2; ++kb)
+            for (int j = 0; j < 3; ++j)  // boxes of 128 weight rows
+              tma_load_2d(base + OFF_W + kb * NQ * 128 + j * XBOX, &tmW, 64 * kb, 128 * j, bars + B_W);
+        }
       }
       __syncwarp();
     }
   } else if (warp == 1) {
     // ================================ MMA issuer ================================
     constexpr uint32_t IDESC_256 = idesc_bf16(256, false), IDESC_128 = idesc_bf16(128, false);
-    mbar_wait(wc, bars + B_W, 0);
+    if ((int)blockIdx.x < ntiles) mbar_wait(wc, bars + B_W, 0);
     int i = 0;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
       mbar_wait(wc, bars + B_HREADY, i & 1);
@@ -130,6 +124,8 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
     const int r = ((warp & 3) << 5) + lane, hf = (warp - 2) >> 2;  // row = TMEM lane; which half of the columns
     const uint32_t tl = tmem + ((uint32_t)((warp & 3) << 5) << 16);
     const uint32_t s_gamma = base + OFF_P, s_beta = s_gamma + D2 * 4, s_bias = s_beta + D2 * 4;
+    stage_parameters<D2, NQ, 256>(prm, gamma, beta, bias, tid - 64);  // while the first rows are on their way
+    t_bar_rows8();
     int i = 0;
     bool real = row_real32(g, row_base + (int)blockIdx.x * TM + r, rows);
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
@@ -282,7 +278,7 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
   tc_fence_after();
   uint32_t tmem;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(bars + SLOT) : "memory");
-  if (warp == 0) {  // the weights do not depend on the kernel before this one
+  if (warp == 0) {  // before the wait: the attention before this kernel has waited for whatever wrote the weights
     if (elect_one()) {
       mbar_expect_tx(bars + B_WO, 2 * XBOX);
       for (int kb = 0; kb < 2; ++kb) tma_load_2d(base + OFF_WO + kb * XBOX, &tmWo, 64 * kb, 0, bars + B_WO);

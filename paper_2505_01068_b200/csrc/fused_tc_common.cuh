@@ -30,6 +30,24 @@ __device__ __forceinline__ float4 ld_v4f(uint32_t addr) {
 __device__ __forceinline__ void stage_vector(float* dst, const float* src, int n, float fill, int tid, int nthreads) {
   for (int i = tid; i < n; i += nthreads) dst[i] = (src != nullptr) ? src[i] : fill;
 }
+// gamma [D] (or ones), beta [D] and bias [NB] (or zeros) side by side in shared memory, by T threads with all their loads in
+// flight at once: the first layer halves may only read them behind their wait, where each latency in a row counts (1.5 us of a
+// launch with one loop per vector).
+template <int D, int NB, int T>
+__device__ __forceinline__ void stage_parameters(float* dst, const float* gamma, const float* beta, const float* bias, int tid) {
+  constexpr int N = 2 * D + NB, K = (N + T - 1) / T;
+  float v[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int e = tid + k * T;
+    const float* src = e < D ? gamma : e < 2 * D ? beta : bias;
+    v[k] = e < D ? 1.f : 0.f;
+    if (src != nullptr && e < N) v[k] = src[e < D ? e : e < 2 * D ? e - D : e - 2 * D];
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+    if (tid + k * T < N) dst[tid + k * T] = v[k];
+}
 // Row validity with 32-bit arithmetic (the library limits B * L to 2^29).
 __device__ __forceinline__ bool row_real32(const Geometry& g, int row, int rows) {
   if (row >= rows) return false;

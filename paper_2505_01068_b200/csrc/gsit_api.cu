@@ -184,6 +184,13 @@ __global__ void expire_wait_kernel(unsigned int* status) {
   __syncthreads();
 }
 
+// Lets its successor start at once, then takes its time before it writes (about delay_us, at most twice that).
+__global__ void late_write_kernel(uint4* dst, const uint4* src, size_t n, int delay_us) {
+  ptx::grid_dep_launch();
+  for (int i = 0; i < delay_us; ++i) __nanosleep(1000);
+  for (size_t i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
+}
+
 // Which kernels run the two halves of a bf16 layer around the attention.
 enum Halves { HALVES_NONE = 0, HALVES_ROWS, HALVES_TC, HALVES_TC128, HALVES_LEGACY };
 Halves pick_halves(const Geometry& g, int d_ff) {
@@ -567,6 +574,12 @@ gsit_status gsit_test_expire_wait(gsit_stream stream) {
   unsigned int* p = nullptr;
   if (status_ptr(&p) != cudaSuccess) return GSIT_ERR_CUDA;
   expire_wait_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(p);
+  return from_cuda(cudaGetLastError());
+}
+
+gsit_status gsit_test_late_write(void* dst, const void* src, size_t bytes, int32_t delay_us, gsit_stream stream) {
+  if (!dst || !src || bytes % 16 != 0 || !aligned16(dst) || !aligned16(src) || delay_us < 0 || delay_us > 1000) return GSIT_ERR_INVALID_ARG;
+  late_write_kernel<<<1, 256, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<uint4*>(dst), static_cast<const uint4*>(src), bytes / 16, delay_us);
   return from_cuda(cudaGetLastError());
 }
 

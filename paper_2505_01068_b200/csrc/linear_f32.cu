@@ -171,10 +171,10 @@ __global__ void __launch_bounds__(FT_THREADS) linear_f32_kernel(const Geometry g
   const float* W = static_cast<const float*>(a.W);
   const int slices = (a.K + FT_K - 1) / FT_K;
   float4 ra[RP];
+  ptx::grid_dep_wait();  // the weights, too: this kernel may be the first of a call, right behind the one that wrote them
+  ptx::grid_dep_launch();
   request(sW[0], Slice{W, a.K, n0, a.N, 0, a.K}, vec_w, tid);
   commit();
-  ptx::grid_dep_wait();
-  ptx::grid_dep_launch();
   const Slice as{static_cast<const float*>(a.A), a.lda, m0, a.M, 0, a.K};
   fetch(as, vec_a, ra, tid);
   put(sA[0], ra, tid);
@@ -272,9 +272,9 @@ ln_qkv_f32_kernel(const Geometry g, const float* __restrict__ x, const int64_t l
   const int m0 = blockIdx.x * BM, chunks = (N + FT_N - 1) / FT_N;
   const int my = (chunks - (int)blockIdx.y + (int)gridDim.y - 1) / (int)gridDim.y;  // column chunks of this CTA
   auto next = [&](int i) { return Slice{w, d, ((int)blockIdx.y + (i / KD) * (int)gridDim.y) * FT_N, N, (i % KD) * FT_K, d}; };
-  auto stream = weight_stream(sW, next, my * KD, tid);
-  ptx::grid_dep_wait();
+  ptx::grid_dep_wait();  // the weights, too: this kernel may be the first of a call, right behind the one that wrote them
   ptx::grid_dep_launch();
+  auto stream = weight_stream(sW, next, my * KD, tid);
   const bool work = tile_has_rows<BM>(g, m0, M, tid);
   if (work) {
     // LayerNorm: eight threads per row, 16 rows at a time; a thread holds float4s 8 apart
@@ -371,7 +371,7 @@ proj_mlp_f32_kernel(const Geometry g, const float* __restrict__ att, const float
     if (j < KD) return Slice{w_1, d, c * FT_N, d_ff, j * FT_K, d};
     return Slice{w_2, d_ff, ((j - KD) >> 1) * FT_N, d, c * FT_N + ((j - KD) & 1) * FT_K, d_ff};
   };
-  auto stream = weight_stream(sW, next, first + nf * per_chunk, tid);
+  auto stream = weight_stream(sW, next, first + nf * per_chunk, tid);  // before the wait: the attention before it has waited
   ptx::grid_dep_wait();
   ptx::grid_dep_launch();
   bool real[2 * RP];

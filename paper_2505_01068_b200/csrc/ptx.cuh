@@ -144,9 +144,12 @@ __device__ __forceinline__ void fence_reads_before_release() { asm volatile("fen
 
 // Programmatic dependent launch.  A kernel launched with the "programmatic stream serialization" attribute may start
 // while the kernel before it in the stream is still running; grid_dep_wait() blocks until that kernel has completed and
-// its writes are visible (a no-op for an ordinary launch), so everything above it -- barrier set-up, TMEM allocation,
-// loads of weights -- overlaps the predecessor's tail.  Every kernel launched that way calls it, in every thread, before
-// its first access to memory an earlier kernel of the stream wrote or read: completion then chains through the stream.
+// its writes are visible (a no-op for an ordinary launch), so everything above it -- barrier set-up, TMEM allocation --
+// overlaps the predecessor's tail.  Every kernel launched that way calls it, in every thread, before its first access to
+// memory an earlier kernel of the stream wrote or read: completion then chains through the stream.  That goes for weights
+// and parameters, too, in a kernel that can be the first of a call: the kernel before it may be the caller's, and may be
+// the very one that writes them.  Only a kernel whose predecessor is always one of the same call that has waited itself
+// (the second layer halves, behind the attention) may read weights above its own wait.
 // grid_dep_launch() lets the next kernel's CTAs be placed as soon as every CTA of this one has called it (or exited).
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
