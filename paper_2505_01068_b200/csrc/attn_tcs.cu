@@ -473,6 +473,7 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
             if (!redo) lsum += part;
           }
           if (redo) {
+            if (j > 0) tmem_wait_st();  // the weights already stored are stored over below, and two tcgen05.st keep no order by themselves
             // ---- pass 1: row maximum ----
             float mx4[4];
 #pragma unroll
