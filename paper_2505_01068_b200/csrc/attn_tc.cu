@@ -292,7 +292,7 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         uint32_t sr[2][32];
 #pragma unroll
         for (int c = 0; c < 2; ++c) tmem_ld32(tl + COL_S + 64 * sb + 32 * c, sr[c]);
-        tmem_wait_ld();
+        tmem_wait_ld(sr[0], sr[1]);
         if (RAGGED) {  // keys past the valid length get weight exactly zero
 #pragma unroll
           for (int c = 0; c < 2; ++c)
@@ -322,7 +322,7 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           for (int c = 0; c < 4; ++c) {
             uint32_t o[16];
             tmem_ld16(tl + COL_O + 16 * c, o);
-            tmem_wait_ld();
+            tmem_wait_ld(o);
 #pragma unroll
             for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
             tmem_st16(tl + COL_O + 16 * c, o);
@@ -384,7 +384,7 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       for (int c = 0; c < 2; ++c) {
         uint32_t o[32];
         tmem_ld32(tl + COL_O + 32 * c, o);
-        tmem_wait_ld();
+        tmem_wait_ld(o);
         if (r < it.rows_in_tile) {
 #pragma unroll
           for (int e = 0; e < 32; e += 8) {

@@ -442,26 +442,25 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
           // 2^59 (bf16 and float keep their precision there), and only when a row's sum says that one did are the scores,
           // still in TMEM, read again for their maximum.  What is left is the hand-over per tile: 32 x (30, 480, 230), 8 heads of
           // 16, no mask 55.7 -> 53.9 us; 32 x (128, 1024, 1024), 8 of 32, intra 136.8 -> 129.8.
-          auto ready = [&](uint32_t (&a)[16]) { tmem_wait_ld(); tmem_regs_ready(a); };
           bool redo = j == 0;
           if (!redo) {
             tmem_ld16(tS, sa);
-            ready(sa);
+            tmem_wait_ld(sa);
             if (16 < krem) tmem_ld16(tS + 16, sb);
             fix(sa, 0);
             weights(sa, 0);
             if (16 < krem) {
-              ready(sb);
+              tmem_wait_ld(sb);
               if (32 < krem) tmem_ld16(tS + 32, sa);
               fix(sb, 1);
               weights(sb, 1);
               if (32 < krem) {
-                ready(sa);
+                tmem_wait_ld(sa);
                 if (48 < krem) tmem_ld16(tS + 48, sb);
                 fix(sa, 2);
                 weights(sa, 2);
                 if (48 < krem) {
-                  ready(sb);
+                  tmem_wait_ld(sb);
                   fix(sb, 3);
                   weights(sb, 3);
                 }
@@ -485,17 +484,17 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
             };
             tmem_ld16(tS + 0, sa);
             if (16 < krem) tmem_ld16(tS + 16, sb);
-            tmem_wait_ld();
+            tmem_wait_ld(sa);
             fix(sa, 0);
             maxc(sa);
-            if (16 < krem) { fix(sb, 1); maxc(sb); }
+            if (16 < krem) { tmem_regs_ready(sb); fix(sb, 1); maxc(sb); }
             if (32 < krem) {
               tmem_ld16(tS + 32, sa);
               if (48 < krem) tmem_ld16(tS + 48, sb);
-              tmem_wait_ld();
+              tmem_wait_ld(sa);
               fix(sa, 2);
               maxc(sa);
-              if (48 < krem) { fix(sb, 3); maxc(sb); }
+              if (48 < krem) { tmem_regs_ready(sb); fix(sb, 3); maxc(sb); }
             }
             const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
             // rescale only when the maximum has grown by more than 2^8 (P stays below 256: exact enough in bf16 and f32)
@@ -509,7 +508,7 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
               for (int c = 0; c < HD / 8; ++c) {
                 uint32_t o[8];
                 tmem_ld8(tO + 8 * c, o);
-                tmem_wait_ld();
+                tmem_wait_ld(o);
 #pragma unroll
                 for (int e = 0; e < 8; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
                 tmem_st8(tO + 8 * c, o);
@@ -524,10 +523,10 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
               weights(sa, 2);
               tmem_ld16(tS + 0, sa);
               if (48 < krem) weights(sb, 3);
-              tmem_wait_ld();
+              tmem_wait_ld(sa);
               tmem_ld16(tS + 16, sb);
               weights(sa, 0);
-              tmem_wait_ld();
+              tmem_wait_ld(sb);
               weights(sb, 1);
             } else {
               // at most two groups: both are still in registers from pass 1 (masked already)
@@ -557,7 +556,7 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
         for (int c = 0; c < HD / 8; ++c) {
           uint32_t o[8];
           tmem_ld8(tO + 8 * c, o);
-          tmem_wait_ld();
+          tmem_wait_ld(o);
 #pragma unroll
           for (int e = 0; e < 8; e += 2)
             orow[(c * 8 + e) >> 1] = pack_bf16(__uint_as_float(o[e]) * inv, __uint_as_float(o[e + 1]) * inv);

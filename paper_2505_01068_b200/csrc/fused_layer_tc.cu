@@ -213,8 +213,7 @@ ln_qkv_tc_kernel(const __grid_constant__ LnQkvArgs arg0, const __grid_constant__
       for (int c0 = 0; c0 < NQ; c0 += 32) {
         uint32_t a[32];
         tmem_ld32(tl + c0, a);
-        tmem_wait_ld();
-        tmem_regs_ready(a);
+        tmem_wait_ld(a);
         uint32_t pk[16];
 #pragma unroll
         for (int e = 0; e < 32; e += 4) {
@@ -428,8 +427,7 @@ proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_consta
       {
         uint32_t a[32];
         tmem_ld32(tl + COL_1 + 32 * hf, a);
-        tmem_wait_ld();
-        tmem_regs_ready(a);
+        tmem_wait_ld(a);
 #pragma unroll
         for (int e = 0; e < 32; e += 4) {
           const float4 bb = ld_v4f(s_bo + (32 * hf + e) * 4);
@@ -469,8 +467,7 @@ proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_consta
       for (int c0 = 32 * hf; c0 < d_ff; c0 += 64) {  // alternate groups of 32 hidden units
         uint32_t a[32];
         tmem_ld32(tl + COL_F + c0, a);
-        tmem_wait_ld();
-        tmem_regs_ready(a);
+        tmem_wait_ld(a);
         uint32_t pk[16];
 #pragma unroll
         for (int e = 0; e < 32; e += 4) {
@@ -498,8 +495,7 @@ proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_consta
       {
         uint32_t a[32];
         tmem_ld32(tl + COL_Y + 32 * hf, a);
-        tmem_wait_ld();
-        tmem_regs_ready(a);
+        tmem_wait_ld(a);
         const uint32_t box = base + OFF_F + hf * (TM * 128);
 #pragma unroll
         for (int ch = 0; ch < 8; ++ch) {

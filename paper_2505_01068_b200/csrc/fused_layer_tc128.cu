@@ -164,8 +164,7 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
           const int col = pass * (NQ / 2) + c0;
           uint32_t a[32];
           tmem_ld32(tl + col, a);
-          tmem_wait_ld();
-          tmem_regs_ready(a);
+          tmem_wait_ld(a);
           uint32_t pk[16];
 #pragma unroll
           for (int e = 0; e < 32; e += 4) {
@@ -431,8 +430,7 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
       for (int c = 0; c < 2; ++c) {
         uint32_t a[32];
         tmem_ld32(tl + COL_1 + 64 * hf + 32 * c, a);
-        tmem_wait_ld();
-        tmem_regs_ready(a);
+        tmem_wait_ld(a);
 #pragma unroll
         for (int e = 0; e < 32; e += 4) {
           const float4 bb = ld_v4f(s_bo + (64 * hf + 32 * c + e) * 4);
@@ -463,8 +461,7 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
         {
           uint32_t a[32];
           tmem_ld32(tl + COL_F + 64 * (n & 1) + 32 * hf, a);
-          tmem_wait_ld();
-          tmem_regs_ready(a);
+          tmem_wait_ld(a);
 #pragma unroll
           for (int e = 0; e < 32; e += 4) {
             const float4 bb = ld_v4f(s_b1 + (64 * c + 32 * hf + e) * 4);
@@ -495,8 +492,7 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
       for (int c = 0; c < 2; ++c) {
         uint32_t a[32];
         tmem_ld32(tl + COL_Y + 64 * hf + 32 * c, a);
-        tmem_wait_ld();
-        tmem_regs_ready(a);
+        tmem_wait_ld(a);
 #pragma unroll
         for (int sub = 0; sub < 2; ++sub) {
 #pragma unroll

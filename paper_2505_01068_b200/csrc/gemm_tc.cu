@@ -290,9 +290,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         uint32_t v[CW];
 #pragma unroll
         for (int h = 0; h < CW / 32; ++h) tmem_ld32(tl + ab * 256 + c * CW + 32 * h, *reinterpret_cast<uint32_t(*)[32]>(v + 32 * h));
-        tmem_wait_ld();
-#pragma unroll
-        for (int h = 0; h < CW / 32; ++h) tmem_regs_ready(*reinterpret_cast<uint32_t(*)[32]>(v + 32 * h));
+        tmem_wait_ld(*reinterpret_cast<uint32_t(*)[32]>(v), *reinterpret_cast<uint32_t(*)[32]>(v + CW - 32));
         if (c + 2 >= p.bn / CW || col0 + 2 * CW >= p.N) {  // this warp has read its last column of the accumulator
           tc_fence_before();
           __syncwarp();
