@@ -12,6 +12,8 @@
 // K and V tiles arrive through cp.async, double-buffered; keys past the valid length are filled with zeros and masked.
 // Where a launch would leave SMs idle, the warps of a CTA split the keys (2 or 4 ways) and merge at the end.
 // At 32 x (50, 375, 500) x 8 heads of 8, intra: 2324 us (a warp per row, lanes over features) -> 81 us, the FMA pipe 55 % busy.
+#include <float.h>
+
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -78,7 +80,7 @@ attn_f32_kernel(const Geometry g, const float* __restrict__ q, const float* __re
       qv[r][i] = make_float2(t.x * sl2, t.y * sl2);
       o[r][i] = make_float2(0.f, 0.f);
     }
-    m[r] = -INFINITY;
+    m[r] = -FLT_MAX;  // not -inf: keys whose scores are all -inf (a -inf in k or q) then weigh exp2(-inf) = 0 and not NaN
     l[r] = 0.f;
   }
 
@@ -173,7 +175,7 @@ attn_f32_kernel(const Geometry g, const float* __restrict__ q, const float* __re
         }
 #pragma unroll
         for (int r = 0; r < F32_R; ++r) {
-          float mx = sc[r][0];                          // the group's first key is real, so mx is finite
+          float mx = sc[r][0];
 #pragma unroll
           for (int kk = 1; kk < F32_G; ++kk) mx = fmaxf(mx, sc[r][kk]);
           if (mx > m[r]) {

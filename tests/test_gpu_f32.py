@@ -46,6 +46,26 @@ def test_attention_key_splits(g, B):
     check_close(to_np64(out), ref, "f32", pad_mask(seg, valid, B), f"B {B}")
 
 
+@pytest.mark.parametrize("hd", [3, 8, 40])
+@pytest.mark.parametrize("masked", [1, 8, 40, 199])
+def test_keys_with_scores_of_minus_infinity(g, hd, masked):
+    """Keys that an infinite feature takes out of the softmax: whole groups of them, first in their segment, weigh nothing."""
+    rng = np.random.default_rng(masked)
+    seg, H, B = (10, 200, 90), 2, 2
+    q, k, v = wk.draw_qkv(rng, B, sum(seg), H, hd, "f32")
+    q[..., 0] = np.abs(q[..., 0]) + 0.1
+    k[:, 10:10 + masked, :, 0] = -np.inf
+    out, lse = g.im_attention_fwd(*[to_dev(t) for t in (q, k, v)], seg, None, g.PHASE_INTER_FWD, want_lse=True)
+    # rows of segment 0 attend to segment 1
+    s = np.einsum("bqhe,bkhe->bhqk", q[:, :10].astype(np.float64), k[:, 10:210].astype(np.float64)) / np.sqrt(hd)
+    m = s.max(-1, keepdims=True)
+    p = np.exp(s - m)
+    want = np.einsum("bhqk,bkhe->bqhe", p / p.sum(-1, keepdims=True), v[:, 10:210].astype(np.float64))
+    assert np.abs(to_np64(out)[:, :10].reshape(B, 10, H, hd) - want).max() <= 1e-4
+    assert np.abs(to_np64(lse)[:, :, :10] - (m + np.log(p.sum(-1, keepdims=True)))[..., 0]).max() <= 1e-4
+    assert np.isfinite(to_np64(out)).all()
+
+
 @pytest.mark.parametrize("B,H", [(65535, 2), (65536, 2), (131072, 2), (2, 65537)])
 def test_batches_and_heads_beyond_one_grid_dimension(g, B, H):
     """A grid's y and z hold 65535 blocks each; attention and layer take larger batches, and attention more heads."""
