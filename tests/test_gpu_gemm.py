@@ -74,3 +74,41 @@ def test_wide_layer_against_legacy_kernels(g, d, heads, d_ff, seg, B):
     err = (first - ref).abs()
     assert float(err.max()) <= 4e-2 and float(err.mean()) <= 4e-3, (float(err.max()), float(err.mean()))
     assert g.last_device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("d,heads,seg,B", [(64, 8, (9, 50, 30), 2), (128, 8, (50, 300, 270), 60), (192, 3, (37, 129, 300), 5), (512, 8, (60, 511, 700), 18)])
+def test_projection_on_packed_rows(g, d, heads, seg, B):
+    """Tiles inside a call's rows, tiles shared with the samples before and after, tiles outside; one CTA per tile and pairs.  Same
+    bits as the padded layout; nothing written beyond the call's rows."""
+    rng = np.random.default_rng(d + B)
+    L, cap = sum(seg), B * sum(seg) + 128
+    x = torch.randn((B, L, d), device="cuda", generator=torch.Generator("cuda").manual_seed(B)).bfloat16()
+    w, bias = to_dev(wk.xavier_uniform(rng, 3 * d, d), "bf16"), to_dev(rng.standard_normal(3 * d).astype(np.float32))
+    valid = np.stack([rng.integers(0, n + 1, size=B) for n in seg], axis=1).astype(np.int32)
+    valid[B // 2] = 0
+    vl = torch.from_numpy(valid).cuda()
+    plan = g.plan_rows(vl, seg)
+    want = torch.empty((cap, 3 * d), device="cuda")
+    g.pack_rows(g.im_qkv_proj(x, w, bias, seg, heads, vl).reshape(B, L, 3 * d).float(), want, seg, vl, plan)
+    xp = torch.full((cap, d), float("nan"), device="cuda")
+    xp = g.pack_rows(x.float(), xp, seg, vl, plan).bfloat16()
+    starts = plan.cpu().numpy()
+    for lo, hi in {(0, B), (0, 1), (B - 1, B), (1, (B + 1) // 2), (B // 3, B)}:
+        if lo >= hi:
+            continue
+        for bare in (False, True):
+            out = torch.full((cap, 3, heads, d // heads), 7.0, dtype=torch.bfloat16, device="cuda")
+            g.im_qkv_proj(xp, w, None if bare else bias, seg, heads, vl[lo:hi], out=out, row_start=plan[3 * lo:])
+            first = out.clone()
+            for _ in range(3):
+                g.im_qkv_proj(xp, w, None if bare else bias, seg, heads, vl[lo:hi], out=out, row_start=plan[3 * lo:])
+                assert torch.equal(out, first)
+            a, b = int(starts[3 * lo]), int(starts[3 * hi])
+            flat = out.reshape(cap, 3 * d).float()
+            assert bool((flat[:a] == 7.0).all()) and bool((flat[b:] == 7.0).all()), (lo, hi)
+            if bare:
+                ref = xp[a:b].float() @ w.float().T
+                assert a == b or float((flat[a:b] - ref).abs().max()) <= 1e-2 * float(ref.abs().max())
+            else:
+                assert torch.equal(flat[a:b], want[a:b]), (lo, hi)
+    assert g.last_device_status() == (0, 0)
