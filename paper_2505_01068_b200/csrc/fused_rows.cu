@@ -353,19 +353,41 @@ cudaError_t launch_proj_mlp(const Geometry& g, const Pair& p, int n, float eps, 
 bool fused_rows_supported(const Geometry& g, int d_ff) {
   return (g.d == 32 || g.d == 64 || g.d == 128) && d_ff % 64 == 0 && d_ff <= ROWS_MAX_FF;
 }
-// Where these kernels are the better ones: always at width 32 (which no tcgen05 half covers); at 64 and 128 as long as a launch is
-// about the latency of a tile.  One layer without open blocks: d 64 14.3 (tcgen05) -> 9.3 us at 1050 rows, 14.4 -> 10.6 at 2100,
-// 14.7 -> 13.0 at 4200, 16.3 -> 16.2 at 8400, 33 -> 70 at 67200; d 128 23.8 -> 14.7, 23.9 -> 17.6, 24.2 -> 21.9, 24.6 -> 30.
-bool fused_rows_preferred(const Geometry& g) { return g.d == 32 || (int64_t)g.batch * g.L <= 6400; }
+// Where these kernels are chosen: always at width 32 (which no tcgen05 half covers); at 64 and 128 up to 43 padded rows per SM.
+// One layer without open blocks, us, these kernels / tcgen05 (148 SMs; lengths between half and full):
+//   rows               2100         3150         4200         5250         6300         8400
+//   d 64  padded    12.3/14.3    14.3/14.4    15.5/14.1    16.5/14.5    17.2/14.8    18.8/16.0
+//   d 64  packed    10.7/14.4    11.8/14.4    13.4/14.7    14.0/14.5    14.4/15.0    16.2/16.2
+//   d 64  packed, pair 13.5/14.5 14.8/15.0    17.2/16.3    17.7/16.8    22.4/17.9    27.1/17.9
+//   d 128 padded    20.4/23.8    23.4/23.8    24.1/23.9    27.3/24.7    35.3/25.1    35.2/24.9
+//   d 128 packed    17.8/23.9    19.1/23.8    21.9/24.0    23.0/25.0    30.7/25.3    31.9/24.8
+//   d 128 packed, pair 21.7/47.5 24.7/47.4    32.7/47.7    33.9/49.8    50.3/50.3    53.8/49.2
+// and at a quarter of the positions real (packed) these are the faster ones up to 8400 rows throughout but for pairs at d 64 (17.0 /
+// 16.7 at 6300).  So the two meet anywhere between 20 and 57 rows per SM, depending on what the host does not know (the lengths) or
+// must not look at: a sample gets the same bits alone, in a pair, padded, packed, and in any grouping of a batch within the limit.
+// The line lies at the upper end, where that holds for batches up to six samples of 1050 rows.  By the figures above a stack of four
+// pairs at d 64 and two layers at d 128 (packed) loses 29 us by it at 6300 rows, nothing at 5250, and wins 8 at a quarter real.
+constexpr int ROWS_PER_SM = 43;
+static int sm_count() {
+  int n = 0;
+  return sm_count_and_smem_once(nullptr, 0, &n) == cudaSuccess ? n : 0;
+}
+bool fused_rows_preferred(const Geometry& g) { return g.d == 32 || (int64_t)g.batch * g.L <= (int64_t)ROWS_PER_SM * sm_count(); }
 
-// n problems (1 or 2) of one geometry in one launch each.  Rows per tile: 16 for the shortest chain while there are few tiles,
-// more where the weight reads of many tiles (through L1) become what counts.
+// n problems (1 or 2) of one geometry in one launch each.  Rows per tile: 16 (d 32: 32) for the shortest chain while a launch is about
+// the latency of a tile, twice as many where the weight reads of many tiles (through L1) become what counts.  Limits in rows per
+// SM; a layer without open blocks, us, small tile / large tile, full lengths:
+//   first half,  d 32   284: 28.6/29.5   341: 31.6/31.3   454: 40.6/39.8     -> 320
+//   second half, d 32    57: 11.7/11.7    71: 13.0/12.7    85: 13.7/13.4   114: 15.9/14.2   -> 72 (half-full lengths meet at 75)
+//   second half, d 64    28: 14.6/14.7    35: 15.5/16.0    43: 16.5/16.4    50: 20.5/17.2   -> 40
+//   second half, d 128  8.5: 17.1/18.3   9.9: 18.7/18.5  11.4: 19.2/19.0    14: 20.9/19.2   -> 10
+// A row's bits do not depend on it, so the number of problems may count here.
 cudaError_t launch_ln_qkv_rows(const Geometry& g, const FusedHalfArgs* h, int n, float eps, int* zero_word, cudaStream_t st) {
   Pair p;
   p.a[0] = h[0];
   p.a[1] = h[n - 1];
-  const int64_t rows = (int64_t)g.batch * g.L * n;
-  if (g.d == 32) return rows > 48000 ? launch_ln_qkv<32, 4>(g, p, n, eps, zero_word, st) : launch_ln_qkv<32, 2>(g, p, n, eps, zero_word, st);
+  const int64_t rows = (int64_t)g.batch * g.L * n, sms = sm_count();
+  if (g.d == 32) return rows > 320 * sms ? launch_ln_qkv<32, 4>(g, p, n, eps, zero_word, st) : launch_ln_qkv<32, 2>(g, p, n, eps, zero_word, st);
   if (g.d == 64) return launch_ln_qkv<64, 1>(g, p, n, eps, zero_word, st);
   return launch_ln_qkv<128, 1>(g, p, n, eps, zero_word, st);
 }
@@ -373,10 +395,10 @@ cudaError_t launch_proj_mlp_rows(const Geometry& g, const FusedHalfArgs* h, int 
   Pair p;
   p.a[0] = h[0];
   p.a[1] = h[n - 1];
-  const int64_t rows = (int64_t)g.batch * g.L * n;
-  if (g.d == 32) return rows > 12000 ? launch_proj_mlp<32, 4>(g, p, n, eps, d_ff, st) : launch_proj_mlp<32, 2>(g, p, n, eps, d_ff, st);
-  if (g.d == 64) return rows > 5000 ? launch_proj_mlp<64, 2>(g, p, n, eps, d_ff, st) : launch_proj_mlp<64, 1>(g, p, n, eps, d_ff, st);
-  return rows > 1600 ? launch_proj_mlp<128, 2>(g, p, n, eps, d_ff, st) : launch_proj_mlp<128, 1>(g, p, n, eps, d_ff, st);
+  const int64_t rows = (int64_t)g.batch * g.L * n, sms = sm_count();
+  if (g.d == 32) return rows > 72 * sms ? launch_proj_mlp<32, 4>(g, p, n, eps, d_ff, st) : launch_proj_mlp<32, 2>(g, p, n, eps, d_ff, st);
+  if (g.d == 64) return rows > 40 * sms ? launch_proj_mlp<64, 2>(g, p, n, eps, d_ff, st) : launch_proj_mlp<64, 1>(g, p, n, eps, d_ff, st);
+  return rows > 10 * sms ? launch_proj_mlp<128, 2>(g, p, n, eps, d_ff, st) : launch_proj_mlp<128, 1>(g, p, n, eps, d_ff, st);
 }
 
 }  // namespace gsit

@@ -61,3 +61,38 @@ def test_layer_on_row_tiles(g, d, heads, d_ff, seg, B):
     assert torch.equal(ya, y.contiguous())
     assert torch.equal(yb, g.im_layer_fwd(xc, w2, seg, heads, vl, g.PHASE_INTER_FWD))
     assert g.last_device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("d,heads", [(64, 8), (128, 8)])
+@pytest.mark.parametrize("above", [0, 1])
+def test_layer_on_either_side_of_the_row_limit(g, d, heads, above):
+    """The last row count on small row tiles (43 per SM) and the first on tcgen05: both against the oracle, and on either side the
+    padded layout, the packed one and the pair call agree bit for bit.  Up to the limit so do a batch and its halves; above it
+    the halves run on other kernels and agree as closely as each does with the oracle."""
+    rng = np.random.default_rng(d)
+    B, L = 4, 43 * torch.cuda.get_device_properties(0).multi_processor_count // 4 + above
+    seg = (70, (L - 70) // 2, L - 70 - (L - 70) // 2)
+    x = rng.standard_normal((B, L, d), dtype=np.float32)
+    w = wk.draw_layer_weights(rng, d, 4 * d, "bf16", affine=True)
+    wd = weights_to_dev(w, "bf16")
+    valid = np.stack([rng.integers(n // 2, n + 1, size=B) for n in seg], axis=1).astype(np.int32)
+    pm, vl, xd = pad_mask(seg, valid, B), torch.from_numpy(valid).cuda(), to_dev(x)
+    y = g.im_layer_fwd(xd, wd, seg, heads, vl, g.PHASE_INTRA)
+    for b in (0, B - 1):
+        ref = oracle.im_layer_fwd(x[b:b + 1], w, seg, heads, valid[b:b + 1], g.PHASE_INTRA)
+        check_close(to_np64(y[b:b + 1]), ref, "bf16", pm[b:b + 1], f"sample {b}")
+    cap = B * L + 128
+    plan = g.plan_rows(vl, seg)
+    xp, yp = torch.zeros((cap, d), device="cuda"), torch.empty((cap, d), device="cuda")
+    g.pack_rows(xd, xp, seg, vl, plan)
+    g.im_layer_fwd(xp, wd, seg, heads, vl, g.PHASE_INTRA, out=yp, row_start=plan)
+    assert torch.equal(g.unpack_rows(yp, torch.empty_like(y), seg, vl, plan), y)
+    for t in g.im_layer_pair_fwd(xd, xd, wd, wd, seg, heads, vl, g.PHASE_INTRA, g.PHASE_INTRA):
+        assert torch.equal(t, y)
+    halves = torch.cat([g.im_layer_fwd(xd[i:i + 2], wd, seg, heads, vl[i:i + 2], g.PHASE_INTRA) for i in (0, 2)])
+    if above:
+        check_close(to_np64(halves), to_np64(y), "bf16", pm, "halves")
+        assert not torch.equal(halves, y)   # the limit lies where this test puts it
+    else:
+        assert torch.equal(halves, y)
+    assert g.last_device_status() == (0, 0)
