@@ -66,9 +66,18 @@ cudaError_t launch_attn_bf16_n(const Geometry& g, const AttnOperands* ops, int n
   };
   // Which kernel, decided for each problem by itself, so that a launch for two problems gives the bits of two launches.
   // The tensor-memory kernels take long to set up and to hand over a work item, the mma.sync kernel takes longer per score: what
-  // counts is the number of units (128 query rows x 64 keys of one head) that the padded lengths amount to.
-  //   head_dim 16: they meet at about 110 units per SM (32 samples of (50, 500, 500), 8 heads, intra: both 46 us; one sample: 8
-  //   against 16 us; 64 samples: 83 against 77).  head_dim 32: at about 55 (16 samples, 8 heads: 34 us).
+  // counts is the number of units (128 query rows x 64 keys of one head) that the padded lengths amount to; the real lengths are on
+  // the device only.  us on mma.sync / tensor memory at B x (50, 500, 500), intra, 8 heads of 16 (a call of its own, which clears
+  // the work counter first; then a whole layer at d 128, where the first half clears it):
+  //   units per SM             56           84          112          141          225
+  //   full lengths          33.6/33.2    48.6/45.6    58.7/51.4    72.3/62.8     114/94.5
+  //   half to full          28.7/29.8    36.2/36.9    43.7/42.9    53.2/51.0    83.8/75.2
+  //   a quarter real        12.3/18.3    13.3/19.1    16.3/21.1    19.4/23.1    30.4/33.3
+  //   layer, half to full   52.7/48.8    73.9/68.9    83.5/76.6    94.1/85.1     142/127
+  //   layer, a quarter      34.6/34.9    35.5/37.1    39.0/38.8    42.5/41.6    56.7/53.2
+  // -> 110: from there on the tensor-memory kernel is no slower at half-to-full lengths nor in a layer at any; a call of its own at a
+  // quarter real loses 3 - 5 us up to 225 units.  4 heads of 32: half to full 27.7/27.6 at 42, 32.5/30.9 at 56, 63.1/47.5 at 112; a
+  // quarter 10.5/16.4, 12.9/18.4, 24.1/25.4; layer, a quarter 34.4/35.8 at 56, 41.2/41.0 at 84 -> 55.
   //   head_dim 64 is a dense contraction; there only a few short walks (at most two key tiles per row) are over sooner in the
   //   mma.sync kernel (32 x (50, 50, 50), 2 heads: 4.8 against 6.1 us; 128 samples: 14.8 against 11.5).
   //   head_dim 8: the tensor-memory kernel is slower throughout (55 against 44 us at 64 x (50, 500, 500)): a tcgen05 hand-over
