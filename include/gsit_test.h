@@ -13,8 +13,8 @@
 extern "C" {
 #endif
 
-/* Kernel selection (process-wide host state; 0 restores the defaults).  Every choice computes the same result up to
- * floating-point summation order.
+/* Kernel selection (process-wide host state; 0 restores the defaults; any other number than those below is answered with
+ * GSIT_ERR_INVALID_ARG).  Every choice computes the same result up to floating-point summation order.
  *   GSIT_ATTN_DEFAULT   head_dim 64, 32, 16: tcgen05 / tensor-memory attention for all but small problems, mma.sync attention
  *                       for those and at head_dim 8;
  *                       layer at d_model 64 / 128: fused tcgen05 halves; linear layers: tcgen05 GEMM where it applies

@@ -583,9 +583,10 @@ gsit_status gsit_test_late_write(void* dst, const void* src, size_t bytes, int32
   return from_cuda(cudaGetLastError());
 }
 
-gsit_status gsit_tune_attention(int variant) {
-  if (variant < 0) return GSIT_ERR_INVALID_ARG;
-  g_attn_variant = variant;
+gsit_status gsit_tune_attention(int choice) {
+  if (choice != GSIT_ATTN_DEFAULT && choice != GSIT_ATTN_UNFUSED && choice != GSIT_ATTN_LEGACY && choice != GSIT_ATTN_TMEM)
+    return GSIT_ERR_INVALID_ARG;
+  g_attn_variant = choice;
   return GSIT_OK;
 }
 

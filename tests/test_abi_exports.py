@@ -51,3 +51,20 @@ def test_workspace_query_needs_no_gpu():
         raise AssertionError("expected an error")
     except g.GsitError:
         pass
+
+
+def test_kernel_choice_takes_its_four_values_only():
+    import paper_2505_01068_b200 as g
+
+    try:
+        for choice in (g.ATTN_UNFUSED, g.ATTN_LEGACY, g.ATTN_TMEM, g.ATTN_DEFAULT):
+            g.tune_attention(choice)
+        for choice in (-1, 1, 2, 3, 4, 5, 6, 7, 11):
+            try:
+                g.tune_attention(choice)
+            except g.GsitError as e:
+                assert e.code == 1
+            else:
+                raise AssertionError(f"{choice} was accepted")
+    finally:
+        g.tune_attention(g.ATTN_DEFAULT)
