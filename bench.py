@@ -255,17 +255,24 @@ def run_only(args):
     vl = None if valid is None else torch.from_numpy(valid).cuda()
     d, heads = args.d or wl.d_model, args.heads or wl.heads
     gen = torch.Generator(device="cuda").manual_seed(1)
-    nsets = 3
-    if args.only == "attention":
-        bufs = [torch.randn((B, wl.L, 3, heads, d // heads), device="cuda", generator=gen).bfloat16() for _ in range(nsets)]
-        outs = [torch.empty((B, wl.L, d), device="cuda", dtype=torch.bfloat16) for _ in range(nsets)]
+    nsets, dtype = 3, args.dtype or wl.dtype
+    td = torch.bfloat16 if dtype == "bf16" else torch.float32
+    dev_w = lambda w: {k: (None if v is None else torch.from_numpy(v).cuda().to(td if k.startswith("w_") else torch.float32)) for k, v in w.items()}
+    if args.only == "stack":
+        layers = lambda n, width: [dev_w(wk.draw_layer_weights(rng, width, wl.d_ff_mult * width, dtype)) for _ in range(n)]
+        n_f, n_b, n_i, intra_heads = wl.stack
+        stack = g.GsitStack(layers(n_f, d), layers(n_b, d), layers(n_i, 2 * d), wl.seg_len, heads, intra_heads)
+        bufs = [torch.randn((B, wl.L, d), device="cuda", generator=gen) for _ in range(nsets)]
+        outs = [torch.empty((B, wl.L, 2 * d), device="cuda") for _ in range(nsets)]
+        run = lambda i: stack.forward(bufs[i], vl, out=outs[i])
+    elif args.only == "attention":
+        bufs = [torch.randn((B, wl.L, 3, heads, d // heads), device="cuda", generator=gen).to(td) for _ in range(nsets)]
+        outs = [torch.empty((B, wl.L, d), device="cuda", dtype=td) for _ in range(nsets)]
         ws = torch.empty(256, dtype=torch.uint8, device="cuda")
         run = lambda i: g.im_attention_fwd(bufs[i][:, :, 0], bufs[i][:, :, 1], bufs[i][:, :, 2], wl.seg_len, vl, args.phase,
                                            out=outs[i], workspace=ws)
     else:
-        w = wk.draw_layer_weights(rng, d, wl.d_ff_mult * d, wl.dtype)
-        wd = {k: (None if v is None else (torch.from_numpy(v).cuda().bfloat16() if (k.startswith("w_") and wl.dtype == "bf16")
-                                          else torch.from_numpy(v).cuda())) for k, v in w.items()}
+        wd = dev_w(wk.draw_layer_weights(rng, d, wl.d_ff_mult * d, dtype))
         bufs = [torch.randn((B, wl.L, d), device="cuda", generator=gen) for _ in range(nsets)]
         outs = [torch.empty((B, wl.L, d), device="cuda") for _ in range(nsets)]
         sh = g.make_shape(B, wl.seg_len, d, heads, vl, g.binding._dtype_code(wd["w_qkv"].dtype), args.phase)
@@ -456,9 +463,9 @@ def run_gpu(args):
         end.record()
         torch.cuda.synchronize()
         sec = beg.elapsed_time(end) * 1e-3 / 10
-        fl = 2.0 * wl5.batch * wl5.L * wl5.d_model * 3 * wl5.d_model
-        scaled["qkv_proj"] = {"us": sec * 1e6, "tflops": fl / sec / 1e12, "frac_tensor_peak": fl / sec / 1e12 / pk["bf16_tflops"],
-                              "note": "padded layout: all B*L rows multiplied (padded rows are zeroed in the epilogue)"}
+        fl_real = 2.0 * tok5 * wl5.d_model * 3 * wl5.d_model
+        scaled["qkv_proj"] = {"us": sec * 1e6, "tflops_real_rows": fl_real / sec / 1e12, "frac_tensor_peak": fl_real / sec / 1e12 / pk["bf16_tflops"],
+                              "real_rows": tok5, "note": "padded layout; operations of the real rows (tiles of padding are written, not multiplied)"}
         # the same projection on the packed row layout: real rows only
         cap5 = wl5.batch * wl5.L + 128
         plan5 = g.plan_rows(vl5, wl5.seg_len)
@@ -474,10 +481,9 @@ def run_gpu(args):
         end.record()
         torch.cuda.synchronize()
         sec_p = beg.elapsed_time(end) * 1e-3 / 10
-        fl_real = 2.0 * tok5 * wl5.d_model * 3 * wl5.d_model
         scaled["qkv_proj_packed"] = {"us": sec_p * 1e6, "tflops_real_rows": fl_real / sec_p / 1e12,
-                                     "padded_layout_tflops_real_rows": fl_real / sec / 1e12, "real_rows": tok5,
-                                     "note": "packed layout: real rows only, rows stored one by one instead of by TMA"}
+                                     "frac_tensor_peak": fl_real / sec_p / 1e12 / pk["bf16_tflops"], "real_rows": tok5,
+                                     "note": "packed layout: real rows only"}
         del xp5, qp5
         del vl5, xs5, qs5
         torch.cuda.empty_cache()
@@ -555,7 +561,8 @@ def main():
     ap.add_argument("--workload", type=int, default=4)
     ap.add_argument("--ref-batch", type=int, default=16, help="samples per step of the CPU oracle")
     ap.add_argument("--no-scaled", action="store_true", help="skip the extra timings (other configs, head_dim 64, length statistics)")
-    ap.add_argument("--only", choices=["attention", "layer"], help="profiler driver: launch one call a few times and exit")
+    ap.add_argument("--only", choices=["attention", "layer", "stack"], help="profiler driver: launch one call a few times and exit")
+    ap.add_argument("--dtype", choices=["bf16", "f32"], help="--only: type of weights and activations (default: the workload's)")
     ap.add_argument("--batch", type=int, default=0)
     ap.add_argument("--phase", type=int, default=0)
     ap.add_argument("--d", type=int, default=0)
