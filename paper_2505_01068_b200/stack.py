@@ -60,10 +60,9 @@ class GsitStack:
     def _workspace_need(self, Bn, d, valid_len, plan=None, capacity=0):
         """Bytes that the most demanding layer of the stack asks for (layers may differ in type and MLP width)."""
         need = 0
-        for layers, width, heads, phase in ((self.fwd, d, self.heads, B.PHASE_INTER_FWD), (self.bwd, d, self.heads, B.PHASE_INTER_BWD),
-                                            (self.intra, 2 * d, self.intra_heads, B.PHASE_INTRA)):
-            for code, d_ff in {(B._dtype_code(w["w_qkv"].dtype), int(w["w_1"].shape[0])) for w in layers}:
-                sh = B.make_shape(Bn, self.seg_len, width, heads, valid_len, code, phase, row_start=plan, capacity=capacity)
+        for layers, width, heads, phase in ((self.fwd + self.bwd, d, self.heads, B.PHASE_INTER_FWD), (self.intra, 2 * d, self.intra_heads, B.PHASE_INTRA)):
+            for t, d_ff in {(w["w_qkv"].dtype, w["w_1"].shape[0]) for w in layers}:
+                sh = B.make_shape(Bn, self.seg_len, width, heads, valid_len, B._dtype_code(t), phase, row_start=plan, capacity=capacity)
                 need = max(need, B.workspace_bytes(sh, B.CALL_LAYER, d_ff))
         return need
 
