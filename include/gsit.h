@@ -87,8 +87,9 @@ typedef struct gsit_shape {
    * gsit_plan_rows (entry 3 B = the row after the last one); valid_len must be given.  Accepted by
    * gsit_im_attention_fwd (bf16, every head_dim), gsit_im_layer_fwd (bf16, d_model 32, 64 or 128, head_dim <= 32) and gsit_im_qkv_proj
    * (bf16, d_model a multiple of 64); other calls and shapes answer GSIT_ERR_UNSUPPORTED.  A call on samples
-   * b0 .. b1 - 1 passes valid_len + 3 b0 and row_start + 3 b0 with the same matrices (rows are absolute) and reads
-   * and writes the rows of those samples only. */
+   * b0 .. b1 - 1 passes valid_len + 3 b0 and row_start + 3 b0 with the same matrices (rows are absolute) and writes the
+   * rows of those samples only -- but gsit_im_layer_fwd may also write zeros behind them, up to the end of a 128-row
+   * tile counted from the call's first row, which is what the split of gsit_plan_rows keeps free. */
   const int32_t* row_start;
   int32_t packed_capacity;  /* rows of the packed matrices (>= the plan's last entry rounded up to 128) */
 } gsit_shape;

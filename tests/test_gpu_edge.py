@@ -124,7 +124,8 @@ def test_bf16_both_kernel_families_at_every_head_width(g, choice):
 
 
 def test_attention_with_and_without_scratch_gives_the_same_bits(g):
-    """The optional scratch of gsit_im_attention_fwd only changes which SM takes which work item."""
+    """The optional scratch of gsit_im_attention_fwd only changes which SM takes which work item (of the tensor-memory kernels,
+    which test_gpu_kernel_families.py selects for this; the kernel of a problem this small does not use it)."""
     rng = np.random.default_rng(78)
     seg, B, H, hd = (50, 300, 270), 4, 8, 16
     q, k, v = (to_dev(a, "bf16") for a in wk.draw_qkv(rng, B, sum(seg), H, hd, "bf16"))

@@ -177,9 +177,9 @@ def test_cfg5_scaled_hd64_bf16(g):
                                                 (128, 8, 320, (50, 201, 93), 2), (64, 8, 192, (300, 20, 333), 2)])
 def test_layer_bf16_affine_biases_ragged(g, d, heads, d_ff, seg, B):
     """One IM layer with LayerNorm affine parameters and every bias set, ragged valid lengths, NaN in the padded input
-    rows and a row count that is not a multiple of any tile: d = 64 / 128 take the fused tcgen05 kernels, d = 32 the separate
-    LayerNorm / mma.sync linear kernels, d = 192 the separate kernels with every linear layer on the tcgen05 GEMM (bias,
-    ReLU, float output with residual, TMA-stored bf16 output)."""
+    rows and a row count that is not a multiple of any tile: d = 32 / 64 / 128 take the fused halves on row tiles at these sizes
+    (those on tcgen05: test_gpu_kernel_families.py), d = 192 the separate kernels with every linear layer on the tcgen05 GEMM
+    (bias, ReLU, float output with residual, TMA-stored bf16 output)."""
     rng = np.random.default_rng(d * 1000 + d_ff)
     x = rng.standard_normal((B, sum(seg), d), dtype=np.float32)
     w = wk.draw_layer_weights(rng, d, d_ff, "bf16", affine=True)
@@ -224,7 +224,8 @@ def test_qkv_proj_tcgen05_matches_mma_sync_kernel(g):
 
 @pytest.mark.parametrize("d,heads,d_ff", [(64, 8, 256), (128, 8, 512)])
 def test_fused_layer_tcgen05_matches_mma_sync_fused_kernels(g, d, heads, d_ff):
-    """The tcgen05 fused halves and the mma.sync fused halves (kernel choice ATTN_LEGACY) compute the same layer."""
+    """The default fused halves -- row tiles at this size, on tcgen05 in test_gpu_kernel_families.py -- and the mma.sync ones of
+    kernel choice ATTN_LEGACY compute the same layer."""
     rng = np.random.default_rng(d)
     seg, B = (50, 333, 190), 2
     x = rng.standard_normal((B, sum(seg), d), dtype=np.float32)
@@ -247,8 +248,8 @@ def test_fused_layer_tcgen05_matches_mma_sync_fused_kernels(g, d, heads, d_ff):
 
 @pytest.mark.parametrize("d,heads,d_ff", [(64, 8, 256), (64, 4, 128), (128, 8, 512), (32, 4, 128)])
 def test_layer_pair_call_equals_two_layer_calls(g, d, heads, d_ff):
-    """gsit_im_layer_pair_fwd (both ring encoders' layers of one depth in one call; one launch per kernel at d_model 64,
-    the two layers in sequence elsewhere) gives the bits of two gsit_im_layer_fwd calls, padded and packed layout, and the
+    """gsit_im_layer_pair_fwd (both ring encoders' layers of one depth in one call; one launch per kernel on row tiles, as
+    here, and at d_model 64, the two layers in sequence elsewhere) gives the bits of two gsit_im_layer_fwd calls, padded and packed layout, and the
     forward-ring member is held to the oracle."""
     rng = np.random.default_rng(d + d_ff)
     seg, B = (50, 300, 170), 3

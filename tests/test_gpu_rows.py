@@ -23,6 +23,11 @@ def g():
                                                 (64, 2, 512, (50, 300, 270), 9), (128, 8, 512, (7, 1, 1), 1), (128, 4, 320, (50, 130, 77), 6),
                                                 (128, 8, 512, (50, 300, 270), 2)])
 def test_layer_on_row_tiles(g, d, heads, d_ff, seg, B):
+    check_layer(g, d, heads, d_ff, seg, B)
+
+
+def check_layer(g, d, heads, d_ff, seg, B, tile=1):
+    """tile: in the packed layout the rows up to the end of the last tile of this many may be written (as zero)."""
     rng = np.random.default_rng(d + d_ff + B)
     L = sum(seg)
     x = rng.standard_normal((B, L, d), dtype=np.float32)
@@ -49,7 +54,7 @@ def test_layer_on_row_tiles(g, d, heads, d_ff, seg, B):
     g.pack_rows(wide[:, :, d:].contiguous(), xp, seg, vl, plan)
     yp = torch.full((cap, d), 7.0, device="cuda")
     g.im_layer_fwd(xp, wd, seg, heads, vl, g.PHASE_INTER_BWD, out=yp, row_start=plan)
-    used = int(plan[-1])
+    used = -(-int(plan[-1]) // tile) * tile
     assert bool((yp[used:] == 7.0).all())
     back = torch.empty((B, L, d), device="cuda")
     g.unpack_rows(yp, back, seg, vl, plan)
