@@ -313,7 +313,7 @@ gsit_status gsit_im_layer_fwd(const gsit_shape* shape, const gsit_layer_weights*
     return from_cuda(second(g, h.att, x, x_row_stride, h.w_o, h.b_o, h.ln2_gamma, h.ln2_beta, eps, h.w_1, h.b_1, h.w_2, h.b_2, w->d_ff, y,
                             y_row_stride, cs));
   }
-  if (!bf && fused_layer_f32_supported(g, w->d_ff)) {  // the same three launches for float operands
+  if (!bf && g_attn_variant != GSIT_ATTN_UNFUSED && fused_layer_f32_supported(g, w->d_ff)) {  // the same three launches for float operands
     auto f32 = [](const void* p) { return static_cast<const float*>(p); };
     float *fq = static_cast<float*>(qkv), *fa = static_cast<float*>(att);
     {

@@ -123,3 +123,25 @@ def test_projection_odd_widths(g, d, heads):
     ref = x.astype(np.float64) @ w.T.astype(np.float64) + b
     ref[pad_mask(seg, valid, 2)] = 0
     check_close(to_np64(qkv).reshape(ref.shape), ref, "f32", pad_mask(seg, valid, 2), f"d {d}")
+
+
+@pytest.mark.parametrize("d,heads,d_ff,B", [(32, 4, 128, 3), (64, 8, 256, 40), (128, 8, 320, 9)])
+def test_separate_kernels_on_request(g, d, heads, d_ff, B):
+    """Kernel choice ATTN_UNFUSED: the separate float kernels at widths that the fused halves cover.  Both within the float
+    tolerance of the oracle; other orders of summation, so within its sum of each other and not equal."""
+    rng = np.random.default_rng(d)
+    seg = (20, 170, 133)
+    x = rng.standard_normal((B, sum(seg), d), dtype=np.float32)
+    w = wk.draw_layer_weights(rng, d, d_ff, "f32", affine=True)
+    valid = np.stack([rng.integers(0, n + 1, size=B) for n in seg], axis=1).astype(np.int32)
+    vl, pm, wd, ys = torch.from_numpy(valid).cuda(), pad_mask(seg, valid, B), weights_to_dev(w, "f32"), []
+    for choice in (g.ATTN_DEFAULT, g.ATTN_UNFUSED):
+        g.tune_attention(choice)
+        try:
+            ys.append(to_np64(g.im_layer_fwd(to_dev(x), wd, seg, heads, vl, g.PHASE_INTRA)))
+        finally:
+            g.tune_attention(g.ATTN_DEFAULT)
+        ref = oracle.im_layer_fwd(x[:2], w, seg, heads, valid[:2], g.PHASE_INTRA)
+        check_close(ys[-1][:2], ref, "f32", pm[:2], f"choice {choice}")
+    diff = np.abs(ys[0] - ys[1]).max()
+    assert 0 < diff <= 2e-4
