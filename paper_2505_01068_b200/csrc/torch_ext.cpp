@@ -92,6 +92,9 @@ void read_segments(PyObject* seg, int32_t (&out)[3]) {
   Py_DECREF(f);
 }
 
+void require_vector(const at::Tensor* bias) {
+  require(bias == nullptr || (bias->scalar_type() == at::kFloat && bias->is_contiguous()), "bias: contiguous float32");
+}
 int32_t dtype_code(const at::Tensor& t) {
   if (t.scalar_type() == at::kFloat) return GSIT_F32;
   if (t.scalar_type() == at::kBFloat16) return GSIT_BF16;
@@ -204,6 +207,8 @@ PyObject* im_qkv_proj(PyObject* const* a) {
   const at::Tensor *bias = opt_tensor(a[2]), *valid = opt_tensor(a[5]), *out = opt_tensor(a[6]), *row_start = opt_tensor(a[7]);
   const int64_t heads = as_int(a[4]);
   require(x.is_cuda() && w.is_contiguous(), "x on the device, contiguous w_qkv");
+  require(w.scalar_type() == x.scalar_type(), "x and w_qkv of one type");  // the call reads both in the type of x
+  require_vector(bias);
   at::Tensor made;
   gsit_shape s;
   int64_t ldx;
@@ -324,6 +329,7 @@ PyObject* stack_head_fwd(PyObject* const* a) {
   require(c.is_cuda() && c.scalar_type() == at::kFloat && c.dim() == 3 && c.stride(2) == 1 && c.stride(0) == c.size(1) * c.stride(1),
           "c: float32 [B, L, dc] on the device with a uniform row stride");
   require(w.is_contiguous() && w.dim() == 2 && w.size(1) == 3 * c.size(2), "w_f: contiguous [out_features, 3 * dc]");
+  require_vector(bias);
   const gsit_shape s = make_shape(c.size(0), a[3], 16, 1, valid, dtype_code(w), GSIT_PHASE_INTRA, 0, 0.0);
   at::Tensor made;
   if (out == nullptr) made = empty({c.size(0), w.size(0)}, at::kFloat, c.device());

@@ -96,3 +96,18 @@ def test_weights_of_two_types_in_one_layer_are_refused(g):
         g.im_layer_fwd(x, dict(w[1], w_2=w[0]["w_2"]), seg, 4)
     with pytest.raises(AssertionError):
         g.im_layer_pair_fwd(x, x, w[0], w[1], seg, 4)
+
+
+def test_projection_and_read_out_refuse_other_types(g):
+    """The projection reads its weights in the type of x, biases are float32: anything else would be read past its end."""
+    seg, d = (5, 9, 3), 64
+    x, w, b = torch.randn((1, sum(seg), d), device="cuda"), torch.randn((3 * d, d), device="cuda"), torch.randn(3 * d, device="cuda")
+    g.im_qkv_proj(x, w, b, seg, 8)
+    g.im_qkv_proj(x.bfloat16(), w.bfloat16(), b, seg, 8)
+    for args in ((x, w.bfloat16(), b), (x.bfloat16(), w, b), (x, w, b.bfloat16()), (x, w, torch.randn(6 * d, device="cuda")[::2])):
+        with pytest.raises(AssertionError):
+            g.im_qkv_proj(*args, seg, 8)
+    w_f = torch.randn((7, 3 * d), device="cuda")
+    g.stack_head_fwd(x, w_f, b[:7].contiguous(), seg)
+    with pytest.raises(AssertionError):
+        g.stack_head_fwd(x, w_f, b[:7].bfloat16(), seg)
