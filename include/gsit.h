@@ -160,6 +160,21 @@ gsit_status gsit_im_layer_pair_fwd(const gsit_shape* shape_a, const gsit_shape* 
                                    int64_t x_b_row_stride, float* y_a, int64_t y_a_row_stride, float* y_b, int64_t y_b_row_stride,
                                    void* workspace, size_t workspace_bytes, gsit_stream stream);
 
+/* `depth` layers of one encoder, or of two side by side (problems = 2: the fusion encoder pair), in one call: exactly what
+ * gsit_im_layer_fwd / gsit_im_layer_pair_fwd compute layer by layer, bit for bit.  Where small row tiles serve the layers and
+ * mma.sync their attention (gsit_encoder_runs_chained), everything of a layer behind its attention and the next layer's LN1 + QKV
+ * projection go into the attention's launch, so that a layer is one launch; other shapes run layer by layer.
+ *   shapes, weights, x, x_row_stride   one per problem (weights[i][j]: layer j of problem i); the shapes as for a pair call
+ *   y, y_row_stride                    y[i][j] receives the output of layer j of problem i and is the input of layer j + 1; no y may
+ *                                      overlap an x or the y of another problem or of the next layer
+ *   workspace                          problems * gsit_workspace_bytes(shapes[0], GSIT_CALL_LAYER, largest d_ff) bytes, 256-byte aligned */
+gsit_status gsit_im_encoder_fwd(const gsit_shape* const* shapes, int32_t problems, const gsit_layer_weights* const* const* weights, int32_t depth,
+                                const float* const* x, const int64_t* x_row_stride, float* const* const* y, const int64_t* const* y_row_stride,
+                                void* workspace, size_t workspace_bytes, gsit_stream stream);
+/* 1 if layers of these shapes (one per problem) and this MLP width run as one launch each inside gsit_im_encoder_fwd (on the current
+ * device), else 0.  Such layers do no work for padding in the padded layout either, so packing rows for them gains nothing. */
+int32_t gsit_encoder_runs_chained(const gsit_shape* const* shapes, int32_t problems, int32_t d_ff);
+
 /* Packed row layout, the helpers (Section "Inner Decomposition for Efficiency": padded positions take no part in
  * the computation; here they take no memory either).  All run on the device, asynchronously on `stream`, and need no
  * host knowledge of the lengths, so a captured sequence of calls stays valid when valid_len changes.

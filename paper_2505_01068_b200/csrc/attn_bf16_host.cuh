@@ -4,20 +4,6 @@
 namespace gsit {
 namespace {
 
-// Query segments in descending order of the keys their tiles walk (longest work first), two bits per segment index.
-int segment_order(const Geometry& g, uint32_t allowed) {
-  int cost[3], ord[3] = {0, 1, 2};
-  for (int s = 0; s < 3; ++s) {
-    cost[s] = 0;
-    for (int r = 0; r < 3; ++r)
-      if ((allowed >> (3 * s + r)) & 1u) cost[s] += g.seg_len[r];
-  }
-  for (int i = 0; i < 3; ++i)
-    for (int j = i + 1; j < 3; ++j)
-      if (cost[ord[j]] > cost[ord[i]]) { const int t = ord[i]; ord[i] = ord[j]; ord[j] = t; }
-  return ord[0] | (ord[1] << 2) | (ord[2] << 4);
-}
-
 // n = 1 or 2 problems of the geometry g (g.allowed is ignored: every problem brings its own pattern).
 template <typename C>
 cudaError_t launch_one(const Geometry& g, const AttnOperands* ops, int n, int64_t row_stride, float scale, cudaStream_t st) {
@@ -39,7 +25,7 @@ cudaError_t launch_one(const Geometry& g, const AttnOperands* ops, int n, int64_
     if (e != cudaSuccess) return e;
   }
   int tiles = 0;
-  for (int s = 0; s < 3; ++s) tiles += (g.seg_len[s] + C::QT - 1) / C::QT;
+  for (int s = 0; s < 3; ++s) tiles += (g.len(s) + C::QT - 1) / C::QT;
   if ((int64_t)tiles * g.batch * n > 0x7fffffffLL) return cudaErrorNotSupported;
   const dim3 grid((unsigned)(tiles * g.batch * n), (unsigned)(g.d / CW), 1u);
   const float sl2 = scale * 1.4426950408889634f;
@@ -50,57 +36,60 @@ cudaError_t launch_one(const Geometry& g, const AttnOperands* ops, int n, int64_
 
 int g_attn_variant = 0;  // gsit_kernel_choice
 
+// Which kernel, decided for each problem by itself, so that a launch for two problems gives the bits of two launches.
+// The tensor-memory kernels take long to set up and to hand over a work item, the mma.sync kernel takes longer per score: what
+// counts is the number of units (128 query rows x 64 keys of one head) that the padded lengths amount to; the real lengths are on
+// the device only.  us on mma.sync / tensor memory at B x (50, 500, 500), intra, 8 heads of 16 (a call of its own, which clears
+// the work counter first; then a whole layer at d 128, where the first half clears it):
+//   units per SM             56           84          112          141          225
+//   full lengths          33.6/33.2    48.6/45.6    58.7/51.4    72.3/62.8     114/94.5
+//   half to full          28.7/29.8    36.2/36.9    43.7/42.9    53.2/51.0    83.8/75.2
+//   a quarter real        12.3/18.3    13.3/19.1    16.3/21.1    19.4/23.1    30.4/33.3
+//   layer, half to full   52.7/48.8    73.9/68.9    83.5/76.6    94.1/85.1     142/127
+//   layer, a quarter      34.6/34.9    35.5/37.1    39.0/38.8    42.5/41.6    56.7/53.2
+// -> 110: from there on the tensor-memory kernel is no slower at half-to-full lengths nor in a layer at any; a call of its own at a
+// quarter real loses 3 - 5 us up to 225 units.  4 heads of 32: half to full 27.7/27.6 at 42, 32.5/30.9 at 56, 63.1/47.5 at 112; a
+// quarter 10.5/16.4, 12.9/18.4, 24.1/25.4; layer, a quarter 34.4/35.8 at 56, 41.2/41.0 at 84 -> 55.
+//   head_dim 64 is a dense contraction; there only a few short walks (at most two key tiles per row) are over sooner in the
+//   mma.sync kernel (32 x (50, 50, 50), 2 heads: 4.8 against 6.1 us; 128 samples: 14.8 against 11.5).
+//   head_dim 8: the tensor-memory kernel is slower throughout (55 against 44 us at 64 x (50, 500, 500)): a tcgen05 hand-over
+//   per 64 keys of one head costs more than the 8192 exponentials it feeds.
+bool attn_uses_tensor_memory(const Geometry& g, uint32_t allowed) {
+  const int var = g_attn_variant;
+  int n_sm = 0;
+  if (sm_count_and_smem_once(nullptr, 0, &n_sm) != cudaSuccess) return false;
+  if (var == GSIT_ATTN_LEGACY || (g.hd != 64 && !attn_tcs_supported(g))) return false;
+  if (var == GSIT_ATTN_TMEM) return true;
+  if (g.hd == 8) return false;
+  int64_t units = 0;
+  int longest = 0;  // most key tiles that a row walks
+  for (int s = 0; s < 3; ++s) {
+    int kt = 0;
+    for (int r = 0; r < 3; ++r)
+      if ((allowed >> (3 * s + r)) & 1u) kt += (g.len(r) + KT - 1) / KT;
+    units += (int64_t)((g.len(s) + 127) / 128) * kt;
+    if (kt > longest) longest = kt;
+  }
+  units *= (int64_t)g.batch * g.heads;
+  if (g.hd == 64) return longest > 2 || units > 2LL * n_sm;
+  return units > (g.hd == 16 ? 110LL : 55LL) * n_sm;
+}
+
 cudaError_t launch_attn_bf16_n(const Geometry& g, const AttnOperands* ops, int n, int64_t row_stride, float scale, int* next_item,
                                cudaStream_t st, bool counter_cleared) {
   if (n < 1 || n > 2) return cudaErrorInvalidValue;
   if (g.batch > 65535 || g.d % 16 != 0) return cudaErrorNotSupported;
   const int cw = (g.d % 64 == 0) ? 64 : (g.d % 32 == 0) ? 32 : 16;
-  const int var = g_attn_variant;
   int n_sm = 0;
   cudaError_t e = sm_count_and_smem_once(nullptr, 0, &n_sm);
   if (e != cudaSuccess) return e;
   auto tiles = [&](int rows) {  // query tiles of one head of one problem
     int64_t t = 0;
-    for (int s = 0; s < 3; ++s) t += (g.seg_len[s] + rows - 1) / rows;
+    for (int s = 0; s < 3; ++s) t += (g.len(s) + rows - 1) / rows;
     return t * g.batch;
   };
-  // Which kernel, decided for each problem by itself, so that a launch for two problems gives the bits of two launches.
-  // The tensor-memory kernels take long to set up and to hand over a work item, the mma.sync kernel takes longer per score: what
-  // counts is the number of units (128 query rows x 64 keys of one head) that the padded lengths amount to; the real lengths are on
-  // the device only.  us on mma.sync / tensor memory at B x (50, 500, 500), intra, 8 heads of 16 (a call of its own, which clears
-  // the work counter first; then a whole layer at d 128, where the first half clears it):
-  //   units per SM             56           84          112          141          225
-  //   full lengths          33.6/33.2    48.6/45.6    58.7/51.4    72.3/62.8     114/94.5
-  //   half to full          28.7/29.8    36.2/36.9    43.7/42.9    53.2/51.0    83.8/75.2
-  //   a quarter real        12.3/18.3    13.3/19.1    16.3/21.1    19.4/23.1    30.4/33.3
-  //   layer, half to full   52.7/48.8    73.9/68.9    83.5/76.6    94.1/85.1     142/127
-  //   layer, a quarter      34.6/34.9    35.5/37.1    39.0/38.8    42.5/41.6    56.7/53.2
-  // -> 110: from there on the tensor-memory kernel is no slower at half-to-full lengths nor in a layer at any; a call of its own at a
-  // quarter real loses 3 - 5 us up to 225 units.  4 heads of 32: half to full 27.7/27.6 at 42, 32.5/30.9 at 56, 63.1/47.5 at 112; a
-  // quarter 10.5/16.4, 12.9/18.4, 24.1/25.4; layer, a quarter 34.4/35.8 at 56, 41.2/41.0 at 84 -> 55.
-  //   head_dim 64 is a dense contraction; there only a few short walks (at most two key tiles per row) are over sooner in the
-  //   mma.sync kernel (32 x (50, 50, 50), 2 heads: 4.8 against 6.1 us; 128 samples: 14.8 against 11.5).
-  //   head_dim 8: the tensor-memory kernel is slower throughout (55 against 44 us at 64 x (50, 500, 500)): a tcgen05 hand-over
-  //   per 64 keys of one head costs more than the 8192 exponentials it feeds.
-  auto tensor_memory = [&](uint32_t allowed) {
-    if (var == GSIT_ATTN_LEGACY || (g.hd != 64 && !attn_tcs_supported(g))) return false;
-    if (var == GSIT_ATTN_TMEM) return true;
-    if (g.hd == 8) return false;
-    int64_t units = 0;
-    int longest = 0;  // most key tiles that a row walks
-    for (int s = 0; s < 3; ++s) {
-      int kt = 0;
-      for (int r = 0; r < 3; ++r)
-        if ((allowed >> (3 * s + r)) & 1u) kt += (g.seg_len[r] + KT - 1) / KT;
-      units += (int64_t)((g.seg_len[s] + 127) / 128) * kt;
-      if (kt > longest) longest = kt;
-    }
-    units *= (int64_t)g.batch * g.heads;
-    if (g.hd == 64) return longest > 2 || units > 2LL * n_sm;
-    return units > (g.hd == 16 ? 110LL : 55LL) * n_sm;
-  };
-  const bool tm = tensor_memory(ops[0].allowed);
-  if (n == 2 && tm != tensor_memory(ops[1].allowed)) {
+  const bool tm = attn_uses_tensor_memory(g, ops[0].allowed);
+  if (n == 2 && tm != attn_uses_tensor_memory(g, ops[1].allowed)) {
     for (int i = 0; i < n; ++i)
       if ((e = launch_attn_bf16_n(g, ops + i, 1, row_stride, scale, nullptr, st)) != cudaSuccess) return e;
     return cudaSuccess;

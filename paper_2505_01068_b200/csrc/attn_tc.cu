@@ -71,12 +71,12 @@ __device__ __forceinline__ Item decode_item(const Geometry& g, int w, int tiles_
   int s = 0;
 #pragma unroll
   for (int ss = 0; ss < 2; ++ss) {
-    const int nts = (g.seg_len[s] + TQ - 1) / TQ;
+    const int nts = (g.len(s) + TQ - 1) / TQ;
     if (tile >= nts) { tile -= nts; ++s; }
   }
   it.s = s;
   it.q0 = tile * TQ;
-  const int in_seg = min(TQ, g.seg_len[s] - it.q0);
+  const int in_seg = min(TQ, g.len(s) - it.q0);
   const int q_real_all = max(0, min(in_seg, valid_rows(g, it.b, s) - it.q0));
   // rows of the tile this CTA writes: in the padded layout all that belong to the segment (padding as +0); in the packed
   // layout only the real ones exist -- what follows them in memory is another segment
@@ -135,7 +135,7 @@ __device__ __forceinline__ Item fetch_item(const WaitCtx& wc, uint32_t base, int
 
 __global__ void __launch_bounds__(TC_THREADS, 2)
 attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                    const __grid_constant__ CUtensorMap tmV, const Geometry g, __nv_bfloat16* __restrict__ out,
+                    const __grid_constant__ CUtensorMap tmV, const __grid_constant__ Geometry g, __nv_bfloat16* __restrict__ out,
                     float* __restrict__ lse, const float sl2 /* scale * log2(e) */, const int tiles_per_sample,
                     const int n_items) {
   extern __shared__ uint8_t smem_raw[];
@@ -273,7 +273,7 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       const Item it = fetch_item(wc, base, k, lane);
       const int64_t grow = (int64_t)it.grow0 + r;
       uint4* dst = reinterpret_cast<uint4*>(out + grow * g.d + it.h * HD64);
-      float* lse_row = (lse != nullptr) ? lse + ((int64_t)it.b * g.heads + it.h) * g.L + g.seg_off[it.s] + it.q0 + r : nullptr;
+      float* lse_row = (lse != nullptr) ? lse + ((int64_t)it.b * g.heads + it.h) * g.L + g.off(it.s) + it.q0 + r : nullptr;
       if (it.T == 0) {  // nothing to attend (padding rows only, or an empty key set): exact zeros, lse = -inf
         if (r < it.rows_in_tile) {
 #pragma unroll
@@ -432,7 +432,7 @@ cudaError_t launch_attn_tc_hd64(const Geometry& g, const __nv_bfloat16* q, const
     if (e != cudaSuccess) return e;
   }
   int tiles = 0;
-  for (int s = 0; s < 3; ++s) tiles += (g.seg_len[s] + TQ - 1) / TQ;
+  for (int s = 0; s < 3; ++s) tiles += (g.len(s) + TQ - 1) / TQ;
   const int64_t n_items = (int64_t)tiles * g.heads * g.batch;
   if (n_items > 0x7fffffffLL) return cudaErrorNotSupported;
   const unsigned grid = (unsigned)((n_items < 2 * n_sm) ? n_items : 2 * n_sm);  // two resident CTAs per SM

@@ -104,7 +104,7 @@ struct SProblem {
 };
 constexpr int WHICH_SHIFT = 30;  // the problem index rides in bit 30 of the item's slice field
 
-__device__ __forceinline__ SItem decode_item(const Geometry& g, int w, int slices, int seg_order, int which) {
+__device__ __forceinline__ SItem decode_item(const Geometry& g, uint32_t allowed, int w, int slices, int seg_order, int which) {
   SItem it;
   it.b = w % g.batch;
   int t = w / g.batch;
@@ -112,17 +112,17 @@ __device__ __forceinline__ SItem decode_item(const Geometry& g, int w, int slice
   int tile = t / slices, s = seg_order & 3;
 #pragma unroll
   for (int rank = 0; rank < 2; ++rank) {
-    const int nts = (g.seg_len[s] + SQ - 1) / SQ;
+    const int nts = (g.len(s) + SQ - 1) / SQ;
     if (tile >= nts) { tile -= nts; s = (seg_order >> (2 * rank + 2)) & 3; }
   }
   it.s = s;
   it.q0 = tile * SQ;
-  const int in_seg = min(SQ, g.seg_len[s] - it.q0);
+  const int in_seg = min(SQ, g.len(s) - it.q0);
   const int q_real_all = max(0, min(in_seg, valid_rows(g, it.b, s) - it.q0));
   it.rows_in_tile = (g.row_start != nullptr) ? q_real_all : in_seg;
-  it.kn0 = ((g.allowed >> (3 * s + 0)) & 1u) ? valid_rows(g, it.b, 0) : 0;
-  it.kn1 = ((g.allowed >> (3 * s + 1)) & 1u) ? valid_rows(g, it.b, 1) : 0;
-  it.kn2 = ((g.allowed >> (3 * s + 2)) & 1u) ? valid_rows(g, it.b, 2) : 0;
+  it.kn0 = ((allowed >> (3 * s + 0)) & 1u) ? valid_rows(g, it.b, 0) : 0;
+  it.kn1 = ((allowed >> (3 * s + 1)) & 1u) ? valid_rows(g, it.b, 1) : 0;
+  it.kn2 = ((allowed >> (3 * s + 2)) & 1u) ? valid_rows(g, it.b, 2) : 0;
   it.nk0 = (it.kn0 + SK - 1) / SK;
   it.nk1 = (it.kn1 + SK - 1) / SK;
   const int nk2 = (it.kn2 + SK - 1) / SK;
@@ -178,7 +178,7 @@ __device__ __forceinline__ SItem fetch_item(const WaitCtx& wc, uint32_t bars, in
 
 template <int HD>
 __global__ void __launch_bounds__(S_THREADS, S_CTAS_PER_SM)
-attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ SProblem prob1, const Geometry g0,
+attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ SProblem prob1, const __grid_constant__ Geometry g,
                 const float sl2 /* scale * log2(e) */, const int slices, const int n_items /* of all problems */,
                 const int problems, int* __restrict__ next_item /* zeroed counter, or nullptr = static round robin */) {
   using C = SCfg<HD>;
@@ -187,7 +187,6 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t sQ = base, sK = base + C::OFF_K, sV = base + C::OFF_V, bars = base + C::OFF_BAR;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const Geometry& g = g0;
   const WaitCtx wc{g.status, bars + B_GAVE_UP};
 
   // ---- set-up, once per CTA: barriers, the zero blocks of the Q layout, tensor memory ----
@@ -221,12 +220,19 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
     for (int i = tid; i < 2 * 128; i += S_THREADS) st_shared_v4(sQ + (i >> 7) * S_QBUF + 2048 + (i & 127) * 16, 0, 0, 0, 0);
     fence_async_smem();
   }
+  if (tid < 2 && tid < problems) {
+    const SProblem& pr = tid ? prob1 : prob0;
+    map_early(pr.tmQ);
+    map_early(pr.tmK);
+    map_early(pr.tmV);
+  }
   if (warp == 1) tmem_alloc(bars + B_TMEM_SLOT, S_TMEM_COLS);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   uint32_t tmem;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(bars + B_TMEM_SLOT) : "memory");
+  load_params_early(g, next_item);
   grid_dep_wait();
   grid_dep_launch();
 
@@ -251,9 +257,7 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
       }
       const int which = (problems == 2) ? (w & 1) : 0;
       const SProblem& prob = which ? prob1 : prob0;
-      Geometry g = g0;
-      g.allowed = prob.allowed;
-      SItem it = decode_item(g, (problems == 2) ? (w >> 1) : w, slices, prob.seg_order, which);
+      SItem it = decode_item(g, prob.allowed, (problems == 2) ? (w >> 1) : w, slices, prob.seg_order, which);
       publish_item(bars, it, k, lane);
       if (it.T == 0) continue;
       it.c &= (1 << WHICH_SHIFT) - 1;
@@ -367,7 +371,7 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
       __nv_bfloat16* __restrict__ out = prob.out;
       float* __restrict__ lse = prob.lse;
       uint4* dst = reinterpret_cast<uint4*>(out + grow * g.d + slice * C::SLW + h * HD);
-      float* lse_row = (lse != nullptr) ? lse + ((int64_t)it.b * g.heads + slice * 2 + h) * g.L + g.seg_off[it.s] + it.q0 + r : nullptr;
+      float* lse_row = (lse != nullptr) ? lse + ((int64_t)it.b * g.heads + slice * 2 + h) * g.L + g.off(it.s) + it.q0 + r : nullptr;
       const bool warp_active = (wq << 5) < it.q_real;  // some row of this warp receives a result
       if (it.T == 0 || !warp_active) {
         // nothing to compute for these rows (padding only, or an empty key set): exact zeros, lse = -inf.  A warp without
@@ -603,7 +607,7 @@ cudaError_t launch_tcs(const Geometry& g, const AttnOperands* ops, int n, int64_
     for (int s = 0; s < 3; ++s) {
       cost[s] = 0;
       for (int r = 0; r < 3; ++r)
-        if ((ops[i].allowed >> (3 * s + r)) & 1u) cost[s] += g.seg_len[r];
+        if ((ops[i].allowed >> (3 * s + r)) & 1u) cost[s] += g.len(r);
     }
     for (int a = 0; a < 3; ++a)
       for (int b = a + 1; b < 3; ++b)
@@ -615,7 +619,7 @@ cudaError_t launch_tcs(const Geometry& g, const AttnOperands* ops, int n, int64_
   cudaError_t e = sm_count_and_smem_once(reinterpret_cast<const void*>(attn_tcs_kernel<HD>), C::SMEM, &n_sm);
   if (e != cudaSuccess) return e;
   int tiles = 0;
-  for (int s = 0; s < 3; ++s) tiles += (g.seg_len[s] + SQ - 1) / SQ;
+  for (int s = 0; s < 3; ++s) tiles += (g.len(s) + SQ - 1) / SQ;
   const int slices = g.d / C::SLW;
   const int64_t n_items = (int64_t)tiles * slices * g.batch * n;
   if (n_items > 0x3fffffffLL || slices >= (1 << WHICH_SHIFT)) return cudaErrorNotSupported;

@@ -21,24 +21,26 @@ struct Geometry {
   // segment s of sample b in a [capacity, d] matrix that holds real rows only, entry 3 B is the row after the last one.
   const int32_t* row_start;
   int capacity;              // rows of the packed matrices (host value, for the tensor maps)
+  __host__ __device__ __forceinline__ int len(int s) const { return seg_len[s]; }
+  __host__ __device__ __forceinline__ int off(int s) const { return seg_off[s]; }
 };
 
 __device__ __forceinline__ void raise_flag(const Geometry& g, unsigned int f) { atomicOr(g.status, f); }
 
 // Real-row count of segment s in sample b, clamped to [0, seg_len[s]].
 __device__ __forceinline__ int valid_rows(const Geometry& g, int b, int s) {
-  if (g.valid_len == nullptr) return g.seg_len[s];
+  if (g.valid_len == nullptr) return g.len(s);
   int n = g.valid_len[3 * b + s];
-  if (n < 0 || n > g.seg_len[s]) {
+  if (n < 0 || n > g.len(s)) {
     raise_flag(g, GSIT_DEVFLAG_CLAMPED);
-    n = n < 0 ? 0 : g.seg_len[s];
+    n = n < 0 ? 0 : g.len(s);
   }
   return n;
 }
 
 // First row of segment s of sample b in the activation matrices, and the range of rows that belongs to this problem.
 __device__ __forceinline__ int seg_row0(const Geometry& g, int b, int s) {
-  return (g.row_start != nullptr) ? g.row_start[3 * b + s] : b * g.L + g.seg_off[s];
+  return (g.row_start != nullptr) ? g.row_start[3 * b + s] : b * g.L + g.off(s);
 }
 __device__ __forceinline__ int rows_begin(const Geometry& g) { return (g.row_start != nullptr) ? g.row_start[0] : 0; }
 __device__ __forceinline__ int rows_end(const Geometry& g) {
@@ -56,7 +58,7 @@ __device__ __forceinline__ bool row_is_real(const Geometry& g, int64_t row) {
   const int b = (int)(row / g.L);
   const int p = (int)(row - (int64_t)b * g.L);
   const int s = segment_of(g, p);
-  return (p - g.seg_off[s]) < valid_rows(g, b, s);
+  return (p - g.off(s)) < valid_rows(g, b, s);
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -120,6 +122,7 @@ struct AttnOperands {
   float* lse;
   uint32_t allowed;
 };
+bool attn_uses_tensor_memory(const Geometry& g, uint32_t allowed);  // which kernel family a problem gets
 cudaError_t launch_attn_bf16_n(const Geometry& g, const AttnOperands* ops, int n, int64_t row_stride, float scale, int* next_item,
                                cudaStream_t st, bool counter_cleared = false);
 // bf16 attention, mma.sync tiles fed by TMA (attn_bf16.cu); returns cudaErrorNotSupported for shapes it lacks
@@ -207,6 +210,18 @@ bool fused_rows_supported(const Geometry& g, int d_ff);
 bool fused_rows_preferred(const Geometry& g);
 cudaError_t launch_ln_qkv_rows(const Geometry& g, const FusedHalfArgs* h, int n, float eps, int* zero_word, cudaStream_t st);
 cudaError_t launch_proj_mlp_rows(const Geometry& g, const FusedHalfArgs* h, int n, float eps, int d_ff, cudaStream_t st);
+
+// Attention and second half of a layer, and the first half of the next one, in one launch for one or two problems of one geometry
+// (attn_mlp_rows.cu): qkv is the projection [rows, 3 d] the attention reads; of h, x is the layer's input, ln2 / w_o / w_1 / w_2 its
+// second half, y its output, and ln1 / w_qkv the next layer's first half, which writes h.qkv (another buffer than qkv; null: none).
+struct LayerTailArgs {
+  const __nv_bfloat16* qkv;
+  FusedHalfArgs h;
+  uint32_t allowed;
+};
+bool layer_tail_supported(const Geometry& g, int d_ff);
+bool layer_tail_preferred(const Geometry& g, const uint32_t* allowed, int n);
+cudaError_t launch_layer_tail(const Geometry& g, const LayerTailArgs* args, int n, float scale, float eps, float next_eps, int d_ff, cudaStream_t st);
 
 // ... and at d_model 128 (d_ff <= 512), with the MLP weights streamed in chunks (fused_layer_tc128.cu)
 bool fused_layer_tc128_supported(const Geometry& g, int d_ff);

@@ -99,7 +99,7 @@ struct LnQkvArgs {
 };
 
 __global__ void __launch_bounds__(T_THREADS, 2)
-ln_qkv_tc_kernel(const __grid_constant__ LnQkvArgs arg0, const __grid_constant__ LnQkvArgs arg1, const Geometry g,
+ln_qkv_tc_kernel(const __grid_constant__ LnQkvArgs arg0, const __grid_constant__ LnQkvArgs arg1, const __grid_constant__ Geometry g,
                  const float eps, const int problems, int* const zero_word) {
   using namespace qk;
   const int which = (problems == 2) ? (int)(blockIdx.x & 1u) : 0;
@@ -136,6 +136,7 @@ ln_qkv_tc_kernel(const __grid_constant__ LnQkvArgs arg0, const __grid_constant__
   tc_fence_after();
   uint32_t tmem;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(bars + SLOT) : "memory");
+  load_params_early(g);
   grid_dep_wait();  // the weights, too, are read behind it: this kernel may be the first of a call, right after the one that wrote them
   grid_dep_launch();
   const int row_base = rows_begin(g), rows = rows_end(g);  // this problem's rows of the activation matrices
@@ -277,7 +278,7 @@ struct ProjMlpArgs {
 };
 
 __global__ void __launch_bounds__(T_THREADS8, 1)
-proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_constant__ ProjMlpArgs arg1, const Geometry g,
+proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_constant__ ProjMlpArgs arg1, const __grid_constant__ Geometry g,
                    const float eps, const int d_ff, const int problems) {
   using namespace pm;
   const int which = (problems == 2) ? (int)(blockIdx.x & 1u) : 0;
@@ -332,6 +333,7 @@ proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_consta
     }
     __syncwarp();
   }
+  load_params_early(g);
   grid_dep_wait();
   grid_dep_launch();
   const int row_base = rows_begin(g), rows = rows_end(g);  // this problem's rows of the activation matrices

@@ -42,7 +42,7 @@ static_assert(SMEM <= 227 * 1024, "shared memory budget");
 
 __global__ void __launch_bounds__(T_THREADS8, 1)
 ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
-                    const __grid_constant__ CUtensorMap tmOut, const Geometry g, const float* __restrict__ gamma,
+                    const __grid_constant__ CUtensorMap tmOut, const __grid_constant__ Geometry g, const float* __restrict__ gamma,
                     const float* __restrict__ beta, const float eps, const float* __restrict__ bias, int* const zero_word) {
   using namespace qk2;
   extern __shared__ uint8_t smem_raw[];
@@ -73,6 +73,7 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
   tc_fence_after();
   uint32_t tmem;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(bars + SLOT) : "memory");
+  load_params_early(g);
   grid_dep_wait();  // the weights, too, are read behind it: this kernel may be the first of a call, right after the one that wrote them
   grid_dep_launch();
   const int row_base = rows_begin(g), rows = rows_end(g);  // this problem's rows of the activation matrices
@@ -227,7 +228,7 @@ static_assert(SMEM <= 227 * 1024, "shared memory budget");
 __global__ void __launch_bounds__(T_THREADS8, 1)
 proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_constant__ CUtensorMap tmX,
                       const __grid_constant__ CUtensorMap tmWo, const __grid_constant__ CUtensorMap tmW1,
-                      const __grid_constant__ CUtensorMap tmW2, const Geometry g, const float* __restrict__ bo,
+                      const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ Geometry g, const float* __restrict__ bo,
                       const float* __restrict__ gamma, const float* __restrict__ beta, const float eps,
                       const float* __restrict__ b1, const float* __restrict__ b2, const int d_ff, float* __restrict__ y,
                       const int64_t ldy) {
@@ -284,6 +285,7 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
     }
     __syncwarp();
   }
+  load_params_early(g);
   grid_dep_wait();
   grid_dep_launch();
   const int row_base = rows_begin(g), rows = rows_end(g);  // this problem's rows of the activation matrices

@@ -4,47 +4,13 @@
 //
 // A CTA of eight warps takes 16 R rows through the whole half.  What bounds the halves at these widths is not arithmetic but
 // latency: the chain load - LayerNorm - product - product - product - store of a tile, and how many tiles are in flight to
-// cover it.  So tiles are small and many, nothing is handed from role to role, and the weights take the shortest way there
-// is: each lane loads its B fragments straight from global memory as 16-byte pieces (all CTAs read the same few tens of
-// kilobytes: they stay in L1), no shared-memory staging, no barrier per weight chunk.  For that the k index of a product is
-// permuted, the same way in both operands: lane t of a quad holds k = 32 i + 8 t .. + 7 of its rows, which serve two
-// m16n8k16 steps.  The A operand lies in shared memory as bf16 rows in 16-byte pieces, swizzled so that the fragment reads
-// (16 bytes per lane) and the writes from accumulators (4 bytes per lane) are both free of bank conflicts.
+// cover it.  So tiles are small and many, and nothing is handed from role to role.
 // Row statistics of LN2 are merged over the warps with the pairwise update of Chan, Golub and LeVeque.
 // A row's result does not depend on R, on the tile it falls into or on the layout.
-#include "common.cuh"
-#include "ptx.cuh"
+#include "rows_tile.cuh"
 
 namespace gsit {
 namespace {
-
-constexpr int THREADS = 256, WARPS = 8, ROWS_MAX_FF = 512;
-
-__device__ __forceinline__ void mma(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-// Byte offset of 16-byte piece c of row r in a tile of K bf16 columns.
-template <int K>
-__device__ __forceinline__ uint32_t piece(int r, int c) {
-  if constexpr (K == 32) return (uint32_t)(r * 64 + ((c ^ ((r >> 1) & 3)) << 4));
-  else return (uint32_t)(r * (K * 2) + ((c ^ (((r & 1) << 2) | ((r >> 1) & 3))) << 4));
-}
-__device__ __forceinline__ uint4 lds16(uint32_t a) {
-  uint4 v;
-  asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
-  return v;
-}
-__device__ __forceinline__ void sts4(uint32_t a, uint32_t v) { asm volatile("st.shared.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
-__device__ __forceinline__ void sts8(uint32_t a, uint32_t v, uint32_t w) { asm volatile("st.shared.v2.b32 [%0], {%1,%2};" ::"r"(a), "r"(v), "r"(w) : "memory"); }
-
-// Two k-steps (32 k's): rows of the slab at `lo` (row g) and `hi` (row g + 8), weights w of one n-tile.
-__device__ __forceinline__ void step(float (&c)[4], const uint4& lo, const uint4& hi, const uint4& w) {
-  mma(c, lo.x, hi.x, lo.y, hi.y, w.x, w.y);
-  mma(c, lo.z, hi.z, lo.w, hi.w, w.z, w.w);
-}
-__device__ __forceinline__ uint4 ldw(const __nv_bfloat16* p) { return __ldg(reinterpret_cast<const uint4*>(p)); }
 
 // Rows of this CTA: m0 .. m0 + 16 R - 1, those at or past `end` are not its own.
 struct Rows { int m0, end; };
@@ -57,7 +23,7 @@ __device__ __forceinline__ bool is_real(const Geometry& g, int m, int end) {
   if (m >= end) return false;
   if (g.row_start != nullptr) return true;  // packed layout: every row is
   const int b = m / g.L, p = m - b * g.L, s = segment_of(g, p);
-  return p - g.seg_off[s] < valid_rows(g, b, s);
+  return p - g.off(s) < valid_rows(g, b, s);
 }
 
 struct Pair { FusedHalfArgs a[2]; };
@@ -65,97 +31,31 @@ struct Pair { FusedHalfArgs a[2]; };
 // ------------------------------------------------------------------------------------------------ LN1 + QKV
 template <int D, int R>
 __global__ void __launch_bounds__(THREADS)
-ln_qkv_rows_kernel(const Geometry g, const __grid_constant__ Pair pair, const float eps, int* __restrict__ zero_word) {
-  constexpr int BM = 16 * R, V = D / 32;            // rows of a tile; float4s per thread of a row (eight threads)
-  constexpr int GROUPS = 3 * D / 16, UNITS = GROUPS * R;
+ln_qkv_rows_kernel(const __grid_constant__ Geometry g, const __grid_constant__ Pair pair, const float eps, int* __restrict__ zero_word) {
+  constexpr int BM = 16 * R;
   __shared__ __align__(128) uint8_t sH[BM * D * 2];
   const FusedHalfArgs& a = pair.a[blockIdx.y];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gr = lane >> 2, t = lane & 3;
+  const int tid = threadIdx.x;
   const uint32_t h = smem_u32(sH);
+  ptx::load_params_early(g, a, zero_word);
   ptx::grid_dep_wait();
   ptx::grid_dep_launch();
   if (zero_word != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *zero_word = 0;
   const Rows rows = rows_of<BM>(g);
   if (rows.m0 >= rows.end) return;
-  // LayerNorm, eight threads per row, 32 rows at a time
-  bool any = false;
-#pragma unroll
-  for (int pass = 0; pass < (BM + 31) / 32; ++pass) {
-    const int r = pass * 32 + (tid >> 3), m = rows.m0 + r;
-    const bool real = r < BM && is_real(g, m, rows.end);
-    any |= real;
-    float4 v[V];
-    float s = 0.f;
-#pragma unroll
-    for (int c = 0; c < V; ++c) v[c] = real ? *reinterpret_cast<const float4*>(a.x + (int64_t)m * a.ldx + 4 * ((tid & 7) + 8 * c)) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int c = 0; c < V; ++c) s += (v[c].x + v[c].y) + (v[c].z + v[c].w);
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    const float mean = s * (1.f / D);
-    float q = 0.f;
-#pragma unroll
-    for (int c = 0; c < V; ++c) {
-      v[c].x -= mean; v[c].y -= mean; v[c].z -= mean; v[c].w -= mean;
-      q += fmaf(v[c].x, v[c].x, v[c].y * v[c].y) + fmaf(v[c].z, v[c].z, v[c].w * v[c].w);
-    }
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-    const float rstd = rsqrtf(q * (1.f / D) + eps);
-    if (r < BM) {
-#pragma unroll
-      for (int c = 0; c < V; ++c) {
-        const int e = 4 * ((tid & 7) + 8 * c);
-        const float4 ga = a.ln1_gamma != nullptr ? make_float4(a.ln1_gamma[e], a.ln1_gamma[e + 1], a.ln1_gamma[e + 2], a.ln1_gamma[e + 3]) : make_float4(1.f, 1.f, 1.f, 1.f);
-        const float4 be = a.ln1_beta != nullptr ? make_float4(a.ln1_beta[e], a.ln1_beta[e + 1], a.ln1_beta[e + 2], a.ln1_beta[e + 3]) : make_float4(0.f, 0.f, 0.f, 0.f);
-        const uint32_t lo = ptx::pack_bf16(fmaf(v[c].x * rstd, ga.x, be.x), fmaf(v[c].y * rstd, ga.y, be.y));
-        const uint32_t hi = ptx::pack_bf16(fmaf(v[c].z * rstd, ga.z, be.z), fmaf(v[c].w * rstd, ga.w, be.w));
-        sts8(h + piece<D>(r, e >> 3) + (e & 4) * 2, real ? lo : 0u, real ? hi : 0u);
-      }
-    }
-  }
+  auto real = [&](int r) { return is_real(g, rows.m0 + r, rows.end); };
+  const bool any = normalise_tile<D, BM>(a.ln1_gamma, a.ln1_beta, eps, h, tid, real,
+                                         [&](int r, int e) { return *reinterpret_cast<const float4*>(a.x + (int64_t)(rows.m0 + r) * a.ldx + e); });
   const bool work = __syncthreads_or(any) != 0;
-  // units of 16 columns x one slab of 16 rows.  The two n-tiles of a unit take their columns interleaved, so that a lane ends up
-  // with four consecutive ones: 8-byte stores, 32-byte sectors written whole.
-#pragma unroll
-  for (int u = warp; u < UNITS; u += WARPS) {
-    const int grp = u % GROUPS, slab = u / GROUPS, n0 = grp * 16;
-    float c[2][4] = {};
-    if (work) {
-      uint4 w[2][D / 32];
-#pragma unroll
-      for (int j = 0; j < 2; ++j)
-#pragma unroll
-        for (int k = 0; k < D / 32; ++k) w[j][k] = ldw(a.w_qkv + (int64_t)(n0 + 4 * (gr >> 1) + (gr & 1) + 2 * j) * D + 32 * k + 8 * t);
-#pragma unroll
-      for (int k = 0; k < D / 32; ++k) {
-        const uint4 lo = lds16(h + piece<D>(slab * 16 + gr, 4 * k + t)), hi = lds16(h + piece<D>(slab * 16 + gr + 8, 4 * k + t));
-        step(c[0], lo, hi, w[0][k]);
-        step(c[1], lo, hi, w[1][k]);
-      }
-    }
-    float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (a.b_qkv != nullptr) {
-      const float* p = a.b_qkv + n0 + 4 * t;
-      b = make_float4(p[0], p[1], p[2], p[3]);
-    }
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      const int m = rows.m0 + slab * 16 + gr + 8 * half;
-      if (m >= rows.end) continue;
-      const bool real = work && is_real(g, m, rows.end);
-      const uint32_t lo = ptx::pack_bf16(c[0][2 * half] + b.x, c[0][2 * half + 1] + b.y), hi = ptx::pack_bf16(c[1][2 * half] + b.z, c[1][2 * half + 1] + b.w);
-      *reinterpret_cast<uint2*>(a.qkv + (int64_t)m * (3 * D) + n0 + 4 * t) = real ? make_uint2(lo, hi) : make_uint2(0u, 0u);
-    }
-  }
+  qkv_units<D, R>([&](int row, int k) { return ldw(a.w_qkv + (int64_t)row * D + 32 * k + 8 * (tid & 3)); }, a.b_qkv, a.qkv, rows.m0, h, work, tid, [&](int r) { return rows.m0 + r < rows.end; }, real);
 }
 
 // ------------------------------------------------------------------------------------------------ out-projection + LN2 + MLP
 template <int D, int R>
-__global__ void __launch_bounds__(THREADS, R <= 2 && D <= 64 ? 2 : 1)
-proj_mlp_rows_kernel(const Geometry g, const __grid_constant__ Pair pair, const float eps, const int d_ff) {
+__global__ void __launch_bounds__(THREADS, R <= 2 && D <= 64 ? (R == 1 ? 3 : 2) : 1)
+proj_mlp_rows_kernel(const __grid_constant__ Geometry g, const __grid_constant__ Pair pair, const float eps, const int d_ff) {
   constexpr int BM = 16 * R, KD = D / 32;
-  constexpr int WN = D / 8 < WARPS ? D / 8 : WARPS, WM = WARPS / WN;   // warps along the D output columns, along the slabs
+  constexpr int WN = D / 8 < ROW_WARPS ? D / 8 : ROW_WARPS, WM = ROW_WARPS / WN;   // warps along the D output columns, along the slabs
   constexpr int NT = D / 8 / WN, SW = R / WM;                          // n-tiles and slabs of a warp in the D-wide products
   static_assert(R % WM == 0, "slabs");
   extern __shared__ __align__(128) uint8_t sm[];
@@ -171,6 +71,7 @@ proj_mlp_rows_kernel(const Geometry g, const __grid_constant__ Pair pair, const 
   for (int j = 0; j < NT; ++j)
 #pragma unroll
     for (int k = 0; k < KD; ++k) wo[j][k] = ldw(a.w_o + (int64_t)((wn * NT + j) * 8 + gr) * D + 32 * k + 8 * t);
+  ptx::load_params_early(g, a);
   ptx::grid_dep_wait();
   ptx::grid_dep_launch();
   const Rows rows = rows_of<BM>(g);
@@ -279,9 +180,9 @@ proj_mlp_rows_kernel(const Geometry g, const __grid_constant__ Pair pair, const 
 #pragma unroll
     for (int k = 0; k < KD; ++k) w[k] = ldw(a.w_1 + (int64_t)(warp * 8 + gr) * D + 32 * k + 8 * t);
 #pragma unroll 2
-    for (int nt = warp; nt < tiles; nt += WARPS) {
+    for (int nt = warp; nt < tiles; nt += ROW_WARPS) {
       uint4 next[KD];
-      const int ahead = nt + WARPS < tiles ? nt + WARPS : nt;
+      const int ahead = nt + ROW_WARPS < tiles ? nt + ROW_WARPS : nt;
 #pragma unroll
       for (int k = 0; k < KD; ++k) next[k] = ldw(a.w_1 + (int64_t)(ahead * 8 + gr) * D + 32 * k + 8 * t);
       const int n = nt * 8 + 2 * t;
@@ -304,9 +205,18 @@ proj_mlp_rows_kernel(const Geometry g, const __grid_constant__ Pair pair, const 
   __syncthreads();
 
   // ---- y = y1 + f W_2^T + b_2 ----
-  float acc[SW][NT][4] = {};
+  // (the two halves of the hidden units are summed by themselves, because elsewhere two warps share them)
+  float acc[SW][NT][4] = {}, lower[SW][NT][4];
 #pragma unroll 4
   for (int k = 0; k < d_ff / 32; ++k) {
+    if (k == d_ff / 64) {
+#pragma unroll
+      for (int s = 0; s < SW; ++s)
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) { lower[s][j][i] = acc[s][j][i]; acc[s][j][i] = 0.f; }
+    }
     uint4 w[NT];
 #pragma unroll
     for (int j = 0; j < NT; ++j) w[j] = ldw(w2[j] + 32 * k);
@@ -318,6 +228,12 @@ proj_mlp_rows_kernel(const Geometry g, const __grid_constant__ Pair pair, const 
       for (int j = 0; j < NT; ++j) step(acc[s][j], lo, hi, w[j]);
     }
   }
+#pragma unroll
+  for (int s = 0; s < SW; ++s)
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[s][j][i] = lower[s][j][i] + acc[s][j][i];
 #pragma unroll
   for (int s = 0; s < SW; ++s)
 #pragma unroll

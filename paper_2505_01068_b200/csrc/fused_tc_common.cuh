@@ -54,7 +54,7 @@ __device__ __forceinline__ bool row_real32(const Geometry& g, int row, int rows)
   if (g.row_start != nullptr) return true;  // packed layout: every row below the end is taken as real
   const int b = row / g.L, p = row - b * g.L;
   const int sgm = segment_of(g, p);
-  return (p - g.seg_off[sgm]) < valid_rows(g, b, sgm);
+  return (p - g.off(sgm)) < valid_rows(g, b, sgm);
 }
 
 // Kernels whose rows are split between two threads -- the same TMEM lane in warps w and w + 4, each owning half of the

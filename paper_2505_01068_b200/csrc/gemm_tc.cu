@@ -67,8 +67,8 @@ __device__ __forceinline__ bool tile_real(const Geometry& g, int m0, int rows, i
   const int end = min(m0 + rows, M);
   for (int pos = m0; pos < end;) {
     const int b = pos / g.L, p = pos - b * g.L, s = segment_of(g, p);
-    if (p - g.seg_off[s] < valid_rows(g, b, s)) return true;
-    pos = b * g.L + g.seg_off[s] + g.seg_len[s];
+    if (p - g.off(s) < valid_rows(g, b, s)) return true;
+    pos = b * g.L + g.off(s) + g.len(s);
   }
   return false;
 }
@@ -133,7 +133,7 @@ __device__ __forceinline__ void commit(uint32_t bar) {  // in a pair: the barrie
 template <bool PAIR, int MODE>
 __global__ void __launch_bounds__(G_THREADS, 1)
 linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
-                 const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmR, const Geometry g, const GemmParams p) {
+                 const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmR, const __grid_constant__ Geometry g, const __grid_constant__ GemmParams p) {
   constexpr int CTAS = PAIR ? 2 : 1, CW = (MODE == STORE_F32) ? 32 : 64;  // columns per epilogue box
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -149,6 +149,9 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const bool res = MODE == STORE_F32 && p.has_residual;
 
   if (tid == 0) {
+    map_early(tmA);
+    map_early(tmW);
+    map_early(tmC);
     for (int i = 0; i < p.stages; ++i) { mbar_init(bar_full + 8 * i, 1); mbar_init(bar_empty + 8 * i, 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(bar_accf + 8 * i, 1); mbar_init(bar_acce + 8 * i, 8 * CTAS); }
     for (int i = 0; i < 2 * MAX_BOXES; ++i) { mbar_init(bar_resf + 8 * i, 1); mbar_init(bar_rese + 8 * i, 1); }
@@ -169,6 +172,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   tc_fence_after();
   uint32_t tmem;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(slot) : "memory");
+  load_params_early(g, p);
   grid_dep_wait();
   grid_dep_launch();
 
@@ -275,7 +279,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       bool real = row >= row_lo && row < row_hi;
       if (real && p.mask_rows && !p.packed) {
         const int b = row / g.L, q = row - b * g.L, s = segment_of(g, q);
-        real = q - g.seg_off[s] < valid_rows(g, b, s);
+        real = q - g.off(s) < valid_rows(g, b, s);
       }
       // the bias of this group's columns, by way of shared memory: read from global memory column by column in the loop below
       // it was what bounded the bf16 layers (572 us against 368 without a bias at M 278528, N 1536, K 512)

@@ -210,8 +210,62 @@ FusedHalfArgs half_args(const gsit_layer_weights* w, const float* x, int64_t ldx
                        b(w->w_1), w->b_1, b(w->w_2), w->b_2, y, ldy};
 }
 
+// Do `n` layers of this geometry, side by side, run as one launch behind their first projection?  (The row-tile kernels on mma.sync, for a problem
+// whose attention is the mma.sync kernel as well: the same bits as three launches.)
+bool one_launch_layers(const Geometry& g, int dtype, const uint32_t* allowed, int n, int d_ff) {
+  if (dtype != GSIT_BF16 || g_attn_variant != GSIT_ATTN_DEFAULT || pick_halves(g, d_ff) != HALVES_ROWS) return false;
+  if (!layer_tail_supported(g, d_ff) || !layer_tail_preferred(g, allowed, n)) return false;
+  for (int i = 0; i < n; ++i)
+    if (attn_uses_tensor_memory(g, allowed[i])) return false;
+  return true;
+}
+
 float pick_scale(const gsit_shape* s, const Geometry& g) {
   return (s->scale > 0.f) ? s->scale : 1.0f / sqrtf((float)g.hd);
+}
+
+// `depth` layers of n (1 or 2) problems of geometry g side by side, each layer behind the first projection in one launch.  The layers of
+// problem i read x[i] and write y[i * depth + j]; ws holds one layer_scratch per problem.
+struct LayerChain {
+  const gsit_layer_weights* const* w[2];
+  const float* x[2];
+  int64_t ldx[2];
+  float* const* y[2];
+  const int64_t* ldy[2];
+  uint32_t allowed[2];
+};
+float eps_of(const gsit_layer_weights* w) { return (w->ln_eps > 0.f) ? w->ln_eps : 1e-5f; }
+
+gsit_status run_chain(const Geometry& g, const LayerChain& c, int n, int depth, float scale, uint8_t* ws, size_t ws_stride, const LayerScratch& sc,
+                      cudaStream_t cs) {
+  // a launch reads one projection and writes the next layer's: they take turns in the scratch of qkv and that of att and y1, which lie
+  // side by side (2 d + 4 d bytes a row) and have no other use here
+  static_assert(sizeof(float) == 2 * sizeof(__nv_bfloat16), "att and y1 together hold the three projections");
+  auto qkv = [&](int i, int j) { return reinterpret_cast<__nv_bfloat16*>(ws + i * ws_stride + ((j & 1) ? sc.att : sc.qkv)); };
+  FusedHalfArgs h[2];
+  for (int i = 0; i < n; ++i) h[i] = half_args(c.w[i][0], c.x[i], c.ldx[i], qkv(i, 0), nullptr, nullptr, 0);
+  {
+    TraceScope t(GSIT_KERNEL_LINEAR, cs);
+    const gsit_status st = from_cuda(launch_ln_qkv_rows(g, h, n, eps_of(c.w[0][0]), nullptr, cs));
+    if (st != GSIT_OK) return st;
+  }
+  for (int j = 0; j < depth; ++j) {
+    LayerTailArgs a[2];
+    for (int i = 0; i < n; ++i) {
+      const bool next = j + 1 < depth;
+      a[i].qkv = qkv(i, j);
+      a[i].h = half_args(c.w[i][j], j == 0 ? c.x[i] : c.y[i][j - 1], j == 0 ? c.ldx[i] : c.ldy[i][j - 1], nullptr, nullptr, c.y[i][j], c.ldy[i][j]);
+      a[i].allowed = c.allowed[i];
+      const FusedHalfArgs nx = half_args(c.w[i][next ? j + 1 : j], nullptr, 0, nullptr, nullptr, nullptr, 0);
+      a[i].h.ln1_gamma = nx.ln1_gamma; a[i].h.ln1_beta = nx.ln1_beta;
+      a[i].h.w_qkv = nx.w_qkv; a[i].h.b_qkv = nx.b_qkv;
+      a[i].h.qkv = next ? qkv(i, j + 1) : nullptr;
+    }
+    TraceScope t(GSIT_KERNEL_ATTENTION, cs);
+    const gsit_status st = from_cuda(launch_layer_tail(g, a, n, scale, eps_of(c.w[0][j]), eps_of(c.w[0][j + 1 < depth ? j + 1 : j]), c.w[0][j]->d_ff, cs));
+    if (st != GSIT_OK) return st;
+  }
+  return GSIT_OK;
 }
 
 }  // namespace
@@ -292,6 +346,10 @@ gsit_status gsit_im_layer_fwd(const gsit_shape* shape, const gsit_layer_weights*
   if (g.row_start != nullptr && (halves == HALVES_NONE || g.hd > 32))
     return GSIT_ERR_UNSUPPORTED;  // the packed layout is implemented by the fused halves and the mma.sync / tensor-memory attention
 
+  if (one_launch_layers(g, dtype, &g.allowed, 1, w->d_ff)) {
+    const LayerChain c = {{&w, nullptr}, {x, nullptr}, {x_row_stride, 0}, {&y, nullptr}, {&y_row_stride, nullptr}, {g.allowed, 0}};
+    return run_chain(g, c, 1, 1, pick_scale(shape, g), ws, 0, sc, cs);
+  }
   if (halves != HALVES_NONE) {
     // three launches: LN1 + shared projection, IM attention, out-projection + residual + LN2 + MLP + residual
     const FusedHalfArgs h = half_args(w, x, x_row_stride, static_cast<__nv_bfloat16*>(qkv), static_cast<__nv_bfloat16*>(att), y, y_row_stride);
@@ -400,6 +458,10 @@ gsit_status gsit_im_layer_pair_fwd(const gsit_shape* shape_a, const gsit_shape* 
   FusedHalfArgs h[2];
   AttnOperands ops[2];
   const uint32_t allowed[2] = {ga.allowed, gb.allowed};
+  if (one_launch_layers(ga, shape_a->dtype, allowed, 2, w_a->d_ff)) {
+    const LayerChain c = {{&w_a, &w_b}, {x_a, x_b}, {x_a_row_stride, x_b_row_stride}, {&y_a, &y_b}, {&y_a_row_stride, &y_b_row_stride}, {allowed[0], allowed[1]}};
+    return run_chain(ga, c, 2, 1, pick_scale(shape_a, ga), ws, sc.total, sc, cs);
+  }
   for (int i = 0; i < 2; ++i) {
     uint8_t* wsi = ws + i * sc.total;
     __nv_bfloat16* qkv = reinterpret_cast<__nv_bfloat16*>(wsi + sc.qkv);
@@ -421,6 +483,72 @@ gsit_status gsit_im_layer_pair_fwd(const gsit_shape* shape_a, const gsit_shape* 
   }
   TraceScope t(GSIT_KERNEL_LINEAR, cs);
   return from_cuda(halves == HALVES_ROWS ? launch_proj_mlp_rows(ga, h, 2, eps_a, w_a->d_ff, cs) : launch_proj_mlp_tc_pair(ga, h, eps_a, w_a->d_ff, cs));
+}
+
+int32_t gsit_encoder_runs_chained(const gsit_shape* const* shapes, int32_t problems, int32_t d_ff) {
+  Geometry g[2];
+  if (!shapes || problems < 1 || problems > 2 || d_ff < 1) return 0;
+  uint32_t allowed[2];
+  for (int i = 0; i < problems; ++i) {
+    if (make_geometry(shapes[i], &g[i]) != GSIT_OK) return 0;
+    allowed[i] = g[i].allowed;
+  }
+  return one_launch_layers(g[0], shapes[0]->dtype, allowed, problems, d_ff);
+}
+
+gsit_status gsit_im_encoder_fwd(const gsit_shape* const* shapes, int32_t problems, const gsit_layer_weights* const* const* weights, int32_t depth,
+                                const float* const* x, const int64_t* x_row_stride, float* const* const* y, const int64_t* const* y_row_stride,
+                                void* workspace, size_t workspace_bytes, gsit_stream stream) {
+  if (!shapes || !weights || !x || !x_row_stride || !y || !y_row_stride || problems < 1 || problems > 2 || depth < 1) return GSIT_ERR_INVALID_ARG;
+  for (int i = 0; i < problems; ++i) {
+    if (!shapes[i] || !weights[i] || !y[i] || !y_row_stride[i]) return GSIT_ERR_INVALID_ARG;
+    for (int j = 0; j < depth; ++j)
+      if (!weights[i][j]) return GSIT_ERR_INVALID_ARG;
+  }
+  // the layers one call each, unless they can follow each other launch by launch; the calls also report what is wrong with an argument
+  Geometry g[2] = {};
+  LayerChain c = {};
+  bool chained = depth > 1;
+  int max_ff = 1;
+  for (int i = 0; i < problems && chained; ++i) {
+    chained = make_geometry(shapes[i], &g[i]) == GSIT_OK;
+    c.w[i] = weights[i]; c.x[i] = x[i]; c.ldx[i] = x_row_stride[i]; c.y[i] = y[i]; c.ldy[i] = y_row_stride[i];
+    c.allowed[i] = g[i].allowed;
+    const Geometry &a = g[0], &b = g[i];
+    chained = chained && a.batch == b.batch && a.d == b.d && a.heads == b.heads && a.valid_len == b.valid_len && a.row_start == b.row_start &&
+              a.capacity == b.capacity && shapes[0]->dtype == shapes[i]->dtype && shapes[0]->scale == shapes[i]->scale &&
+              a.seg_len[0] == b.seg_len[0] && a.seg_len[1] == b.seg_len[1] && a.seg_len[2] == b.seg_len[2];
+    chained = chained && x[i] && aligned16(x[i]) && x_row_stride[i] >= a.d && x_row_stride[i] % 4 == 0;
+    for (int j = 0; j < depth && chained; ++j) {
+      const gsit_layer_weights *w = weights[i][j], *w0 = weights[0][j];
+      chained = w->w_qkv && w->w_o && w->w_1 && w->w_2 && aligned16(w->w_qkv) && aligned16(w->w_o) && aligned16(w->w_1) && aligned16(w->w_2) &&
+                w->d_ff >= 1 && w->d_ff == w0->d_ff && eps_of(w) == eps_of(w0) && y[i][j] && aligned16(y[i][j]) && y_row_stride[i][j] >= a.d &&
+                y_row_stride[i][j] % 4 == 0;
+      if (chained && w->d_ff > max_ff) max_ff = w->d_ff;
+    }
+  }
+  for (int j = 0; j < depth && chained; ++j) chained = one_launch_layers(g[0], shapes[0]->dtype, c.allowed, problems, weights[0][j]->d_ff);
+  if (chained) {
+    const LayerScratch sc = layer_scratch(g[0], shapes[0]->dtype, max_ff);
+    if (!workspace || workspace_bytes < problems * sc.total || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return GSIT_ERR_WORKSPACE;
+    if (from_cuda(status_ptr(&g[0].status)) != GSIT_OK) return GSIT_ERR_CUDA;
+    return run_chain(g[0], c, problems, depth, pick_scale(shapes[0], g[0]), static_cast<uint8_t*>(workspace), sc.total, sc,
+                     static_cast<cudaStream_t>(stream));
+  }
+  for (int j = 0; j < depth; ++j) {
+    const float* in[2];
+    int64_t ld[2];
+    for (int i = 0; i < problems; ++i) {
+      in[i] = j == 0 ? x[i] : y[i][j - 1];
+      ld[i] = j == 0 ? x_row_stride[i] : y_row_stride[i][j - 1];
+    }
+    const gsit_status st =
+        problems == 1 ? gsit_im_layer_fwd(shapes[0], weights[0][j], in[0], ld[0], y[0][j], y_row_stride[0][j], workspace, workspace_bytes, stream)
+                      : gsit_im_layer_pair_fwd(shapes[0], shapes[1], weights[0][j], weights[1][j], in[0], ld[0], in[1], ld[1], y[0][j],
+                                               y_row_stride[0][j], y[1][j], y_row_stride[1][j], workspace, workspace_bytes, stream);
+    if (st != GSIT_OK) return st;
+  }
+  return GSIT_OK;
 }
 
 gsit_status gsit_plan_rows(const gsit_shape* shape, int32_t split_sample, int32_t* row_start, gsit_stream stream) {

@@ -132,15 +132,16 @@ __global__ void __launch_bounds__(256) linear_bf16_kernel(Geometry g, LinearArgs
 // once, and a warp keeps gamma and beta in registers over many rows (loading them for every row costs more L1 cycles than
 // the row itself: 217 us; 4-byte loads in three passes: 201 us; now 143 us at 278528 x 512).  CHUNKS = 0: any d.
 template <typename OutT, int CHUNKS>
-__global__ void __launch_bounds__(256) layernorm_kernel(const Geometry g, const float* __restrict__ x, const int64_t ldx,
+__global__ void __launch_bounds__(256) layernorm_kernel(const __grid_constant__ Geometry g, const float* __restrict__ x, const int64_t ldx,
                                                         const float* __restrict__ gamma, const float* __restrict__ beta,
                                                         const float eps, OutT* __restrict__ y, const int rows) {
   const int lane = threadIdx.x & 31, d = g.d;
   int row = (int)(blockIdx.x * 8 + (threadIdx.x >> 5));
   auto is_real = [&](int r) {
     const int b = r / g.L, p = r - b * g.L, s = segment_of(g, p);
-    return p - g.seg_off[s] < valid_rows(g, b, s);
+    return p - g.off(s) < valid_rows(g, b, s);
   };
+  ptx::load_params_early(g, x, ldx, gamma, beta, y);
   ptx::grid_dep_wait();
   ptx::grid_dep_launch();
   if constexpr (CHUNKS > 0) {

@@ -52,9 +52,10 @@ __global__ void __launch_bounds__(1024) plan_rows_kernel(const Geometry g, const
 // All index arithmetic is 32-bit (the library limits B * L to 2^29 rows).
 constexpr int MOVE_UNROLL = 4;
 template <bool PACK>
-__global__ void __launch_bounds__(256) move_rows_kernel(const Geometry g, const float* __restrict__ src, const int64_t src_stride,
+__global__ void __launch_bounds__(256) move_rows_kernel(const __grid_constant__ Geometry g, const float* __restrict__ src, const int64_t src_stride,
                                                         float* __restrict__ dst, const int64_t dst_stride, const int cpr /* chunks per row */,
                                                         const unsigned total /* chunks in all */, const unsigned quarter) {
+  ptx::load_params_early(g, src, src_stride, dst, dst_stride);
   ptx::grid_dep_wait();  // the source comes from the kernel before this one (and the row plan from an earlier one)
   ptx::grid_dep_launch();
   const unsigned idx0 = blockIdx.x * 256u + threadIdx.x;
@@ -69,7 +70,7 @@ __global__ void __launch_bounds__(256) move_rows_kernel(const Geometry g, const 
     if (idx >= total) continue;
     const unsigned w = idx / (unsigned)cpr, c = idx - w * (unsigned)cpr;  // padded-layout row, chunk in the row
     const int b = (int)(w / (unsigned)g.L), p = (int)(w - (unsigned)b * (unsigned)g.L);
-    const int s = segment_of(g, p), i = p - g.seg_off[s];
+    const int s = segment_of(g, p), i = p - g.off(s);
     const bool real = i < valid_rows(g, b, s);
     if (PACK) {
       if (!real) continue;
@@ -89,11 +90,12 @@ __global__ void __launch_bounds__(256) move_rows_kernel(const Geometry g, const 
 // Plan and gather in one launch: every CTA scans the valid lengths itself (3 B integers, a microsecond) instead of waiting for a
 // kernel that does nothing else, and CTA 0 writes the plan down for the kernels that follow.
 constexpr int PLAN_MAX = 3072;  // entries (samples x segments) a CTA can hold
-__global__ void __launch_bounds__(256) plan_pack_kernel(const Geometry g, int32_t* __restrict__ row_start, const float* __restrict__ src,
+__global__ void __launch_bounds__(256) plan_pack_kernel(const __grid_constant__ Geometry g, int32_t* __restrict__ row_start, const float* __restrict__ src,
                                                         const int64_t src_stride, float* __restrict__ dst, const int64_t dst_stride, const int cpr,
                                                         const unsigned total, const unsigned quarter) {
   __shared__ int starts[PLAN_MAX + 1];
   __shared__ int warp_sum[8];
+  ptx::load_params_early(g, src, src_stride, dst, dst_stride);
   ptx::grid_dep_wait();
   ptx::grid_dep_launch();
   const int n = 3 * g.batch, tid = threadIdx.x, lane = tid & 31;
@@ -129,7 +131,7 @@ __global__ void __launch_bounds__(256) plan_pack_kernel(const Geometry g, int32_
     if (idx >= total) continue;
     const unsigned w = idx / (unsigned)cpr, c = idx - w * (unsigned)cpr;  // padded-layout row, chunk in the row
     const int b = (int)(w / (unsigned)g.L), p = (int)(w - (unsigned)b * (unsigned)g.L);
-    const int s = segment_of(g, p), i = p - g.seg_off[s], at = starts[3 * b + s];
+    const int s = segment_of(g, p), i = p - g.off(s), at = starts[3 * b + s];
     if (i >= starts[3 * b + s + 1] - at) continue;
     out[u] = reinterpret_cast<float4*>(dst + (int64_t)(at + i) * dst_stride) + c;
     v[u] = __ldg(reinterpret_cast<const float4*>(src + (int64_t)w * src_stride) + c);

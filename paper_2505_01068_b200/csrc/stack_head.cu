@@ -28,18 +28,19 @@ __device__ __forceinline__ float dot_chunk(const float* z, const uint4& u, const
 // VEC: the weight rows are whole numbers of 16-byte chunks
 template <typename WT, bool VEC>
 __global__ void __launch_bounds__(HEAD_WARPS * 32)
-stack_head_kernel(const Geometry g, const float* __restrict__ c, const int64_t ldc, const int dc, const WT* __restrict__ w,
+stack_head_kernel(const __grid_constant__ Geometry g, const float* __restrict__ c, const int64_t ldc, const int dc, const WT* __restrict__ w,
                   const float* __restrict__ bias, float* __restrict__ out, const int n_out) {
   extern __shared__ __align__(16) float z[];  // [3 * dc]
   const int b = blockIdx.x, K = 3 * dc;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int o0 = (blockIdx.y * HEAD_WARPS + warp) * HEAD_PER_WARP;
+  ptx::load_params_early(g, c, ldc, w, bias, out);
   ptx::grid_dep_wait();
   ptx::grid_dep_launch();
   for (int i = threadIdx.x; i < K; i += blockDim.x) {
     const int s = i / dc, e = i - s * dc;
     const int n = valid_rows(g, b, s);
-    z[i] = (n > 0) ? c[((int64_t)b * g.L + g.seg_off[s] + n - 1) * ldc + e] : 0.f;
+    z[i] = (n > 0) ? c[((int64_t)b * g.L + g.off(s) + n - 1) * ldc + e] : 0.f;
   }
   __syncthreads();
   float acc[HEAD_PER_WARP] = {};

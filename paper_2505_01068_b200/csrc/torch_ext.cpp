@@ -14,6 +14,7 @@
 
 #include <deque>
 #include <exception>
+#include <vector>
 
 #include "gsit.h"
 
@@ -403,6 +404,28 @@ std::deque<Layer> all_layers(PyObject* list, double eps) {
   return layers;
 }
 
+// Are all layers of one type, of equal MLP width in a pair?  Then an encoder (pair) goes through one call.
+bool uniform(const std::deque<Layer>& a, const std::deque<Layer>& b) {
+  for (size_t i = 0; i < a.size(); ++i)
+    if (a[i].dtype != a[0].dtype || b[i].dtype != a[0].dtype || a[i].w.d_ff != b[i].w.d_ff) return false;
+  return true;
+}
+bool chained(const at::Tensor& x, PyObject* seg, int64_t heads, int64_t intra_heads, const at::Tensor* valid, const std::deque<Layer>& fwd,
+             const std::deque<Layer>& bwd, const std::deque<Layer>& intra) {
+  if (!uniform(fwd, bwd) || !uniform(intra, intra)) return false;
+  auto all = [&](const std::deque<Layer>& layers, int64_t width, int64_t h, int problems) {
+    for (const Layer& l : layers) {
+      gsit_shape s[2];
+      for (int i = 0; i < 2; ++i)
+        s[i] = make_shape(x.size(0), seg, width, h, valid, l.dtype, problems == 1 ? GSIT_PHASE_INTRA : i ? GSIT_PHASE_INTER_BWD : GSIT_PHASE_INTER_FWD, 0, 0.0);
+      const gsit_shape* shapes[2] = {&s[0], &s[1]};
+      if (!gsit_encoder_runs_chained(shapes, problems, l.w.d_ff)) return false;
+    }
+    return true;
+  };
+  return all(fwd, x.size(2), heads, 2) && all(intra, 2 * x.size(2), intra_heads, 1);
+}
+
 // x, valid_len, y, fwd, bwd, intra, seg_len, heads, intra_heads, ln_eps, buffers
 //   buffers = (plan or None, workspace, ring_a0, ring_a1, ring_b0, ring_b1, x_packed or None, wide_0, wide_1): with a plan the
 //   packed row layout is used (x gathered into x_packed, the result scattered into y), without one the padded layout.
@@ -421,7 +444,9 @@ PyObject* stack_forward(PyObject* const* a) {
   require(PyTuple_Check(a[10]) && PyTuple_GET_SIZE(a[10]) == 9, "buffers: nine tensors");
   const at::Tensor* b[9];
   for (int i = 0; i < 9; ++i) b[i] = opt_tensor(PyTuple_GET_ITEM(a[10], i));
+  // layers that run as one launch each do no work for padding in the padded layout either: no plan, no copies between layouts then
   const at::Tensor* plan = b[0];
+  if (plan != nullptr && chained(x, a[6], as_int(a[7]), as_int(a[8]), valid, fwd, bwd, intra)) plan = nullptr;
   const int64_t B = x.size(0), d = x.size(2), cap = plan != nullptr ? b[6]->size(0) : 0;
   const gsit_shape ring_shape = make_shape(B, a[6], d, as_int(a[7]), valid, fwd[0].dtype, GSIT_PHASE_INTER_FWD, 0, 0.0, plan, cap);
   const gsit_shape intra_shape = make_shape(B, a[6], 2 * d, as_int(a[8]), valid, fwd[0].dtype, GSIT_PHASE_INTRA, 0, 0.0, plan, cap);
@@ -443,36 +468,69 @@ PyObject* stack_forward(PyObject* const* a) {
       x_in = xp;
       ldx = d;
     }
-    // both rings, layers of equal depth in one call each; the last pair writes the halves of the concatenated rows
+    // both rings side by side; the last layers write the halves of the concatenated rows
     float* c = (plan == nullptr && intra.empty()) ? out : wide[0];
     gsit_shape sa = ring_shape, sb = ring_shape;
     sb.phase = GSIT_PHASE_INTER_BWD;
-    const float *cur_a = x_in, *cur_b = x_in;
-    int64_t ld = ldx;
+    std::vector<float*> ya, yb, yi;
+    std::vector<int64_t> ldr, ldi;
+    std::vector<const gsit_layer_weights*> wf, wb, wi;
     for (size_t i = 0; i < fwd.size(); ++i) {
       const bool last = i + 1 == fwd.size();
-      float *dst_a = last ? c : ping_a[i & 1], *dst_b = last ? c + d : ping_b[i & 1];
-      const int64_t ldy = last ? 2 * d : d;
-      // every layer in the type of its own weights; a pair of one type goes through one call
-      sa.dtype = fwd[i].dtype;
-      sb.dtype = bwd[i].dtype;
-      if (sa.dtype == sb.dtype && fwd[i].w.d_ff == bwd[i].w.d_ff) {
-        st = gsit_im_layer_pair_fwd(&sa, &sb, &fwd[i].w, &bwd[i].w, cur_a, ld, cur_b, ld, dst_a, ldy, dst_b, ldy, ws, ws_n, cs);
-      } else {
-        st = gsit_im_layer_fwd(&sa, &fwd[i].w, cur_a, ld, dst_a, ldy, ws, ws_half, cs);
-        if (st == GSIT_OK) st = gsit_im_layer_fwd(&sb, &bwd[i].w, cur_b, ld, dst_b, ldy, ws + ws_half, ws_half, cs);
-      }
+      ya.push_back(last ? c : ping_a[i & 1]);
+      yb.push_back(last ? c + d : ping_b[i & 1]);
+      ldr.push_back(last ? 2 * d : d);
+      wf.push_back(&fwd[i].w);
+      wb.push_back(&bwd[i].w);
+    }
+    if (uniform(fwd, bwd)) {
+      const gsit_shape* shapes[2] = {&sa, &sb};
+      const gsit_layer_weights* const* w[2] = {wf.data(), wb.data()};
+      const float* xs[2] = {x_in, x_in};
+      const int64_t ldxs[2] = {ldx, ldx};
+      float* const* ys[2] = {ya.data(), yb.data()};
+      const int64_t* ldys[2] = {ldr.data(), ldr.data()};
+      st = gsit_im_encoder_fwd(shapes, 2, w, (int32_t)fwd.size(), xs, ldxs, ys, ldys, ws, ws_n, cs);
       if (st != GSIT_OK) return st;
-      cur_a = dst_a; cur_b = dst_b; ld = ldy;
+    } else {
+      for (size_t i = 0; i < fwd.size(); ++i) {  // every layer in the type of its own weights; a pair of one type goes through one call
+        const float *cur_a = i == 0 ? x_in : ya[i - 1], *cur_b = i == 0 ? x_in : yb[i - 1];
+        const int64_t ld = i == 0 ? ldx : ldr[i - 1];
+        sa.dtype = fwd[i].dtype;
+        sb.dtype = bwd[i].dtype;
+        if (sa.dtype == sb.dtype && fwd[i].w.d_ff == bwd[i].w.d_ff) {
+          st = gsit_im_layer_pair_fwd(&sa, &sb, wf[i], wb[i], cur_a, ld, cur_b, ld, ya[i], ldr[i], yb[i], ldr[i], ws, ws_n, cs);
+        } else {
+          st = gsit_im_layer_fwd(&sa, wf[i], cur_a, ld, ya[i], ldr[i], ws, ws_half, cs);
+          if (st == GSIT_OK) st = gsit_im_layer_fwd(&sb, wb[i], cur_b, ld, yb[i], ldr[i], ws + ws_half, ws_half, cs);
+        }
+        if (st != GSIT_OK) return st;
+      }
     }
     int in_wide = 0;
     for (size_t i = 0; i < intra.size(); ++i) {
-      float* dst = (i + 1 == intra.size() && plan == nullptr) ? out : wide[in_wide ^ 1];
-      gsit_shape si = intra_shape;
-      si.dtype = intra[i].dtype;
-      st = gsit_im_layer_fwd(&si, &intra[i].w, wide[in_wide], 2 * d, dst, 2 * d, ws, ws_n, cs);
-      if (st != GSIT_OK) return st;
+      yi.push_back((i + 1 == intra.size() && plan == nullptr) ? out : wide[in_wide ^ 1]);
+      ldi.push_back(2 * d);
+      wi.push_back(&intra[i].w);
       in_wide ^= 1;
+    }
+    gsit_shape si = intra_shape;
+    if (!intra.empty() && uniform(intra, intra)) {
+      si.dtype = intra[0].dtype;
+      const gsit_shape* shape = &si;
+      const gsit_layer_weights* const* w = wi.data();
+      const float* xs = wide[0];
+      const int64_t ldxs = 2 * d;
+      float* const* ys = yi.data();
+      const int64_t* ldys = ldi.data();
+      st = gsit_im_encoder_fwd(&shape, 1, &w, (int32_t)intra.size(), &xs, &ldxs, &ys, &ldys, ws, ws_n, cs);
+      if (st != GSIT_OK) return st;
+    } else {
+      for (size_t i = 0; i < intra.size(); ++i) {
+        si.dtype = intra[i].dtype;
+        st = gsit_im_layer_fwd(&si, wi[i], i == 0 ? wide[0] : yi[i - 1], 2 * d, yi[i], 2 * d, ws, ws_n, cs);
+        if (st != GSIT_OK) return st;
+      }
     }
     if (plan != nullptr) st = gsit_unpack_rows(&ring_shape, wide[in_wide], 2 * d, out, 2 * d, (int32_t)(2 * d), cs);
     return st;
