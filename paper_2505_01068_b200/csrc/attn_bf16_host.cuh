@@ -51,7 +51,7 @@ int g_attn_variant = 0;  // gsit_kernel_choice
 // quarter real loses 3 - 5 us up to 225 units.  4 heads of 32: half to full 27.7/27.6 at 42, 32.5/30.9 at 56, 63.1/47.5 at 112; a
 // quarter 10.5/16.4, 12.9/18.4, 24.1/25.4; layer, a quarter 34.4/35.8 at 56, 41.2/41.0 at 84 -> 55.
 //   head_dim 64 is a dense contraction; there only a few short walks (at most two key tiles per row) are over sooner in the
-//   mma.sync kernel (32 x (50, 50, 50), 2 heads: 4.8 against 6.1 us; 128 samples: 14.8 against 11.5).
+//   mma.sync kernel (32 x (50, 50, 50), 2 heads: 4.4 against 5.1 us; 64 samples: 7.7 against 6.8; 128: 11.5 against 9.0).
 //   head_dim 8: the tensor-memory kernel is slower throughout (55 against 44 us at 64 x (50, 500, 500)): a tcgen05 hand-over
 //   per 64 keys of one head costs more than the 8192 exponentials it feeds.
 bool attn_uses_tensor_memory(const Geometry& g, uint32_t allowed) {

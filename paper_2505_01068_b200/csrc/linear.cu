@@ -19,7 +19,7 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool p
 }
 
 template <int BN>
-__global__ void __launch_bounds__(256) linear_bf16_kernel(Geometry g, LinearArgs a) {
+__global__ void __launch_bounds__(256) linear_bf16_kernel(const __grid_constant__ Geometry g, const __grid_constant__ LinearArgs a) {
   constexpr int WGN = (BN == 128) ? 4 : 2, WGM = 8 / WGN;
   constexpr int WTM = BM / WGM, WTN = BN / WGN;  // warp tile
   constexpr int MT = WTM / 16, NTL = WTN / 8;
@@ -32,6 +32,9 @@ __global__ void __launch_bounds__(256) linear_bf16_kernel(Geometry g, LinearArgs
   const int wm = warp / WGN, wn = warp % WGN;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
   const int KT_ = (a.K + BK - 1) / BK;
+  ptx::load_params_early(g, a);
+  ptx::grid_dep_wait();  // the weights, too: this kernel may be the first of a call, right behind the one that wrote them
+  ptx::grid_dep_launch();
 
   auto load_stage = [&](int kt, int st) {
     const int k0 = kt * BK;
@@ -236,9 +239,7 @@ cudaError_t launch_linear_bf16(const Geometry& g, const LinearArgs& a, cudaStrea
   const int bn = wide ? 128 : 64;
   const dim3 grid((a.N + bn - 1) / bn, (a.M + BM - 1) / BM);
   if (grid.y > 65535) return cudaErrorNotSupported;
-  if (wide) linear_bf16_kernel<128><<<grid, 256, 0, st>>>(g, a);
-  else linear_bf16_kernel<64><<<grid, 256, 0, st>>>(g, a);
-  return cudaGetLastError();
+  return launch_overlapped(wide ? linear_bf16_kernel<128> : linear_bf16_kernel<64>, grid, dim3(256), 0, st, g, a);
 }
 
 cudaError_t launch_layernorm(const Geometry& g, const float* x, int64_t ldx, const float* gamma, const float* beta,
