@@ -237,6 +237,9 @@ typedef enum { GSIT_CALL_QKV_PROJ = 0, GSIT_CALL_ATTENTION = 1, GSIT_CALL_LAYER 
 /* Scratch bytes the given call needs for this shape (d_ff is read for GSIT_CALL_LAYER only).
  * Returns 0 for calls that need none and (size_t)-1 for an invalid shape. */
 size_t gsit_workspace_bytes(const gsit_shape* shape, int which_call, int32_t d_ff);
+/* Would gsit_im_attention_fwd read its workspace for this shape (on the current device)?  1 or 0; -1 for an invalid shape.  Where it would
+ * not, passing none saves the caller an allocation. */
+int32_t gsit_attention_uses_workspace(const gsit_shape* shape);
 
 /* Device status flags, accumulated by kernels of this library on the current device. */
 #define GSIT_DEVFLAG_CLAMPED 1u  /* a valid_len value was outside [0, seg_len] and was clamped */

@@ -389,12 +389,13 @@ int64_t tail_ctas(const Geometry& g, int n, int rows) {
 int small_tile(const Geometry& g) { return g.d == 32 ? 32 : 16; }
 }  // namespace
 
-// One CTA fills an SM, and a second wave of long walks costs more than two launches less: one wave, or up to three of walks over at
-// most eight key tiles.  Layer of one kernel behind the projection / of two, us (the half, full and sparse lengths of 0.05 - 0.4):
+// One CTA fills an SM, and a second wave of long walks costs more than two launches less: one wave, or up to three (d 32: two) of walks
+// over at most eight key tiles.  Layer of one kernel behind the projection / of two, us (the half, full and sparse lengths of 0.05 - 0.4):
 //   4200 rows of (50, 500, 500), d 64: half 18.4/24.5, full 19.6/26.0, sparse 13.1/16.4      (one wave of 32-row tiles)
 //   6300 rows, two waves:              half 21.4/27.4, full 32.1/28.8, sparse 13.9/19.2;     pair, three: 32.4/34.5, 43.9/42.8, 16.6/22.9
 //   5358 rows of (850, 34, 9), intra, full, two waves of 14 key tiles: 43.8/36.0
-//   d 128, 6300 rows of (50, 500, 500): half 32.3/43.0, full 49.8/50.6; d 32, 26400 rows of (50, 250, 250), full: 31.9/32.4, pair (six) 57/49
+//   d 128, 6300 rows of (50, 500, 500): half 32.3/43.0, full 49.8/50.6; d 32, pair, 8800 rows of (50, 250, 250), full 22.6/22.1,
+//   sparse 12.6/16.8; a stack of 8650 rows, two and a half waves: 132.6/130
 bool layer_tail_preferred(const Geometry& g, const uint32_t* allowed, int n) {
   int n_sm = 0;
   if (sm_count_and_smem_once(nullptr, 0, &n_sm) != cudaSuccess) return false;
@@ -408,7 +409,7 @@ bool layer_tail_preferred(const Geometry& g, const uint32_t* allowed, int n) {
         if ((allowed[i] >> (3 * s + r)) & 1u) kt += (g.len(r) + KT - 1) / KT;
       if (g.len(s) > 0 && kt > longest) longest = kt;
     }
-  return ctas <= 3 * n_sm && longest <= 8;
+  return ctas <= (g.d == 32 ? 2 : 3) * n_sm && longest <= 8;
 }
 
 cudaError_t launch_layer_tail(const Geometry& g, const LayerTailArgs* args, int n, float scale, float eps, float next_eps, int d_ff, cudaStream_t st) {

@@ -211,6 +211,10 @@ bool fused_rows_preferred(const Geometry& g);
 cudaError_t launch_ln_qkv_rows(const Geometry& g, const FusedHalfArgs* h, int n, float eps, int* zero_word, cudaStream_t st);
 cudaError_t launch_proj_mlp_rows(const Geometry& g, const FusedHalfArgs* h, int n, float eps, int d_ff, cudaStream_t st);
 
+// The shared projection alone on the same row tiles (bf16 at d_model 32 and 64): where it is chosen, and its launch.
+bool qkv_rows_preferred(const Geometry& g);
+cudaError_t launch_qkv_rows(const Geometry& g, const LinearArgs& a, cudaStream_t st);
+
 // Attention and second half of a layer, and the first half of the next one, in one launch for one or two problems of one geometry
 // (attn_mlp_rows.cu): qkv is the projection [rows, 3 d] the attention reads; of h, x is the layer's input, ln2 / w_o / w_1 / w_2 its
 // second half, y its output, and ln1 / w_qkv the next layer's first half, which writes h.qkv (another buffer than qkv; null: none).

@@ -50,6 +50,38 @@ ln_qkv_rows_kernel(const __grid_constant__ Geometry g, const __grid_constant__ P
   qkv_units<D, R>([&](int row, int k) { return ldw(a.w_qkv + (int64_t)row * D + 32 * k + 8 * (tid & 3)); }, a.b_qkv, a.qkv, rows.m0, h, work, tid, [&](int r) { return rows.m0 + r < rows.end; }, real);
 }
 
+// ------------------------------------------------------------------------------------------------ QKV alone
+// The shared projection by itself, for bf16 rows: what bounds a few thousand rows of these widths is the latency of one launch, and this
+// one has no tensor memory, barriers or tensor maps to set up and fits beside its neighbours on an SM.
+struct ProjArgs { const __nv_bfloat16* x; int64_t ldx; const __nv_bfloat16* w; const float* bias; __nv_bfloat16* qkv; };
+
+template <int D, int R>
+__global__ void __launch_bounds__(THREADS)
+qkv_rows_kernel(const __grid_constant__ Geometry g, const __grid_constant__ ProjArgs a) {
+  constexpr int BM = 16 * R, CPR = D / 8;
+  __shared__ __align__(128) uint8_t sX[BM * D * 2];
+  const int tid = threadIdx.x;
+  const uint32_t h = smem_u32(sX);
+  ptx::load_params_early(g, a);
+  ptx::grid_dep_wait();
+  ptx::grid_dep_launch();
+  const Rows rows = rows_of<BM>(g);
+  if (rows.m0 >= rows.end) return;
+  auto real = [&](int r) { return is_real(g, rows.m0 + r, rows.end); };
+  bool any = false;
+#pragma unroll
+  for (int i = tid; i < BM * CPR; i += THREADS) {
+    const int r = i / CPR, c = i % CPR;
+    const bool ok = real(r);
+    any |= ok;
+    const uint4 v = ok ? *reinterpret_cast<const uint4*>(a.x + (int64_t)(rows.m0 + r) * a.ldx + 8 * c) : make_uint4(0, 0, 0, 0);
+    ptx::st_shared_v4(h + piece<D>(r, c), v.x, v.y, v.z, v.w);
+  }
+  const bool work = __syncthreads_or(any) != 0;
+  qkv_units<D, R>([&](int row, int k) { return ldw(a.w + (int64_t)row * D + 32 * k + 8 * (tid & 3)); }, a.bias, a.qkv, rows.m0, h, work, tid,
+                  [&](int r) { return rows.m0 + r < rows.end; }, real);
+}
+
 // ------------------------------------------------------------------------------------------------ out-projection + LN2 + MLP
 template <int D, int R>
 __global__ void __launch_bounds__(THREADS, R <= 2 && D <= 64 ? (R == 1 ? 3 : 2) : 1)
@@ -256,6 +288,10 @@ cudaError_t launch_ln_qkv(const Geometry& g, const Pair& p, int n, float eps, in
   return launch_overlapped(ln_qkv_rows_kernel<D, R>, dim3((unsigned)tiles, n), dim3(THREADS), 0, st, g, p, eps, zero_word);
 }
 template <int D, int R>
+cudaError_t launch_qkv(const Geometry& g, const ProjArgs& a, cudaStream_t st) {
+  return launch_overlapped(qkv_rows_kernel<D, R>, dim3((unsigned)((matrix_rows(g) + 16 * R - 1) / (16 * R))), dim3(THREADS), 0, st, g, a);
+}
+template <int D, int R>
 cudaError_t launch_proj_mlp(const Geometry& g, const Pair& p, int n, float eps, int d_ff, cudaStream_t st) {
   constexpr int BM = 16 * R;
   const int64_t tiles = (matrix_rows(g) + BM - 1) / BM;
@@ -289,6 +325,22 @@ static int sm_count() {
   return sm_count_and_smem_once(nullptr, 0, &n) == cudaSuccess ? n : 0;
 }
 bool fused_rows_preferred(const Geometry& g) { return g.d == 32 || (int64_t)g.batch * g.L <= (int64_t)ROWS_PER_SM * sm_count(); }
+
+// Where the projection alone runs here: always at width 32; at 64 up to 2000 rows, where both kernels take the same time but the
+// tcgen05 GEMM's three tensor maps are encoded on the host first (6.2 us a call there, 5.4 here); at 128 never.  us here / on the kernel
+// for other widths (mma.sync at d 32, tcgen05 at 64 and 128), every position real:
+//   rows      500       2000      4000      8000      16000     32000
+//   d 32    2.7/4.4   2.7/4.6   2.8/4.7   3.1/4.7   4.0/5.3   6.3/7.3    (64 rows a tile from 8192 rows on; 32 there: 4.7 at 16000)
+//   d 64    3.5/3.5   3.6/3.6   3.9/3.7   5.1/5.1   8.7/5.8  11.9/6.4
+//   d 128   5.0/4.0   5.2/4.1   6.2/5.6   9.5/6.2  17.4/7.2  29.3/14.6
+// The rows counted are those of the matrices, packed or padded: a call on part of a packed batch takes the kernel of the whole.
+bool qkv_rows_preferred(const Geometry& g) { return g.d == 32 || (g.d == 64 && matrix_rows(g) <= 2000); }
+cudaError_t launch_qkv_rows(const Geometry& g, const LinearArgs& l, cudaStream_t st) {
+  const ProjArgs a = {static_cast<const __nv_bfloat16*>(l.A), l.lda, static_cast<const __nv_bfloat16*>(l.W), l.bias, static_cast<__nv_bfloat16*>(l.C)};
+  if (g.d == 32) return matrix_rows(g) >= 8192 ? launch_qkv<32, 4>(g, a, st) : launch_qkv<32, 2>(g, a, st);
+  if (g.d == 64) return launch_qkv<64, 1>(g, a, st);
+  return cudaErrorNotSupported;
+}
 
 // n problems (1 or 2) of one geometry in one launch each.  Rows per tile: 16 (d 32: 32) for the shortest chain while a launch is about
 // the latency of a tile, twice as many where the weight reads of many tiles (through L1) become what counts.  Limits in rows per

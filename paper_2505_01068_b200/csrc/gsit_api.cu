@@ -289,6 +289,10 @@ gsit_status gsit_im_qkv_proj(const gsit_shape* shape, const void* x, int64_t x_r
   a.C = qkv; a.ldc = 3 * (int64_t)g.d;
   a.M = (int)matrix_rows(g); a.N = 3 * g.d; a.K = g.d;
   a.mask_rows = 1;
+  if (shape->dtype == GSIT_BF16 && g_attn_variant == GSIT_ATTN_DEFAULT && qkv_rows_preferred(g)) {
+    TraceScope t(GSIT_KERNEL_LINEAR, static_cast<cudaStream_t>(stream));
+    return from_cuda(launch_qkv_rows(g, a, static_cast<cudaStream_t>(stream)));
+  }
   if (g.row_start != nullptr) {
     // packed rows: the tcgen05 kernel computes and writes this call's row range only (widths it covers: multiples of 64)
     if (shape->dtype != GSIT_BF16 || !linear_tc_supported(a)) return GSIT_ERR_UNSUPPORTED;
@@ -632,6 +636,12 @@ size_t gsit_workspace_bytes(const gsit_shape* shape, int which_call, int32_t d_f
   if (which_call == GSIT_CALL_ATTENTION) return (shape->dtype == GSIT_BF16) ? ATTENTION_SCRATCH : 0;
   if (which_call == GSIT_CALL_QKV_PROJ) return 0;
   return (size_t)-1;
+}
+
+int32_t gsit_attention_uses_workspace(const gsit_shape* shape) {
+  Geometry g;
+  if (make_geometry(shape, &g) != GSIT_OK) return -1;
+  return shape->dtype == GSIT_BF16 && g.hd != 64 && attn_uses_tensor_memory(g, g.allowed);
 }
 
 gsit_status gsit_last_device_status(gsit_stream stream, uint32_t* flags) {

@@ -249,10 +249,12 @@ PyObject* im_attention_fwd(PyObject* const* a) {
   at::Tensor made, lse, made_ws;
   if (out == nullptr) made = empty({B, L, H * hd}, q.scalar_type(), q.device());
   if (want_lse) lse = empty({B, H, L}, at::kFloat, q.device());
-  const size_t need = scratch_bytes(s, GSIT_CALL_ATTENTION, 0);
-  if (ws == nullptr && need > 0) {
-    made_ws = empty({(int64_t)need}, at::kByte, q.device());
-    ws = &made_ws;
+  // (an allocation is a quarter of what a small call takes on the host: only for the kernels that read their scratch)
+  if (const int uses = ws == nullptr ? gsit_attention_uses_workspace(&s) : 0; uses != 0) {
+    if (const size_t need = scratch_bytes(s, GSIT_CALL_ATTENTION, 0); need > 0) {  // an invalid shape raises here
+      made_ws = empty({(int64_t)need}, at::kByte, q.device());
+      ws = &made_ws;
+    }
   }
   void* dst = out != nullptr ? out->data_ptr() : made.data_ptr();
   float* lse_p = want_lse ? static_cast<float*>(lse.data_ptr()) : nullptr;

@@ -101,3 +101,34 @@ def test_layer_on_either_side_of_the_row_limit(g, d, heads, above):
     else:
         assert torch.equal(halves, y)
     assert g.last_device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("d,heads,seg,B", [(32, 4, (3, 1, 2), 1), (32, 1, (17, 130, 45), 5), (32, 4, (33, 257, 300), 15), (64, 8, (3, 5, 9), 1), (64, 2, (40, 193, 267), 4)])
+def test_projection_on_row_tiles(g, d, heads, seg, B):
+    """The projection alone on row tiles (32 and, from 8192 rows on, 64 rows at d 32; 16 at d 64 up to 2000 rows): strided input with NaN
+    in the padding against a float product of the same operands (bf16 result: 2^-8 relative), and the packed layout bit for bit."""
+    rng = np.random.default_rng(B)
+    L, cap = sum(seg), B * sum(seg)
+    valid = np.stack([rng.integers(0, n + 1, size=B) for n in seg], axis=1).astype(np.int32)
+    vl, pm = torch.from_numpy(valid).cuda(), torch.from_numpy(pad_mask(seg, valid, B)).cuda()
+    x = to_dev(rng.standard_normal((B, L, d), dtype=np.float32), "bf16")
+    x[pm] = float("nan")
+    wide = torch.full((B, L, 2 * d), float("nan"), dtype=torch.bfloat16, device="cuda")
+    wide[:, :, d:] = x
+    w, bias = to_dev(wk.xavier_uniform(rng, 3 * d, d), "bf16"), to_dev(rng.standard_normal(3 * d).astype(np.float32))
+    for b in (bias, None):
+        got = g.im_qkv_proj(wide[:, :, d:], w, b, seg, heads, vl).reshape(B, L, 3 * d)
+        ref = torch.nan_to_num(x.float()) @ w.float().T + (0 if b is None else b)
+        assert bool((got[pm] == 0).all())
+        assert float((got.float() - ref)[~pm].abs().max()) <= 2.0 ** -8 * max(1.0, float(ref[~pm].abs().max()))
+    plan = g.plan_rows(vl, seg)
+    xp = g.pack_rows(torch.nan_to_num(x.float()), torch.zeros((cap, d), device="cuda"), seg, vl, plan).bfloat16()
+    for lo, hi in {(0, B), (B // 2, B)}:
+        out = torch.full((cap, 3, heads, d // heads), 7.0, dtype=torch.bfloat16, device="cuda")
+        g.im_qkv_proj(xp, w, None, seg, heads, vl[lo:hi], out=out, row_start=plan[3 * lo:])
+        want = torch.full((cap, 3 * d), 7.0, device="cuda")
+        first, last = int(plan[3 * lo]), int(plan[3 * hi])
+        whole = g.pack_rows(got.float(), torch.zeros((cap, 3 * d), device="cuda"), seg, vl, plan)
+        want[first:last] = whole[first:last]
+        assert torch.equal(out.reshape(cap, 3 * d).float(), want), (lo, hi)
+    assert g.last_device_status() == (0, 0)
