@@ -587,6 +587,14 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
   }
 }
 
+// Clears the work counter of a call that has no earlier kernel to do it.  (A memset breaks the chain of overlapped launches: the
+// attention then starts only once it is over, and the memset once the kernel before it is.)
+__global__ void clear_counter_kernel(int* next_item) {
+  grid_dep_wait();
+  grid_dep_launch();
+  if (threadIdx.x == 0) *next_item = 0;
+}
+
 template <int HD>
 cudaError_t launch_tcs(const Geometry& g, const AttnOperands* ops, int n, int64_t row_stride, float scale, int* next_item,
                        cudaStream_t st, bool counter_cleared) {
@@ -625,8 +633,9 @@ cudaError_t launch_tcs(const Geometry& g, const AttnOperands* ops, int n, int64_
   if (n_items > 0x3fffffffLL || slices >= (1 << WHICH_SHIFT)) return cudaErrorNotSupported;
   const int64_t resident = (int64_t)S_CTAS_PER_SM * n_sm;
   const unsigned grid = (unsigned)((n_items < resident) ? n_items : resident);
+  if (n_items <= resident) next_item = nullptr;  // an item per CTA: nothing to hand out
   if (next_item != nullptr && !counter_cleared) {
-    e = cudaMemsetAsync(next_item, 0, sizeof(int), st);
+    e = launch_overlapped(clear_counter_kernel, dim3(1), dim3(32), 0, st, next_item);
     if (e != cudaSuccess) return e;
   }
   return launch_overlapped(attn_tcs_kernel<HD>, dim3(grid), dim3(S_THREADS), C::SMEM, st, pr[0], pr[1], g,
