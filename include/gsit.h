@@ -194,6 +194,17 @@ gsit_status gsit_pack_rows(const gsit_shape* shape, const float* x, int64_t x_ro
                            int64_t packed_row_stride, int32_t cols, gsit_stream stream);
 gsit_status gsit_plan_pack_rows(const gsit_shape* shape, int32_t* row_start, const float* x, int64_t x_row_stride, float* x_packed,
                                 int64_t packed_row_stride, int32_t cols, gsit_stream stream);
+/* gsit_plan_pack_map_rows does the same and prepares a result [B, L, 2 cols] for gsit_im_layer_scatter_fwd: row_map (int32 [capacity])
+ *   receives the row b * L + position of every packed row, and the padding rows of y are set to +0 (its other rows are left alone).
+ *   GSIT_ERR_UNSUPPORTED above 1024 samples.
+ * gsit_im_layer_scatter_fwd is gsit_im_layer_fwd on packed rows whose result goes straight to the padded matrix: packed row i to row
+ *   row_map[i] of y.  Covered (gsit_layer_scatters returns 1) where the tcgen05 halves at d_model 128 serve the layer. */
+gsit_status gsit_plan_pack_map_rows(const gsit_shape* shape, int32_t* row_start, int32_t* row_map, const float* x, int64_t x_row_stride,
+                                    float* x_packed, int64_t packed_row_stride, int32_t cols, float* y, int64_t y_row_stride, gsit_stream stream);
+int32_t gsit_layer_scatters(const gsit_shape* shape, int32_t d_ff);
+gsit_status gsit_im_layer_scatter_fwd(const gsit_shape* shape, const gsit_layer_weights* weights, const float* x, int64_t x_row_stride,
+                                      const int32_t* row_map, float* y, int64_t y_row_stride, void* workspace, size_t workspace_bytes,
+                                      gsit_stream stream);
 gsit_status gsit_unpack_rows(const gsit_shape* shape, const float* y_packed, int64_t packed_row_stride, float* y,
                              int64_t y_row_stride, int32_t cols, gsit_stream stream);
 

@@ -21,6 +21,8 @@ struct Geometry {
   // segment s of sample b in a [capacity, d] matrix that holds real rows only, entry 3 B is the row after the last one.
   const int32_t* row_start;
   int capacity;              // rows of the packed matrices (host value, for the tensor maps)
+  // Packed layout, one layer call only: row i of the result goes to row out_rows[i] of a padded matrix (nullptr: to row i)
+  const int32_t* out_rows;
   __host__ __device__ __forceinline__ int len(int s) const { return seg_len[s]; }
   __host__ __device__ __forceinline__ int off(int s) const { return seg_off[s]; }
 };
@@ -247,8 +249,9 @@ cudaError_t launch_stack_head(const Geometry& g, int dtype, const float* c, int6
 // packed row layout (rows.cu)
 cudaError_t launch_plan_rows(const Geometry& g, int split_sample, int32_t* row_start, cudaStream_t st);
 bool plan_pack_supported(const Geometry& g);
+// row_map (may be null): the padded row of every packed one; y (may be null): its padded rows of 2 cols columns are zeroed
 cudaError_t launch_plan_pack(const Geometry& g, int32_t* row_start, const float* src, int64_t src_stride, float* dst, int64_t dst_stride, int cols,
-                             cudaStream_t st);
+                             int32_t* row_map, float* y, int64_t y_stride, cudaStream_t st);
 cudaError_t launch_move_rows(const Geometry& g, bool pack, const float* src, int64_t src_stride, float* dst, int64_t dst_stride,
                              int cols, cudaStream_t st);
 

@@ -490,6 +490,12 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
       // written swizzled and read back with four lanes per row -- each store then covers 8 rows x 64 contiguous bytes.
       const uint32_t scr = base + OFF_F + (uint32_t)(warp - 2) * 2048u;
       const int jj = lane & 3, rr0 = lane >> 2;
+      int to[4];  // where this lane's rows go: a padded matrix, when the geometry names the places, saves the stack a scatter
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int grow = row0 + ((warp & 3) << 5) + 8 * k + rr0;
+        to[k] = grow >= rows ? -1 : g.out_rows != nullptr ? g.out_rows[grow] : grow;
+      }
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         uint32_t a[32];
@@ -512,8 +518,7 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
           for (int k = 0; k < 4; ++k) {
             const int rr = 8 * k + rr0;
             const float4 o = ld_v4f(scr + rr * 64 + ((jj ^ ((rr >> 1) & 3)) << 4));
-            const int grow = row0 + ((warp & 3) << 5) + rr;
-            if (grow < rows) *reinterpret_cast<float4*>(y + (int64_t)grow * ldy + 64 * hf + 32 * c + 16 * sub + 4 * jj) = o;
+            if (to[k] >= 0) *reinterpret_cast<float4*>(y + (int64_t)to[k] * ldy + 64 * hf + 32 * c + 16 * sub + 4 * jj) = o;
           }
           __syncwarp();
         }

@@ -73,6 +73,7 @@ gsit_status make_geometry(const gsit_shape* s, Geometry* g) {
   g->valid_len = s->valid_len;
   g->status = nullptr;
   g->row_start = s->row_start;
+  g->out_rows = nullptr;
   g->capacity = 0;
   if (s->row_start != nullptr) {  // packed row layout
     if (s->valid_len == nullptr || s->packed_capacity < 1) return GSIT_ERR_INVALID_ARG;
@@ -320,9 +321,8 @@ gsit_status gsit_im_attention_fwd(const gsit_shape* shape, const void* q, const 
                        static_cast<cudaStream_t>(stream));
 }
 
-gsit_status gsit_im_layer_fwd(const gsit_shape* shape, const gsit_layer_weights* w, const float* x,
-                              int64_t x_row_stride, float* y, int64_t y_row_stride, void* workspace,
-                              size_t workspace_bytes, gsit_stream stream) {
+static gsit_status layer_fwd(const gsit_shape* shape, const gsit_layer_weights* w, const float* x, int64_t x_row_stride, float* y,
+                             int64_t y_row_stride, const int32_t* row_map, void* workspace, size_t workspace_bytes, gsit_stream stream) {
   Geometry g;
   gsit_status st = make_geometry(shape, &g);
   if (st != GSIT_OK) return st;
@@ -347,6 +347,8 @@ gsit_status gsit_im_layer_fwd(const gsit_shape* shape, const gsit_layer_weights*
   const int es = bf ? 2 : 4;
   const int M = g.batch * g.L, d = g.d;
   const Halves halves = bf ? pick_halves(g, w->d_ff) : HALVES_NONE;
+  if (row_map != nullptr && (g.row_start == nullptr || halves != HALVES_TC128)) return GSIT_ERR_UNSUPPORTED;
+  g.out_rows = row_map;
   if (g.row_start != nullptr && (halves == HALVES_NONE || g.hd > 32))
     return GSIT_ERR_UNSUPPORTED;  // the packed layout is implemented by the fused halves and the mma.sync / tensor-memory attention
 
@@ -417,6 +419,24 @@ gsit_status gsit_im_layer_fwd(const gsit_shape* shape, const gsit_layer_weights*
   a.A = f; a.lda = w->d_ff; a.W = w->w_2; a.bias = w->b_2; a.residual = y1; a.ldr = d;
   a.C = y; a.ldc = y_row_stride; a.M = M; a.N = d; a.K = w->d_ff; a.out_f32 = 1; a.mask_rows = 1;
   return run_linear(g, dtype, a, cs);
+}
+
+gsit_status gsit_im_layer_fwd(const gsit_shape* shape, const gsit_layer_weights* w, const float* x, int64_t x_row_stride, float* y,
+                              int64_t y_row_stride, void* workspace, size_t workspace_bytes, gsit_stream stream) {
+  return layer_fwd(shape, w, x, x_row_stride, y, y_row_stride, nullptr, workspace, workspace_bytes, stream);
+}
+
+int32_t gsit_layer_scatters(const gsit_shape* shape, int32_t d_ff) {
+  Geometry g;
+  return make_geometry(shape, &g) == GSIT_OK && g.row_start != nullptr && shape->dtype == GSIT_BF16 && d_ff >= 1 && d_ff % 8 == 0 && g.hd <= 32 &&
+         pick_halves(g, d_ff) == HALVES_TC128;
+}
+
+gsit_status gsit_im_layer_scatter_fwd(const gsit_shape* shape, const gsit_layer_weights* w, const float* x, int64_t x_row_stride,
+                                      const int32_t* row_map, float* y, int64_t y_row_stride, void* workspace, size_t workspace_bytes,
+                                      gsit_stream stream) {
+  if (!row_map) return GSIT_ERR_INVALID_ARG;
+  return layer_fwd(shape, w, x, x_row_stride, y, y_row_stride, row_map, workspace, workspace_bytes, stream);
 }
 
 gsit_status gsit_im_layer_pair_fwd(const gsit_shape* shape_a, const gsit_shape* shape_b, const gsit_layer_weights* w_a,
@@ -587,8 +607,8 @@ gsit_status gsit_pack_rows(const gsit_shape* shape, const float* x, int64_t x_ro
   return move_rows(shape, true, x, x_row_stride, x_packed, packed_row_stride, cols, stream);
 }
 
-gsit_status gsit_plan_pack_rows(const gsit_shape* shape, int32_t* row_start, const float* x, int64_t x_row_stride, float* x_packed,
-                                int64_t packed_row_stride, int32_t cols, gsit_stream stream) {
+static gsit_status plan_pack(const gsit_shape* shape, int32_t* row_start, const float* x, int64_t x_row_stride, float* x_packed,
+                             int64_t packed_row_stride, int32_t cols, int32_t* row_map, float* y, int64_t y_row_stride, gsit_stream stream) {
   if (shape == nullptr || row_start == nullptr || shape->valid_len == nullptr || !x || !x_packed) return GSIT_ERR_INVALID_ARG;
   if (cols < 4 || cols % 4 != 0 || x_row_stride < cols || packed_row_stride < cols || x_row_stride % 4 != 0 || packed_row_stride % 4 != 0)
     return GSIT_ERR_INVALID_ARG;
@@ -600,10 +620,23 @@ gsit_status gsit_plan_pack_rows(const gsit_shape* shape, int32_t* row_start, con
   if (st != GSIT_OK) return st;
   if (from_cuda(status_ptr(&g.status)) != GSIT_OK) return GSIT_ERR_CUDA;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
-  if (plan_pack_supported(g)) return from_cuda(launch_plan_pack(g, row_start, x, x_row_stride, x_packed, packed_row_stride, cols, cs));
+  if (plan_pack_supported(g))
+    return from_cuda(launch_plan_pack(g, row_start, x, x_row_stride, x_packed, packed_row_stride, cols, row_map, y, y_row_stride, cs));
+  if (row_map != nullptr) return GSIT_ERR_UNSUPPORTED;
   if ((st = from_cuda(launch_plan_rows(g, 0, row_start, cs))) != GSIT_OK) return st;
   g.row_start = row_start;
   return from_cuda(launch_move_rows(g, true, x, x_row_stride, x_packed, packed_row_stride, cols, cs));
+}
+
+gsit_status gsit_plan_pack_rows(const gsit_shape* shape, int32_t* row_start, const float* x, int64_t x_row_stride, float* x_packed,
+                                int64_t packed_row_stride, int32_t cols, gsit_stream stream) {
+  return plan_pack(shape, row_start, x, x_row_stride, x_packed, packed_row_stride, cols, nullptr, nullptr, 0, stream);
+}
+
+gsit_status gsit_plan_pack_map_rows(const gsit_shape* shape, int32_t* row_start, int32_t* row_map, const float* x, int64_t x_row_stride,
+                                    float* x_packed, int64_t packed_row_stride, int32_t cols, float* y, int64_t y_row_stride, gsit_stream stream) {
+  if (!row_map || !y || !aligned16(y) || y_row_stride < 2 * (int64_t)cols || y_row_stride % 4 != 0) return GSIT_ERR_INVALID_ARG;
+  return plan_pack(shape, row_start, x, x_row_stride, x_packed, packed_row_stride, cols, row_map, y, y_row_stride, stream);
 }
 
 gsit_status gsit_unpack_rows(const gsit_shape* shape, const float* y_packed, int64_t packed_row_stride, float* y,

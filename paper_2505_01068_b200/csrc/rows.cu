@@ -92,7 +92,8 @@ __global__ void __launch_bounds__(256) move_rows_kernel(const __grid_constant__ 
 constexpr int PLAN_MAX = 3072;  // entries (samples x segments) a CTA can hold
 __global__ void __launch_bounds__(256) plan_pack_kernel(const __grid_constant__ Geometry g, int32_t* __restrict__ row_start, const float* __restrict__ src,
                                                         const int64_t src_stride, float* __restrict__ dst, const int64_t dst_stride, const int cpr,
-                                                        const unsigned total, const unsigned quarter) {
+                                                        const unsigned total, const unsigned quarter, int32_t* __restrict__ row_map,
+                                                        float* __restrict__ y, const int64_t y_stride) {
   __shared__ int starts[PLAN_MAX + 1];
   __shared__ int warp_sum[8];
   ptx::load_params_early(g, src, src_stride, dst, dst_stride);
@@ -132,7 +133,14 @@ __global__ void __launch_bounds__(256) plan_pack_kernel(const __grid_constant__ 
     const unsigned w = idx / (unsigned)cpr, c = idx - w * (unsigned)cpr;  // padded-layout row, chunk in the row
     const int b = (int)(w / (unsigned)g.L), p = (int)(w - (unsigned)b * (unsigned)g.L);
     const int s = segment_of(g, p), i = p - g.off(s), at = starts[3 * b + s];
-    if (i >= starts[3 * b + s + 1] - at) continue;
+    if (i >= starts[3 * b + s + 1] - at) {
+      if (y != nullptr) {  // the result's padding, twice as wide: nobody else writes it
+        float4* z = reinterpret_cast<float4*>(y + (int64_t)w * y_stride) + 2 * c;
+        z[0] = z[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+      continue;
+    }
+    if (row_map != nullptr && c == 0) row_map[at + i] = (int)w;
     out[u] = reinterpret_cast<float4*>(dst + (int64_t)(at + i) * dst_stride) + c;
     v[u] = __ldg(reinterpret_cast<const float4*>(src + (int64_t)w * src_stride) + c);
   }
@@ -146,13 +154,13 @@ __global__ void __launch_bounds__(256) plan_pack_kernel(const __grid_constant__ 
 bool plan_pack_supported(const Geometry& g) { return 3 * g.batch <= PLAN_MAX; }
 
 cudaError_t launch_plan_pack(const Geometry& g, int32_t* row_start, const float* src, int64_t src_stride, float* dst, int64_t dst_stride, int cols,
-                             cudaStream_t st) {
+                             int32_t* row_map, float* y, int64_t y_stride, cudaStream_t st) {
   const int cpr = cols / 4;
   const int64_t total = (int64_t)g.batch * g.L * cpr;
   if (total > 0xffffffffLL || !plan_pack_supported(g)) return cudaErrorNotSupported;
   const unsigned quarter = (unsigned)((total + MOVE_UNROLL - 1) / MOVE_UNROLL);
   return launch_overlapped(plan_pack_kernel, dim3((quarter + 255u) / 256u), dim3(256), 0, st, g, row_start, src, src_stride, dst, dst_stride, cpr,
-                           (unsigned)total, quarter);
+                           (unsigned)total, quarter, row_map, y, y_stride);
 }
 
 cudaError_t launch_plan_rows(const Geometry& g, int split_sample, int32_t* row_start, cudaStream_t st) {

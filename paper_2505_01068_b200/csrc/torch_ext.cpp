@@ -429,8 +429,9 @@ bool chained(const at::Tensor& x, PyObject* seg, int64_t heads, int64_t intra_he
 }
 
 // x, valid_len, y, fwd, bwd, intra, seg_len, heads, intra_heads, ln_eps, buffers
-//   buffers = (plan or None, workspace, ring_a0, ring_a1, ring_b0, ring_b1, x_packed or None, wide_0, wide_1): with a plan the
-//   packed row layout is used (x gathered into x_packed, the result scattered into y), without one the padded layout.
+//   buffers = (plan or None, workspace, ring_a0, ring_a1, ring_b0, ring_b1, x_packed or None, wide_0, wide_1, row_map or None): with a
+//   plan the packed row layout is used (x gathered into x_packed; the result scattered into y, by the last layer itself where it
+//   can), without one the padded layout.
 // Everything runs on the caller's stream, the whole batch per launch: every kernel then starts under the tail of the one
 // before it.  (Halves of the batch on two streams in the intra encoder, 820 us against 784 at 64 x 1050 rows, 234 against
 // 225 at 2 x 1050: the fork and the join each cost one such overlap.)
@@ -443,9 +444,9 @@ PyObject* stack_forward(PyObject* const* a) {
   const double eps = as_float(a[9]);
   const std::deque<Layer> intra = all_layers(a[5], eps), fwd = all_layers(a[3], eps), bwd = all_layers(a[4], eps);
   require(fwd.size() == bwd.size() && !fwd.empty(), "rings of equal depth");
-  require(PyTuple_Check(a[10]) && PyTuple_GET_SIZE(a[10]) == 9, "buffers: nine tensors");
-  const at::Tensor* b[9];
-  for (int i = 0; i < 9; ++i) b[i] = opt_tensor(PyTuple_GET_ITEM(a[10], i));
+  require(PyTuple_Check(a[10]) && PyTuple_GET_SIZE(a[10]) == 10, "buffers: ten tensors");
+  const at::Tensor* b[10];
+  for (int i = 0; i < 10; ++i) b[i] = opt_tensor(PyTuple_GET_ITEM(a[10], i));
   // layers that run as one launch each do no work for padding in the padded layout either: no plan, no copies between layouts then
   const at::Tensor* plan = b[0];
   if (plan != nullptr && chained(x, a[6], as_int(a[7]), as_int(a[8]), valid, fwd, bwd, intra)) plan = nullptr;
@@ -463,9 +464,17 @@ PyObject* stack_forward(PyObject* const* a) {
 
   auto issue = [&]() -> gsit_status {
     gsit_status st = GSIT_OK;
+    int32_t* row_map = nullptr;  // the last layer writes the padded result itself
     if (plan != nullptr) {
       float* xp = f(b[6]);
-      st = gsit_plan_pack_rows(&ring_shape, static_cast<int32_t*>(plan->data_ptr()), x_in, ldx, xp, d, (int32_t)d, cs);
+      int32_t* starts = static_cast<int32_t*>(plan->data_ptr());
+      if (!intra.empty() && B <= 1024) {
+        gsit_shape last = intra_shape;
+        last.dtype = intra.back().dtype;
+        if (gsit_layer_scatters(&last, intra.back().w.d_ff)) row_map = static_cast<int32_t*>(b[9]->data_ptr());
+      }
+      st = row_map != nullptr ? gsit_plan_pack_map_rows(&ring_shape, starts, row_map, x_in, ldx, xp, d, (int32_t)d, out, 2 * d, cs)
+                              : gsit_plan_pack_rows(&ring_shape, starts, x_in, ldx, xp, d, (int32_t)d, cs);
       if (st != GSIT_OK) return st;
       x_in = xp;
       ldx = d;
@@ -517,7 +526,8 @@ PyObject* stack_forward(PyObject* const* a) {
       in_wide ^= 1;
     }
     gsit_shape si = intra_shape;
-    if (!intra.empty() && uniform(intra, intra)) {
+    const size_t plain = intra.size() - (row_map != nullptr ? 1 : 0);  // layers before the one that scatters
+    if (plain > 0 && uniform(intra, intra)) {
       si.dtype = intra[0].dtype;
       const gsit_shape* shape = &si;
       const gsit_layer_weights* const* w = wi.data();
@@ -525,14 +535,18 @@ PyObject* stack_forward(PyObject* const* a) {
       const int64_t ldxs = 2 * d;
       float* const* ys = yi.data();
       const int64_t* ldys = ldi.data();
-      st = gsit_im_encoder_fwd(&shape, 1, &w, (int32_t)intra.size(), &xs, &ldxs, &ys, &ldys, ws, ws_n, cs);
+      st = gsit_im_encoder_fwd(&shape, 1, &w, (int32_t)plain, &xs, &ldxs, &ys, &ldys, ws, ws_n, cs);
       if (st != GSIT_OK) return st;
     } else {
-      for (size_t i = 0; i < intra.size(); ++i) {
+      for (size_t i = 0; i < plain; ++i) {
         si.dtype = intra[i].dtype;
         st = gsit_im_layer_fwd(&si, wi[i], i == 0 ? wide[0] : yi[i - 1], 2 * d, yi[i], 2 * d, ws, ws_n, cs);
         if (st != GSIT_OK) return st;
       }
+    }
+    if (row_map != nullptr) {
+      si.dtype = intra[plain].dtype;
+      return gsit_im_layer_scatter_fwd(&si, wi[plain], plain == 0 ? wide[0] : yi[plain - 1], 2 * d, row_map, out, 2 * d, ws, ws_n, cs);
     }
     if (plan != nullptr) st = gsit_unpack_rows(&ring_shape, wide[in_wide], 2 * d, out, 2 * d, (int32_t)(2 * d), cs);
     return st;

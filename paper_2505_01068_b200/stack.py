@@ -205,7 +205,7 @@ class GsitStack:
         return res
 
     def _native_buffers(self, x, valid_len, packed):
-        """Buffers of the natively issued forward, kept per problem size: (the nine tensors stack_forward takes, result)."""
+        """Buffers of the natively issued forward, kept per problem size: (the ten tensors stack_forward takes, result)."""
         key = ("native", packed, x.shape, x.device)
         got = None if self._bufs is None else self._bufs.get(key)
         if got is not None:
@@ -217,7 +217,7 @@ class GsitStack:
         # rows past the last real one are read by the last row tile (and discarded): they start out as zeros
         z = lambda cols: torch.zeros((cap, cols), dtype=torch.float32, device=x.device)
         bufs = (plan, torch.empty(2 * need, dtype=torch.uint8, device=x.device), z(d), z(d), z(d), z(d), z(d) if packed else None,
-                z(2 * d), z(2 * d))
+                z(2 * d), z(2 * d), torch.empty(cap, dtype=torch.int32, device=x.device) if packed else None)
         if self._bufs is None:
             self._bufs = {}
         got = self._bufs[key] = (bufs, torch.empty((Bn, L, 2 * d), dtype=torch.float32, device=x.device))

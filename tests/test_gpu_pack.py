@@ -1,7 +1,8 @@
 """Row plan and gather in one launch against the two separate calls, on both sides of the number of samples that one
-CTA can scan (1024)."""
+CTA can scan (1024); the stack whose last layer writes the padded result itself."""
 import ctypes
 
+import numpy as np
 import pytest
 import torch
 
@@ -26,3 +27,30 @@ def test_plan_pack_matches_separate_calls(batch, seg_len, cols):
                                       ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
     assert st == 0
     assert torch.equal(plan, want_plan) and torch.equal(got, want)
+
+
+@pytest.mark.parametrize("intra_depth", [1, 2])
+@pytest.mark.parametrize("d", [32, 64])
+def test_stack_result_in_the_padded_layout(d, intra_depth):
+    """Above the row limit of the small tiles the stack packs rows; at width 64 its last layer (128 wide) writes the padded result itself, at
+    32 a scatter does.  Padded layout throughout and packed: equal bit for bit, padding +0 in a buffer that held NaN, input a view
+    of the result buffer of the call before."""
+    import paper_2505_01068_b200 as g
+    import workloads as wk
+    from gpu_util import weights_to_dev
+    rng = np.random.default_rng(d)
+    seg, B = (50, 300, 270), 12
+    layers = lambda width, n: [weights_to_dev(wk.draw_layer_weights(rng, width, 2 * width, "bf16", affine=True), "bf16") for _ in range(n)]
+    fwd, bwd, intra = layers(d, 1), layers(d, 1), layers(2 * d, intra_depth)
+    valid = np.stack([rng.integers(0, n + 1, size=B) for n in seg], axis=1).astype(np.int32)
+    valid[3], valid[7] = 0, seg
+    vl = torch.from_numpy(valid).cuda()
+    x = torch.from_numpy(rng.standard_normal((B, sum(seg), d), dtype=np.float32)).cuda()
+    want = g.GsitStack(fwd, bwd, intra, seg, 4, 4, packed=False).forward(x, vl).clone()
+    out = torch.full((B, sum(seg), 2 * d), float("nan"), device="cuda")
+    out[:, :, d:] = x
+    st = g.GsitStack(fwd, bwd, intra, seg, 4, 4)
+    got = st.forward(out[:, :, d:], vl, out=out)
+    assert st.packed and torch.equal(got, want)
+    assert not torch.signbit(got[torch.from_numpy(wk.padded_row_mask(seg, valid, B)).cuda()]).any()
+    assert g.last_device_status() == (0, 0)
