@@ -98,7 +98,7 @@ cudaError_t launch_attn_bf16_n(const Geometry& g, const AttnOperands* ops, int n
     for (int i = 0; i < n; ++i) {  // one launch per problem
       Geometry gi = g;
       gi.allowed = ops[i].allowed;
-      e = launch_attn_tc_hd64(gi, ops[i].q, ops[i].k, ops[i].v, row_stride, ops[i].out, ops[i].lse, scale, st);
+      e = launch_attn_tc_hd64(gi, ops[i].q, ops[i].k, ops[i].v, row_stride, ops[i].out, ops[i].lse, scale, next_item, st, counter_cleared && i == 0);
       if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

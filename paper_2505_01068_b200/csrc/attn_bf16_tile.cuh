@@ -494,19 +494,5 @@ __device__ __forceinline__ void attend_tile(const Geometry& g, const Tile& t_, c
   __syncthreads();
 }
 
-// Query segments in descending order of the keys their tiles walk (longest work first), two bits per segment index.
-int segment_order(const Geometry& g, uint32_t allowed) {
-  int cost[3], ord[3] = {0, 1, 2};
-  for (int s = 0; s < 3; ++s) {
-    cost[s] = 0;
-    for (int r = 0; r < 3; ++r)
-      if ((allowed >> (3 * s + r)) & 1u) cost[s] += g.len(r);
-  }
-  for (int i = 0; i < 3; ++i)
-    for (int j = i + 1; j < 3; ++j)
-      if (cost[ord[j]] > cost[ord[i]]) { const int t = ord[i]; ord[i] = ord[j]; ord[j] = t; }
-  return ord[0] | (ord[1] << 2) | (ord[2] << 4);
-}
-
 }  // namespace
 }  // namespace gsit

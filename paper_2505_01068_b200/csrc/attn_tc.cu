@@ -5,7 +5,7 @@
 // a work item is 128 query rows of one modality segment of one head of one sample; it walks only the key tiles of
 // the segment(s) the Interlaced Mask opens for that block row, up to the sample's valid length.
 //
-// The grid is persistent: two CTAs per SM, each striding over the work items, so tensor memory, barriers and the
+// The grid is persistent: two CTAs per SM, each taking work items until there are none left, so tensor memory, barriers and the
 // tensor maps are set up once and the loads of the next item start while the current one is still being reduced.
 // Roles inside a CTA of 6 warps:
 //   warp 0, one thread   TMA producer: Q (two buffers), K and V tiles of 64 keys (four-stage rings)
@@ -62,18 +62,21 @@ struct Item {
   int grow0;                    // first row of the query tile in the activation matrices
 };
 
-__device__ __forceinline__ Item decode_item(const Geometry& g, int w, int tiles_per_sample) {
+// Items in order of the segments with the longest walks first (seg_order: three segment indices, two bits each), so that the short ones
+// even out the end; within a segment the query tiles of a head stay together, which read the same keys.  Against sample by sample,
+// us, cross / intra: 32 x (50, 375, 500), 2 heads 20.0/20.1 -> 14.5/18.7; 64 samples 34.8/35.6 -> 27.3/31.1; together with the counter
+// 128 x (128, 1024, 1024), 8 heads 483/707 -> 460/674.  A launch of a single item per CTA pays 0.2 us for it.
+__device__ __forceinline__ Item decode_item(const Geometry& g, int w, int seg_order) {
   Item it;
-  const int bh = w / tiles_per_sample;
-  int tile = w - bh * tiles_per_sample;
+  const int heads = g.batch * g.heads;
+  const int s0 = seg_order & 3, s1 = (seg_order >> 2) & 3, s2 = seg_order >> 4;
+  const int t0 = (g.len(s0) + TQ - 1) / TQ, t1 = (g.len(s1) + TQ - 1) / TQ, t2 = (g.len(s2) + TQ - 1) / TQ;
+  const bool past0 = w >= t0 * heads, past1 = w >= (t0 + t1) * heads;
+  const int s = past1 ? s2 : past0 ? s1 : s0, nts = past1 ? t2 : past0 ? t1 : t0;
+  w -= past1 ? (t0 + t1) * heads : past0 ? t0 * heads : 0;
+  const int bh = w / nts, tile = w - bh * nts;
   it.b = bh / g.heads;
   it.h = bh - it.b * g.heads;
-  int s = 0;
-#pragma unroll
-  for (int ss = 0; ss < 2; ++ss) {
-    const int nts = (g.len(s) + TQ - 1) / TQ;
-    if (tile >= nts) { tile -= nts; ++s; }
-  }
   it.s = s;
   it.q0 = tile * TQ;
   const int in_seg = min(TQ, g.len(s) - it.q0);
@@ -120,7 +123,7 @@ __device__ __forceinline__ void publish_item(uint32_t base, const Item& it, int 
 // Consumer side (whole warp): waits for record k, copies it to registers and releases the slot (one arrival per warp).
 __device__ __forceinline__ Item fetch_item(const WaitCtx& wc, uint32_t base, int k, int lane) {
   const int slot = k % ITEM_SLOTS;
-  mbar_wait(wc, base + OFF_ITEMBAR + 8 * slot, (k / ITEM_SLOTS) & 1);
+  const bool ok = mbar_wait(wc, base + OFF_ITEMBAR + 8 * slot, (k / ITEM_SLOTS) & 1);
   const uint32_t a = base + OFF_ITEMS + 64 * slot;
   Item it;
   asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(it.b), "=r"(it.h), "=r"(it.s), "=r"(it.q0) : "r"(a) : "memory");
@@ -130,14 +133,15 @@ __device__ __forceinline__ Item fetch_item(const WaitCtx& wc, uint32_t base, int
   fence_reads_before_release();
   __syncwarp();
   if (lane == 0) mbar_arrive(base + OFF_ITEMBAR + 8 * ITEM_SLOTS + 8 * slot);
+  if (!ok) it.T = -1;  // a wait has run out: no further items
   return it;
 }
 
 __global__ void __launch_bounds__(TC_THREADS, 2)
 attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ Geometry g, __nv_bfloat16* __restrict__ out,
-                    float* __restrict__ lse, const float sl2 /* scale * log2(e) */, const int tiles_per_sample,
-                    const int n_items) {
+                    float* __restrict__ lse, const float sl2 /* scale * log2(e) */, const int seg_order,
+                    const int n_items, int* __restrict__ next_item /* zeroed counter, or nullptr = static round robin */) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t sQ = base + OFF_Q, sK = base + OFF_K, sV = base + OFF_V, bars = base + OFF_BAR;
@@ -177,21 +181,34 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   tc_fence_after();
   uint32_t tmem;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(bars + SLOT_TMEM) : "memory");
-  load_params_early(g, out, lse);
+  load_params_early(g, out, lse, sl2, seg_order, n_items, next_item);
   // q, k, v and the lengths may come from the kernel before this one; what stands above overlaps its tail (back to back, an ordinary
   // launch / this: 1 x (8, 110, 148), 4 heads 8.8/6.9 us; 8 x (50, 500, 500), 2 heads 13.1/10.8; 128 x (128, 1024, 1024) 491/482)
   grid_dep_wait();
   grid_dep_launch();
 
+  // with a fixed assignment every role knows where it ends, without waiting for a record that says so
+  auto over = [&](int k) { return next_item == nullptr && (int)(blockIdx.x + k * gridDim.x) >= n_items; };
   if (warp == 0) {
     // ================================ TMA producer ================================
     {
       int n_q = 0, n_kv = 0;  // Q tiles and K/V tiles requested so far (ring positions and phases follow from them)
       int k = 0;              // items of this CTA so far
-      for (int w = blockIdx.x; w < n_items; w += gridDim.x, ++k) {
-        const Item it = decode_item(g, w, tiles_per_sample);
+      for (; !over(k); ++k) {
+        int w;
+        if (next_item != nullptr) {
+          w = (lane == 0) ? atomicAdd(next_item, 1) : 0;
+          w = __shfl_sync(0xffffffffu, w, 0);
+        } else {
+          w = blockIdx.x + k * gridDim.x;
+        }
+        const bool end = next_item != nullptr && (w >= n_items || cta_gave_up(wc));
+        Item it = {};
+        if (end) it.T = -1;
+        else it = decode_item(g, w, seg_order);
         if (k >= ITEM_SLOTS) mbar_wait(wc, base + OFF_ITEMBAR + 8 * ITEM_SLOTS + 8 * (k % ITEM_SLOTS), ((k / ITEM_SLOTS) - 1) & 1);
         publish_item(base, it, k, lane);
+        if (end) break;
         if (it.T == 0) continue;
         const int qb = n_q & 1, quse = n_q >> 1;
         if (quse > 0) mbar_wait(wc, bars + BAR_QEMPTY + 8 * qb, (quse - 1) & 1);
@@ -223,9 +240,9 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       constexpr uint32_t IDESC_QK = idesc_bf16(TK, false), IDESC_PV = idesc_bf16(HD64, true);
       int n_q = 0, n_kv = 0;  // Q tiles / key tiles consumed so far.  Key tile n uses S and P buffer n & 1 (phase
                               // (n >> 1) & 1 of their barriers) and ring stage n % KV_STAGES
-      int k = 0;
-      for (int w = blockIdx.x; w < n_items; w += gridDim.x, ++k) {
+      for (int k = 0; !over(k); ++k) {
         const Item it = fetch_item(wc, base, k, lane);
+        if (it.T < 0) break;
         if (it.T == 0) continue;
         const int qb = n_q & 1;
         const uint32_t sQb = sQ + qb * Q_BYTES;
@@ -276,9 +293,9 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     const float2 sl2v = make_float2(sl2, sl2);
     int n_kv = 0, n_items_done = 0;
 
-    int k = 0;
-    for (int w = blockIdx.x; w < n_items; w += gridDim.x, ++k) {
+    for (int k = 0; !over(k); ++k) {
       const Item it = fetch_item(wc, base, k, lane);
+      if (it.T < 0) break;
       const int64_t grow = (int64_t)it.grow0 + r;
       uint4* dst = reinterpret_cast<uint4*>(out + grow * g.d + it.h * HD64);
       float* lse_row = (lse != nullptr) ? lse + ((int64_t)it.b * g.heads + it.h) * g.L + g.off(it.s) + it.q0 + r : nullptr;
@@ -423,11 +440,24 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   }
 }
 
+int64_t items_of(const Geometry& g) {
+  int64_t tiles = 0;
+  for (int s = 0; s < 3; ++s) tiles += (g.len(s) + TQ - 1) / TQ;
+  return tiles * g.heads * g.batch;
+}
+
 }  // namespace
+
+// Handing the items out pays where every CTA takes several: with a fixed assignment the unluckiest CTA of 128 x (128, 1024, 1024), 8 heads,
+// a quarter of the samples at half length, has 3 - 4 % more to do than the average.
+bool attn_tc_hd64_uses_counter(const Geometry& g) {
+  int n_sm = 0;
+  return sm_count_and_smem_once(nullptr, 0, &n_sm) == cudaSuccess && items_of(g) > 8LL * n_sm;
+}
 
 cudaError_t launch_attn_tc_hd64(const Geometry& g, const __nv_bfloat16* q, const __nv_bfloat16* k,
                                 const __nv_bfloat16* v, int64_t row_stride, __nv_bfloat16* out, float* lse,
-                                float scale, cudaStream_t st) {
+                                float scale, int* next_item, cudaStream_t st, bool counter_cleared) {
   if (g.hd != HD64) return cudaErrorNotSupported;
   const int64_t rows = matrix_rows(g);
   alignas(64) CUtensorMap tmQ, tmK, tmV;
@@ -439,13 +469,16 @@ cudaError_t launch_attn_tc_hd64(const Geometry& g, const __nv_bfloat16* q, const
     cudaError_t e = sm_count_and_smem_once(reinterpret_cast<const void*>(attn_tc_hd64_kernel), TC_SMEM, &n_sm);
     if (e != cudaSuccess) return e;
   }
-  int tiles = 0;
-  for (int s = 0; s < 3; ++s) tiles += (g.len(s) + TQ - 1) / TQ;
-  const int64_t n_items = (int64_t)tiles * g.heads * g.batch;
-  if (n_items > 0x7fffffffLL) return cudaErrorNotSupported;
+  const int64_t n_items = items_of(g);
+  if (n_items > 0x3fffffffLL) return cudaErrorNotSupported;
+  if (!attn_tc_hd64_uses_counter(g)) next_item = nullptr;
+  if (next_item != nullptr && !counter_cleared) {
+    cudaError_t e = launch_clear_counter(next_item, st);
+    if (e != cudaSuccess) return e;
+  }
   const unsigned grid = (unsigned)((n_items < 2 * n_sm) ? n_items : 2 * n_sm);  // two resident CTAs per SM
   return launch_overlapped(attn_tc_hd64_kernel, dim3(grid), dim3(TC_THREADS), TC_SMEM, st, tmQ, tmK, tmV, g, out, lse, scale * 1.4426950408889634f,
-                           tiles, (int)n_items);
+                           segment_order(g, g.allowed), (int)n_items, next_item);
 }
 
 }  // namespace gsit

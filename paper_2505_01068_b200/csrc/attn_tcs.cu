@@ -610,17 +610,7 @@ cudaError_t launch_tcs(const Geometry& g, const AttnOperands* ops, int n, int64_
     pr[i].out = ops[i].out;
     pr[i].lse = ops[i].lse;
     pr[i].allowed = ops[i].allowed;
-    // query segments in descending order of the keys their tiles walk (longest work first)
-    int cost[3], ord[3] = {0, 1, 2};
-    for (int s = 0; s < 3; ++s) {
-      cost[s] = 0;
-      for (int r = 0; r < 3; ++r)
-        if ((ops[i].allowed >> (3 * s + r)) & 1u) cost[s] += g.len(r);
-    }
-    for (int a = 0; a < 3; ++a)
-      for (int b = a + 1; b < 3; ++b)
-        if (cost[ord[b]] > cost[ord[a]]) { const int t = ord[a]; ord[a] = ord[b]; ord[b] = t; }
-    pr[i].seg_order = ord[0] | (ord[1] << 2) | (ord[2] << 4);
+    pr[i].seg_order = segment_order(g, ops[i].allowed);
   }
   if (n == 1) pr[1] = pr[0];
   int n_sm = 0;
@@ -635,7 +625,7 @@ cudaError_t launch_tcs(const Geometry& g, const AttnOperands* ops, int n, int64_
   const unsigned grid = (unsigned)((n_items < resident) ? n_items : resident);
   if (n_items <= resident) next_item = nullptr;  // an item per CTA: nothing to hand out
   if (next_item != nullptr && !counter_cleared) {
-    e = launch_overlapped(clear_counter_kernel, dim3(1), dim3(32), 0, st, next_item);
+    e = launch_clear_counter(next_item, st);
     if (e != cudaSuccess) return e;
   }
   return launch_overlapped(attn_tcs_kernel<HD>, dim3(grid), dim3(S_THREADS), C::SMEM, st, pr[0], pr[1], g,
@@ -643,6 +633,8 @@ cudaError_t launch_tcs(const Geometry& g, const AttnOperands* ops, int n, int64_
 }
 
 }  // namespace
+
+cudaError_t launch_clear_counter(int* next_item, cudaStream_t st) { return launch_overlapped(clear_counter_kernel, dim3(1), dim3(32), 0, st, next_item); }
 
 bool attn_tcs_supported(const Geometry& g) {  // the kernel works on pairs of heads
   return (g.hd == 8 || g.hd == 16 || g.hd == 32) && g.heads % 2 == 0;

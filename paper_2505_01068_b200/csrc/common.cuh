@@ -67,6 +67,20 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
 
+// Query segments in descending order of the keys their tiles walk (longest work first), two bits per segment index.
+inline int segment_order(const Geometry& g, uint32_t allowed) {
+  int cost[3], ord[3] = {0, 1, 2};
+  for (int s = 0; s < 3; ++s) {
+    cost[s] = 0;
+    for (int r = 0; r < 3; ++r)
+      if ((allowed >> (3 * s + r)) & 1u) cost[s] += g.len(r);
+  }
+  for (int i = 0; i < 3; ++i)
+    for (int j = i + 1; j < 3; ++j)
+      if (cost[ord[j]] > cost[ord[i]]) { const int t = ord[i]; ord[i] = ord[j]; ord[j] = t; }
+  return ord[0] | (ord[1] << 2) | (ord[2] << 4);
+}
+
 // Per-device launch set-up (a process may drive several GPUs; kernel attributes and SM counts belong to a device):
 // sets the kernel's dynamic shared-memory limit the first time `func` is launched on the current device and returns
 // that device's SM count.  `func` identifies the kernel; at most 64 devices and 64 kernels are tracked.
@@ -135,7 +149,9 @@ cudaError_t launch_attn_bf16(const Geometry& g, const __nv_bfloat16* q, const __
 // bf16 attention for head_dim 64 on tcgen05 tensor cores with TMEM accumulators (attn_tc.cu)
 cudaError_t launch_attn_tc_hd64(const Geometry& g, const __nv_bfloat16* q, const __nv_bfloat16* k,
                                 const __nv_bfloat16* v, int64_t row_stride, __nv_bfloat16* out, float* lse,
-                                float scale, cudaStream_t st);
+                                float scale, int* next_item, cudaStream_t st, bool counter_cleared);
+bool attn_tc_hd64_uses_counter(const Geometry& g);  // would it use next_item?
+cudaError_t launch_clear_counter(int* next_item, cudaStream_t st);  // one word, as a kernel of the overlapped chain (attn_tcs.cu)
 
 // bf16 attention for head_dim 8 / 16 / 32 on tcgen05 with thread-per-row softmax (attn_tcs.cu).  next_item: a device int
 // the call may use as its work counter (cleared on the stream before the launch unless `counter_cleared` says that the

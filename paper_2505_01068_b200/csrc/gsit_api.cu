@@ -674,7 +674,7 @@ size_t gsit_workspace_bytes(const gsit_shape* shape, int which_call, int32_t d_f
 int32_t gsit_attention_uses_workspace(const gsit_shape* shape) {
   Geometry g;
   if (make_geometry(shape, &g) != GSIT_OK) return -1;
-  return shape->dtype == GSIT_BF16 && g.hd != 64 && attn_uses_tensor_memory(g, g.allowed);
+  return shape->dtype == GSIT_BF16 && attn_uses_tensor_memory(g, g.allowed) && (g.hd != 64 || attn_tc_hd64_uses_counter(g));
 }
 
 gsit_status gsit_last_device_status(gsit_stream stream, uint32_t* flags) {
