@@ -452,7 +452,7 @@ int64_t items_of(const Geometry& g) {
 // a quarter of the samples at half length, has 3 - 4 % more to do than the average.
 bool attn_tc_hd64_uses_counter(const Geometry& g) {
   int n_sm = 0;
-  return sm_count_and_smem_once(nullptr, 0, &n_sm) == cudaSuccess && items_of(g) > 8LL * n_sm;
+  return sm_count_and_smem_once(nullptr, 0, &n_sm) == cudaSuccess && items_of(g) > 8LL * n_sm && items_of(g) < 0x3fffffffLL;
 }
 
 cudaError_t launch_attn_tc_hd64(const Geometry& g, const __nv_bfloat16* q, const __nv_bfloat16* k,
@@ -470,7 +470,7 @@ cudaError_t launch_attn_tc_hd64(const Geometry& g, const __nv_bfloat16* q, const
     if (e != cudaSuccess) return e;
   }
   const int64_t n_items = items_of(g);
-  if (n_items > 0x3fffffffLL) return cudaErrorNotSupported;
+  if (n_items > 0x7fffffffLL) return cudaErrorNotSupported;
   if (!attn_tc_hd64_uses_counter(g)) next_item = nullptr;
   if (next_item != nullptr && !counter_cleared) {
     cudaError_t e = launch_clear_counter(next_item, st);

@@ -83,9 +83,9 @@ inline int segment_order(const Geometry& g, uint32_t allowed) {
 
 // Per-device launch set-up (a process may drive several GPUs; kernel attributes and SM counts belong to a device):
 // sets the kernel's dynamic shared-memory limit the first time `func` is launched on the current device and returns
-// that device's SM count.  `func` identifies the kernel; at most 64 devices and 64 kernels are tracked.
+// that device's SM count.  `func` identifies the kernel; at most 64 devices and 192 kernels are tracked.
 inline cudaError_t sm_count_and_smem_once(const void* func, int smem_bytes, int* n_sm) {
-  constexpr int MAX_DEV = 64, MAX_FUNC = 64;
+  constexpr int MAX_DEV = 64, MAX_FUNC = 192;
   static int sm_count[MAX_DEV] = {};
   static const void* done[MAX_DEV][MAX_FUNC] = {};
   int dev = 0;

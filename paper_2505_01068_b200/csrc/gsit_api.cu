@@ -290,7 +290,7 @@ gsit_status gsit_im_qkv_proj(const gsit_shape* shape, const void* x, int64_t x_r
   a.C = qkv; a.ldc = 3 * (int64_t)g.d;
   a.M = (int)matrix_rows(g); a.N = 3 * g.d; a.K = g.d;
   a.mask_rows = 1;
-  if (shape->dtype == GSIT_BF16 && g_attn_variant == GSIT_ATTN_DEFAULT && qkv_rows_preferred(g)) {
+  if (shape->dtype == GSIT_BF16 && g_attn_variant == GSIT_ATTN_DEFAULT && qkv_rows_preferred(g) && (g.row_start == nullptr || linear_tc_supported(a))) {
     TraceScope t(GSIT_KERNEL_LINEAR, static_cast<cudaStream_t>(stream));
     return from_cuda(launch_qkv_rows(g, a, static_cast<cudaStream_t>(stream)));
   }

@@ -106,7 +106,8 @@ def test_layer_on_either_side_of_the_row_limit(g, d, heads, above):
 @pytest.mark.parametrize("d,heads,seg,B", [(32, 4, (3, 1, 2), 1), (32, 1, (17, 130, 45), 5), (32, 4, (33, 257, 300), 15), (64, 8, (3, 5, 9), 1), (64, 2, (40, 193, 267), 4)])
 def test_projection_on_row_tiles(g, d, heads, seg, B):
     """The projection alone on row tiles (32 and, from 8192 rows on, 64 rows at d 32; 16 at d 64 up to 2000 rows): strided input with NaN
-    in the padding against a float product of the same operands (bf16 result: 2^-8 relative), and the packed layout bit for bit."""
+    in the padding against a float product of the same operands (bf16 result: 2^-8 relative), and the packed layout bit for bit
+    (at 32, where it is not covered, refused)."""
     rng = np.random.default_rng(B)
     L, cap = sum(seg), B * sum(seg)
     valid = np.stack([rng.integers(0, n + 1, size=B) for n in seg], axis=1).astype(np.int32)
@@ -122,6 +123,11 @@ def test_projection_on_row_tiles(g, d, heads, seg, B):
         assert bool((got[pm] == 0).all())
         assert float((got.float() - ref)[~pm].abs().max()) <= 2.0 ** -8 * max(1.0, float(ref[~pm].abs().max()))
     plan = g.plan_rows(vl, seg)
+    if d == 32:
+        with pytest.raises(g.GsitError) as e:
+            g.im_qkv_proj(torch.zeros((cap, d), dtype=torch.bfloat16, device="cuda"), w, None, seg, heads, vl, row_start=plan)
+        assert e.value.code == 2
+        return
     xp = g.pack_rows(torch.nan_to_num(x.float()), torch.zeros((cap, d), device="cuda"), seg, vl, plan).bfloat16()
     for lo, hi in {(0, B), (B // 2, B)}:
         out = torch.full((cap, 3, heads, d // heads), 7.0, dtype=torch.bfloat16, device="cuda")
