@@ -15,6 +15,7 @@ With --gpus N > 1 and no torchrun environment the script starts N worker process
 from __future__ import annotations
 
 import argparse
+import ctypes
 import json
 import os
 import sys
@@ -322,7 +323,9 @@ def run_gpu(args):
     paired = stack.paired_rings and n_f == n_b and n_f > 0   # one launch per kernel for both rings of a depth
     launches_per_step = 3 * (n_f if paired else n_f + n_b) + 3 * n_i * (1 if paired else 2)
     if stack.packed:
-        launches_per_step += 2   # row plan and gather of the real rows, scatter of the result
+        # row plan and gather of the real rows; scatter of the result, unless the last layer writes it in place
+        sh = g.make_shape(B, wl.seg_len, 2 * wl.d_model, ih, vl, g.DTYPE_BF16, g.PHASE_INTRA, row_start=g.plan_rows(vl, wl.seg_len), capacity=B * sum(wl.seg_len) + 128)
+        launches_per_step += 1 if g.load().gsit_layer_scatters(ctypes.byref(sh), int(inp["intra_layers"][-1]["w_1"].shape[0])) else 2
 
     for i in range(max(1, min(args.warmup, 2))):           # eager warm-up (module load, attributes, buffers)
         stack.forward(xbufs[i % nbuf], vl)
