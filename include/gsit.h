@@ -195,10 +195,12 @@ gsit_status gsit_pack_rows(const gsit_shape* shape, const float* x, int64_t x_ro
 gsit_status gsit_plan_pack_rows(const gsit_shape* shape, int32_t* row_start, const float* x, int64_t x_row_stride, float* x_packed,
                                 int64_t packed_row_stride, int32_t cols, gsit_stream stream);
 /* gsit_plan_pack_map_rows does the same and prepares a result [B, L, 2 cols] for gsit_im_layer_scatter_fwd: row_map (int32 [capacity])
- *   receives the row b * L + position of every packed row, and the padding rows of y are set to +0 (its other rows are left alone).
+ *   receives the row b * L + position of every packed row, and the padding rows of y are set to +0 (its other rows are left alone)
+ *   while x is still being read: y must not overlap x (use gsit_plan_pack_rows and gsit_unpack_rows where it does).
  *   GSIT_ERR_UNSUPPORTED above 1024 samples.
  * gsit_im_layer_scatter_fwd is gsit_im_layer_fwd on packed rows whose result goes straight to the padded matrix: packed row i to row
- *   row_map[i] of y.  Covered (gsit_layer_scatters returns 1) where the tcgen05 halves at d_model 128 serve the layer. */
+ *   row_map[i] of y, which must not overlap x.  Covered (gsit_layer_scatters returns 1) where the tcgen05 halves at d_model 128 serve
+ *   the layer. */
 gsit_status gsit_plan_pack_map_rows(const gsit_shape* shape, int32_t* row_start, int32_t* row_map, const float* x, int64_t x_row_stride,
                                     float* x_packed, int64_t packed_row_stride, int32_t cols, float* y, int64_t y_row_stride, gsit_stream stream);
 int32_t gsit_layer_scatters(const gsit_shape* shape, int32_t d_ff);

@@ -428,6 +428,21 @@ bool chained(const at::Tensor& x, PyObject* seg, int64_t heads, int64_t intra_he
   return all(fwd, x.size(2), heads, 2) && all(intra, 2 * x.size(2), intra_heads, 1);
 }
 
+// Do two float matrices of uniform row stride touch the same bytes anywhere between their first and last element?
+bool overlap(const at::Tensor& a, const at::Tensor& b) {
+  auto range = [](const at::Tensor& t, const char*& lo, const char*& hi) {
+    lo = hi = static_cast<const char*>(t.data_ptr());
+    if (t.numel() == 0) return;
+    int64_t last = 0;
+    for (int64_t i = 0; i < t.dim(); ++i) last += (t.size(i) - 1) * t.stride(i);
+    hi += (last + 1) * t.element_size();
+  };
+  const char *a0, *a1, *b0, *b1;
+  range(a, a0, a1);
+  range(b, b0, b1);
+  return a0 < b1 && b0 < a1;
+}
+
 // x, valid_len, y, fwd, bwd, intra, seg_len, heads, intra_heads, ln_eps, buffers
 //   buffers = (plan or None, workspace, ring_a0, ring_a1, ring_b0, ring_b1, x_packed or None, wide_0, wide_1, row_map or None): with a
 //   plan the packed row layout is used (x gathered into x_packed; the result scattered into y, by the last layer itself where it
@@ -447,9 +462,12 @@ PyObject* stack_forward(PyObject* const* a) {
   require(PyTuple_Check(a[10]) && PyTuple_GET_SIZE(a[10]) == 10, "buffers: ten tensors");
   const at::Tensor* b[10];
   for (int i = 0; i < 10; ++i) b[i] = opt_tensor(PyTuple_GET_ITEM(a[10], i));
+  // x may lie in y (a view of an earlier result): then it is gathered, or copied, before anything of y is written.  The gather must not
+  // clear y's padding in the same launch, and no layer may read x while another kernel of the call writes y.
+  const bool x_in_y = overlap(x, y);
   // layers that run as one launch each do no work for padding in the padded layout either: no plan, no copies between layouts then
   const at::Tensor* plan = b[0];
-  if (plan != nullptr && chained(x, a[6], as_int(a[7]), as_int(a[8]), valid, fwd, bwd, intra)) plan = nullptr;
+  if (plan != nullptr && !x_in_y && chained(x, a[6], as_int(a[7]), as_int(a[8]), valid, fwd, bwd, intra)) plan = nullptr;
   const int64_t B = x.size(0), d = x.size(2), cap = plan != nullptr ? b[6]->size(0) : 0;
   const gsit_shape ring_shape = make_shape(B, a[6], d, as_int(a[7]), valid, fwd[0].dtype, GSIT_PHASE_INTER_FWD, 0, 0.0, plan, cap);
   const gsit_shape intra_shape = make_shape(B, a[6], 2 * d, as_int(a[8]), valid, fwd[0].dtype, GSIT_PHASE_INTRA, 0, 0.0, plan, cap);
@@ -458,8 +476,10 @@ PyObject* stack_forward(PyObject* const* a) {
   auto f = [](const at::Tensor* t) { return static_cast<float*>(t->data_ptr()); };
   float *ping_a[2] = {f(b[2]), f(b[3])}, *ping_b[2] = {f(b[4]), f(b[5])}, *wide[2] = {f(b[7]), f(b[8])};
   float* out = f(&y);
-  const float* x_in = static_cast<const float*>(x.data_ptr());
-  int64_t ldx = x.stride(1);
+  at::Tensor copy;
+  if (x_in_y && plan == nullptr && fwd.size() == 1 && intra.empty()) copy = x.clone(at::MemoryFormat::Contiguous);  // a first layer that is also the last
+  const float* x_in = static_cast<const float*>(copy.defined() ? copy.data_ptr() : x.data_ptr());
+  int64_t ldx = copy.defined() ? d : x.stride(1);
   gsit_stream cs = stream();
 
   auto issue = [&]() -> gsit_status {
@@ -468,7 +488,7 @@ PyObject* stack_forward(PyObject* const* a) {
     if (plan != nullptr) {
       float* xp = f(b[6]);
       int32_t* starts = static_cast<int32_t*>(plan->data_ptr());
-      if (!intra.empty() && B <= 1024) {
+      if (!x_in_y && !intra.empty() && B <= 1024) {
         gsit_shape last = intra_shape;
         last.dtype = intra.back().dtype;
         if (gsit_layer_scatters(&last, intra.back().w.d_ff)) row_map = static_cast<int32_t*>(b[9]->data_ptr());

@@ -190,7 +190,8 @@ class GsitStack:
 
     def forward(self, x, valid_len=None, out=None, check=False):
         """x float32 [B, L, d] -> float32 [B, L, 2d].  The result lives in a buffer owned by this object, or in `out`
-        (float32 [B, L, 2d], contiguous) when one is given.  check=True synchronises the stream afterwards and raises
+        (float32 [B, L, 2d], contiguous) when one is given.  x may lie anywhere in `out`, and with paired rings or packed rows also in
+        the owned buffer (a view of the result before), which then no longer holds it afterwards.  check=True synchronises the stream afterwards and raises
         GsitError if a kernel reported a timed-out device-side wait (not for use under stream capture)."""
         if out is not None:
             assert out.shape == (x.shape[0], x.shape[1], 2 * x.shape[2]) and out.dtype == torch.float32 and out.is_contiguous()

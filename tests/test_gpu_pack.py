@@ -54,3 +54,33 @@ def test_stack_result_in_the_padded_layout(d, intra_depth):
     assert st.packed and torch.equal(got, want)
     assert not torch.signbit(got[torch.from_numpy(wk.padded_row_mask(seg, valid, B)).cuda()]).any()
     assert g.last_device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("B,intra_depth", [(12, 1), (2, 0), (2, 1), (12, 0)])
+@pytest.mark.parametrize("padded", [False, True])
+def test_stack_input_anywhere_in_the_result(B, intra_depth, padded):
+    """The input of a stack may lie in its result, row for row or in any other mapping: packed rows (12 samples; the last layer at width
+    128 could write the padded result itself), layers of one launch (2 samples), rings whose only layer also writes the result."""
+    import paper_2505_01068_b200 as g
+    import workloads as wk
+    from gpu_util import weights_to_dev
+    rng = np.random.default_rng(B)
+    seg, d = (50, 300, 270), 64
+    layers = lambda width, n: [weights_to_dev(wk.draw_layer_weights(rng, width, 2 * width, "bf16", affine=True), "bf16") for _ in range(n)]
+    st = g.GsitStack(layers(d, 1), layers(d, 1), layers(2 * d, intra_depth), seg, 4, 4, packed=not padded)
+    vl = torch.from_numpy(np.stack([rng.integers(0, n + 1, size=B) for n in seg], axis=1).astype(np.int32)).cuda()
+    x = torch.from_numpy(rng.standard_normal((B, sum(seg), d), dtype=np.float32)).cuda()
+    for valid in (vl, None):
+        want = st.forward(x, valid).clone()
+        out = torch.empty((B, sum(seg), 2 * d), device="cuda")
+        flat = out.view(-1)
+        views = [out[:, :, :d], out[:, :, d:], flat[:x.numel()].view(x.shape), flat[x.numel():].view(x.shape), flat[d // 2 * 3:][:x.numel()].view(x.shape)]
+        for v in views:
+            out.fill_(float("nan"))
+            v.copy_(x)
+            assert torch.equal(st.forward(v, valid, out=out), want)
+        mine = st.forward(x, valid)   # the object's own buffer
+        view = mine.view(-1)[x.numel():].view(x.shape)
+        view.copy_(x)
+        assert torch.equal(st.forward(view, valid), want)
+    assert g.last_device_status() == (0, 0)
