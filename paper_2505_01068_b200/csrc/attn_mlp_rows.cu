@@ -389,27 +389,82 @@ int64_t tail_ctas(const Geometry& g, int n, int rows) {
 int small_tile(const Geometry& g) { return g.d == 32 ? 32 : 16; }
 }  // namespace
 
-// One CTA fills an SM, and a second wave of long walks costs more than two launches less: one wave, or up to three (d 32: two) of walks
-// over at most eight key tiles.  Layer of one kernel behind the projection / of two, us (the half, full and sparse lengths of 0.05 - 0.4):
-//   4200 rows of (50, 500, 500), d 64: half 18.4/24.5, full 19.6/26.0, sparse 13.1/16.4      (one wave of 32-row tiles)
-//   6300 rows, two waves:              half 21.4/27.4, full 32.1/28.8, sparse 13.9/19.2;     pair, three: 32.4/34.5, 43.9/42.8, 16.6/22.9
-//   5358 rows of (850, 34, 9), intra, full, two waves of 14 key tiles: 43.8/36.0
-//   d 128, 6300 rows of (50, 500, 500): half 32.3/43.0, full 49.8/50.6; d 32, pair, 8800 rows of (50, 250, 250), full 22.6/22.1,
-//   sparse 12.6/16.8; a stack of 8650 rows, two and a half waves: 132.6/130
+// Full lengths (no valid_len): the time of the launch in key tiles, its CTAs handed to n_sm SMs one at a time, longest walk first (the order
+// of the grid).  A CTA takes its walk and as long as eight key tiles for everything else.
+namespace {
+constexpr int REST_OF_CTA = 8;
+struct Walks { int key_tiles; int64_t ctas; };
+int walks_of(const Geometry& g, const uint32_t* allowed, int n, int rows, Walks (&w)[6]) {  // of each segment and problem, longest first
+  int count = 0;
+  for (int i = 0; i < n; ++i)
+    for (int s = 0; s < 3; ++s) {
+      Walks v = {0, (int64_t)((g.len(s) + rows - 1) / rows) * g.batch};
+      for (int r = 0; r < 3; ++r)
+        if ((allowed[i] >> (3 * s + r)) & 1u) v.key_tiles += (g.len(r) + KT - 1) / KT;
+      if (v.ctas == 0) continue;
+      int at = count++;
+      for (; at > 0 && w[at - 1].key_tiles < v.key_tiles; --at) w[at] = w[at - 1];
+      w[at] = v;
+    }
+  return count;
+}
+int makespan(const Walks* w, int count, int n_sm) {
+  struct { int at, sms; } free_at[8] = {{0, n_sm}};  // SMs by when they are free: a set of walks that runs out splits one entry
+  int groups = 1, end = 0;
+  for (int i = 0; i < count; ++i)
+    for (int64_t left = w[i].ctas; left > 0;) {
+      int k = 0;
+      for (int j = 1; j < groups; ++j)
+        if (free_at[j].at < free_at[k].at) k = j;
+      const int done = free_at[k].at + REST_OF_CTA + w[i].key_tiles;
+      if (left >= free_at[k].sms) {
+        left -= free_at[k].sms;
+        free_at[k].at = done;
+      } else {
+        free_at[k].sms -= (int)left;
+        free_at[groups++] = {done, (int)left};
+        left = 0;
+      }
+      if (done > end) end = done;
+    }
+  return end;
+}
+}  // namespace
+
+// One CTA fills an SM, and a second wave of long walks costs more than two launches less.  One wave always runs here; more (up to three
+// waves, at d 32 two) by what the host knows of the lengths.
+// No valid_len: every length is full.  Then the walks are known, and what decides is when the last CTA ends: not after 5/3 of the longest
+// CTA's time (d 32: 7/4).  us of a layer in one launch behind the projection / in two; the last end in longest CTAs:
+//   d 64   6 x (50, 500, 500), intra 31.7/27.7 (2.0), both rings 42.7/40.9 (2.1);   32 x (50, 52, 52), intra 19.5/17.4 (2.0)
+//          5 x (50, 500, 500), forward ring 21.2/26.7 (1.1);   4 x, both rings 27.2/28.4 (1.6)
+//   d 32   54 x (50, 52, 52), intra 15.6/13.4 (2.0);   8 x (50, 500, 500), both rings 23.8/27.4 (1.6)
+// Over 291 shapes beyond one wave at d 64 (segments of 8 - 1024 steps, one problem or two) this costs 0.4 % on average against the better
+// of both, the rule for unknown lengths 10 %; over 352 at d 32 1.3 % and 13 %.
+// At d 128 the separate second half itself takes two waves above 32 rows per SM.  Below, a second wave here loses throughout (3850 rows of
+// (50, 52, 52) 32.0/27.0, 4230 of (50, 116, 116) 32.9/28.0); above, two waves hold their own up to eight key tiles (5250 rows of (50, 500,
+// 500), intra 47.4/48.1, 4928 of (50, 52, 52) 34.1/35.3; fourteen key tiles 64.2/60.4).
+// With valid_len the lengths are unknown here, and padding cuts the second wave short: walks of up to eight key tiles.  d 64, intra, 1.2 waves,
+// us, one launch / two, by key tiles of the longest walk (lengths full, half to full, 0.05 - 0.4):
+//   tiles     4          6          8          9          10         11         13         14
+//   full  23.5/21.0  27.2/23.9  30.5/26.5  33.1/28.5  34.9/29.8  37.8/31.1  41.8/34.2  44.6/35.3
+//   half  16.3/21.1  18.1/23.3  18.9/26.0  20.3/27.5  20.8/28.4  22.2/30.0  24.3/32.2  26.5/33.3
+//   few   13.2/16.8  13.4/16.9  13.6/17.7  13.9/18.4  13.7/17.9  14.2/18.6  14.9/19.2  15.3/19.2
+// What padding gains stays at a quarter from four tiles on; what a batch whose lengths are full after all loses grows from 12 % at four
+// and 15 % at eight to 26 % at fourteen.  The line lies where one still clearly outweighs the other.
 bool layer_tail_preferred(const Geometry& g, const uint32_t* allowed, int n) {
   int n_sm = 0;
   if (sm_count_and_smem_once(nullptr, 0, &n_sm) != cudaSuccess) return false;
-  const int64_t ctas = tail_ctas(g, n, 2 * small_tile(g));
+  const int rows = 2 * small_tile(g);
+  const int64_t ctas = tail_ctas(g, n, rows);
   if (ctas <= n_sm) return true;
-  int longest = 0;
-  for (int i = 0; i < n; ++i)
-    for (int s = 0; s < 3; ++s) {
-      int kt = 0;
-      for (int r = 0; r < 3; ++r)
-        if ((allowed[i] >> (3 * s + r)) & 1u) kt += (g.len(r) + KT - 1) / KT;
-      if (g.len(s) > 0 && kt > longest) longest = kt;
-    }
-  return ctas <= (g.d == 32 ? 2 : 3) * n_sm && longest <= 8;
+  if (ctas > (g.d == 32 ? 2 : 3) * n_sm) return false;
+  Walks w[6];
+  const int count = walks_of(g, allowed, n, rows, w);
+  const int longest = w[0].key_tiles;
+  if (g.valid_len != nullptr) return longest <= 8;
+  const int end = 12 * makespan(w, count, n_sm), cta = REST_OF_CTA + longest;
+  if (g.d == 128) return (int64_t)g.batch * g.L * n > 32LL * n_sm && (end <= 20 * cta || (end <= 24 * cta && longest <= 8));
+  return end <= (g.d == 32 ? 21 : 20) * cta;
 }
 
 cudaError_t launch_layer_tail(const Geometry& g, const LayerTailArgs* args, int n, float scale, float eps, float next_eps, int d_ff, cudaStream_t st) {

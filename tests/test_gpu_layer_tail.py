@@ -1,5 +1,7 @@
 """A layer behind its projection in one launch (attention, out-projection, LN2, MLP, the next layer's first half): the same bits as the
 separate kernels, which serve the same samples inside a batch whose walks are too long for it, at both heights of its row tiles."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -55,4 +57,30 @@ def test_chained_layers_equal_layer_calls(g, d, heads, intra_heads, B):
             want = g.im_layer_fwd(want, wi, seg, intra_heads, vl, g.PHASE_INTRA)
         for packed in (True, False):
             assert torch.equal(g.GsitStack(fwd, bwd, intra, seg, heads, intra_heads, packed=packed).forward(x, vl), want)
+    assert g.last_device_status() == (0, 0)
+
+
+# Beyond one wave of the one-launch kernel's CTAs; (phases, with no valid_len: one launch?) -- a second wave of long walks costs more than
+# the launches it saves, one of short walks behind them does not
+@pytest.mark.parametrize("B,seg,d,heads,routes", [
+    (6, (50, 500, 500), 64, 8, {(2,): 0, (0,): 1, (0, 1): 0}), (32, (50, 52, 52), 64, 4, {(2,): 0}), (4, (50, 500, 500), 64, 8, {(0, 1): 1}),
+    (25, (50, 52, 52), 128, 8, {(2,): 0}), (5, (50, 500, 500), 128, 8, {(2,): 1}), (54, (50, 52, 52), 32, 4, {(2,): 0}), (8, (50, 500, 500), 32, 4, {(0, 1): 1})])
+def test_full_lengths_known_to_the_host(g, B, seg, d, heads, routes):
+    """Without valid_len every length is full and the launch is chosen by the walks that follow from it; with lengths that are full as
+    well, by what padding usually leaves.  The same bits either way."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("sizes chosen for 148 SMs")
+    rng = np.random.default_rng(B)
+    full = torch.tensor([seg] * B, dtype=torch.int32, device="cuda")
+    x = to_dev(rng.standard_normal((B, sum(seg), d), dtype=np.float32))
+    w = [weights_to_dev(wk.draw_layer_weights(rng, d, 2 * d, "bf16", affine=True), "bf16") for _ in range(2)]
+    fn = g.load().gsit_encoder_runs_chained
+    for phases, one_launch in routes.items():
+        shapes = [g.make_shape(B, seg, d, heads, None, g.DTYPE_BF16, p) for p in phases]
+        assert fn((ctypes.c_void_p * 2)(*[ctypes.addressof(s) for s in shapes]), len(phases), 2 * d) == one_launch, phases
+        if len(phases) == 1:
+            a, b = (g.im_layer_fwd(x, w[0], seg, heads, v, phases[0]) for v in (None, full))
+        else:
+            a, b = (torch.cat(g.im_layer_pair_fwd(x, x, w[0], w[1], seg, heads, v), 2) for v in (None, full))
+        assert torch.equal(a, b), phases
     assert g.last_device_status() == (0, 0)
