@@ -451,6 +451,9 @@ int makespan(const Walks* w, int count, int n_sm) {
 //   few   13.2/16.8  13.4/16.9  13.6/17.7  13.9/18.4  13.7/17.9  14.2/18.6  14.9/19.2  15.3/19.2
 // What padding gains stays at a quarter from four tiles on; what a batch whose lengths are full after all loses grows from 12 % at four
 // and 15 % at eight to 26 % at fourteen.  The line lies where one still clearly outweighs the other.
+// At d 32 walks of one or two key tiles leave nothing to cut short: 54 x (50, 52, 52) half to full 15.9/14.4, few 14.7/13.0; 32 x (50, 116, 116)
+// 16.6/14.6, 12.2/13.0; 23 x (50, 180, 180) 13.3/15.2, 11.4/13.2.  Over 73 shapes of one or two tiles one launch takes 1.11 of the time of two
+// (half to full) and 1.06 (few), over 67 of three or four 0.96 and 0.86 -> from three on.
 bool layer_tail_preferred(const Geometry& g, const uint32_t* allowed, int n) {
   int n_sm = 0;
   if (sm_count_and_smem_once(nullptr, 0, &n_sm) != cudaSuccess) return false;
@@ -461,7 +464,7 @@ bool layer_tail_preferred(const Geometry& g, const uint32_t* allowed, int n) {
   Walks w[6];
   const int count = walks_of(g, allowed, n, rows, w);
   const int longest = w[0].key_tiles;
-  if (g.valid_len != nullptr) return longest <= 8;
+  if (g.valid_len != nullptr) return longest <= 8 && (g.d != 32 || longest > 2);
   const int end = 12 * makespan(w, count, n_sm), cta = REST_OF_CTA + longest;
   if (g.d == 128) return (int64_t)g.batch * g.L * n > 32LL * n_sm && (end <= 20 * cta || (end <= 24 * cta && longest <= 8));
   return end <= (g.d == 32 ? 21 : 20) * cta;

@@ -84,3 +84,19 @@ def test_full_lengths_known_to_the_host(g, B, seg, d, heads, routes):
             a, b = (torch.cat(g.im_layer_pair_fwd(x, x, w[0], w[1], seg, heads, v), 2) for v in (None, full))
         assert torch.equal(a, b), phases
     assert g.last_device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("B,seg,one_launch", [(54, (50, 52, 52), 0), (32, (50, 116, 116), 0), (23, (50, 180, 180), 1), (30, (50, 52, 52), 1)])
+def test_short_walks_at_width_32(g, B, seg, one_launch):
+    """Given lengths, beyond one wave: walks of one or two key tiles leave nothing for padding to cut short.  (30 samples are one wave.)"""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("sizes chosen for 148 SMs")
+    rng = np.random.default_rng(B)
+    vl = torch.from_numpy(np.stack([rng.integers(0, n + 1, size=B) for n in seg], axis=1).astype(np.int32)).cuda()
+    shape = g.make_shape(B, seg, 32, 4, vl, g.DTYPE_BF16, g.PHASE_INTRA)
+    assert g.load().gsit_encoder_runs_chained((ctypes.c_void_p * 1)(ctypes.addressof(shape)), 1, 64) == one_launch
+    x = to_dev(rng.standard_normal((B, sum(seg), 32), dtype=np.float32))
+    w = weights_to_dev(wk.draw_layer_weights(rng, 32, 64, "bf16", affine=True), "bf16")
+    want = torch.cat([g.im_layer_fwd(x[b:b + 1], w, seg, 4, vl[b:b + 1], g.PHASE_INTRA) for b in range(B)])
+    assert torch.equal(g.im_layer_fwd(x, w, seg, 4, vl, g.PHASE_INTRA), want)
+    assert g.last_device_status() == (0, 0)
