@@ -44,7 +44,7 @@ attn_bf16_kernel(const __grid_constant__ AttnProblem prob0, const __grid_constan
   const Tile t = find_tile<C::QT>(g, prob.allowed, bx, prob.seg_order);
   if (t.T > 0) {
     __syncthreads();
-    attend_tile<C>(g, t, prob.tmQ, prob.tmK, prob.tmV, xcol, xcol, xcol, cs, sl2, lse, sQ, [] {});
+    attend_tile<C, NTHREADS / 32>(g, t, prob.tmQ, prob.tmK, prob.tmV, xcol, xcol, xcol, cs, sl2, lse, sQ, [] {});
   }
 
   // ---- coalesced 16-byte stores; padded rows are written as +0, rows of the next segment are left alone ----

@@ -143,7 +143,7 @@ __device__ __forceinline__ void init_walk(uint32_t base, int tid) {
 // Walks the keys of tile t (t.T > 0), by all threads of the CTA: the heads of column slices first_slice .. + SL - 1, whose columns start at
 // xq, xk, xv in the three maps.  Leaves the normalised rows as bf16 where Q was (swizzled rows of CW columns, slice by slice) and ends
 // with a barrier; lse (with the heads of the whole problem) may be null.  meanwhile(): what every thread does once Q is there.
-template <typename C, typename F>
+template <typename C, int CTA_WARPS, typename F>
 __device__ __forceinline__ void attend_tile(const Geometry& g, const Tile& t_, const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                                             const int xq, const int xk, const int xv, const int first_slice, const float sl2, float* __restrict__ lse,
                                             const uint32_t base, F meanwhile) {
@@ -152,7 +152,11 @@ __device__ __forceinline__ void attend_tile(const Geometry& g, const Tile& t_, c
   constexpr bool HOIST = (R > 1);  // several query slabs per warp reuse the K/V fragments of a step
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int head = warp % (G * SL), sg = warp / (G * SL), slice = head / G, head_in_slice = head % G;
-  const bool active = warp < C::WARPS;
+  // Known at compile time where every warp of the CTA attends: a walk behind a branch takes longer (14 key tiles of one 16-row slab at head_dim 8:
+  // 13.75 us, 13.50 without the branch; one sample of (50, 500, 500) 8.96 and 8.80).  Not with four slabs per warp, which then spill
+  // (64 samples of it 42.05 and 42.35).
+  constexpr bool EVERY_WARP = C::WARPS == CTA_WARPS && R < 4;
+  const bool active = EVERY_WARP || warp < C::WARPS;
   const uint32_t sQall = base, sK = base + C::OFF_K, sV = base + C::OFF_V;
   const uint32_t sQ = base + slice * C::Q_SLICE;
   const uint32_t bar_full = base + C::OFF_BAR;          // STAGES barriers of 8 bytes: TMA bytes have landed

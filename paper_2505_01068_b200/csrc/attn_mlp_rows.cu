@@ -141,7 +141,7 @@ attn_mlp_rows_kernel(const __grid_constant__ LayerProblem prob0, const __grid_co
       if (next) rows(sW + M::w_qkv(d_ff), M::PD, a.w_qkv, 3 * D, D / 8);
     }
   };
-  if (t.T > 0) attend_tile<C>(g, t, prob.tmQ, prob.tmKV, prob.tmKV, 0, D, 2 * D, 0, sl2, nullptr, base, stage_weights);
+  if (t.T > 0) attend_tile<C, TAIL_WARPS>(g, t, prob.tmQ, prob.tmKV, prob.tmKV, 0, D, 2 * D, 0, sl2, nullptr, base, stage_weights);
   else stage_weights();
 
   // ---- y1 = x + att W_o^T + b_o, in registers of the warps with wk = 0; the attention rows are where the walk left them ----
