@@ -389,18 +389,20 @@ int64_t tail_ctas(const Geometry& g, int n, int rows) {
 int small_tile(const Geometry& g) { return g.d == 32 ? 32 : 16; }
 }  // namespace
 
-// Full lengths (no valid_len): the time of the launch in key tiles, its CTAs handed to n_sm SMs one at a time, longest walk first (the order
-// of the grid).  A CTA takes its walk and as long as eight key tiles for everything else.
+// Time of the launch in key tiles, its CTAs handed to n_sm SMs one at a time, longest walk first (the order of the grid).  A CTA takes its walk
+// and as long as eight key tiles for everything else.
 namespace {
 constexpr int REST_OF_CTA = 8;
 struct Walks { int key_tiles; int64_t ctas; };
-int walks_of(const Geometry& g, const uint32_t* allowed, int n, int rows, Walks (&w)[6]) {  // of each segment and problem, longest first
+// ... of each segment and problem, longest first, with `thirds` thirds of every length real
+int walks_of(const Geometry& g, const uint32_t* allowed, int n, int rows, int thirds, Walks (&w)[6]) {
+  auto real = [&](int s) { return (int)(((int64_t)g.len(s) * thirds + 2) / 3); };
   int count = 0;
   for (int i = 0; i < n; ++i)
     for (int s = 0; s < 3; ++s) {
-      Walks v = {0, (int64_t)((g.len(s) + rows - 1) / rows) * g.batch};
+      Walks v = {0, (int64_t)((real(s) + rows - 1) / rows) * g.batch};
       for (int r = 0; r < 3; ++r)
-        if ((allowed[i] >> (3 * s + r)) & 1u) v.key_tiles += (g.len(r) + KT - 1) / KT;
+        if ((allowed[i] >> (3 * s + r)) & 1u) v.key_tiles += (real(r) + KT - 1) / KT;
       if (v.ctas == 0) continue;
       int at = count++;
       for (; at > 0 && w[at - 1].key_tiles < v.key_tiles; --at) w[at] = w[at - 1];
@@ -432,29 +434,37 @@ int makespan(const Walks* w, int count, int n_sm) {
 }  // namespace
 
 // One CTA fills an SM, and a second wave of long walks costs more than two launches less.  One wave always runs here; more (up to three
-// waves, at d 32 two) by what the host knows of the lengths.
-// No valid_len: every length is full.  Then the walks are known, and what decides is when the last CTA ends: not after 5/3 of the longest
-// CTA's time (d 32: 7/4).  us of a layer in one launch behind the projection / in two; the last end in longest CTAs:
+// waves, at d 32 two) by when the last CTA ends, in times of the longest CTA.
+//
+// No valid_len: every length is full, the walks are known.  The line lies at 5/3 (d 32: 7/4).  us of a layer in one launch behind the
+// projection / in two; the last end:
 //   d 64   6 x (50, 500, 500), intra 31.7/27.7 (2.0), both rings 42.7/40.9 (2.1);   32 x (50, 52, 52), intra 19.5/17.4 (2.0)
 //          5 x (50, 500, 500), forward ring 21.2/26.7 (1.1);   4 x, both rings 27.2/28.4 (1.6)
 //   d 32   54 x (50, 52, 52), intra 15.6/13.4 (2.0);   8 x (50, 500, 500), both rings 23.8/27.4 (1.6)
 // Over 291 shapes beyond one wave at d 64 (segments of 8 - 1024 steps, one problem or two) this costs 0.4 % on average against the better
-// of both, the rule for unknown lengths 10 %; over 352 at d 32 1.3 % and 13 %.
+// of both, one launch up to the limits above 10 %; over 352 at d 32 1.3 % and 13 %.
 // At d 128 the separate second half itself takes two waves above 32 rows per SM.  Below, a second wave here loses throughout (3850 rows of
 // (50, 52, 52) 32.0/27.0, 4230 of (50, 116, 116) 32.9/28.0); above, two waves hold their own up to eight key tiles (5250 rows of (50, 500,
 // 500), intra 47.4/48.1, 4928 of (50, 52, 52) 34.1/35.3; fourteen key tiles 64.2/60.4).
-// With valid_len the lengths are unknown here, and padding cuts the second wave short: walks of up to eight key tiles.  d 64, intra, 1.2 waves,
-// us, one launch / two, by key tiles of the longest walk (lengths full, half to full, 0.05 - 0.4):
+//
+// With valid_len the lengths are unknown here, and padding cuts the second wave short -- where a segment has several tiles; a segment of
+// one tile keeps its CTA however few rows are real.  So the same sum over walks of two thirds of the lengths, the line at 15/8 (among 110
+// stacks at 1 - 3 waves any share from 5/8 to 3/4 does as well).  us of a stack on these lengths, layers in one launch / in two on packed rows:
+//   d 64   42 x (21, 43, 34), depths 2 and 2   half to full 118.8/93.7, a quarter 81.7/84.0;   63 x (31, 21, 10), 4 and 3   202.5/168.6, 198.6/150.3
+//          14 x (59, 16, 57), 4 and 3 (one wave)   86.3/132.5, 79.8/117.2
+//   d 32   34 x (11, 60, 75), 2 and 1          51.3/47.8, 44.7/41.4;                            17 x (9, 152, 208), 3 and 2  88.2/93.0, 56.2/76.5
+// At d 128 an encoder's other choice is packed rows, whose second half then mostly fits one wave: there two thirds of the lengths must fit
+// one wave here (25 x (30, 26, 146), three layers in the stack's intra encoder, 148.6/124.9, 93.0/101.5).  A layer by itself takes up to
+// three waves (32 x (50, 52, 52) half to full 33.9/36.3, few 23.3/27.6).
+// Longest walk with valid_len: eight key tiles.  d 64, intra, 1.2 waves, us, one launch / two, by key tiles (lengths full, half to full,
+// 0.05 - 0.4):
 //   tiles     4          6          8          9          10         11         13         14
 //   full  23.5/21.0  27.2/23.9  30.5/26.5  33.1/28.5  34.9/29.8  37.8/31.1  41.8/34.2  44.6/35.3
 //   half  16.3/21.1  18.1/23.3  18.9/26.0  20.3/27.5  20.8/28.4  22.2/30.0  24.3/32.2  26.5/33.3
 //   few   13.2/16.8  13.4/16.9  13.6/17.7  13.9/18.4  13.7/17.9  14.2/18.6  14.9/19.2  15.3/19.2
 // What padding gains stays at a quarter from four tiles on; what a batch whose lengths are full after all loses grows from 12 % at four
 // and 15 % at eight to 26 % at fourteen.  The line lies where one still clearly outweighs the other.
-// At d 32 walks of one or two key tiles leave nothing to cut short: 54 x (50, 52, 52) half to full 15.9/14.4, few 14.7/13.0; 32 x (50, 116, 116)
-// 16.6/14.6, 12.2/13.0; 23 x (50, 180, 180) 13.3/15.2, 11.4/13.2.  Over 73 shapes of one or two tiles one launch takes 1.11 of the time of two
-// (half to full) and 1.06 (few), over 67 of three or four 0.96 and 0.86 -> from three on.
-bool layer_tail_preferred(const Geometry& g, const uint32_t* allowed, int n) {
+bool layer_tail_preferred(const Geometry& g, const uint32_t* allowed, int n, bool in_encoder) {
   int n_sm = 0;
   if (sm_count_and_smem_once(nullptr, 0, &n_sm) != cudaSuccess) return false;
   const int rows = 2 * small_tile(g);
@@ -462,12 +472,21 @@ bool layer_tail_preferred(const Geometry& g, const uint32_t* allowed, int n) {
   if (ctas <= n_sm) return true;
   if (ctas > (g.d == 32 ? 2 : 3) * n_sm) return false;
   Walks w[6];
-  const int count = walks_of(g, allowed, n, rows, w);
+  int count = walks_of(g, allowed, n, rows, 3, w);
   const int longest = w[0].key_tiles;
-  if (g.valid_len != nullptr) return longest <= 8 && (g.d != 32 || longest > 2);
-  const int end = 12 * makespan(w, count, n_sm), cta = REST_OF_CTA + longest;
-  if (g.d == 128) return (int64_t)g.batch * g.L * n > 32LL * n_sm && (end <= 20 * cta || (end <= 24 * cta && longest <= 8));
-  return end <= (g.d == 32 ? 21 : 20) * cta;
+  if (g.valid_len == nullptr) {
+    const int end = 12 * makespan(w, count, n_sm), cta = REST_OF_CTA + longest;
+    if (g.d == 128) return (int64_t)g.batch * g.L * n > 32LL * n_sm && (end <= 20 * cta || (end <= 24 * cta && longest <= 8));
+    return end <= (g.d == 32 ? 21 : 20) * cta;
+  }
+  if (longest > 8) return false;
+  count = walks_of(g, allowed, n, rows, 2, w);
+  if (g.d == 128) {
+    int64_t likely = 0;
+    for (int i = 0; i < count; ++i) likely += w[i].ctas;
+    return !in_encoder || likely <= n_sm;
+  }
+  return 8 * makespan(w, count, n_sm) <= 15 * (REST_OF_CTA + w[0].key_tiles);
 }
 
 cudaError_t launch_layer_tail(const Geometry& g, const LayerTailArgs* args, int n, float scale, float eps, float next_eps, int d_ff, cudaStream_t st) {

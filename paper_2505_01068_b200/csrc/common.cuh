@@ -242,7 +242,7 @@ struct LayerTailArgs {
   uint32_t allowed;
 };
 bool layer_tail_supported(const Geometry& g, int d_ff);
-bool layer_tail_preferred(const Geometry& g, const uint32_t* allowed, int n);
+bool layer_tail_preferred(const Geometry& g, const uint32_t* allowed, int n, bool in_encoder);
 cudaError_t launch_layer_tail(const Geometry& g, const LayerTailArgs* args, int n, float scale, float eps, float next_eps, int d_ff, cudaStream_t st);
 
 // ... and at d_model 128 (d_ff <= 512), with the MLP weights streamed in chunks (fused_layer_tc128.cu)

@@ -212,10 +212,10 @@ FusedHalfArgs half_args(const gsit_layer_weights* w, const float* x, int64_t ldx
 }
 
 // Do `n` layers of this geometry, side by side, run as one launch behind their first projection?  (The row-tile kernels on mma.sync, for a problem
-// whose attention is the mma.sync kernel as well: the same bits as three launches.)
-bool one_launch_layers(const Geometry& g, int dtype, const uint32_t* allowed, int n, int d_ff) {
+// whose attention is the mma.sync kernel as well: the same bits as three launches.)  in_encoder: layers of an encoder call, or on packed rows.
+bool one_launch_layers(const Geometry& g, int dtype, const uint32_t* allowed, int n, int d_ff, bool in_encoder) {
   if (dtype != GSIT_BF16 || g_attn_variant != GSIT_ATTN_DEFAULT || pick_halves(g, d_ff) != HALVES_ROWS) return false;
-  if (!layer_tail_supported(g, d_ff) || !layer_tail_preferred(g, allowed, n)) return false;
+  if (!layer_tail_supported(g, d_ff) || !layer_tail_preferred(g, allowed, n, in_encoder || g.row_start != nullptr)) return false;
   for (int i = 0; i < n; ++i)
     if (attn_uses_tensor_memory(g, allowed[i])) return false;
   return true;
@@ -352,7 +352,7 @@ static gsit_status layer_fwd(const gsit_shape* shape, const gsit_layer_weights* 
   if (g.row_start != nullptr && (halves == HALVES_NONE || g.hd > 32))
     return GSIT_ERR_UNSUPPORTED;  // the packed layout is implemented by the fused halves and the mma.sync / tensor-memory attention
 
-  if (one_launch_layers(g, dtype, &g.allowed, 1, w->d_ff)) {
+  if (one_launch_layers(g, dtype, &g.allowed, 1, w->d_ff, false)) {
     const LayerChain c = {{&w, nullptr}, {x, nullptr}, {x_row_stride, 0}, {&y, nullptr}, {&y_row_stride, nullptr}, {g.allowed, 0}};
     return run_chain(g, c, 1, 1, pick_scale(shape, g), ws, 0, sc, cs);
   }
@@ -482,7 +482,7 @@ gsit_status gsit_im_layer_pair_fwd(const gsit_shape* shape_a, const gsit_shape* 
   FusedHalfArgs h[2];
   AttnOperands ops[2];
   const uint32_t allowed[2] = {ga.allowed, gb.allowed};
-  if (one_launch_layers(ga, shape_a->dtype, allowed, 2, w_a->d_ff)) {
+  if (one_launch_layers(ga, shape_a->dtype, allowed, 2, w_a->d_ff, false)) {
     const LayerChain c = {{&w_a, &w_b}, {x_a, x_b}, {x_a_row_stride, x_b_row_stride}, {&y_a, &y_b}, {&y_a_row_stride, &y_b_row_stride}, {allowed[0], allowed[1]}};
     return run_chain(ga, c, 2, 1, pick_scale(shape_a, ga), ws, sc.total, sc, cs);
   }
@@ -517,7 +517,7 @@ int32_t gsit_encoder_runs_chained(const gsit_shape* const* shapes, int32_t probl
     if (make_geometry(shapes[i], &g[i]) != GSIT_OK) return 0;
     allowed[i] = g[i].allowed;
   }
-  return one_launch_layers(g[0], shapes[0]->dtype, allowed, problems, d_ff);
+  return one_launch_layers(g[0], shapes[0]->dtype, allowed, problems, d_ff, true);
 }
 
 gsit_status gsit_im_encoder_fwd(const gsit_shape* const* shapes, int32_t problems, const gsit_layer_weights* const* const* weights, int32_t depth,
@@ -551,7 +551,7 @@ gsit_status gsit_im_encoder_fwd(const gsit_shape* const* shapes, int32_t problem
       if (chained && w->d_ff > max_ff) max_ff = w->d_ff;
     }
   }
-  for (int j = 0; j < depth && chained; ++j) chained = one_launch_layers(g[0], shapes[0]->dtype, c.allowed, problems, weights[0][j]->d_ff);
+  for (int j = 0; j < depth && chained; ++j) chained = one_launch_layers(g[0], shapes[0]->dtype, c.allowed, problems, weights[0][j]->d_ff, true);
   if (chained) {
     const LayerScratch sc = layer_scratch(g[0], shapes[0]->dtype, max_ff);
     if (!workspace || workspace_bytes < problems * sc.total || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return GSIT_ERR_WORKSPACE;

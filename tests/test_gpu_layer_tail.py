@@ -86,17 +86,22 @@ def test_full_lengths_known_to_the_host(g, B, seg, d, heads, routes):
     assert g.last_device_status() == (0, 0)
 
 
-@pytest.mark.parametrize("B,seg,one_launch", [(54, (50, 52, 52), 0), (32, (50, 116, 116), 0), (23, (50, 180, 180), 1), (30, (50, 52, 52), 1)])
-def test_short_walks_at_width_32(g, B, seg, one_launch):
-    """Given lengths, beyond one wave: walks of one or two key tiles leave nothing for padding to cut short.  (30 samples are one wave.)"""
+# Beyond one wave with lengths that only the device knows: by walks of two thirds of the segments.  Segments of one tile keep their CTAs
+# however few rows are real; at width 128 an encoder's other choice are packed rows.
+@pytest.mark.parametrize("B,seg,d,phases,one_launch", [
+    (54, (50, 52, 52), 32, (2,), 0), (23, (50, 180, 180), 32, (2,), 1), (30, (50, 52, 52), 32, (2,), 1), (42, (21, 43, 34), 64, (0, 1), 0),
+    (5, (50, 500, 500), 64, (0, 1), 1), (25, (30, 26, 146), 128, (2,), 0), (5, (50, 500, 500), 128, (2,), 1)])
+def test_lengths_only_the_device_knows(g, B, seg, d, phases, one_launch):
     if torch.cuda.get_device_properties(0).multi_processor_count != 148:
         pytest.skip("sizes chosen for 148 SMs")
     rng = np.random.default_rng(B)
     vl = torch.from_numpy(np.stack([rng.integers(0, n + 1, size=B) for n in seg], axis=1).astype(np.int32)).cuda()
-    shape = g.make_shape(B, seg, 32, 4, vl, g.DTYPE_BF16, g.PHASE_INTRA)
-    assert g.load().gsit_encoder_runs_chained((ctypes.c_void_p * 1)(ctypes.addressof(shape)), 1, 64) == one_launch
-    x = to_dev(rng.standard_normal((B, sum(seg), 32), dtype=np.float32))
-    w = weights_to_dev(wk.draw_layer_weights(rng, 32, 64, "bf16", affine=True), "bf16")
-    want = torch.cat([g.im_layer_fwd(x[b:b + 1], w, seg, 4, vl[b:b + 1], g.PHASE_INTRA) for b in range(B)])
-    assert torch.equal(g.im_layer_fwd(x, w, seg, 4, vl, g.PHASE_INTRA), want)
+    shapes = [g.make_shape(B, seg, d, 8 if d > 32 else 4, vl, g.DTYPE_BF16, p) for p in phases]
+    assert g.load().gsit_encoder_runs_chained((ctypes.c_void_p * 2)(*[ctypes.addressof(s) for s in shapes]), len(phases), 64) == one_launch
+    x = to_dev(rng.standard_normal((B, sum(seg), d), dtype=np.float32))
+    w = [weights_to_dev(wk.draw_layer_weights(rng, d, 64, "bf16", affine=True), "bf16") for _ in phases]
+    run = lambda x, v: torch.cat([g.im_layer_fwd(x, w[0], seg, shapes[0].heads, v, phases[0])] if len(phases) == 1 else
+                                 g.im_layer_pair_fwd(x, x, w[0], w[1], seg, shapes[0].heads, v), 2)
+    want = torch.cat([run(x[b:b + 1], vl[b:b + 1]) for b in range(B)])
+    assert torch.equal(run(x, vl), want)
     assert g.last_device_status() == (0, 0)
