@@ -45,7 +45,8 @@ EXPORTS = ("gsit_im_qkv_proj", "gsit_im_attention_fwd", "gsit_im_layer_fwd", "gs
            "gsit_last_device_status", "gsit_status_string", "gsit_version", "gsit_trace_enable", "gsit_trace_read",
            "gsit_trace_launches", "gsit_trace_reset", "gsit_tune_attention", "gsit_test_expire_wait", "gsit_test_late_write", "gsit_im_layer_fwd_static",
            "gsit_stack_head_fwd", "gsit_im_layer_pair_fwd",
-           "gsit_plan_rows", "gsit_pack_rows", "gsit_unpack_rows", "gsit_plan_pack_rows")
+           "gsit_plan_rows", "gsit_pack_rows", "gsit_unpack_rows", "gsit_plan_pack_rows", "gsit_plan_pack_map_rows",
+           "gsit_im_encoder_fwd", "gsit_encoder_runs_chained", "gsit_im_layer_scatter_fwd", "gsit_layer_scatters", "gsit_attention_uses_workspace")
 STATIC_SCRATCH_BYTES = 4 << 20
 KERNEL_ATTENTION, KERNEL_LINEAR, KERNEL_LAYERNORM = 0, 1, 2
 ATTN_DEFAULT, ATTN_UNFUSED, ATTN_LEGACY, ATTN_TMEM = 0, 8, 9, 10   # gsit_kernel_choice of include/gsit_test.h

@@ -1,6 +1,8 @@
 """Kernels of the library may start while the kernel before them still runs; they must not read what that one writes before it has
 ended.  Each call is issued right behind a kernel that lets its successor start at once and writes the call's inputs -- all of
 them: weights, biases, activations, lengths -- late."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -109,3 +111,64 @@ def test_projection_and_attention_behind_a_kernel_that_writes_late(g, dtype, d, 
             att.check(lambda: list(g.im_attention_fwd(q[0], q[1], q[2], SEG, att.views[1], g.PHASE_INTER_BWD, want_lse=True)))
         finally:
             g.tune_attention(g.ATTN_DEFAULT)
+
+
+@pytest.mark.parametrize("B", [2, 90])
+def test_deep_stack_behind_a_kernel_that_writes_late(g, B):
+    """Three ring layers and two intra layers with weights of their own.  Two samples: every layer behind the first projection is one launch,
+    which reads its parameters above its wait while the launch before it runs; 90: packed rows, the last layer writes the padded result."""
+    rng = np.random.default_rng(B)
+    sets = [_layer(rng, 64, "bf16") for _ in range(6)] + [_layer(rng, 128, "bf16") for _ in range(2)]
+    keys, n = sets[0][0], len(sets[0][0])
+    x = torch.randn((B, sum(SEG), 64), device="cuda")
+    valid = torch.from_numpy(np.stack([rng.integers(1, n + 1, size=B) for n in SEG], axis=1).astype(np.int32)).cuda()
+    late = Late(g, [x, valid] + [t for _, ws in sets for t in ws])
+    w = [dict(zip(keys, late.views[2 + k * n:2 + (k + 1) * n])) for k in range(8)]
+    stack = g.GsitStack(w[0:3], w[3:6], w[6:8], SEG, 8, 8)
+    ring = [g.make_shape(B, SEG, 64, 8, late.views[1], g.DTYPE_BF16, p) for p in (g.PHASE_INTER_FWD, g.PHASE_INTER_BWD)]
+    intra = g.make_shape(B, SEG, 128, 8, late.views[1], g.DTYPE_BF16, g.PHASE_INTRA)
+    for shapes, d_ff in ((ring, 256), ([intra], 512)):
+        p = (ctypes.c_void_p * len(shapes))(*[ctypes.addressof(s) for s in shapes])
+        assert g.load().gsit_encoder_runs_chained(p, len(shapes), d_ff) == (B == 2)
+    if B == 90:
+        plan = g.plan_rows(late.views[1], SEG)
+        packed = g.make_shape(B, SEG, 128, 8, late.views[1], g.DTYPE_BF16, g.PHASE_INTRA, row_start=plan, capacity=B * sum(SEG) + 128)
+        assert g.load().gsit_layer_scatters(ctypes.byref(packed), 512) == 1
+    late.check(lambda: [stack.forward(late.views[0], late.views[1])])
+
+
+# more items than CTAs are resident, so that the kernel hands them out through the counter in its scratch
+@pytest.mark.parametrize("d,heads,choice", [(256, 4, "ATTN_DEFAULT"), (64, 4, "ATTN_TMEM"), (64, 2, "ATTN_TMEM"), (64, 8, "ATTN_TMEM")])
+def test_counter_of_the_attention_behind_a_kernel_that_writes_late(g, d, heads, choice):
+    """The counter is cleared by a kernel of the call: behind one that leaves something else there late, and behind an attention that is
+    still counting."""
+    B, hd = 150, d // heads
+    rng = np.random.default_rng(d)
+    valid = torch.from_numpy(np.stack([rng.integers(1, n + 1, size=B) for n in SEG], axis=1).astype(np.int32)).cuda()
+    qkv = torch.randn((3, B, sum(SEG), heads, hd), device="cuda").bfloat16()
+    late = Late(g, [qkv, valid, torch.full((64,), 1 << 20, dtype=torch.int32, device="cuda")])
+    q, vl, ws = late.views[0], late.views[1], late.views[2].view(torch.uint8)
+    g.tune_attention(getattr(g, choice))
+    try:
+        shape = g.make_shape(B, SEG, d, heads, vl, g.DTYPE_BF16, g.PHASE_INTER_BWD)
+        assert g.load().gsit_attention_uses_workspace(ctypes.byref(shape)) == 1
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
+        tiles = 3 * B   # every segment is one tile of 128 rows
+        assert tiles * heads > 8 * sms if hd == 64 else tiles * heads // 2 > 2 * sms
+        late.now.copy_(late.new)
+        want = g.im_attention_fwd(q[0], q[1], q[2], SEG, vl, g.PHASE_INTER_BWD, out=torch.empty((B, sum(SEG), d), dtype=q.dtype, device="cuda"),
+                                  workspace=torch.zeros(256, dtype=torch.uint8, device="cuda")).clone()
+        outs = [torch.empty_like(want) for _ in range(2)]
+        for _ in range(3):
+            late.now.copy_(late.old)
+            for o in outs:
+                o.fill_(float("nan"))
+            torch.cuda.synchronize()
+            g.late_write(late.now, late.new)
+            for o in outs:
+                g.im_attention_fwd(q[0], q[1], q[2], SEG, vl, g.PHASE_INTER_BWD, out=o, workspace=ws)
+            torch.cuda.synchronize()
+            assert all(torch.equal(o, want) for o in outs)
+    finally:
+        g.tune_attention(g.ATTN_DEFAULT)
+    assert g.last_device_status() == (0, 0)
