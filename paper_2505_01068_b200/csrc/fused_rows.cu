@@ -331,18 +331,22 @@ bool fused_rows_supported(const Geometry& g, int d_ff) {
 }
 // Where these kernels are chosen: always at width 32 (which no tcgen05 half covers); at 64 and 128 up to 43 padded rows per SM.
 // One layer without open blocks, us, these kernels / tcgen05 (148 SMs; lengths between half and full):
-//   rows               2100         3150         4200         5250         6300         8400
-//   d 64  padded    12.3/14.3    14.3/14.4    15.5/14.1    16.5/14.5    17.2/14.8    18.8/16.0
-//   d 64  packed    10.7/14.4    11.8/14.4    13.4/14.7    14.0/14.5    14.4/15.0    16.2/16.2
-//   d 64  packed, pair 13.5/14.5 14.8/15.0    17.2/16.3    17.7/16.8    22.4/17.9    27.1/17.9
-//   d 128 padded    20.4/23.8    23.4/23.8    24.1/23.9    27.3/24.7    35.3/25.1    35.2/24.9
-//   d 128 packed    17.8/23.9    19.1/23.8    21.9/24.0    23.0/25.0    30.7/25.3    31.9/24.8
-//   d 128 packed, pair 21.7/47.5 24.7/47.4    32.7/47.7    33.9/49.8    50.3/50.3    53.8/49.2
-// and at a quarter of the positions real (packed) these are the faster ones up to 8400 rows throughout but for pairs at d 64 (17.0 /
-// 16.7 at 6300).  So the two meet anywhere between 20 and 57 rows per SM, depending on what the host does not know (the lengths) or
-// must not look at: a sample gets the same bits alone, in a pair, padded, packed, and in any grouping of a batch within the limit.
-// The line lies at the upper end, where that holds for batches up to six samples of 1050 rows.  By the figures above a stack of four
-// pairs at d 64 and two layers at d 128 (packed) loses 29 us by it at 6300 rows, nothing at 5250, and wins 8 at a quarter real.
+//   rows                2100         3150         4200         5250         6300         8400
+//   d 64  padded     12.2/13.9    14.1/14.1    15.0/14.3    15.2/14.3    16.3/14.6    17.2/15.1
+//   d 64  packed     10.5/14.0    11.6/14.0    12.8/14.0    13.2/14.1    14.0/14.5    15.1/15.0
+//   d 64  packed, pair 13.3/14.1  14.6/14.6    15.4/15.0    15.9/15.5    16.0/15.8    21.8/17.0
+//   d 128 padded     20.3/23.4    23.0/23.5    23.2/23.6    25.8/24.2    33.7/24.6    33.9/24.2
+//   d 128 packed     17.6/23.4    19.5/23.4    21.1/23.6    22.3/24.2    22.4/24.4    30.6/23.8
+//   d 128 packed, pair 21.2/46.6  23.2/46.6    31.0/46.9    32.3/48.2    32.6/48.6    49.7/47.5
+// and at a quarter of the positions real these are the faster ones up to 8400 packed rows throughout and up to 4200 (d 64) and 5250
+// (d 128) padded ones.  So the two meet anywhere between 21 and 57 rows per SM, depending on what the host does not know (the lengths)
+// or must not look at: a sample gets the same bits alone, in a pair, padded, packed, and in any grouping of a batch within the limit.
+// The line lies at the upper end, where that holds for batches up to six samples of 1050 rows.  What it costs there, a stack of four pairs
+// at d 64 and two layers at d 128 as it runs (layers in one launch where they are chosen) / on the tcgen05 halves, us:
+//   samples               half to full   three quarters full   every length full   a quarter real
+//   4 (28 rows per SM)      144/168           154/172              155/166            101/138
+//   5 (35)                  157/169           207/178              234/186            100/138
+//   6 (43)                  217/184           239/199              260/198            135/142
 constexpr int ROWS_PER_SM = 43;
 static int sm_count() {
   int n = 0;
@@ -354,32 +358,34 @@ bool fused_rows_preferred(const Geometry& g) { return g.d == 32 || (int64_t)g.ba
 // tcgen05 GEMM's three tensor maps are encoded on the host first (6.2 us a call there, 5.4 here); at 128 never.  us here / on the kernel
 // for other widths (mma.sync at d 32, tcgen05 at 64 and 128), every position real:
 //   rows      500       2000      4000      8000      16000     32000
-//   d 32    2.7/4.4   2.7/4.6   2.8/4.7   3.1/4.7   4.0/5.3   6.3/7.3    (64 rows a tile from 8192 rows on; 32 there: 4.7 at 16000)
+//   d 32    2.7/4.4   2.7/4.6   2.7/4.7   3.0/4.7   3.7/5.3   5.4/7.3    (32 / 64 rows a tile: 3.7/3.9 at 16000, 5.9/5.4 at 32000)
 //   d 64    3.5/3.5   3.6/3.6   3.9/3.7   5.1/5.1   8.7/5.8  11.9/6.4
 //   d 128   5.0/4.0   5.2/4.1   6.2/5.6   9.5/6.2  17.4/7.2  29.3/14.6
 // The rows counted are those of the matrices, packed or padded: a call on part of a packed batch takes the kernel of the whole.
 bool qkv_rows_preferred(const Geometry& g) { return g.d == 32 || (g.d == 64 && matrix_rows(g) <= 2000); }
 cudaError_t launch_qkv_rows(const Geometry& g, const LinearArgs& l, cudaStream_t st) {
   const ProjArgs a = {static_cast<const __nv_bfloat16*>(l.A), l.lda, static_cast<const __nv_bfloat16*>(l.W), l.bias, static_cast<__nv_bfloat16*>(l.C)};
-  if (g.d == 32) return matrix_rows(g) >= 8192 ? launch_qkv<32, 4>(g, a, st) : launch_qkv<32, 2>(g, a, st);
+  // 32 rows a tile up to 140 rows per SM, by the figures above
+  if (g.d == 32) return matrix_rows(g) > 140 * (int64_t)sm_count() ? launch_qkv<32, 4>(g, a, st) : launch_qkv<32, 2>(g, a, st);
   if (g.d == 64) return launch_qkv<64, 1>(g, a, st);
   return cudaErrorNotSupported;
 }
 
 // n problems (1 or 2) of one geometry in one launch each.  Rows per tile: 16 (d 32: 32) for the shortest chain while a launch is about
-// the latency of a tile, twice as many where the weight reads of many tiles (through L1) become what counts.  Limits in rows per
-// SM; a layer without open blocks, us, small tile / large tile, full lengths:
-//   first half,  d 32   284: 28.6/29.5   341: 31.6/31.3   454: 40.6/39.8     -> 320
-//   second half, d 32    57: 11.7/11.7    71: 13.0/12.7    85: 13.7/13.4   114: 15.9/14.2   -> 72 (half-full lengths meet at 75)
-//   second half, d 64    28: 14.6/14.7    35: 15.5/16.0    43: 16.5/16.4    50: 20.5/17.2   -> 40
-//   second half, d 128  8.5: 17.1/18.3   9.9: 18.7/18.5  11.4: 19.2/19.0    14: 20.9/19.2   -> 10
+// the latency of a tile, twice as many where the weight reads of many tiles (through L1) become what counts.  For the second half that is
+// one wave of small tiles at d 64 (three CTAs per SM) and 128 (one), and three tiles per SM (two at a time) at d 32.  Limits in rows per SM; a layer without open blocks, us, small tile /
+// large tile, full lengths (half to full):
+//   first half,  d 32   341: 30.7/31.2    600: 49.6/49.7    900: 71.4/71.3 (63.0/62.2)    1500: 119.4/118.9 (104.4/102.8)   -> 800
+//   second half, d 32    78: 12.3/12.8     92: 13.1/12.9     96: 13.2/12.9 (11.7/13.9)      99: 14.0/13.0 (13.6/13.9)       -> 96
+//   second half, d 64    43: 14.7/15.2     48: 14.8/15.7   48.5: 18.6/15.8 (15.4/16.6)      50: 19.7/15.9 (15.5/16.8)       -> 48
+//   second half, d 128   10: 16.4/18.1     14: 17.0/19.2     16: 16.0/19.3 (16.7/20.3)    16.5: 23.1/20.6 (18.3/20.3)       -> 16
 // A row's bits do not depend on it, so the number of problems may count here.
 cudaError_t launch_ln_qkv_rows(const Geometry& g, const FusedHalfArgs* h, int n, float eps, int* zero_word, cudaStream_t st) {
   Pair p;
   p.a[0] = h[0];
   p.a[1] = h[n - 1];
   const int64_t rows = (int64_t)g.batch * g.L * n, sms = sm_count();
-  if (g.d == 32) return rows > 320 * sms ? launch_ln_qkv<32, 4>(g, p, n, eps, zero_word, st) : launch_ln_qkv<32, 2>(g, p, n, eps, zero_word, st);
+  if (g.d == 32) return rows > 800 * sms ? launch_ln_qkv<32, 4>(g, p, n, eps, zero_word, st) : launch_ln_qkv<32, 2>(g, p, n, eps, zero_word, st);
   if (g.d == 64) return launch_ln_qkv<64, 1>(g, p, n, eps, zero_word, st);
   return launch_ln_qkv<128, 1>(g, p, n, eps, zero_word, st);
 }
@@ -388,9 +394,9 @@ cudaError_t launch_proj_mlp_rows(const Geometry& g, const FusedHalfArgs* h, int 
   p.a[0] = h[0];
   p.a[1] = h[n - 1];
   const int64_t rows = (int64_t)g.batch * g.L * n, sms = sm_count();
-  if (g.d == 32) return rows > 72 * sms ? launch_proj_mlp<32, 4>(g, p, n, eps, d_ff, st) : launch_proj_mlp<32, 2>(g, p, n, eps, d_ff, st);
-  if (g.d == 64) return rows > 40 * sms ? launch_proj_mlp<64, 2>(g, p, n, eps, d_ff, st) : launch_proj_mlp<64, 1>(g, p, n, eps, d_ff, st);
-  return rows > 10 * sms ? launch_proj_mlp<128, 2>(g, p, n, eps, d_ff, st) : launch_proj_mlp<128, 1>(g, p, n, eps, d_ff, st);
+  if (g.d == 32) return rows > 96 * sms ? launch_proj_mlp<32, 4>(g, p, n, eps, d_ff, st) : launch_proj_mlp<32, 2>(g, p, n, eps, d_ff, st);
+  if (g.d == 64) return rows > 48 * sms ? launch_proj_mlp<64, 2>(g, p, n, eps, d_ff, st) : launch_proj_mlp<64, 1>(g, p, n, eps, d_ff, st);
+  return rows > 16 * sms ? launch_proj_mlp<128, 2>(g, p, n, eps, d_ff, st) : launch_proj_mlp<128, 1>(g, p, n, eps, d_ff, st);
 }
 
 }  // namespace gsit
