@@ -1,5 +1,7 @@
-"""The fused layer halves on small row tiles: every width, tiles of 16, 32 and 64 rows (chosen by the row count), row counts that end
-inside a tile, tiles of padding only, strided rows, the packed layout and the pair call."""
+"""Layers on small row tiles: every width, tiles of 16, 32 and 64 rows (chosen by the row count), row counts that end inside a tile, tiles of
+padding only, strided rows, the packed layout and the pair call; by layers of one launch, where those are chosen, and by the two halves."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -19,7 +21,7 @@ def g():
 
 
 @pytest.mark.parametrize("d,heads,d_ff,seg,B", [(32, 4, 128, (5, 11, 2), 1), (32, 2, 64, (50, 130, 77), 5), (32, 1, 512, (50, 300, 270), 25),
-                                                (32, 4, 128, (50, 300, 270), 80), (64, 8, 256, (3, 0, 4), 1), (64, 4, 192, (50, 130, 77), 3),
+                                                (32, 4, 128, (50, 300, 270), 80), (32, 4, 64, (50, 300, 270), 200), (64, 8, 256, (3, 0, 4), 1), (64, 4, 192, (50, 130, 77), 3),
                                                 (64, 2, 512, (50, 300, 270), 9), (128, 8, 512, (7, 1, 1), 1), (128, 4, 320, (50, 130, 77), 6),
                                                 (128, 8, 512, (50, 300, 270), 2)])
 def test_layer_on_row_tiles(g, d, heads, d_ff, seg, B):
@@ -68,6 +70,38 @@ def check_layer(g, d, heads, d_ff, seg, B, tile=1):
     assert g.last_device_status() == (0, 0)
 
 
+# Heads of 64 have no layers of one launch: both halves are launches of their own at every size.  Tiles of 16 rows up to 48 (d 64) and 16
+# (d 128) rows per SM, of 32 above; B * L around the edges of tiles and, with 148 SMs, on both sides of 16 rows per SM (2368).
+@pytest.mark.parametrize("d,heads,d_ff,seg,B", [(64, 1, 256, (3, 0, 4), 1), (64, 1, 64, (50, 130, 77), 3), (64, 1, 512, (100, 300, 300), 9), (128, 2, 512, (7, 1, 1), 1),
+                                                (128, 2, 320, (50, 130, 77), 6), (128, 2, 64, (50, 130, 77), 9), (128, 2, 512, (50, 130, 77), 10),
+                                                (128, 2, 512, (50, 500, 500), 6)])
+def test_halves_as_launches_of_their_own(g, d, heads, d_ff, seg, B):
+    rng = np.random.default_rng(d + d_ff + B)
+    x = rng.standard_normal((B, sum(seg), d), dtype=np.float32)
+    w = wk.draw_layer_weights(rng, d, d_ff, "bf16", affine=True)
+    valid = np.stack([rng.integers((n + 1) // 2, n + 1, size=B) for n in seg], axis=1).astype(np.int32)
+    if B > 2:
+        valid[B // 2] = 0
+    pm, vl, wd = pad_mask(seg, valid, B), torch.from_numpy(valid).cuda(), weights_to_dev(w, "bf16")
+    shape = g.make_shape(B, seg, d, heads, vl, g.DTYPE_BF16, g.PHASE_INTRA)
+    assert g.load().gsit_encoder_runs_chained((ctypes.c_void_p * 1)(ctypes.addressof(shape)), 1, d_ff) == 0
+    xd = to_dev(np.where(pm[:, :, None], np.nan, x).astype(np.float32))
+    y = g.im_layer_fwd(xd, wd, seg, heads, vl, g.PHASE_INTRA)
+    assert bool((y[torch.from_numpy(pm).cuda()] == 0).all())
+    for b in {0, B - 1}:
+        ref = oracle.im_layer_fwd(x[b:b + 1], w, seg, heads, valid[b:b + 1], g.PHASE_INTRA)
+        if sum(seg) > 16:
+            check_close(to_np64(y[b:b + 1]), ref, "bf16", pm[b:b + 1], f"sample {b}")
+        else:
+            # rows of a few keys, which average nothing: five roundings to bf16 on a value's way (LN1 row, v, attention row, LN2 row, hidden
+            # unit), each 0.4 x 2^-9 on average of values around one, add up to at most 3.9e-3 on average (1.3 - 2.7e-3 seen, with heads
+            # of 8 to 64 alike); the largest as everywhere
+            err = np.abs(to_np64(y[b:b + 1]) - ref)
+            assert err.mean() <= 3.9e-3 and err.max() <= 2e-2
+        assert torch.equal(g.im_layer_fwd(xd[b:b + 1], wd, seg, heads, vl[b:b + 1], g.PHASE_INTRA), y[b:b + 1])   # at small tiles
+    assert g.last_device_status() == (0, 0)
+
+
 @pytest.mark.parametrize("d,heads", [(64, 8), (128, 8)])
 @pytest.mark.parametrize("above", [0, 1])
 def test_layer_on_either_side_of_the_row_limit(g, d, heads, above):
@@ -103,9 +137,9 @@ def test_layer_on_either_side_of_the_row_limit(g, d, heads, above):
     assert g.last_device_status() == (0, 0)
 
 
-@pytest.mark.parametrize("d,heads,seg,B", [(32, 4, (3, 1, 2), 1), (32, 1, (17, 130, 45), 5), (32, 4, (33, 257, 300), 15), (64, 8, (3, 5, 9), 1), (64, 2, (40, 193, 267), 4)])
+@pytest.mark.parametrize("d,heads,seg,B", [(32, 4, (3, 1, 2), 1), (32, 1, (17, 130, 45), 5), (32, 4, (33, 257, 300), 15), (32, 4, (33, 257, 300), 36), (64, 8, (3, 5, 9), 1), (64, 2, (40, 193, 267), 4)])
 def test_projection_on_row_tiles(g, d, heads, seg, B):
-    """The projection alone on row tiles (32 and, from 8192 rows on, 64 rows at d 32; 16 at d 64 up to 2000 rows): strided input with NaN
+    """The projection alone on row tiles (32 and, above 140 per SM, 64 rows at d 32; 16 at d 64 up to 2000 rows): strided input with NaN
     in the padding against a float product of the same operands (bf16 result: 2^-8 relative), and the packed layout bit for bit
     (at 32, where it is not covered, refused)."""
     rng = np.random.default_rng(B)
