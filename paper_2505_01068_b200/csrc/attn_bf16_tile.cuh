@@ -48,6 +48,7 @@ __device__ __forceinline__ uint32_t swz(uint32_t off) { return off ^ (((off >> 7
 // Bounded wait: gives up after WAIT_SPINS polls, raises GSIT_DEVFLAG_TIMEOUT and lets the CTA run on
 // (its results are then invalid, but nothing hangs).
 __device__ __forceinline__ void mbar_wait(const Geometry& g, uint32_t bar, uint32_t parity) {
+#pragma unroll 1
   for (int it = 0; it < WAIT_SPINS; ++it) {
     if (mbar_test(bar, parity)) return;
     if (it > 64) __nanosleep(64);

@@ -53,6 +53,7 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
 }
 // Bounded wait for a phase of the tile barrier; raises GSIT_DEVFLAG_TIMEOUT instead of hanging.
 __device__ __forceinline__ void mbar_wait(const Geometry& g, uint32_t bar, uint32_t parity) {
+#pragma unroll 1
   for (int it = 0; it < (1 << 16); ++it) {
     uint32_t ok;
     asm volatile(

@@ -91,6 +91,7 @@ __device__ __forceinline__ void arrive_remote(uint32_t cluster_addr) {
 }
 // Bounded wait whose phase other CTAs of the cluster complete with arrive_remote.
 __device__ __forceinline__ bool mbar_wait_cluster(const WaitCtx& w, uint32_t bar, uint32_t parity, int limit = 1 << 16) {
+#pragma unroll 1
   for (int it = 0; it < limit; ++it) {
     uint32_t ok;
     asm volatile(

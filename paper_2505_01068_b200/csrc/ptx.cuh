@@ -71,7 +71,12 @@ __device__ __forceinline__ bool cta_gave_up(const WaitCtx& w) {
 // Bounded wait on a barrier phase.  Returns true when the phase completed; false after `limit` polls (the timeout flag is
 // raised) or as soon as another wait of this CTA has expired.  The caller carries on either way and must still release
 // whatever it holds.
+// The loops of all waits stay rolled.  Left to itself the compiler unrolls them, at every place where they are used: the polls of the
+// waiting warps then stream through kilobytes of instructions and push those of the computing warps out of the instruction caches.  Text of
+// the head_dim 16 attention 54 -> 46 KB, misses of its instruction cache 309 K -> 123 K, 74.9 -> 71.2 us at 64 x (50, 500, 500), 8 heads, intra;
+// head_dim 32, 4 heads, cross 36.5 -> 34.3; a whole stack of that batch 718 -> 701 us, of 32 samples a quarter real 214.6 -> 205.0.
 __device__ __forceinline__ bool mbar_wait(const WaitCtx& w, uint32_t bar, uint32_t parity, int limit = 1 << 16) {
+#pragma unroll 1
   for (int it = 0; it < limit; ++it) {
     if (mbar_try(bar, parity)) return true;
     if ((it & 63) == 63 && cta_gave_up(w)) return false;
@@ -83,6 +88,7 @@ __device__ __forceinline__ bool mbar_wait(const WaitCtx& w, uint32_t bar, uint32
 
 // The same with parked polls of up to ten microseconds each (2^15 of them at most: a third of a second).
 __device__ __forceinline__ bool mbar_wait_parked(const WaitCtx& w, uint32_t bar, uint32_t parity, int limit = 1 << 15) {
+#pragma unroll 1
   for (int it = 0; it < limit; ++it) {
     if (mbar_try_park(bar, parity, 10000u)) return true;
     if ((it & 15) == 15 && cta_gave_up(w)) return false;
@@ -97,6 +103,7 @@ __device__ __forceinline__ bool mbar_wait_parked(const WaitCtx& w, uint32_t bar,
 // slots from the warps that compute.  Here a poll never parks (test_wait) and is followed by a sleep of about `ns`
 // nanoseconds during which the warp issues nothing.  Gives up after `limit` polls like mbar_wait.
 __device__ __forceinline__ bool mbar_wait_sleep(const WaitCtx& w, uint32_t bar, uint32_t parity, unsigned ns, int limit = 1 << 17) {
+#pragma unroll 1
   for (int it = 0; it < limit; ++it) {
     if (mbar_test(bar, parity)) return true;
     if (ns) __nanosleep(ns);
@@ -113,6 +120,7 @@ __device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t count) {
 }
 // Bounded wait that spins on non-parking polls: the shortest hand-over latency, at the price of issue slots.
 __device__ __forceinline__ bool mbar_wait_spin(const WaitCtx& w, uint32_t bar, uint32_t parity, int limit = 1 << 22) {
+#pragma unroll 1
   for (int it = 0; it < limit; ++it) {
     if (mbar_test(bar, parity)) return true;
     if ((it & 1023) == 1023 && cta_gave_up(w)) return false;
