@@ -19,8 +19,8 @@ constexpr int WAIT_SPINS = 1 << 20;
 
 // HD = head_dim, CW = features per column slice, R_ = 16-row query slabs per warp, KSTEP_ = keys per softmax
 // step, MINB_ = CTAs per SM the register allocation must allow, SL_ = column slices per CTA, NSG_ = warps per head,
-// STAGES_ = key tiles in flight.
-template <int HD_, int CW_, int R_, int KSTEP_, int MINB_, int SL_ = 1, int NSG_ = 8 / (CW_ / HD_ * SL_), int STAGES_ = 3>
+// STAGES_ = key tiles in flight (three make the warps of a CTA wait for the slowest: 64 x (50, 500, 500), 8 heads of 8, every block open, 200 us; five 195).
+template <int HD_, int CW_, int R_, int KSTEP_, int MINB_, int SL_ = 1, int NSG_ = 8 / (CW_ / HD_ * SL_), int STAGES_ = 5>
 struct Cfg {
   static constexpr int HD = HD_, CW = CW_, R = R_, KSTEP = KSTEP_, MINB = MINB_, SL = SL_, STAGES = STAGES_;
   static constexpr int G = CW / HD;                 // heads per column slice
@@ -51,6 +51,15 @@ __device__ __forceinline__ void mbar_wait(const Geometry& g, uint32_t bar, uint3
 #pragma unroll 1
   for (int it = 0; it < WAIT_SPINS; ++it) {
     if (mbar_test(bar, parity)) return;
+    if (it > 64) __nanosleep(64);
+  }
+  raise_flag(g, GSIT_DEVFLAG_TIMEOUT);
+}
+// The same by a whole warp, which then knows that its lanes stay together: nothing has to be done to bring them together again.
+__device__ __forceinline__ void mbar_wait_warp(const Geometry& g, uint32_t bar, uint32_t parity) {
+#pragma unroll 1
+  for (int it = 0; it < WAIT_SPINS; ++it) {
+    if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return;
     if (it > 64) __nanosleep(64);
   }
   raise_flag(g, GSIT_DEVFLAG_TIMEOUT);
@@ -151,7 +160,7 @@ __device__ __forceinline__ void attend_tile(const Geometry& g, const Tile& t_, c
   constexpr int HD = C::HD, CW = C::CW, G = C::G, R = C::R, PITCH = C::PITCH, SWZ = C::SWZ,
                 KSTEP = C::KSTEP, NT = C::NT, KSQ = C::KSQ, NTO = C::NTO, SL = C::SL, STAGES = C::STAGES;
   constexpr bool HOIST = (R > 1);  // several query slabs per warp reuse the K/V fragments of a step
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   const int head = warp % (G * SL), sg = warp / (G * SL), slice = head / G, head_in_slice = head % G;
   // Known at compile time where every warp of the CTA attends: a walk behind a branch takes longer (14 key tiles of one 16-row slab at head_dim 8:
   // 13.75 us, 13.50 without the branch; one sample of (50, 500, 500) 8.96 and 8.80).  Not with four slabs per warp, which then spill
@@ -164,7 +173,7 @@ __device__ __forceinline__ void attend_tile(const Geometry& g, const Tile& t_, c
   const uint32_t bar_empty = bar_full + 8 * STAGES;     // STAGES barriers: all attending warps are done with the stage
   const uint32_t bar_q = bar_empty + 8 * STAGES;
   const int cb = head_in_slice * (HD / 8);  // first 16-byte chunk of this warp's head inside a tile row
-  const int b = t_.b, s = t_.s, q0 = t_.q0, kn0 = t_.kn0, kn1 = t_.kn1, kn2 = t_.kn2, nk0 = t_.nk0, nk1 = t_.nk1, T = t_.T, q_real = t_.q_real;
+  const int b = t_.b, s = t_.s, q0 = t_.q0, kn0 = t_.kn0, kn1 = t_.kn1, kn2 = t_.kn2, nk0 = t_.nk0, nk1 = t_.nk1, T = uniform(t_.T), q_real = uniform(t_.q_real);
   const int kbase0 = t_.kbase0, kbase1 = t_.kbase1, kbase2 = t_.kbase2;
   const int64_t grow0 = t_.grow0;
 
@@ -212,7 +221,7 @@ __device__ __forceinline__ void attend_tile(const Geometry& g, const Tile& t_, c
   // ---- query fragments, kept in registers for the whole key walk ----
   uint32_t QF[R][KSQ][4];
   if (active) {
-    mbar_wait(g, bar_q, 0);
+    mbar_wait_warp(g, bar_q, 0);
 #pragma unroll
     for (int r_ = 0; r_ < R; ++r_) {
       const int row0 = (sg * R + r_) * 16;
@@ -434,9 +443,10 @@ __device__ __forceinline__ void attend_tile(const Geometry& g, const Tile& t_, c
         }
       }
       __syncwarp();
-      mbar_wait(g, bar_full + 8 * st, (i / STAGES) & 1);
+      mbar_wait_warp(g, bar_full + 8 * st, (i / STAGES) & 1);
       int krem, yrow;
       locate(i - from, krem, yrow);
+      krem = uniform(krem);
       const bool first = i == from;
       const uint32_t sKs = sK + (st * SL + slice) * C::KV_BYTES, sVs = sV + (st * SL + slice) * C::KV_BYTES;
       if (krem >= KT) {

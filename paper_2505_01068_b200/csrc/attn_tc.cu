@@ -108,6 +108,11 @@ __device__ __forceinline__ void locate(const Geometry& g, const Item& it, int i,
   yrow = ((r == 0) ? it.kb0 : (r == 1) ? it.kb1 : it.kb2) + t * TK;
 }
 
+// The same item in uniform registers.
+__device__ __forceinline__ Item uniform_item(const Item& a) {
+  return Item{uniform(a.b), uniform(a.h), uniform(a.s), uniform(a.q0), uniform(a.rows_in_tile), uniform(a.q_real), uniform(a.T), uniform(a.kn0),
+              uniform(a.kn1), uniform(a.kn2), uniform(a.nk0), uniform(a.nk1), uniform(a.kb0), uniform(a.kb1), uniform(a.kb2), uniform(a.grow0)};
+}
 // Producer side: lane 0 writes record k of this CTA, then the slot's "written" barrier is released.
 __device__ __forceinline__ void publish_item(uint32_t base, const Item& it, int k, int lane) {
   if (lane == 0) {
@@ -123,13 +128,14 @@ __device__ __forceinline__ void publish_item(uint32_t base, const Item& it, int 
 // Consumer side (whole warp): waits for record k, copies it to registers and releases the slot (one arrival per warp).
 __device__ __forceinline__ Item fetch_item(const WaitCtx& wc, uint32_t base, int k, int lane) {
   const int slot = k % ITEM_SLOTS;
-  const bool ok = mbar_wait(wc, base + OFF_ITEMBAR + 8 * slot, (k / ITEM_SLOTS) & 1);
+  const bool ok = mbar_wait_warp(wc, base + OFF_ITEMBAR + 8 * slot, (k / ITEM_SLOTS) & 1);
   const uint32_t a = base + OFF_ITEMS + 64 * slot;
   Item it;
   asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(it.b), "=r"(it.h), "=r"(it.s), "=r"(it.q0) : "r"(a) : "memory");
   asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(it.rows_in_tile), "=r"(it.q_real), "=r"(it.T), "=r"(it.kn0) : "r"(a + 16) : "memory");
   asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(it.kn1), "=r"(it.kn2), "=r"(it.nk0), "=r"(it.nk1) : "r"(a + 32) : "memory");
   asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(it.kb0), "=r"(it.kb1), "=r"(it.kb2), "=r"(it.grow0) : "r"(a + 48) : "memory");
+  it = uniform_item(it);
   fence_reads_before_release();
   __syncwarp();
   if (lane == 0) mbar_arrive(base + OFF_ITEMBAR + 8 * ITEM_SLOTS + 8 * slot);
@@ -145,7 +151,7 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t sQ = base + OFF_Q, sK = base + OFF_K, sV = base + OFF_V, bars = base + OFF_BAR;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   const WaitCtx wc{g.status, bars + SLOT_GAVE_UP};
 
   // ---- set-up, once per CTA: barriers, tensor memory ----
@@ -202,16 +208,16 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         } else {
           w = blockIdx.x + k * gridDim.x;
         }
-        const bool end = next_item != nullptr && (w >= n_items || cta_gave_up(wc));
+        const bool end = next_item != nullptr && __any_sync(0xffffffffu, w >= n_items || cta_gave_up(wc));
         Item it = {};
         if (end) it.T = -1;
-        else it = decode_item(g, w, seg_order);
-        if (k >= ITEM_SLOTS) mbar_wait(wc, base + OFF_ITEMBAR + 8 * ITEM_SLOTS + 8 * (k % ITEM_SLOTS), ((k / ITEM_SLOTS) - 1) & 1);
+        else it = uniform_item(decode_item(g, w, seg_order));
+        if (k >= ITEM_SLOTS) mbar_wait_warp(wc, base + OFF_ITEMBAR + 8 * ITEM_SLOTS + 8 * (k % ITEM_SLOTS), ((k / ITEM_SLOTS) - 1) & 1);
         publish_item(base, it, k, lane);
         if (end) break;
         if (it.T == 0) continue;
         const int qb = n_q & 1, quse = n_q >> 1;
-        if (quse > 0) mbar_wait(wc, bars + BAR_QEMPTY + 8 * qb, (quse - 1) & 1);
+        if (quse > 0) mbar_wait_warp(wc, bars + BAR_QEMPTY + 8 * qb, (quse - 1) & 1);
         if (elect_one()) {
           mbar_expect_tx(bars + BAR_QFULL + 8 * qb, Q_BYTES);
           tma_load_2d(sQ + qb * Q_BYTES, &tmQ, it.h * HD64, it.grow0, bars + BAR_QFULL + 8 * qb);
@@ -221,12 +227,12 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           int krem, yrow;
           locate(g, it, i, krem, yrow);
           const int st = n_kv % KV_STAGES, use = n_kv / KV_STAGES;
-          if (use > 0) mbar_wait(wc, bars + BAR_KEMPTY + 8 * st, (use - 1) & 1);
+          if (use > 0) mbar_wait_warp(wc, bars + BAR_KEMPTY + 8 * st, (use - 1) & 1);
           if (elect_one()) {
             mbar_expect_tx(bars + BAR_KFULL + 8 * st, KV_BYTES);
             tma_load_2d(sK + st * KV_BYTES, &tmK, it.h * HD64, yrow, bars + BAR_KFULL + 8 * st);
           }
-          if (use > 0) mbar_wait(wc, bars + BAR_VEMPTY + 8 * st, (use - 1) & 1);
+          if (use > 0) mbar_wait_warp(wc, bars + BAR_VEMPTY + 8 * st, (use - 1) & 1);
           if (elect_one()) {
             mbar_expect_tx(bars + BAR_VFULL + 8 * st, KV_BYTES);
             tma_load_2d(sV + st * KV_BYTES, &tmV, it.h * HD64, yrow, bars + BAR_VFULL + 8 * st);
@@ -250,7 +256,7 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         // read by the softmax of key tile n - 2, whose P this thread has already waited for.
         auto issue_qk = [&](int n, bool last) {
           const int st = n % KV_STAGES;
-          mbar_wait(wc, bars + BAR_KFULL + 8 * st, (n / KV_STAGES) & 1);
+          mbar_wait_warp(wc, bars + BAR_KFULL + 8 * st, (n / KV_STAGES) & 1);
           tc_fence_after();
           if (elect_one()) {
 #pragma unroll
@@ -263,14 +269,14 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           }
           __syncwarp();
         };
-        mbar_wait(wc, bars + BAR_QFULL + 8 * qb, (n_q >> 1) & 1);
+        mbar_wait_warp(wc, bars + BAR_QFULL + 8 * qb, (n_q >> 1) & 1);
         issue_qk(n_kv, it.T == 1);
         for (int j = 0; j < it.T; ++j) {
           const int n = n_kv + j, st = n % KV_STAGES;
           if (j + 1 < it.T) issue_qk(n + 1, j + 2 == it.T);  // scores of the next tile, ahead of this tile's P V
           // P[n & 1] is in TMEM (and, for the first tile of an item, the previous item's O has been read)
-          mbar_wait(wc, bars + BAR_PFULL + 8 * (n & 1), (n >> 1) & 1);
-          mbar_wait(wc, bars + BAR_VFULL + 8 * st, (n / KV_STAGES) & 1);
+          mbar_wait_warp(wc, bars + BAR_PFULL + 8 * (n & 1), (n >> 1) & 1);
+          mbar_wait_warp(wc, bars + BAR_VFULL + 8 * st, (n / KV_STAGES) & 1);
           tc_fence_after();
           if (elect_one()) {
 #pragma unroll
@@ -312,7 +318,7 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       auto tile_step = [&](auto ragged_tag, const int j, const int n, const int krem) {
         constexpr bool RAGGED = decltype(ragged_tag)::value;
         const int sb = n & 1;
-        mbar_wait(wc, bars + BAR_SFULL + 8 * sb, (n >> 1) & 1);
+        mbar_wait_warp(wc, bars + BAR_SFULL + 8 * sb, (n >> 1) & 1);
         tc_fence_after();
         uint32_t sr[2][32];
 #pragma unroll
@@ -341,7 +347,7 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           const float alpha = grow_m ? ex2((m_used - mx) * sl2) : 1.f;
           l *= alpha;
           // O must hold every earlier tile of the item before it is rescaled: wait for the P V of tile n - 1
-          mbar_wait(wc, bars + BAR_VEMPTY + 8 * ((n - 1) % KV_STAGES), ((n - 1) / KV_STAGES) & 1);
+          mbar_wait_warp(wc, bars + BAR_VEMPTY + 8 * ((n - 1) % KV_STAGES), ((n - 1) / KV_STAGES) & 1);
           tc_fence_after();
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
@@ -376,7 +382,7 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           // Rows of the V tile past the valid length hold whatever follows in memory; a zero weight times NaN or Inf
           // would still poison the accumulator, so clear them before the MMA reads the tile.
           const int st = n % KV_STAGES;
-          mbar_wait(wc, bars + BAR_VFULL + 8 * st, (n / KV_STAGES) & 1);
+          mbar_wait_warp(wc, bars + BAR_VFULL + 8 * st, (n / KV_STAGES) & 1);
           const int row = krem + (tid - 64);
           if (row < TK) {
             const uint32_t a = sV + st * KV_BYTES + row * 128;
@@ -400,7 +406,7 @@ attn_tc_hd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       n_kv += it.T;
 
       // ---- epilogue: O / l -> bf16, each thread its own 128-byte row; padded rows +0 ----
-      mbar_wait(wc, bars + BAR_OFINAL, n_items_done & 1);
+      mbar_wait_warp(wc, bars + BAR_OFINAL, n_items_done & 1);
       ++n_items_done;
       tc_fence_after();
       const float inv = (l > 0.f) ? 1.f / l : 0.f;

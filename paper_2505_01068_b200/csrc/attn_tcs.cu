@@ -155,6 +155,11 @@ __device__ __forceinline__ void publish_item(uint32_t bars, const SItem& it, int
   }
   __syncwarp();
 }
+// The same item in uniform registers.
+__device__ __forceinline__ SItem uniform_item(const SItem& a) {
+  return SItem{uniform(a.b), uniform(a.c), uniform(a.s), uniform(a.q0), uniform(a.rows_in_tile), uniform(a.q_real), uniform(a.T), uniform(a.kn0),
+               uniform(a.kn1), uniform(a.kn2), uniform(a.nk0), uniform(a.nk1), uniform(a.kb0), uniform(a.kb1), uniform(a.kb2), uniform(a.grow0)};
+}
 // Copies record `slot` to registers and releases the slot (one arrival per warp).
 __device__ __forceinline__ SItem read_item(uint32_t bars, int slot, int lane) {
   const uint32_t a = bars + B_ITEMS + 64 * slot;
@@ -163,6 +168,7 @@ __device__ __forceinline__ SItem read_item(uint32_t bars, int slot, int lane) {
   asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(it.rows_in_tile), "=r"(it.q_real), "=r"(it.T), "=r"(it.kn0) : "r"(a + 16) : "memory");
   asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(it.kn1), "=r"(it.kn2), "=r"(it.nk0), "=r"(it.nk1) : "r"(a + 32) : "memory");
   asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(it.kb0), "=r"(it.kb1), "=r"(it.kb2), "=r"(it.grow0) : "r"(a + 48) : "memory");
+  it = uniform_item(it);
   fence_reads_before_release();
   __syncwarp();
   if (lane == 0) mbar_arrive(bars + B_ITEMBAR + 8 * S_ITEM_SLOTS + 8 * slot);
@@ -170,7 +176,7 @@ __device__ __forceinline__ SItem read_item(uint32_t bars, int slot, int lane) {
 }
 __device__ __forceinline__ SItem fetch_item(const WaitCtx& wc, uint32_t bars, int k, int lane) {
   const int slot = k % S_ITEM_SLOTS;
-  const bool ok = mbar_wait(wc, bars + B_ITEMBAR + 8 * slot, (k / S_ITEM_SLOTS) & 1);
+  const bool ok = mbar_wait_warp(wc, bars + B_ITEMBAR + 8 * slot, (k / S_ITEM_SLOTS) & 1);
   SItem it = read_item(bars, slot, lane);
   if (!ok) it.T = -1;  // the hand-over itself timed out: stop (the flag has been raised)
   return it;
@@ -186,7 +192,7 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t sQ = base, sK = base + C::OFF_K, sV = base + C::OFF_V, bars = base + C::OFF_BAR;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   const WaitCtx wc{g.status, bars + B_GAVE_UP};
 
   // ---- set-up, once per CTA: barriers, the zero blocks of the Q layout, tensor memory ----
@@ -248,8 +254,8 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
         w = blockIdx.x + k * gridDim.x;
       }
       if (k >= S_ITEM_SLOTS)
-        mbar_wait(wc, bars + B_ITEMBAR + 8 * S_ITEM_SLOTS + 8 * (k % S_ITEM_SLOTS), ((k / S_ITEM_SLOTS) - 1) & 1);
-      if (w >= n_items || cta_gave_up(wc)) {
+        mbar_wait_warp(wc, bars + B_ITEMBAR + 8 * S_ITEM_SLOTS + 8 * (k % S_ITEM_SLOTS), ((k / S_ITEM_SLOTS) - 1) & 1);
+      if (__any_sync(0xffffffffu, w >= n_items || cta_gave_up(wc))) {
         SItem end = {};
         end.T = -1;
         publish_item(bars, end, k, lane);
@@ -257,13 +263,13 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
       }
       const int which = (problems == 2) ? (w & 1) : 0;
       const SProblem& prob = which ? prob1 : prob0;
-      SItem it = decode_item(g, prob.allowed, (problems == 2) ? (w >> 1) : w, slices, prob.seg_order, which);
+      SItem it = uniform_item(decode_item(g, prob.allowed, (problems == 2) ? (w >> 1) : w, slices, prob.seg_order, which));
       publish_item(bars, it, k, lane);
       if (it.T == 0) continue;
       it.c &= (1 << WHICH_SHIFT) - 1;
       const CUtensorMap &tmQ = prob.tmQ, &tmK = prob.tmK, &tmV = prob.tmV;
       const int qb = n_q & 1;
-      if (n_q >= 2) mbar_wait(wc, bars + B_QEMPTY + 8 * qb, ((n_q >> 1) - 1) & 1);
+      if (n_q >= 2) mbar_wait_warp(wc, bars + B_QEMPTY + 8 * qb, ((n_q >> 1) - 1) & 1);
       if (elect_one()) {
         mbar_expect_tx(bars + B_QFULL + 8 * qb, C::Q_TX);
         if constexpr (HD == 8) {
@@ -278,7 +284,7 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
         int krem, yrow;
         locate(it, i, krem, yrow);
         const int st = n_kv % STAGES, use = n_kv / STAGES;
-        if (use > 0) mbar_wait(wc, bars + B_KVEMPTY + 8 * st, (use - 1) & 1);
+        if (use > 0) mbar_wait_warp(wc, bars + B_KVEMPTY + 8 * st, (use - 1) & 1);
         if (elect_one()) {
           mbar_expect_tx(bars + B_KFULL + 8 * st, KVB);
           tma_load_2d(sK + st * KVB, &tmK, it.c * C::SLW, yrow, bars + B_KFULL + 8 * st);
@@ -297,7 +303,7 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
       if (it.T == 0) continue;
       const int qb = n_q & 1;
       const uint32_t sQb = sQ + qb * S_QBUF;
-      mbar_wait(wc, bars + B_QFULL + 8 * qb, (n_q >> 1) & 1);
+      mbar_wait_warp(wc, bars + B_QFULL + 8 * qb, (n_q >> 1) & 1);
       // Round (j, h): the P V of key tile j - 1 of head h (once its weights are in TMEM), then the scores of key tile j of
       // head h.  The softmax warps of the head have finished reading S_h before they release P_h, so S_h may be
       // overwritten then; tcgen05.mma instructions of one thread execute in issue order, so P_h is read by the P V
@@ -311,15 +317,15 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
         if (j < it.T) {
           int yrow;
           locate(it, j, krem, yrow);
-          mbar_wait(wc, bars + B_KFULL + 8 * st, (n / STAGES) & 1);
+          mbar_wait_warp(wc, bars + B_KFULL + 8 * st, (n / STAGES) & 1);
         }
-        if (j > 0) mbar_wait(wc, bars + B_VFULL + 8 * pst, ((n - 1) / STAGES) & 1);
+        if (j > 0) mbar_wait_warp(wc, bars + B_VFULL + 8 * pst, ((n - 1) / STAGES) & 1);
         const int ncols = (krem >= SK) ? SK : ((krem + 15) >> 4) << 4;
         const int ksteps = (krem_prev >= SK) ? SK / 16 : (krem_prev + 15) >> 4;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           // P_h of key tile j - 1 is in TMEM (and, for the first tile of an item, the previous item's O_h has been read)
-          if (j > 0) mbar_wait(wc, bars + B_PFULL + 8 * h, (n - 1) & 1);
+          if (j > 0) mbar_wait_warp(wc, bars + B_PFULL + 8 * h, (n - 1) & 1);
           tc_fence_after();
           if (elect_one()) {
             if (j > 0) {
@@ -385,7 +391,7 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
         if (it.T > 0) {
           // ... but it may not run ahead into the next item: a barrier phase is told from the one two phases later only
           // by the order of events, so every warp stays within one item of the others
-          mbar_wait(wc, bars + B_OFINAL, n_items_done & 1);
+          mbar_wait_warp(wc, bars + B_OFINAL, n_items_done & 1);
           n_kv += it.T;
           ++n_items_done;
         }
@@ -398,7 +404,7 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
         const int n = n_kv + j;
         int krem, yrow;
         locate(it, j, krem, yrow);
-        mbar_wait(wc, bars + B_SFULL + 8 * h, n & 1);
+        mbar_wait_warp(wc, bars + B_SFULL + 8 * h, n & 1);
         tc_fence_after();
         if (krem < SK && h == 0) {
           // Rows of the V tile past the valid length hold whatever follows in memory; a zero weight times NaN or Inf
@@ -406,7 +412,7 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
           // multiplied) before the first P V of the tile reads them: the MMA warp issues head 0's product first, after
           // this group's release of P_0.
           const int st = n % STAGES;
-          mbar_wait(wc, bars + B_VFULL + 8 * st, (n / STAGES) & 1);
+          mbar_wait_warp(wc, bars + B_VFULL + 8 * st, (n / STAGES) & 1);
           const int row = krem + r;
           if (row < (((krem + 15) >> 4) << 4)) {
             const uint32_t a = sV + st * KVB + row * ROWB;
@@ -549,7 +555,7 @@ attn_tcs_kernel(const __grid_constant__ SProblem prob0, const __grid_constant__ 
       n_kv += it.T;
 
       // ---- epilogue: O_h / l -> bf16, each thread the 16 (32, 64) bytes of its row and head; padded rows +0 ----
-      mbar_wait(wc, bars + B_OFINAL, n_items_done & 1);
+      mbar_wait_warp(wc, bars + B_OFINAL, n_items_done & 1);
       ++n_items_done;
       tc_fence_after();
       if (warp_active) {
