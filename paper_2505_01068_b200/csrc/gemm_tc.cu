@@ -40,7 +40,8 @@ constexpr int G_THREADS = 352;
 constexpr int A_STAGE = GM * GK * 2;      // 16 KB
 constexpr int BOX = GM * 128;             // one epilogue box: 128 rows of 128 bytes
 constexpr int G_MAX_STAGES = 8, MAX_BOXES = 3;  // boxes per epilogue group
-constexpr int G_BAR_BYTES = 512 + 1024;   // barriers, and each epilogue group's half of the tile's bias
+constexpr int G_TABLE = 512;              // tiles of a CTA whose state is looked up once
+constexpr int G_BAR_BYTES = 512 + 1024 + G_TABLE;   // barriers, each epilogue group's half of the tile's bias, and that table
 constexpr int G_MIN_SMEM = 120 * 1024;    // more than half an SM's shared memory: one CTA per SM, so 512 TMEM columns fit
 
 // STORE_PACKED: bf16, rows of the packed layout: a tile whose rows are all this call's leaves by TMA like the others; in the (at
@@ -89,7 +90,7 @@ __device__ __forceinline__ void cluster_sync() {
 __device__ __forceinline__ void arrive_remote(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
-// Bounded wait whose phase other CTAs of the cluster complete with arrive_remote.
+// Bounded wait of a whole warp whose phase other CTAs of the cluster complete with arrive_remote.
 __device__ __forceinline__ bool mbar_wait_cluster(const WaitCtx& w, uint32_t bar, uint32_t parity, int limit = 1 << 16) {
 #pragma unroll 1
   for (int it = 0; it < limit; ++it) {
@@ -99,8 +100,8 @@ __device__ __forceinline__ bool mbar_wait_cluster(const WaitCtx& w, uint32_t bar
         "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    if (ok) return true;
-    if ((it & 63) == 63 && cta_gave_up(w)) return false;
+    if (__all_sync(0xffffffffu, ok != 0)) return true;
+    if ((it & 63) == 63 && __any_sync(0xffffffffu, cta_gave_up(w))) return false;
   }
   asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(w.gave_up), "r"(1u) : "memory");
   atomicOr(w.status, GSIT_DEVFLAG_TIMEOUT);
@@ -142,8 +143,8 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const uint32_t bars = s_box + 2 * p.boxes * BOX;
   const uint32_t bar_full = bars, bar_empty = bar_full + 8 * G_MAX_STAGES, bar_accf = bar_empty + 8 * G_MAX_STAGES,
                  bar_acce = bar_accf + 16, bar_resf = bar_acce + 16, bar_rese = bar_resf + 16 * MAX_BOXES, slot = bar_rese + 16 * MAX_BOXES,
-                 slot_gave_up = slot + 4, s_bias = bars + 512;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+                 slot_gave_up = slot + 4, s_bias = bars + 512, s_table = s_bias + 1024;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   const uint32_t rank = PAIR ? cta_rank() : 0;
   const WaitCtx wc{g.status, slot_gave_up};
   const int kblocks = p.K / GK;
@@ -178,21 +179,40 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   grid_dep_launch();
 
   // The walk over the tiles, the same in every role: first row of the tile (of the pair), first column.
-  const int row_lo = p.packed ? rows_begin(g) : 0, row_hi = p.packed ? rows_end(g) : p.M;
+  const int row_lo = uniform(p.packed ? rows_begin(g) : 0), row_hi = uniform(p.packed ? rows_end(g) : p.M);
   const int t0 = PAIR ? blockIdx.x >> 1 : blockIdx.x, dt = PAIR ? gridDim.x >> 1 : gridDim.x;
-  auto outside = [&](int m0) { return m0 + GM * CTAS <= row_lo || m0 >= row_hi; };            // not touched at all
-  auto padding = [&](int m0) { return p.mask_rows && !p.packed && !tile_real(g, m0, GM * CTAS, p.M); };  // zero, not multiplied
+  // What is done with tile t, the i-th of this CTA: multiplied, zeroed (padding only) or left alone.  Which of the first two needs the lengths and
+  // divisions, the better part of a thousand clocks, and the MMA warp stood still for them at every tile (a tile's products at K 512
+  // take 4256): all threads together look the first tiles up ahead.  With this and warp-uniform control flow a layer of 128 x
+  // (128, 1024, 1024), d 512, a quarter of the samples at half length, 2985 -> 2784 us (attention part of it 679 -> 637), the projection of 32
+  // x (39, 55, 400) at d 128 with its attention 23.9 -> 22.3.
+  enum { MULTIPLY = 0, PADDING = 1, OUTSIDE = 2 };
+  auto look_up = [&](int t) -> int {
+    const int m0 = (t / p.tiles_n) * GM * CTAS;
+    if (m0 + GM * CTAS <= row_lo || m0 >= row_hi) return OUTSIDE;
+    return p.mask_rows && !p.packed && !tile_real(g, m0, GM * CTAS, p.M) ? PADDING : MULTIPLY;
+  };
+  for (int i = tid; i < G_TABLE && t0 + i * (int64_t)dt < p.n_tiles; i += G_THREADS)
+    asm volatile("st.shared.u8 [%0], %1;" ::"r"(s_table + i), "r"(look_up(t0 + i * dt)) : "memory");
+  __syncthreads();
+  auto state = [&](int t, int i) {
+    if (i >= G_TABLE) return uniform(look_up(t));
+    int v;
+    asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(s_table + i) : "memory");
+    return uniform(v);
+  };
 
   if (warp == 0) {
     // ================================ TMA producer ================================
     const int wrows = p.bn / CTAS;
-    int n = 0;  // k-blocks requested so far
-    for (int t = t0; t < p.n_tiles; t += dt) {
+    int st = 0, use = 0;  // stage of the next k-block, times round the ring
+#pragma unroll 1
+    for (int t = t0, j = 0; t < p.n_tiles; t += dt, ++j) {
+      if (state(t, j) != MULTIPLY) continue;
       const int m0 = (t / p.tiles_n) * GM * CTAS, n0 = (t % p.tiles_n) * p.bn;
-      if (outside(m0) || padding(m0)) continue;
-      for (int kb = 0; kb < kblocks; ++kb, ++n) {
-        const int st = n % p.stages, use = n / p.stages;
-        if (use > 0) mbar_wait(wc, bar_empty + 8 * st, (use - 1) & 1);
+#pragma unroll 1
+      for (int kb = 0; kb < kblocks; ++kb) {
+        if (use > 0) mbar_wait_warp(wc, bar_empty + 8 * st, (use - 1) & 1);
         if (elect_one()) {
           const uint32_t sA = base + st * p.stage_bytes, bytes = (uint32_t)(A_STAGE + wrows * GK * 2);
           if constexpr (PAIR) {
@@ -207,22 +227,23 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           }
         }
         __syncwarp();
+        if (++st == p.stages) { st = 0; ++use; }
       }
     }
   } else if (warp == 1) {
     // ================================ MMA issuer ================================
     if (rank == 0) {
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.bn >> 3) << 17) | ((uint32_t)((GM * CTAS) >> 4) << 24);
-      int n = 0, i = 0;  // k-blocks consumed, tiles multiplied
-      for (int t = t0; t < p.n_tiles; t += dt) {
-        const int m0 = (t / p.tiles_n) * GM * CTAS;
-        if (outside(m0) || padding(m0)) continue;
+      int st = 0, use = 0, i = 0;  // stage of the next k-block, times round the ring; tiles multiplied
+#pragma unroll 1
+      for (int t = t0, j = 0; t < p.n_tiles; t += dt, ++j) {
+        if (state(t, j) != MULTIPLY) continue;
         const int ab = i & 1;
         if (i >= 2) mbar_wait_cluster(wc, bar_acce + 8 * ab, ((i >> 1) - 1) & 1);  // the epilogues have drained this accumulator
         tc_fence_after();
-        for (int kb = 0; kb < kblocks; ++kb, ++n) {
-          const int st = n % p.stages;
-          mbar_wait(wc, bar_full + 8 * st, (n / p.stages) & 1);
+#pragma unroll 1
+        for (int kb = 0; kb < kblocks; ++kb) {
+          mbar_wait_warp(wc, bar_full + 8 * st, use & 1);
           tc_fence_after();
           if (elect_one()) {
             const uint32_t sA = base + st * p.stage_bytes;
@@ -233,6 +254,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             if (kb + 1 == kblocks) commit<PAIR>(bar_accf + 8 * ab);
           }
           __syncwarp();
+          if (++st == p.stages) { st = 0; ++use; }
         }
         ++i;
       }
@@ -241,12 +263,14 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     // ================================ residual loader ================================
     if (res) {
       int use[2] = {0, 0};
-      for (int t = t0; t < p.n_tiles; t += dt) {
+#pragma unroll 1
+      for (int t = t0, j = 0; t < p.n_tiles; t += dt, ++j) {
+        if (state(t, j) != MULTIPLY) continue;
         const int m0 = (t / p.tiles_n) * GM * CTAS, n0 = (t % p.tiles_n) * p.bn;
-        if (outside(m0) || padding(m0)) continue;
+#pragma unroll 1
         for (int c = 0; c < p.bn / CW && n0 + c * CW < p.N; ++c) {
           const int grp = c & 1, u = grp ? use[1]++ : use[0]++, box = grp * MAX_BOXES + u % p.boxes;
-          if (u >= p.boxes) mbar_wait(wc, bar_rese + 8 * box, (u / p.boxes - 1) & 1);
+          if (u >= p.boxes) mbar_wait_warp(wc, bar_rese + 8 * box, (u / p.boxes - 1) & 1);
           if (elect_one()) {
             mbar_expect_tx(bar_resf + 8 * box, BOX);
             tma_load_2d(s_box + (grp * p.boxes + u % p.boxes) * BOX, &tmR, n0 + c * CW, m0 + rank * GM, bar_resf + 8 * box);
@@ -262,10 +286,12 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const uint32_t tl = tmem + ((uint32_t)(quarter << 5) << 16);
     auto group_sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory"); };
     int i = 0, u = 0;  // tiles with an accumulator, boxes of this group so far
-    for (int t = t0; t < p.n_tiles; t += dt) {
+#pragma unroll 1
+    for (int t = t0, j = 0; t < p.n_tiles; t += dt, ++j) {
+      const int what = state(t, j);
+      if (what == OUTSIDE) continue;
       const int mp = (t / p.tiles_n) * GM * CTAS, n0 = (t % p.tiles_n) * p.bn, m0 = mp + rank * GM;
-      if (outside(mp)) continue;
-      if (padding(mp)) {  // zeros, eight threads per 128-byte line
+      if (what == PADDING) {  // zeros, eight threads per 128-byte line
         constexpr int ES = MODE == STORE_F32 ? 4 : 2;
         for (int c = grp; c < p.bn / CW; c += 2)
           for (int k = tid & 127; k < GM * 8; k += 128) {
@@ -291,8 +317,9 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         asm volatile("st.shared.f32 [%0], %1;" ::"r"(my_bias + 4 * j), "f"(col < p.N ? p.bias[col] : 0.f) : "memory");
         group_sync();
       }
-      mbar_wait(wc, bar_accf + 8 * ab, (i >> 1) & 1);
+      mbar_wait_warp(wc, bar_accf + 8 * ab, (i >> 1) & 1);
       tc_fence_after();
+#pragma unroll 1
       for (int c = grp; c < p.bn / CW && n0 + c * CW < p.N; c += 2) {
         const int col0 = n0 + c * CW, bi = u % p.boxes;
         const uint32_t box = s_box + (grp * p.boxes + bi) * BOX + r * 128;
@@ -336,7 +363,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           }
           continue;  // no box was used: u stands
         }
-        if (res) mbar_wait(wc, bar_resf + 8 * (grp * MAX_BOXES + bi), (u / p.boxes) & 1);
+        if (res) mbar_wait_warp(wc, bar_resf + 8 * (grp * MAX_BOXES + bi), (u / p.boxes) & 1);
         else group_sync();  // the leader has seen to it that this box's previous store has been read
 #pragma unroll
         for (int q = 0; q < 8; ++q) {  // 16-byte pieces of the row, swizzled with the row
