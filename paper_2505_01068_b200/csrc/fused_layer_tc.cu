@@ -113,7 +113,7 @@ ln_qkv_tc_kernel(const __grid_constant__ LnQkvArgs arg0, const __grid_constant__
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
   const uint32_t bars = base + OFF_BAR;
   const WaitCtx wc{g.status, bars + SLOT + 4};
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
 
   float* prm = reinterpret_cast<float*>(base_ptr + OFF_P);
   if (tid == 0) {
@@ -139,7 +139,7 @@ ln_qkv_tc_kernel(const __grid_constant__ LnQkvArgs arg0, const __grid_constant__
   load_params_early(g);
   grid_dep_wait();  // the weights, too, are read behind it: this kernel may be the first of a call, right after the one that wrote them
   grid_dep_launch();
-  const int row_base = rows_begin(g), rows = rows_end(g);  // this problem's rows of the activation matrices
+  const int row_base = uniform(rows_begin(g)), rows = uniform(rows_end(g));  // this problem's rows of the activation matrices
   const int ntiles = (rows - row_base + TM - 1) / TM;
   if (zero_word != nullptr && blockIdx.x == 0 && tid == 0) *zero_word = 0;  // work counter of the attention kernel that follows
 
@@ -147,7 +147,7 @@ ln_qkv_tc_kernel(const __grid_constant__ LnQkvArgs arg0, const __grid_constant__
     // ================================ producer ================================
     int i = 0;
     for (int t = cta; t < ntiles; t += ctas, ++i) {
-      if (i >= 1) mbar_wait(wc, bars + B_XFREE, (i - 1) & 1);  // the row warps hold the previous tile in registers
+      if (i >= 1) mbar_wait_warp(wc, bars + B_XFREE, (i - 1) & 1);  // the row warps hold the previous tile in registers
       if (elect_one()) {
         mbar_expect_tx(bars + B_XFULL, 2 * XBOX);
         tma_load_2d(base + OFF_X, &tmX, 0, row_base + t * TM, bars + B_XFULL);
@@ -162,11 +162,11 @@ ln_qkv_tc_kernel(const __grid_constant__ LnQkvArgs arg0, const __grid_constant__
   } else if (warp == 1) {
     // ================================ MMA issuer ================================
     constexpr uint32_t IDESC = idesc_bf16(NQ, false);
-    if (cta < ntiles) mbar_wait(wc, bars + B_W, 0);
+    if (cta < ntiles) mbar_wait_warp(wc, bars + B_W, 0);
     int i = 0;
     for (int t = cta; t < ntiles; t += ctas, ++i) {
-      mbar_wait(wc, bars + B_HREADY, i & 1);
-      if (i > 0) mbar_wait(wc, bars + B_ACCFREE, (i - 1) & 1);
+      mbar_wait_warp(wc, bars + B_HREADY, i & 1);
+      if (i > 0) mbar_wait_warp(wc, bars + B_ACCFREE, (i - 1) & 1);
       tc_fence_after();
       if (elect_one()) {
 #pragma unroll
@@ -187,7 +187,7 @@ ln_qkv_tc_kernel(const __grid_constant__ LnQkvArgs arg0, const __grid_constant__
     bool real = row_real32(g, row_base + cta * TM + r, rows);
     for (int t = cta; t < ntiles; t += ctas, ++i) {
       const int row0 = row_base + t * TM;
-      mbar_wait(wc, bars + B_XFULL, i & 1);
+      mbar_wait_warp(wc, bars + B_XFULL, i & 1);
       float v[TD];
       if (real) {
         load_row64(base + OFF_X, r, v);
@@ -208,7 +208,7 @@ ln_qkv_tc_kernel(const __grid_constant__ LnQkvArgs arg0, const __grid_constant__
       }
       const bool real_next = row_real32(g, row_base + (t + ctas) * TM + r, rows);  // overlaps the MMA
 
-      mbar_wait(wc, bars + B_ACCFULL, i & 1);  // the MMA has also finished reading the normalised rows
+      mbar_wait_warp(wc, bars + B_ACCFULL, i & 1);  // the MMA has also finished reading the normalised rows
       tc_fence_after();
 #pragma unroll 1
       for (int c0 = 0; c0 < NQ; c0 += 32) {
@@ -292,7 +292,7 @@ proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_consta
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
   const uint32_t bars = base + OFF_BAR;
   const WaitCtx wc{g.status, bars + SLOT + 4};
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   const int nh = d_ff / 64;  // k-blocks of hidden units
 
   float* prm = reinterpret_cast<float*>(base_ptr + OFF_P);
@@ -336,7 +336,7 @@ proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_consta
   load_params_early(g);
   grid_dep_wait();
   grid_dep_launch();
-  const int row_base = rows_begin(g), rows = rows_end(g);  // this problem's rows of the activation matrices
+  const int row_base = uniform(rows_begin(g)), rows = uniform(rows_end(g));  // this problem's rows of the activation matrices
   const int ntiles = (rows - row_base + TM - 1) / TM;
 
   if (warp == 0) {
@@ -345,13 +345,13 @@ proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_consta
     for (int t = cta; t < ntiles; t += ctas, ++i) {
       const int row0 = row_base + t * TM;
       const int b = i & 1;
-      if (i >= 2) mbar_wait(wc, bars + B_ATTFREE + 8 * b, ((i >> 1) - 1) & 1);
+      if (i >= 2) mbar_wait_warp(wc, bars + B_ATTFREE + 8 * b, ((i >> 1) - 1) & 1);
       if (elect_one()) {
         mbar_expect_tx(bars + B_ATTFULL + 8 * b, TM * 128);
         tma_load_2d(base + OFF_ATT + b * TM * 128, &tmAtt, 0, row0, bars + B_ATTFULL + 8 * b);
       }
       __syncwarp();
-      if (i > 0) mbar_wait(wc, bars + B_XFREE, (i - 1) & 1);
+      if (i > 0) mbar_wait_warp(wc, bars + B_XFREE, (i - 1) & 1);
       if (elect_one()) {
         mbar_expect_tx(bars + B_XFULL, 2 * XBOX);
         tma_load_2d(base + OFF_X, &tmX, 0, row0, bars + B_XFULL);
@@ -363,11 +363,11 @@ proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_consta
     // ================================ MMA issuer ================================
     constexpr uint32_t IDESC_D = idesc_bf16(TD, false);
     const uint32_t idesc_f = idesc_bf16(d_ff, false);
-    mbar_wait(wc, bars + B_W, 0);
+    mbar_wait_warp(wc, bars + B_W, 0);
     // y1 accumulator of tile number i_ = att W_o^T
     auto out_proj = [&](int i_) {
       const int b = i_ & 1;
-      mbar_wait(wc, bars + B_ATTFULL + 8 * b, (i_ >> 1) & 1);
+      mbar_wait_warp(wc, bars + B_ATTFULL + 8 * b, (i_ >> 1) & 1);
       tc_fence_after();
       if (elect_one()) {
 #pragma unroll
@@ -384,7 +384,7 @@ proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_consta
     if (cta < ntiles) out_proj(0);
     for (int t = cta; t < ntiles; t += ctas, ++i) {
       // hidden accumulator = LN2(y1) W_1^T
-      mbar_wait(wc, bars + B_HREADY, i & 1);  // (the rows have also read the y1 accumulator of this tile)
+      mbar_wait_warp(wc, bars + B_HREADY, i & 1);  // (the rows have also read the y1 accumulator of this tile)
       tc_fence_after();
       if (elect_one()) {
 #pragma unroll
@@ -395,7 +395,7 @@ proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_consta
       __syncwarp();
       if (t + ctas < ntiles) out_proj(i + 1);
       // output accumulator = relu(hidden) W_2^T
-      mbar_wait(wc, bars + B_FREADY, i & 1);
+      mbar_wait_warp(wc, bars + B_FREADY, i & 1);
       tc_fence_after();
       if (elect_one()) {
         for (int kb = 0; kb < nh; ++kb)
@@ -417,14 +417,14 @@ proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_consta
     // A operand of the first MLP product.  It runs one tile ahead of the rest, while the tensor core is still busy with
     // the tile before (whose first MLP product has completed, so the LN2 buffer is free).
     auto first_part = [&](int i_, bool real_, float (&v_)[32]) {
-      mbar_wait(wc, bars + B_XFULL, i_ & 1);
+      mbar_wait_warp(wc, bars + B_XFULL, i_ & 1);
       if (real_) {
         load_half_row(base + OFF_X + hf * XBOX, r, v_);
       } else {
 #pragma unroll
         for (int e = 0; e < 32; ++e) v_[e] = 0.f;
       }
-      mbar_wait(wc, bars + B_ACC1, i_ & 1);
+      mbar_wait_warp(wc, bars + B_ACC1, i_ & 1);
       tc_fence_after();
       {
         uint32_t a[32];
@@ -459,7 +459,7 @@ proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_consta
       const bool has_next = t + ctas < ntiles;
       const bool real_next = row_real32(g, row_base + (t + ctas) * TM + r, rows);
       // ---- f = relu(h W_1^T + b_1) -> A operand of the second MLP product ----
-      mbar_wait(wc, bars + B_ACCF, i & 1);
+      mbar_wait_warp(wc, bars + B_ACCF, i & 1);
       tc_fence_after();
       if (i > 0) {  // the previous tile's output stores must have finished reading the staging rows (they overlay f)
         if (tid == 64) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -492,7 +492,7 @@ proj_mlp_tc_kernel(const __grid_constant__ ProjMlpArgs arg0, const __grid_consta
       float vn[32];
       if (has_next) first_part(i + 1, real_next, vn);
       // ---- y = y1 + f W_2^T + b_2 -> staging rows (this thread's box of 32 floats) -> TMA stores; padded rows +0 ----
-      mbar_wait(wc, bars + B_ACCY, i & 1);
+      mbar_wait_warp(wc, bars + B_ACCY, i & 1);
       tc_fence_after();
       {
         uint32_t a[32];

@@ -50,7 +50,7 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
   const uint32_t bars = base + OFF_BAR;
   const WaitCtx wc{g.status, bars + SLOT + 4};
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
 
   float* prm = reinterpret_cast<float*>(base_ptr + OFF_P);
   if (tid == 0) {
@@ -76,7 +76,7 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
   load_params_early(g);
   grid_dep_wait();  // the weights, too, are read behind it: this kernel may be the first of a call, right after the one that wrote them
   grid_dep_launch();
-  const int row_base = rows_begin(g), rows = rows_end(g);  // this problem's rows of the activation matrices
+  const int row_base = uniform(rows_begin(g)), rows = uniform(rows_end(g));  // this problem's rows of the activation matrices
   const int ntiles = (rows - row_base + TM - 1) / TM;
   if (zero_word != nullptr && blockIdx.x == 0 && tid == 0) *zero_word = 0;  // work counter of the attention kernel that follows
 
@@ -84,7 +84,7 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
     // ================================ producer ================================
     int i = 0;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
-      if (i > 0) mbar_wait(wc, bars + B_XFREE, (i - 1) & 1);  // the row warps hold the previous tile in registers
+      if (i > 0) mbar_wait_warp(wc, bars + B_XFREE, (i - 1) & 1);  // the row warps hold the previous tile in registers
       if (elect_one()) {
         mbar_expect_tx(bars + B_XFULL, 4 * XBOX);
         for (int j = 0; j < 4; ++j) tma_load_2d(base + OFF_X + j * XBOX, &tmX, 32 * j, row_base + t * TM, bars + B_XFULL);
@@ -100,11 +100,11 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
   } else if (warp == 1) {
     // ================================ MMA issuer ================================
     constexpr uint32_t IDESC_256 = idesc_bf16(256, false), IDESC_128 = idesc_bf16(128, false);
-    if ((int)blockIdx.x < ntiles) mbar_wait(wc, bars + B_W, 0);
+    if ((int)blockIdx.x < ntiles) mbar_wait_warp(wc, bars + B_W, 0);
     int i = 0;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
-      mbar_wait(wc, bars + B_HREADY, i & 1);
-      if (i > 0) mbar_wait(wc, bars + B_ACCFREE, (i - 1) & 1);
+      mbar_wait_warp(wc, bars + B_HREADY, i & 1);
+      if (i > 0) mbar_wait_warp(wc, bars + B_ACCFREE, (i - 1) & 1);
       tc_fence_after();
       if (elect_one()) {
 #pragma unroll
@@ -131,7 +131,7 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
     bool real = row_real32(g, row_base + (int)blockIdx.x * TM + r, rows);
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
       const int row0 = row_base + t * TM;
-      mbar_wait(wc, bars + B_XFULL, i & 1);
+      mbar_wait_warp(wc, bars + B_XFULL, i & 1);
       float v[64];
       if (real) {
         load_half_row128(base + OFF_X + 2 * hf * XBOX, r, v);
@@ -152,7 +152,7 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
       }
       const bool real_next = row_real32(g, row_base + (t + (int)gridDim.x) * TM + r, rows);  // overlaps the MMA
 
-      mbar_wait(wc, bars + B_ACCFULL, i & 1);  // the MMA has also finished reading the normalised rows
+      mbar_wait_warp(wc, bars + B_ACCFULL, i & 1);  // the MMA has also finished reading the normalised rows
       tc_fence_after();
 #pragma unroll 1
       for (int pass = 0; pass < 2; ++pass) {
@@ -238,7 +238,7 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
   const uint32_t bars = base + OFF_BAR;
   const WaitCtx wc{g.status, bars + SLOT + 4};
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   const int nc = d_ff / 64;  // chunks of 64 hidden units
 
   float* prm = reinterpret_cast<float*>(base_ptr + OFF_P);
@@ -288,7 +288,7 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
   load_params_early(g);
   grid_dep_wait();
   grid_dep_launch();
-  const int row_base = rows_begin(g), rows = rows_end(g);  // this problem's rows of the activation matrices
+  const int row_base = uniform(rows_begin(g)), rows = uniform(rows_end(g));  // this problem's rows of the activation matrices
   const int ntiles = (rows - row_base + TM - 1) / TM;
 
   if (warp == 0) {
@@ -299,7 +299,7 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
     int i = 0, n = 0;  // tiles, weight chunks whose W_1 half has been requested
     auto request_w1 = [&](int m) {
       const int st = m & 1, use = m >> 1, c = m % nc;
-      if (use > 0) mbar_wait(wc, bars + B_W1FREE + 8 * st, (use - 1) & 1);
+      if (use > 0) mbar_wait_warp(wc, bars + B_W1FREE + 8 * st, (use - 1) & 1);
       if (elect_one()) {
         const uint32_t dst = base + OFF_WC + st * WC_STAGE;
         mbar_expect_tx(bars + B_W1FULL + 8 * st, 2 * 64 * 128);
@@ -310,7 +310,7 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
     };
     auto request_w2 = [&](int m) {
       const int st = m & 1, use = m >> 1, c = m % nc;
-      if (use > 0) mbar_wait(wc, bars + B_W2FREE + 8 * st, (use - 1) & 1);
+      if (use > 0) mbar_wait_warp(wc, bars + B_W2FREE + 8 * st, (use - 1) & 1);
       if (elect_one()) {
         const uint32_t dst = base + OFF_WC + st * WC_STAGE + 2 * 64 * 128;
         mbar_expect_tx(bars + B_W2FULL + 8 * st, XBOX);
@@ -325,13 +325,13 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
         if (n > 0) request_w2(n - 1);
         if (c == 0) {
           // the attention buffer also holds the LN2 rows of the previous tile until its last first-MLP product is done
-          if (i > 0) mbar_wait(wc, bars + B_ATTFREE, (i - 1) & 1);
+          if (i > 0) mbar_wait_warp(wc, bars + B_ATTFREE, (i - 1) & 1);
           if (elect_one()) {
             mbar_expect_tx(bars + B_ATTFULL, 2 * XBOX);
             for (int kb = 0; kb < 2; ++kb) tma_load_2d(base + OFF_ATT + kb * XBOX, &tmAtt, 64 * kb, row0, bars + B_ATTFULL);
           }
           __syncwarp();
-          if (i > 0) mbar_wait(wc, bars + B_XFREE, (i - 1) & 1);
+          if (i > 0) mbar_wait_warp(wc, bars + B_XFREE, (i - 1) & 1);
           if (elect_one()) {
             mbar_expect_tx(bars + B_XFULL, 4 * XBOX);
             for (int j = 0; j < 4; ++j) tma_load_2d(base + OFF_X + j * XBOX, &tmX, 32 * j, row0, bars + B_XFULL);
@@ -344,11 +344,11 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
   } else if (warp == 1) {
     // ================================ MMA issuer ================================
     constexpr uint32_t IDESC_128 = idesc_bf16(128, false), IDESC_64 = idesc_bf16(64, false);
-    mbar_wait(wc, bars + B_WO, 0);
+    mbar_wait_warp(wc, bars + B_WO, 0);
     int i = 0, n = 0;  // tiles done, chunks whose first product has been issued
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
       // y1 accumulator = att W_o^T
-      mbar_wait(wc, bars + B_ATTFULL, i & 1);
+      mbar_wait_warp(wc, bars + B_ATTFULL, i & 1);
       tc_fence_after();
       if (elect_one()) {
 #pragma unroll
@@ -360,11 +360,11 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
         umma_commit(bars + B_ACC1);
       }
       __syncwarp();
-      mbar_wait(wc, bars + B_HREADY, i & 1);
+      mbar_wait_warp(wc, bars + B_HREADY, i & 1);
       // first product of chunk m (global index): hidden accumulator (m & 1) = LN2(y1) W_1c^T
       auto first = [&](int m, bool last_of_tile) {
         const int st = m & 1;
-        mbar_wait(wc, bars + B_W1FULL + 8 * st, (m >> 1) & 1);
+        mbar_wait_warp(wc, bars + B_W1FULL + 8 * st, (m >> 1) & 1);
         tc_fence_after();
         if (elect_one()) {
           const uint32_t w1 = base + OFF_WC + st * WC_STAGE;
@@ -382,8 +382,8 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
       };
       // second product of chunk m: accY += relu-hidden(m) W_2c^T
       auto second = [&](int m, bool first_of_tile, bool last_of_tile) {
-        mbar_wait(wc, bars + B_FREADY, m & 1);
-        mbar_wait(wc, bars + B_W2FULL + 8 * (m & 1), (m >> 1) & 1);
+        mbar_wait_warp(wc, bars + B_FREADY, m & 1);
+        mbar_wait_warp(wc, bars + B_W2FULL + 8 * (m & 1), (m >> 1) & 1);
         tc_fence_after();
         if (elect_one()) {
           const uint32_t w2 = base + OFF_WC + (m & 1) * WC_STAGE + 2 * 64 * 128;
@@ -418,7 +418,7 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
       const int row0 = row_base + t * TM;
       // ---- y1 = x + att W_o^T + b_o (this thread's 64 columns, in registers) ----
-      mbar_wait(wc, bars + B_XFULL, i & 1);
+      mbar_wait_warp(wc, bars + B_XFULL, i & 1);
       float v[64];
       if (real) {
         load_half_row128(base + OFF_X + 2 * hf * XBOX, r, v);
@@ -426,7 +426,7 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
 #pragma unroll
         for (int e = 0; e < 64; ++e) v[e] = 0.f;
       }
-      mbar_wait(wc, bars + B_ACC1, i & 1);
+      mbar_wait_warp(wc, bars + B_ACC1, i & 1);
       tc_fence_after();
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
@@ -457,7 +457,7 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
       // ---- hidden chunks: f = relu(h W_1c^T + b_1c) -> A operand of the second product (32 of the 64 units each) ----
 #pragma unroll 1
       for (int c = 0; c < nc; ++c, ++n) {
-        mbar_wait(wc, bars + B_ACCF + 8 * (n & 1), (n >> 1) & 1);
+        mbar_wait_warp(wc, bars + B_ACCF + 8 * (n & 1), (n >> 1) & 1);
         tc_fence_after();
         uint32_t pk[16];
         {
@@ -473,7 +473,7 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
             pk[(e >> 1) + 1] = pack_bf16_relu(h1.x, h1.y);
           }
         }
-        if (n > 0) mbar_wait(wc, bars + B_FFREE, (n - 1) & 1);  // the previous second product has read the hidden chunk
+        if (n > 0) mbar_wait_warp(wc, bars + B_FFREE, (n - 1) & 1);  // the previous second product has read the hidden chunk
 #pragma unroll
         for (int q = 0; q < 4; ++q) st_shared_v4(sw128(base + OFF_F, r, 4 * hf + q), pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
         fence_async_smem();
@@ -482,7 +482,7 @@ proj_mlp_tc128_kernel(const __grid_constant__ CUtensorMap tmAtt, const __grid_co
         if (lane == 0) mbar_arrive(bars + B_FREADY);
       }
       // ---- y = y1 + f W_2^T + b_2; padded rows +0 ----
-      mbar_wait(wc, bars + B_ACCY, i & 1);
+      mbar_wait_warp(wc, bars + B_ACCY, i & 1);
       tc_fence_after();
       // The rows leave through a per-warp transpose in shared memory (2 KB of the hidden-chunk buffer per warp, which
       // nothing reads between the last second product and the next tile's first chunk): a thread owns a row, but a store
