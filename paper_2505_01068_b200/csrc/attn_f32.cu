@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(F32_WARPS * 32)
 attn_f32_kernel(const Geometry g, const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
                 const int64_t row_stride, float* __restrict__ out, float* __restrict__ lse, const float sl2 /* scale * log2(e) */,
                 const int key_splits) {
-  constexpr int HP = DT * T, KT = (HP <= 64) ? 64 : (HP <= 128) ? 32 : 16;  // padded head width, keys per tile
+  constexpr int HP = DT * T, KT = (HP <= 32) ? 2048 / HP : (HP <= 64) ? 64 : (HP <= 128) ? 32 : 16;  // padded head width, keys per tile
   constexpr int TILE = KT * HP, C4 = HP / 4, NT = F32_WARPS * 32;
   extern __shared__ __align__(16) float sm[];                              // [2 buffers][K, V][KT][HP]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -270,7 +270,7 @@ attn_f32_kernel(const Geometry g, const float* __restrict__ q, const float* __re
 template <int DT, int T, int F32_R>
 cudaError_t launch(const Geometry& g, const float* q, const float* k, const float* v, int64_t row_stride, float* out, float* lse,
                    float scale, cudaStream_t st) {
-  constexpr int HP = DT * T, KT = (HP <= 64) ? 64 : (HP <= 128) ? 32 : 16;
+  constexpr int HP = DT * T, KT = (HP <= 32) ? 2048 / HP : (HP <= 64) ? 64 : (HP <= 128) ? 32 : 16;
   // tiles, double-buffered; the merge of key splits needs at most 3 * F32_R * (DT + 2) * 32 floats
   constexpr int FLOATS = 4 * KT * HP, MERGE = 3 * F32_R * (DT + 2) * 32;
   constexpr int smem = (FLOATS > MERGE ? FLOATS : MERGE) * 4;
