@@ -109,15 +109,32 @@ cudaError_t launch_attn_bf16_n(const Geometry& g, const AttnOperands* ops, int n
 #define GSIT_LAUNCH(HD_, CW_, R_, KS_, MB_) return launch_one<Cfg<HD_, CW_, R_, KS_, MB_>>(g, ops, n, row_stride, scale, st)
   const int64_t slices = (int64_t)n * (g.d / cw);
   if (g.hd == 8 && cw == 64) {
-    // 16 us with 64 rows per CTA, 10 with 32, 8 with 16 for one sample of (50, 500, 500); from three CTAs per SM on 64 is best
+    // Rows per CTA x CTAs per SM: 16 x 3 for few tiles, 32 x 2 (keys five tiles ahead), 32 x 3 beyond.  us at B x (50, 500, 500), 8 heads, for
+    // CTAs of 64 rows per SM (which the lines count) 0.9, 1.4, 1.8, 2.3, 2.8, 3.7 (B = 8, 12, 16, 20, 24, 32):
+    //   16 x 3, intra, every position real    19.4  24.9  30.0  35.9  43.0  54.1    cross, half to full  13.9  13.2  15.3  19.3  21.5  26.9
+    //   32 x 2                                15.9  23.4  28.8  35.6  41.3  48.5                         14.2  15.0  15.2  16.8  20.8  24.6
+    //   32 x 3                                21.8  22.2  28.5  33.2  38.8  45.0                         17.3  19.2  20.4  20.9  20.8  22.8
+    //   64 x 2                                22.3  27.4  27.5  39.1  39.4  50.1                         20.0  24.1  25.2  25.9  25.8  26.0
+    // 64 samples, cross, half to full: 32 x 3 40.5, 64 x 2 42.0; 32 x (50, 375, 500) 18.3 and 21.1.  64 x 2 is left for many short walks, where
+    // the CTAs' own cost counts (the pattern's average below six key tiles): cross at 9.2, 11, 14.7 per SM 50.0/49.4, 58.3/57.4, 75.2/73.9, a quarter
+    // real at 14.7 30.0/27.8; the ring pair of a stack of 40 and 64 samples (the same counts) 452/451, 668/663, of 32 397/402; but intra 109.7/110.7.
     const int64_t ctas = tiles(64) * slices;
-    if (2 * ctas <= 3LL * n_sm) GSIT_LAUNCH(8, 64, 1, 64, 3);
-    if (ctas <= 3LL * n_sm) GSIT_LAUNCH(8, 64, 2, 64, 2);
-    GSIT_LAUNCH(8, 64, 4, 64, 2);
+    if (4 * ctas <= 5LL * n_sm) return launch_one<Cfg<8, 64, 1, 64, 3, 1, 1, 3>>(g, ops, n, row_stride, scale, st);
+    if (2 * ctas <= 5LL * n_sm) GSIT_LAUNCH(8, 64, 2, 64, 2);
+    int64_t walks = 0;  // key tiles of all query tiles of a sample
+    for (int s = 0; s < 3; ++s)
+      for (int r = 0; r < 3; ++r)
+        if ((ops[0].allowed >> (3 * s + r)) & 1u) walks += (int64_t)((g.len(s) + 63) / 64) * ((g.len(r) + KT - 1) / KT);
+    if (ctas > 8LL * n_sm && walks * g.batch < 6 * tiles(64)) GSIT_LAUNCH(8, 64, 4, 64, 2);
+    return launch_one<Cfg<8, 64, 2, 64, 3, 1, 1, 3>>(g, ops, n, row_stride, scale, st);
   }
   if (g.hd == 8 && cw == 32) {
-    if (tiles(64) * slices <= n_sm) GSIT_LAUNCH(8, 32, 1, 64, 3);
-    GSIT_LAUNCH(8, 32, 2, 64, 2);
+    // 32 rows per CTA up to four CTAs of 64 per SM, 64 rows beyond, three CTAs per SM both.  us at B x (50, 500, 500), 4 heads, 32 / 64 rows, for
+    // 1.4, 2.8, 3.7, 5.5, 7.4, 14.7 of them per SM (B = 12, 24, 32, 48, 64, 128): intra, every position real 13.0/16.1, 23.1/21.8, 27.6/28.1,
+    // 39.7/38.6, 49.7/45.0, 95.0/84.1; cross, half to full 10.7/14.6, 12.5/19.6, 15.4/19.6, 20.3/20.7, 26.3/24.8, 48.2/39.8.
+    // (64 rows, two CTAs per SM, was taken from one per SM on: 15.3, 23.4, 28.6, 40.9, 48.1, 91.6 and 13.9, 14.7, 15.2, 20.9, 25.3, 45.3.)
+    if (tiles(64) * slices <= 4LL * n_sm) GSIT_LAUNCH(8, 32, 1, 64, 3);
+    return launch_one<Cfg<8, 32, 2, 64, 3, 1, 2, 4>>(g, ops, n, row_stride, scale, st);
   }
   if (g.hd == 8) GSIT_LAUNCH(8, 16, 1, 64, 2);
   if (g.hd == 16 && cw == 64) {
