@@ -125,6 +125,7 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
     const int r = ((warp & 3) << 5) + lane, hf = (warp - 2) >> 2;  // row = TMEM lane; which half of the columns
     const uint32_t tl = tmem + ((uint32_t)((warp & 3) << 5) << 16);
     const uint32_t s_gamma = base + OFF_P, s_beta = s_gamma + D2 * 4, s_bias = s_beta + D2 * 4;
+    const int quarter = warp & 3, limit = map_rows(g);
     stage_parameters<D2, NQ, 256>(prm, gamma, beta, bias, tid - 64);  // while the first rows are on their way
     t_bar_rows8();
     int i = 0;
@@ -139,8 +140,8 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
 #pragma unroll
         for (int e = 0; e < 64; ++e) v[e] = 0.f;
       }
-      if (i > 0 && tid == 64) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-      // the barrier inside: the previous tile's stores have finished reading the staging rows the normalised rows overlay
+      if (i > 0 && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+      // the barrier inside: the pair's stores of the previous tile have finished reading the staging rows the normalised rows overlay
       float mean, rstd;
       split_row_stats<64>(v, base + OFF_STAT, r, hf, eps, real, mean, rstd);
       normalise_to_tile<64>(v, mean, rstd, real, s_gamma, s_beta, 64 * hf, base + OFF_H + hf * XBOX, r, 0);
@@ -156,46 +157,49 @@ ln_qkv_tc128_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
       tc_fence_after();
 #pragma unroll 1
       for (int pass = 0; pass < 2; ++pass) {
-        if (pass > 0) {  // the first pass's stores must have finished reading the staging rows
-          if (tid == 64) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-          t_bar_rows8();
+        if (pass > 0) {  // the pair's stores of the first pass must have finished reading the staging rows
+          if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+          t_bar_pair(quarter);
         }
+        // Boxes of 64 columns in turn between the two warps of a row, three to each over both passes; a box leaves as soon as the warp has
+        // written its 32 rows of it.
 #pragma unroll 1
-        for (int c0 = 32 * hf; c0 < NQ / 2; c0 += 64) {  // alternate groups of 32 output columns
-          const int col = pass * (NQ / 2) + c0;
-          uint32_t a[32];
-          tmem_ld32(tl + col, a);
-          tmem_wait_ld(a);
-          uint32_t pk[16];
+        for (int j = hf ^ pass; j < 3; j += 2) {
+#pragma unroll 1
+          for (int c0 = 64 * j; c0 < 64 * j + 64; c0 += 32) {
+            const int col = pass * (NQ / 2) + c0;
+            uint32_t a[32];
+            tmem_ld32(tl + col, a);
+            tmem_wait_ld(a);
+            uint32_t pk[16];
 #pragma unroll
-          for (int e = 0; e < 32; e += 4) {
-            const float4 bb = ld_v4f(s_bias + (col + e) * 4);
-            const float2 h0 = __fadd2_rn(make_float2(__uint_as_float(a[e]), __uint_as_float(a[e + 1])), make_float2(bb.x, bb.y));
-            const float2 h1 = __fadd2_rn(make_float2(__uint_as_float(a[e + 2]), __uint_as_float(a[e + 3])), make_float2(bb.z, bb.w));
-            pk[e >> 1] = real ? pack_bf16(h0.x, h0.y) : 0u;
-            pk[(e >> 1) + 1] = real ? pack_bf16(h1.x, h1.y) : 0u;
+            for (int e = 0; e < 32; e += 4) {
+              const float4 bb = ld_v4f(s_bias + (col + e) * 4);
+              const float2 h0 = __fadd2_rn(make_float2(__uint_as_float(a[e]), __uint_as_float(a[e + 1])), make_float2(bb.x, bb.y));
+              const float2 h1 = __fadd2_rn(make_float2(__uint_as_float(a[e + 2]), __uint_as_float(a[e + 3])), make_float2(bb.z, bb.w));
+              pk[e >> 1] = real ? pack_bf16(h0.x, h0.y) : 0u;
+              pk[(e >> 1) + 1] = real ? pack_bf16(h1.x, h1.y) : 0u;
+            }
+            const int ch0 = (c0 & 32) >> 3;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) st_shared_v4(sw128(base + OFF_OUT + j * XBOX, r, ch0 + q), pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
           }
-          const uint32_t box = base + OFF_OUT + (c0 >> 6) * XBOX;
-          const int ch0 = (c0 & 32) >> 3;
-#pragma unroll
-          for (int q = 0; q < 4; ++q) st_shared_v4(sw128(box, r, ch0 + q), pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+          fence_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            store_warp_rows(&tmOut, base + OFF_OUT + j * XBOX, quarter, pass * (NQ / 2) + 64 * j, row0, limit);
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+          }
         }
         if (pass == 1) {
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(bars + B_ACCFREE);
         }
-        fence_async_smem();
-        t_bar_rows8();
-        if (tid == 64) {
-#pragma unroll
-          for (int j = 0; j < 3; ++j) tma_store_2d(&tmOut, base + OFF_OUT + j * XBOX, pass * (NQ / 2) + 64 * j, row0);
-          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-        }
       }
       real = real_next;
     }
-    if (tid == 64) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
   }
 
   tc_fence_before();
@@ -548,7 +552,7 @@ cudaError_t launch_ln_qkv_tc128(const Geometry& g, const float* x, int64_t ldx, 
   if (nsm == 0) return cudaErrorUnknown;
   alignas(64) CUtensorMap tmW, tmX, tmOut;
   if (!make_map(&tmW, w_qkv, 3 * D2, D2, D2, 64, 128) || !make_map_f32(&tmX, x, rows, D2, ldx, TM) ||
-      !make_map(&tmOut, qkv, rows, 3 * D2, 3 * D2, 64, TM))
+      !make_map(&tmOut, qkv, rows, 3 * D2, 3 * D2, 64, 32))
     return cudaErrorInvalidValue;
   {
     cudaError_t e = sm_count_and_smem_once(reinterpret_cast<const void*>(ln_qkv_tc128_kernel), qk2::SMEM, nullptr);

@@ -61,11 +61,22 @@ __device__ __forceinline__ bool row_real32(const Geometry& g, int row, int rows)
 // columns -- have eight row warps.
 constexpr int T_THREADS8 = 320;
 __device__ __forceinline__ void t_bar_rows8() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// The two warps that share 32 rows (`quarter`: which of the tile's four).  Only they exchange statistics and write the same staging rows, so the
+// others need not wait for them.
+__device__ __forceinline__ void t_bar_pair(int quarter) { asm volatile("bar.sync %0, 64;" ::"r"(2 + quarter) : "memory"); }
+
+// Rows leave warp by warp: a box of 32 rows x 128 bytes of the staging tile at `tile` (column box), whose first matrix row is row0; `limit`: rows of the
+// tensor map.  Behind a warp-wide fence and barrier, by one lane, which commits.
+__device__ __forceinline__ void store_warp_rows(const CUtensorMap* tm, uint32_t tile, int quarter, int col, int row0, int limit) {
+  if (row0 + 32 * quarter < limit) tma_store_2d(tm, tile + quarter * 32 * 128, col, row0 + 32 * quarter);
+}
+// Rows that the tensor maps over activations span.
+__device__ __forceinline__ int map_rows(const Geometry& g) { return g.row_start != nullptr ? g.capacity : g.batch * g.L; }
 
 // LayerNorm statistics of a row whose columns are split between two threads.  Each takes the mean and the centred sum
 // of squares of its own NC values; the pair exchanges them through `s_stat` (2 x 128 float pairs) and merges them with
 // the pairwise update of Chan, Golub and LeVeque, which is symmetric in the two halves, so both threads get the same
-// bits.  Every row thread calls it (it contains a barrier of the eight row warps).
+// bits.  Every row thread calls it (it contains a barrier of the two warps).
 template <int NC>
 __device__ __forceinline__ void split_row_stats(const float (&v)[NC], uint32_t s_stat, int r, int hf, float eps, bool real,
                                                 float& mean, float& rstd) {
@@ -87,7 +98,7 @@ __device__ __forceinline__ void split_row_stats(const float (&v)[NC], uint32_t s
   }
   const float m2_h = (q0.x + q0.y) + (q1.x + q1.y);
   asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(s_stat + (uint32_t)(hf * TM + r) * 8u), "f"(mean_h), "f"(m2_h) : "memory");
-  t_bar_rows8();
+  t_bar_pair(uniform(r >> 5));
   float mean_p, m2_p;
   asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(mean_p), "=f"(m2_p) : "r"(s_stat + (uint32_t)((hf ^ 1) * TM + r) * 8u) : "memory");
   const float delta = mean_p - mean_h;
