@@ -31,12 +31,12 @@ __device__ __forceinline__ void cp_async4_zfill(uint32_t dst, const void* src, b
 
 // DT features per thread, T threads per row, F32_R rows per thread: head widths up to DT * T (narrower ones are padded with zeros).
 // key_splits (1, 2 or 4): how many ways the warps of the CTA share out the keys.  VEC: rows are 16-byte aligned and hd % 4 == 0.
-template <int DT, int T, int F32_R, bool VEC>
+template <int DT, int T, int F32_R, bool VEC, int KT /* keys per tile */>
 __global__ void __launch_bounds__(F32_WARPS * 32)
 attn_f32_kernel(const Geometry g, const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
                 const int64_t row_stride, float* __restrict__ out, float* __restrict__ lse, const float sl2 /* scale * log2(e) */,
                 const int key_splits) {
-  constexpr int HP = DT * T, KT = (HP <= 32) ? 2048 / HP : (HP <= 64) ? 64 : (HP <= 128) ? 32 : 16;  // padded head width, keys per tile
+  constexpr int HP = DT * T;                                                // padded head width
   constexpr int TILE = KT * HP, C4 = HP / 4, NT = F32_WARPS * 32;
   extern __shared__ __align__(16) float sm[];                              // [2 buffers][K, V][KT][HP]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -267,17 +267,17 @@ attn_f32_kernel(const Geometry g, const float* __restrict__ q, const float* __re
   }
 }
 
-template <int DT, int T, int F32_R>
-cudaError_t launch(const Geometry& g, const float* q, const float* k, const float* v, int64_t row_stride, float* out, float* lse,
+template <int DT, int T, int F32_R, int KT>
+cudaError_t launch_tiles(const Geometry& g, const float* q, const float* k, const float* v, int64_t row_stride, float* out, float* lse,
                    float scale, cudaStream_t st) {
-  constexpr int HP = DT * T, KT = (HP <= 32) ? 2048 / HP : (HP <= 64) ? 64 : (HP <= 128) ? 32 : 16;
+  constexpr int HP = DT * T;
   // tiles, double-buffered; the merge of key splits needs at most 3 * F32_R * (DT + 2) * 32 floats
   constexpr int FLOATS = 4 * KT * HP, MERGE = 3 * F32_R * (DT + 2) * 32;
   constexpr int smem = (FLOATS > MERGE ? FLOATS : MERGE) * 4;
   const bool vec = g.hd % 4 == 0 && row_stride % 4 == 0 && g.d % 4 == 0 &&
                    ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(k) | reinterpret_cast<uintptr_t>(v) |
                      reinterpret_cast<uintptr_t>(out)) & 15u) == 0;
-  auto kernel = vec ? attn_f32_kernel<DT, T, F32_R, true> : attn_f32_kernel<DT, T, F32_R, false>;
+  auto kernel = vec ? attn_f32_kernel<DT, T, F32_R, true, KT> : attn_f32_kernel<DT, T, F32_R, false, KT>;
   int n_sm = 0;
   cudaError_t e = sm_count_and_smem_once(reinterpret_cast<const void*>(kernel), smem, &n_sm);
   if (e != cudaSuccess) return e;
@@ -308,6 +308,18 @@ cudaError_t launch(const Geometry& g, const float* q, const float* k, const floa
       if (e != cudaSuccess) return e;
     }
   return cudaSuccess;
+}
+
+// Key tiles of 32 KB (256 keys at head_dim 8, 128 at 16, 64 at 32) need a quarter of the barriers of 64 keys, but their places are filled with
+// zeros where a segment is shorter: 32 x (50, 375, 500), 8 heads of 8, intra 78.0 -> 75.5 us, 4 x (50, 300, 200) 14.0 -> 13.6, 8 x (20, 100, 60), 4 of
+// 16 6.4 -> 6.2, but 16 x (50, 50, 50), 8 of 8 6.7 -> 7.05.
+template <int DT, int T, int F32_R>
+cudaError_t launch(const Geometry& g, const float* q, const float* k, const float* v, int64_t row_stride, float* out, float* lse,
+                   float scale, cudaStream_t st) {
+  constexpr int HP = DT * T, KT = (HP <= 64) ? 64 : (HP <= 128) ? 32 : 16, WIDE = (HP <= 32) ? 2048 / HP : KT;
+  if constexpr (WIDE > KT)
+    if (g.seg_len[0] > KT || g.seg_len[1] > KT || g.seg_len[2] > KT) return launch_tiles<DT, T, F32_R, WIDE>(g, q, k, v, row_stride, out, lse, scale, st);
+  return launch_tiles<DT, T, F32_R, KT>(g, q, k, v, row_stride, out, lse, scale, st);
 }
 
 }  // namespace
