@@ -33,17 +33,6 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
       : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
-// One poll that lets the hardware park the thread for up to `ns` nanoseconds (it wakes as soon as the phase completes):
-// for roles that wait long, so that their polling does not take issue slots from the warps that compute.
-__device__ __forceinline__ bool mbar_try_park(uint32_t bar, uint32_t parity, uint32_t ns) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity), "r"(ns) : "memory");
-  return ok != 0;
-}
 // One poll that never parks the thread.
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
   uint32_t ok;
@@ -105,48 +94,9 @@ __device__ __forceinline__ bool mbar_wait_warp(const WaitCtx& w, uint32_t bar, u
   return false;
 }
 
-// The same with parked polls of up to ten microseconds each (2^15 of them at most: a third of a second).
-__device__ __forceinline__ bool mbar_wait_parked(const WaitCtx& w, uint32_t bar, uint32_t parity, int limit = 1 << 15) {
-#pragma unroll 1
-  for (int it = 0; it < limit; ++it) {
-    if (mbar_try_park(bar, parity, 10000u)) return true;
-    if ((it & 15) == 15 && cta_gave_up(w)) return false;
-  }
-  asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(w.gave_up), "r"(1u) : "memory");
-  atomicOr(w.status, GSIT_DEVFLAG_TIMEOUT);
-  return false;
-}
-
-// Bounded wait that sleeps between polls.  A try_wait that fails comes back within tens of clocks, so a warp that waits
-// by polling alone keeps issuing instructions; with several waiting warps per scheduler that takes most of the issue
-// slots from the warps that compute.  Here a poll never parks (test_wait) and is followed by a sleep of about `ns`
-// nanoseconds during which the warp issues nothing.  Gives up after `limit` polls like mbar_wait.
-__device__ __forceinline__ bool mbar_wait_sleep(const WaitCtx& w, uint32_t bar, uint32_t parity, unsigned ns, int limit = 1 << 17) {
-#pragma unroll 1
-  for (int it = 0; it < limit; ++it) {
-    if (mbar_test(bar, parity)) return true;
-    if (ns) __nanosleep(ns);
-    if ((it & 63) == 63 && cta_gave_up(w)) return false;
-  }
-  asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(w.gave_up), "r"(1u) : "memory");
-  atomicOr(w.status, GSIT_DEVFLAG_TIMEOUT);
-  return false;
-}
-
 // Arrival that counts for `count` participants (a warp arriving on behalf of warps that have nothing to contribute).
 __device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-// Bounded wait that spins on non-parking polls: the shortest hand-over latency, at the price of issue slots.
-__device__ __forceinline__ bool mbar_wait_spin(const WaitCtx& w, uint32_t bar, uint32_t parity, int limit = 1 << 22) {
-#pragma unroll 1
-  for (int it = 0; it < limit; ++it) {
-    if (mbar_test(bar, parity)) return true;
-    if ((it & 1023) == 1023 && cta_gave_up(w)) return false;
-  }
-  asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(w.gave_up), "r"(1u) : "memory");
-  atomicOr(w.status, GSIT_DEVFLAG_TIMEOUT);
-  return false;
 }
 
 // ---------------------------------------------------------------- TMA
