@@ -37,11 +37,18 @@ gsit_status gsit_trace_read(int kernel_kind, float* total_ms, int32_t* launches)
 gsit_status gsit_trace_launches(int kernel_kind, float* out_ms, int32_t capacity, int32_t* launches);
 gsit_status gsit_trace_reset(void);
 
-/* Runs a one-CTA kernel whose only action is a bounded wait (the same routine the tcgen05 kernels wait with, limited to
+/* Runs a one-CTA kernel whose only action are bounded waits (the same routine the tcgen05 kernels wait with, limited to
  * 4096 polls) on a barrier that nothing will ever complete.  The wait runs out, the kernel raises GSIT_DEVFLAG_TIMEOUT
  * and returns normally: nothing traps, faults or spins without limit, and the context stays usable.  Afterwards
  * gsit_last_device_status() answers GSIT_ERR_TIMEOUT once and clears the flag.  Asynchronous on `stream`. */
 gsit_status gsit_test_expire_wait(gsit_stream stream);
+
+/* The same kernel with what its two warps were answered.  answers (DEVICE, 130 words): warp 0's answers for a phase that is over
+ * and for one that never will be (32 lanes each: 1, then 0), the same of warp 1, which waits after warp 0 has run out and must leave
+ * without running out itself; then the flags that warp 0 raised (GSIT_DEVFLAG_TIMEOUT) and those of warp 1 (none), both OR-ed to
+ * what stands there.  cluster_form: 1 for the wait on barriers of a CTA pair, else 0.  The library's own status word is left alone.
+ * Asynchronous on `stream`. */
+gsit_status gsit_test_wait_answers(uint32_t* answers, int32_t cluster_form, gsit_stream stream);
 
 /* Copies `bytes` (a multiple of 16; both DEVICE pointers 16-byte aligned) from src to dst in a one-CTA kernel that allows
  * the kernel after it in the stream to start at once and writes only some delay_us (at most 1000) microseconds later: a

@@ -43,7 +43,8 @@ class LayerWeights(ctypes.Structure):
 
 EXPORTS = ("gsit_im_qkv_proj", "gsit_im_attention_fwd", "gsit_im_layer_fwd", "gsit_workspace_bytes",
            "gsit_last_device_status", "gsit_status_string", "gsit_version", "gsit_trace_enable", "gsit_trace_read",
-           "gsit_trace_launches", "gsit_trace_reset", "gsit_tune_attention", "gsit_test_expire_wait", "gsit_test_late_write", "gsit_im_layer_fwd_static",
+           "gsit_trace_launches", "gsit_trace_reset", "gsit_tune_attention", "gsit_test_expire_wait", "gsit_test_wait_answers",
+           "gsit_test_late_write", "gsit_im_layer_fwd_static",
            "gsit_stack_head_fwd", "gsit_im_layer_pair_fwd",
            "gsit_plan_rows", "gsit_pack_rows", "gsit_unpack_rows", "gsit_plan_pack_rows", "gsit_plan_pack_map_rows",
            "gsit_im_encoder_fwd", "gsit_encoder_runs_chained", "gsit_im_layer_scatter_fwd", "gsit_layer_scatters", "gsit_attention_uses_workspace")
@@ -176,6 +177,16 @@ def expire_wait_selftest():
     lib = load()
     lib.gsit_test_expire_wait.argtypes = [ctypes.c_void_p]
     _check(lib.gsit_test_expire_wait(_stream()), "gsit_test_expire_wait")
+
+
+def wait_answers(cluster_form: bool):
+    """Test hook: (answers [2 warps, 2 waits, 32 lanes], flags [2]) of the kernel behind expire_wait_selftest (see include/gsit_test.h)."""
+    out = torch.zeros(130, dtype=torch.int32, device="cuda")
+    lib = load()
+    lib.gsit_test_wait_answers.argtypes = [ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p]
+    _check(lib.gsit_test_wait_answers(_ptr(out), int(cluster_form), _stream()), "gsit_test_wait_answers")
+    out = out.cpu()
+    return out[:128].reshape(2, 2, 32), out[128:].tolist()
 
 
 def late_write(dst, src, delay_us: int = 100):

@@ -90,23 +90,6 @@ __device__ __forceinline__ void cluster_sync() {
 __device__ __forceinline__ void arrive_remote(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
-// Bounded wait of a whole warp whose phase other CTAs of the cluster complete with arrive_remote.
-__device__ __forceinline__ bool mbar_wait_cluster(const WaitCtx& w, uint32_t bar, uint32_t parity, int limit = 1 << 16) {
-#pragma unroll 1
-  for (int it = 0; it < limit; ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    if (__all_sync(0xffffffffu, ok != 0)) return true;
-    if ((it & 63) == 63 && __any_sync(0xffffffffu, cta_gave_up(w))) return false;
-  }
-  asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(w.gave_up), "r"(1u) : "memory");
-  atomicOr(w.status, GSIT_DEVFLAG_TIMEOUT);
-  return false;
-}
 // A tensor copy into this CTA's shared memory that completes on a barrier of either CTA of the pair.
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t cluster_bar) {
   asm volatile(

@@ -169,20 +169,34 @@ gsit_status run_attention(const Geometry& g, int dtype, const void* q, const voi
                                    static_cast<const float*>(v), row_stride, static_cast<float*>(out), lse, scale, st));
 }
 
-// A bounded wait that must run out: the barrier expects one arrival and nobody arrives.
-__global__ void expire_wait_kernel(unsigned int* status) {
-  __shared__ __align__(8) uint64_t bar;
+// Bounded waits whose barrier expects one arrival that nobody makes, by the loop that the kernels wait with: warp 0 must run out after 4096
+// polls; warp 1, whose own limit is sixteen times that, must then see that the CTA has given up.  Both also wait for a phase that is over.
+// `status` and `drained` take the flags of warps 0 and 1; answers (may be null): 2 warps x (phase over, phase never over) x 32 lanes.
+__global__ void expire_wait_kernel(unsigned int* status, unsigned int* drained, uint32_t* answers, int cluster_form) {
+  __shared__ __align__(8) uint64_t bar[2];
   __shared__ uint32_t gave_up;
-  const uint32_t b = smem_u32(&bar);
+  const uint32_t never = smem_u32(&bar[0]), over = smem_u32(&bar[1]);
   if (threadIdx.x == 0) {
     gave_up = 0;
-    ptx::mbar_init(b, 1);
+    ptx::mbar_init(never, 1);
+    ptx::mbar_init(over, 1);
     ptx::mbar_init_fence();
+    ptx::mbar_arrive(over);
   }
   __syncthreads();
-  const ptx::WaitCtx wc{status, smem_u32(&gave_up)};
-  if (threadIdx.x == 0) ptx::mbar_wait(wc, b, 0, 1 << 12);
-  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const ptx::WaitCtx wc{warp == 0 ? status : drained, smem_u32(&gave_up)};
+  auto wait = [&](uint32_t b, int limit) { return cluster_form ? ptx::mbar_wait_cluster(wc, b, 0, limit) : ptx::mbar_wait_warp(wc, b, 0, limit); };
+  for (int w = 0; w < 2; ++w) {
+    if (warp == w) {
+      const bool first = wait(over, 1 << 12), second = wait(never, w == 0 ? 1 << 12 : 1 << 16);
+      if (answers != nullptr) {
+        answers[64 * w + lane] = first;
+        answers[64 * w + 32 + lane] = second;
+      }
+    }
+    __syncthreads();
+  }
 }
 
 // Lets its successor start at once, then takes its time before it writes (about delay_us, at most twice that).
@@ -744,7 +758,13 @@ const char* gsit_status_string(gsit_status s) {
 gsit_status gsit_test_expire_wait(gsit_stream stream) {
   unsigned int* p = nullptr;
   if (status_ptr(&p) != cudaSuccess) return GSIT_ERR_CUDA;
-  expire_wait_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(p);
+  expire_wait_kernel<<<1, 64, 0, static_cast<cudaStream_t>(stream)>>>(p, p, nullptr, 0);
+  return from_cuda(cudaGetLastError());
+}
+
+gsit_status gsit_test_wait_answers(uint32_t* answers, int32_t cluster_form, gsit_stream stream) {
+  if (!answers || (cluster_form != 0 && cluster_form != 1)) return GSIT_ERR_INVALID_ARG;
+  expire_wait_kernel<<<1, 64, 0, static_cast<cudaStream_t>(stream)>>>(answers + 128, answers + 129, answers, cluster_form);
   return from_cuda(cudaGetLastError());
 }
 

@@ -57,22 +57,39 @@ __device__ __forceinline__ bool cta_gave_up(const WaitCtx& w) {
   asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(v) : "r"(w.gave_up) : "memory");
   return v != 0;
 }
-// Bounded wait on a barrier phase.  Returns true when the phase completed; false after `limit` polls (the timeout flag is
-// raised) or as soon as another wait of this CTA has expired.  The caller carries on either way and must still release
-// whatever it holds.
+// Bounded wait of a whole warp, with the same answer in all lanes: until poll() is true in every lane.  Returns true when it was; false after
+// `limit` polls (the timeout flag is raised) or as soon as another wait of this CTA has expired.  The caller carries on either way and must still
+// release whatever it holds.
 // The loops of all waits stay rolled.  Left to itself the compiler unrolls them, at every place where they are used: the polls of the
 // waiting warps then stream through kilobytes of instructions and push those of the computing warps out of the instruction caches.  Text of
 // the head_dim 16 attention 54 -> 46 KB, misses of its instruction cache 309 K -> 123 K, 74.9 -> 71.2 us at 64 x (50, 500, 500), 8 heads, intra;
 // head_dim 32, 4 heads, cross 36.5 -> 34.3; a whole stack of that batch 718 -> 701 us, of 32 samples a quarter real 214.6 -> 205.0.
-__device__ __forceinline__ bool mbar_wait(const WaitCtx& w, uint32_t bar, uint32_t parity, int limit = 1 << 16) {
+template <typename Poll>
+__device__ __forceinline__ bool wait_warp(const WaitCtx& w, int limit, Poll poll) {
 #pragma unroll 1
   for (int it = 0; it < limit; ++it) {
-    if (mbar_try(bar, parity)) return true;
-    if ((it & 63) == 63 && cta_gave_up(w)) return false;
+    if (__all_sync(0xffffffffu, poll())) return true;
+    if ((it & 63) == 63 && __any_sync(0xffffffffu, cta_gave_up(w))) return false;
   }
   asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(w.gave_up), "r"(1u) : "memory");
   atomicOr(w.status, GSIT_DEVFLAG_TIMEOUT);
   return false;
+}
+// ... on a barrier phase.
+__device__ __forceinline__ bool mbar_wait_warp(const WaitCtx& w, uint32_t bar, uint32_t parity, int limit = 1 << 16) {
+  return wait_warp(w, limit, [&] { return mbar_try(bar, parity); });
+}
+// ... on a phase that other CTAs of the cluster complete.
+__device__ __forceinline__ bool mbar_wait_cluster(const WaitCtx& w, uint32_t bar, uint32_t parity, int limit = 1 << 16) {
+  return wait_warp(w, limit, [&] {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+  });
 }
 
 // A value that is the same in all lanes of the (whole) warp, made visible as such to the compiler: what depends on it stays in uniform
@@ -82,17 +99,6 @@ __device__ __forceinline__ bool mbar_wait(const WaitCtx& w, uint32_t bar, uint32
 // us without / with this and mbar_wait_warp below, B200: 64 x (50, 500, 500), 8 heads of 16 intra 71.2/66.1, cross 51.5/47.8, of 4 heads of 32
 // intra 45.2/42.7; 128 x (128, 1024, 1024), 8 of 64 cross 468/439, intra 679/637; 64 x (50, 500, 500), 8 of 8 cross 43.0/41.9.
 __device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
-// mbar_wait by a whole warp, with the same answer in all lanes.
-__device__ __forceinline__ bool mbar_wait_warp(const WaitCtx& w, uint32_t bar, uint32_t parity, int limit = 1 << 16) {
-#pragma unroll 1
-  for (int it = 0; it < limit; ++it) {
-    if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
-    if ((it & 63) == 63 && __any_sync(0xffffffffu, cta_gave_up(w))) return false;
-  }
-  asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(w.gave_up), "r"(1u) : "memory");
-  atomicOr(w.status, GSIT_DEVFLAG_TIMEOUT);
-  return false;
-}
 
 // Arrival that counts for `count` participants (a warp arriving on behalf of warps that have nothing to contribute).
 __device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t count) {
