@@ -104,9 +104,13 @@ attn_f32_kernel(const Geometry g, const float* __restrict__ q, const float* __re
       locate(j, &r, &k0);
       const uint32_t dst = smem_u32(sm) + (uint32_t)((j & 1) * 2 * TILE * 4);
       const int n = nk[r] - k0;
+      // Of a wide tile only the rounds of the CTA that hold a key are fetched or filled: nothing is read behind the last key's group.
+      constexpr bool WIDE = KT > 64;
+      static_assert(!WIDE || NT * 4 / HP % F32_G == 0, "a round of the CTA must hold whole groups");
       const int64_t off = (base + g.seg_off[r] + k0) * row_stride + (int64_t)h * hd;
       if (VEC) {
         for (int i = tid; i < KT * C4; i += NT) {
+          if (WIDE && (i - tid) / C4 >= n) break;
           const int row = i / C4, c = i % C4;
           const bool ok = row < n && 4 * c < hd;
           const int64_t at = ok ? off + (int64_t)row * row_stride + 4 * c : 0;
@@ -114,7 +118,8 @@ attn_f32_kernel(const Geometry g, const float* __restrict__ q, const float* __re
           cp_async16_zfill(dst + (TILE + 4 * i) * 4, v + at, ok);
         }
       } else {
-        for (int i = tid; i < TILE; i += NT) {
+        const int most = WIDE ? min(KT, (n + F32_G - 1) / F32_G * F32_G) * HP : TILE;
+        for (int i = tid; i < most; i += NT) {
           const int row = i / HP, c = i % HP;
           const bool ok = row < n && c < hd;
           const int64_t at = ok ? off + (int64_t)row * row_stride + c : 0;
@@ -310,15 +315,18 @@ cudaError_t launch_tiles(const Geometry& g, const float* q, const float* k, cons
   return cudaSuccess;
 }
 
-// Key tiles of 32 KB (256 keys at head_dim 8, 128 at 16, 64 at 32) need a quarter of the barriers of 64 keys, but their places are filled with
-// zeros where a segment is shorter: 32 x (50, 375, 500), 8 heads of 8, intra 78.0 -> 75.5 us, 4 x (50, 300, 200) 14.0 -> 13.6, 8 x (20, 100, 60), 4 of
-// 16 6.4 -> 6.2, but 16 x (50, 50, 50), 8 of 8 6.7 -> 7.05.
+// Wide key tiles: 256 keys at head_dim 8, 128 at 16 (8 KB each of K and V, twice as many buffers: a quarter and half of the barriers of 64 keys).
+// They are taken where a segment is longer than half of one; of a tile that is not full only the rounds that hold a key are filled (every place
+// filled: 4 x (17, 126, 125), 16 heads of 8, a quarter real, 5.5 -> 5.95 us).  Against 64 keys throughout, us: 32 x (50, 375, 500), 8 heads of 8,
+// intra 78.0 -> 75.5; 4 x (50, 300, 200) 14.0 -> 13.6; geometric means over batches of 1 - 32, all patterns and lengths, 8 and 16 heads of 8:
+// (50, 500, 500) 0.96, (70, 300, 200) 0.97, (10, 256, 129) 0.97 (worst single call 1.04: 80 real keys in one tile, whose load nothing hides);
+// (17, 126, 125) and (30, 120, 90) 0.995, worst 1.04: left to 64 keys.  Heads of 16: (30, 120, 90) 0.98, (17, 126, 125) 0.99, longer 0.985, worst 1.02.
 template <int DT, int T, int F32_R>
 cudaError_t launch(const Geometry& g, const float* q, const float* k, const float* v, int64_t row_stride, float* out, float* lse,
                    float scale, cudaStream_t st) {
   constexpr int HP = DT * T, KT = (HP <= 64) ? 64 : (HP <= 128) ? 32 : 16, WIDE = (HP <= 32) ? 2048 / HP : KT;
   if constexpr (WIDE > KT)
-    if (g.seg_len[0] > KT || g.seg_len[1] > KT || g.seg_len[2] > KT) return launch_tiles<DT, T, F32_R, WIDE>(g, q, k, v, row_stride, out, lse, scale, st);
+    if (2 * g.seg_len[0] > WIDE || 2 * g.seg_len[1] > WIDE || 2 * g.seg_len[2] > WIDE) return launch_tiles<DT, T, F32_R, WIDE>(g, q, k, v, row_stride, out, lse, scale, st);
   return launch_tiles<DT, T, F32_R, KT>(g, q, k, v, row_stride, out, lse, scale, st);
 }
 
