@@ -108,33 +108,64 @@ cudaError_t launch_attn_bf16_n(const Geometry& g, const AttnOperands* ops, int n
   // does not depend on it (the keys per step are the same), so the number of problems may count here.
 #define GSIT_LAUNCH(HD_, CW_, R_, KS_, MB_) return launch_one<Cfg<HD_, CW_, R_, KS_, MB_>>(g, ops, n, row_stride, scale, st)
   const int64_t slices = (int64_t)n * (g.d / cw);
+  const bool full = g.valid_len == nullptr;  // every length is known here
+  // CTAs of 32 rows, of all problems, that walk (three quarters of) the most key tiles.  Where lengths are given, those of segments of one tile
+  // only: they keep their CTAs however few rows are real.
+  auto long_walks = [&]() {
+    int64_t ctas = 0;
+    for (int i = 0; i < n; ++i) {
+      int kt[3] = {0, 0, 0}, most = 0;
+      for (int s = 0; s < 3; ++s) {
+        for (int r = 0; r < 3; ++r)
+          if ((ops[i].allowed >> (3 * s + r)) & 1u) kt[s] += (g.len(r) + KT - 1) / KT;
+        if (kt[s] > most) most = kt[s];
+      }
+      for (int s = 0; s < 3; ++s)
+        if (4 * kt[s] >= 3 * most && (full || g.len(s) <= 64)) ctas += (g.len(s) + 31) / 32;
+    }
+    return ctas * g.batch * (g.d / cw);
+  };
   if (g.hd == 8 && cw == 64) {
-    // Rows per CTA x CTAs per SM: 16 x 3 for few tiles, 32 x 2 (keys five tiles ahead), 32 x 3 beyond.  us at B x (50, 500, 500), 8 heads, for
-    // CTAs of 64 rows per SM (which the lines count) 0.9, 1.4, 1.8, 2.3, 2.8, 3.7 (B = 8, 12, 16, 20, 24, 32):
-    //   16 x 3, intra, every position real    19.4  24.9  30.0  35.9  43.0  54.1    cross, half to full  13.9  13.2  15.3  19.3  21.5  26.9
-    //   32 x 2                                15.9  23.4  28.8  35.6  41.3  48.5                         14.2  15.0  15.2  16.8  20.8  24.6
-    //   32 x 3                                21.8  22.2  28.5  33.2  38.8  45.0                         17.3  19.2  20.4  20.9  20.8  22.8
-    //   64 x 2                                22.3  27.4  27.5  39.1  39.4  50.1                         20.0  24.1  25.2  25.9  25.8  26.0
-    // 64 samples, cross, half to full: 32 x 3 40.5, 64 x 2 42.0; 32 x (50, 375, 500) 18.3 and 21.1.  64 x 2 is left for many short walks, where
-    // the CTAs' own cost counts (the pattern's average below six key tiles): cross at 9.2, 11, 14.7 per SM 50.0/49.4, 58.3/57.4, 75.2/73.9, a quarter
-    // real at 14.7 30.0/27.8; the ring pair of a stack of 40 and 64 samples (the same counts) 452/451, 668/663, of 32 397/402; but intra 109.7/110.7.
+    // Rows per CTA x CTAs per SM: 16 x 3 for few tiles, 32 x 2 (keys five tiles ahead), 32 x 3 beyond.  Times over those of the version without
+    // uniform control flow (16 rows up to 1.5, 32 up to 3, 64 beyond, three key stages), geometric mean and worst over six sets of segments between
+    // (60, 60, 60) and (20, 1000, 300), intra and cross, lengths full, half to full and a quarter, by CTAs of 64 rows per SM, which the lines count:
+    //   per SM      1.0 - 1.25    1.25 - 1.5    1.5 - 2.5     2.5 - 3       3 - 4         4 - 5.6
+    //   16 x 3       0.96 0.99     0.95 0.98     0.96 1.17     0.97 1.11     0.95 1.25     1.03 1.24
+    //   32 x 2       0.99 1.22     0.99 1.19     0.94 1.00     0.93 1.01     0.88 1.15     0.93 1.11
+    //   32 x 3       1.13 1.45     1.17 1.76     0.98 1.27     0.94 1.14     0.86 1.06     0.88 1.03
+    //   64 x 2       1.33 1.70     1.37 1.84     1.14 1.58     1.04 1.41     0.96 0.99     0.96 0.99
+    // So 16 x 3 up to 1.5, 32 x 2 up to 3; but where every length is full 32 x 3 wins from 2.5 on (32 x 2 0.94, 32 x 3 0.88), and loses to 64 x 2
+    // where its long walks make one wave and up to a quarter (28 x (50, 500, 500), cross: 28.5 and 27.1).  Given lengths may do the same
+    // unseen: 22 x (20, 1000, 300), intra, half to full is the 1.06 above.  Four key stages at 32 x 3 and 16 x 3, which fit too, change either
+    // by less than 1 %.
+    // 64 x 2 also for many short walks, where the CTAs' own cost counts (the pattern's average below six key tiles): cross at 9.2, 11, 14.7 per
+    // SM 32 x 3 50.0, 64 x 2 49.4, 58.3/57.4, 75.2/73.9, a quarter real at 14.7 30.0/27.8; the ring pair of a stack of 40 and 64 samples (the
+    // same counts) 452/451, 668/663, of 32 397/402; but intra 109.7/110.7.
     const int64_t ctas = tiles(64) * slices;
-    if (4 * ctas <= 5LL * n_sm) return launch_one<Cfg<8, 64, 1, 64, 3, 1, 1, 3>>(g, ops, n, row_stride, scale, st);
-    if (2 * ctas <= 5LL * n_sm) GSIT_LAUNCH(8, 64, 2, 64, 2);
+    if (2 * ctas <= 3LL * n_sm) return launch_one<Cfg<8, 64, 1, 64, 3, 1, 1, 3>>(g, ops, n, row_stride, scale, st);
+    if (2 * ctas <= (full ? 5LL : 6LL) * n_sm) GSIT_LAUNCH(8, 64, 2, 64, 2);
     int64_t walks = 0;  // key tiles of all query tiles of a sample
     for (int s = 0; s < 3; ++s)
       for (int r = 0; r < 3; ++r)
         if ((ops[0].allowed >> (3 * s + r)) & 1u) walks += (int64_t)((g.len(s) + 63) / 64) * ((g.len(r) + KT - 1) / KT);
-    if (ctas > 8LL * n_sm && walks * g.batch < 6 * tiles(64)) GSIT_LAUNCH(8, 64, 4, 64, 2);
+    const int64_t waves = full ? long_walks() : 0, wave = 3LL * n_sm;
+    if ((ctas > 8LL * n_sm && walks * g.batch < 6 * tiles(64)) || (ctas > 3LL * n_sm && waves > wave && 4 * waves <= 5 * wave)) GSIT_LAUNCH(8, 64, 4, 64, 2);
     return launch_one<Cfg<8, 64, 2, 64, 3, 1, 1, 3>>(g, ops, n, row_stride, scale, st);
   }
   if (g.hd == 8 && cw == 32) {
-    // 32 rows per CTA up to four CTAs of 64 per SM, 64 rows beyond, three CTAs per SM both.  us at B x (50, 500, 500), 4 heads, 32 / 64 rows, for
-    // 1.4, 2.8, 3.7, 5.5, 7.4, 14.7 of them per SM (B = 12, 24, 32, 48, 64, 128): intra, every position real 13.0/16.1, 23.1/21.8, 27.6/28.1,
-    // 39.7/38.6, 49.7/45.0, 95.0/84.1; cross, half to full 10.7/14.6, 12.5/19.6, 15.4/19.6, 20.3/20.7, 26.3/24.8, 48.2/39.8.
-    // (64 rows, two CTAs per SM, was taken from one per SM on: 15.3, 23.4, 28.6, 40.9, 48.1, 91.6 and 13.9, 14.7, 15.2, 20.9, 25.3, 45.3.)
-    if (tiles(64) * slices <= 4LL * n_sm) GSIT_LAUNCH(8, 32, 1, 64, 3);
-    return launch_one<Cfg<8, 32, 2, 64, 3, 1, 2, 4>>(g, ops, n, row_stride, scale, st);
+    // 32 x 3, then 64 x 2, then 64 x 3, five key stages all.  As above, for 4 heads (32 rows up to 1, 64 x 2 beyond, three key stages, is 1):
+    //   per SM      0.9 - 1.5     1.5 - 3       3 - 4.5       4.5 - 5.6     5.6 - 7.5     7.5 - 9.2
+    //   32 x 3       0.84 0.99     0.87 1.20     0.89 1.15     0.93 1.01     0.94 1.10     0.97 1.08
+    //   64 x 2       0.94 1.00     0.94 1.00     0.93 0.98     0.92 0.96     0.93 0.96     0.93 0.96
+    //   64 x 3       0.93 1.04     1.05 1.27     0.98 1.26     0.94 1.12     0.90 1.05     0.87 0.99
+    // (64 x 3 with four stages is 2 % behind.)  32 x 3 up to 4.5, then 64 x 3, which where lengths are given waits for 5.5: half to full it is 1.12 at
+    // 4.6 and 0.92 at 5.3, full 0.85 at both (a quarter real is still 1.05 at 6.9).  64 x 2 between the two, and where the long walks of 32 x 3
+    // make one wave and up to a third (16 x (50, 500, 500), intra, full 17.5 and 15.0 us, every block 36.3 and 30.1; 80 x (60, 60, 60), half to full,
+    // 1.19 and 0.97).  Given lengths of longer segments may do the same unseen (up to 1.09; 22 x (20, 1000, 300), intra, half to full, 1.15).
+    const int64_t ctas = tiles(64) * slices, waves = long_walks(), wave = 3LL * n_sm;
+    if (2 * ctas <= 9LL * n_sm && !(2 * ctas > 3LL * n_sm && waves > wave && 3 * waves <= 4 * wave)) GSIT_LAUNCH(8, 32, 1, 64, 3);
+    if (2 * ctas <= (full ? 9LL : 11LL) * n_sm) GSIT_LAUNCH(8, 32, 2, 64, 2);
+    GSIT_LAUNCH(8, 32, 2, 64, 3);
   }
   if (g.hd == 8) GSIT_LAUNCH(8, 16, 1, 64, 2);
   if (g.hd == 16 && cw == 64) {
