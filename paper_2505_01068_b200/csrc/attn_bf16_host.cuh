@@ -42,17 +42,17 @@ int g_attn_variant = 0;  // gsit_kernel_choice
 // the device only.  us on mma.sync / tensor memory at B x (50, 500, 500), intra, 8 heads of 16 (a call of its own, which clears
 // the work counter first; then a whole layer at d 128, where the first half clears it):
 //   units per SM             56           84          112          141          225
-//   full lengths          33.6/33.2    48.6/45.6    58.7/51.4    72.3/62.8     114/94.5
-//   half to full          28.7/29.8    36.2/36.9    43.7/42.9    53.2/51.0    83.8/75.2
-//   a quarter real        12.3/18.3    13.3/19.1    16.3/21.1    19.4/23.1    30.4/33.3
-//   layer, half to full   52.7/48.8    73.9/68.9    83.5/76.6    94.1/85.1     142/127
-//   layer, a quarter      34.6/34.9    35.5/37.1    39.0/38.8    42.5/41.6    56.7/53.2
+//   full lengths          30.7/28.2    44.8/41.1    54.0/45.8    66.6/56.8    103/85.5
+//   half to full          25.2/24.5    32.9/31.3    40.1/37.5    48.9/44.5    74.4/64.5
+//   a quarter real         9.6/12.6    14.6/16.2    15.6/16.7    19.1/19.7    28.8/26.9
+//   layer, half to full   43.7/41.9    64.5/61.7    72.1/68.1    93.6/87.8     134/123
+//   layer, a quarter      28.5/29.5    46.7/47.3    48.1/48.0    64.5/63.1    88.6/84.3
 // -> 110: from there on the tensor-memory kernel is no slower at half-to-full lengths nor in a layer at any; a call of its own at a
-// quarter real loses 3 - 5 us up to 225 units.  4 heads of 32: half to full 27.7/27.6 at 42, 32.5/30.9 at 56, 63.1/47.5 at 112; a
-// quarter 10.5/16.4, 12.9/18.4, 24.1/25.4; layer, a quarter 34.4/35.8 at 56, 41.2/41.0 at 84 -> 55.
+// quarter real loses 1 us up to 141 units.  4 heads of 32: half to full 25.2/23.7 at 42, 30.6/26.6 at 56, 56.7/41.1 at 112; a
+// quarter 11.9/14.1, 12.5/14.7, 23.2/21.6; layer, a quarter 44.6/45.8 at 56, 62.9/62.1 at 84 -> 55.
 //   head_dim 64 is a dense contraction; there only a few short walks (at most two key tiles per row) are over sooner in the
-//   mma.sync kernel (32 x (50, 50, 50), 2 heads: 4.4 against 5.1 us; 64 samples: 7.7 against 6.8; 128: 11.5 against 9.0).
-//   head_dim 8: the tensor-memory kernel is slower throughout (55 against 44 us at 64 x (50, 500, 500)): a tcgen05 hand-over
+//   mma.sync kernel (32 x (50, 50, 50), 2 heads: 4.3 against 4.8 us; 64 samples: 6.7 against 6.3; 128: 10.9 against 8.5).
+//   head_dim 8: the tensor-memory kernel is slower throughout (44.5 against 39.5 us at 64 x (50, 500, 500)): a tcgen05 hand-over
 //   per 64 keys of one head costs more than the 8192 exponentials it feeds.
 bool attn_uses_tensor_memory(const Geometry& g, uint32_t allowed) {
   const int var = g_attn_variant;

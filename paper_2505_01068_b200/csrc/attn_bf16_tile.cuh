@@ -21,8 +21,8 @@ constexpr int WAIT_SPINS = 1 << 20;
 // step, MINB_ = CTAs per SM the register allocation must allow, SL_ = column slices per CTA, NSG_ = warps per head,
 // STAGES_ = key tiles in flight.  Three make the warps of a CTA wait for the slowest; five over three, geometric means (and worst) over (50, 500, 500)
 // and (30, 120, 90), 1 - 64 samples, intra and every block, full and half to full: head_dim 8 x 2 heads 0.95 (1.01), 16 x 2 heads 0.95 (1.02), 16 x 4
-// 0.96 (1.03), 32 x 1 and 32 x 4 0.96 (1.02), 64 x 2 1.00 (1.04).  With more, larger CTAs the second kernel of a layer starts later beside them: layers
-// of width 32 at 32 x (30, 120, 90), full, are up to 4 % slower for it, at (50, 500, 500) 4 % faster.
+// 0.96 (1.03), 32 x 1 and 32 x 4 0.96 (1.02); at 64 the walks have one or two key tiles and it is the same.  In a layer of width 32 at (50, 500, 500)
+// 4 % as well, but around one wave of short walks five can lose what the next kernel's early start gains (40 x (30, 120, 90), full, 13.8 -> 14.4).
 template <int HD_, int CW_, int R_, int KSTEP_, int MINB_, int SL_ = 1, int NSG_ = 8 / (CW_ / HD_ * SL_), int STAGES_ = 5>
 struct Cfg {
   static constexpr int HD = HD_, CW = CW_, R = R_, KSTEP = KSTEP_, MINB = MINB_, SL = SL_, STAGES = STAGES_;

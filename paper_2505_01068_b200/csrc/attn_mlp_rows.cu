@@ -438,32 +438,33 @@ int makespan(const Walks* w, int count, int n_sm) {
 //
 // No valid_len: every length is full, the walks are known.  The line lies at 5/3 (d 32: 7/4).  us of a layer in one launch behind the
 // projection / in two; the last end:
-//   d 64   6 x (50, 500, 500), intra 31.7/27.7 (2.0), both rings 42.7/40.9 (2.1);   32 x (50, 52, 52), intra 19.5/17.4 (2.0)
-//          5 x (50, 500, 500), forward ring 21.2/26.7 (1.1);   4 x, both rings 27.2/28.4 (1.6)
-//   d 32   54 x (50, 52, 52), intra 15.6/13.4 (2.0);   8 x (50, 500, 500), both rings 23.8/27.4 (1.6)
+//   d 64   6 x (50, 500, 500), intra 30.7/26.5 (2.0), both rings 41.7/40.5 (2.1);   32 x (50, 52, 52), intra 19.5/17.2 (2.0)
+//          5 x (50, 500, 500), forward ring 21.0/25.8 (1.1);   4 x, both rings 26.8/27.9 (1.6)
+//   d 32   54 x (50, 52, 52), intra 15.4/12.7 (2.0);   8 x (50, 500, 500), both rings 23.3/24.2 (1.6)
 // Over 291 shapes beyond one wave at d 64 (segments of 8 - 1024 steps, one problem or two) this costs 0.4 % on average against the better
 // of both, one launch up to the limits above 10 %; over 352 at d 32 1.3 % and 13 %.
 // At d 128 the separate second half itself takes two waves above 32 rows per SM.  Below, a second wave here loses throughout (3850 rows of
-// (50, 52, 52) 32.0/27.0, 4230 of (50, 116, 116) 32.9/28.0); above, two waves hold their own up to eight key tiles (5250 rows of (50, 500,
-// 500), intra 47.4/48.1, 4928 of (50, 52, 52) 34.1/35.3; fourteen key tiles 64.2/60.4).
+// (50, 52, 52) 31.8/26.5, 4230 of (50, 116, 116) 32.4/27.2); above, two waves nearly hold their own up to eight key tiles (5250 rows of (50,
+// 500, 500), intra 46.4/44.6, 4928 of (50, 52, 52) 33.8/34.1).
 //
 // With valid_len the lengths are unknown here, and padding cuts the second wave short -- where a segment has several tiles; a segment of
 // one tile keeps its CTA however few rows are real.  So the same sum over walks of two thirds of the lengths, the line at 15/8 (among 110
-// stacks at 1 - 3 waves any share from 5/8 to 3/4 does as well).  us of a stack on these lengths, layers in one launch / in two on packed rows:
-//   d 64   42 x (21, 43, 34), depths 2 and 2   half to full 118.8/93.7, a quarter 81.7/84.0;   63 x (31, 21, 10), 4 and 3   202.5/168.6, 198.6/150.3
-//          14 x (59, 16, 57), 4 and 3 (one wave)   86.3/132.5, 79.8/117.2
-//   d 32   34 x (11, 60, 75), 2 and 1          51.3/47.8, 44.7/41.4;                            17 x (9, 152, 208), 3 and 2  88.2/93.0, 56.2/76.5
+// stacks at 1 - 3 waves any share from 5/8 to 3/4 does as well).  us of a stack on these lengths, the layers of this width in
+// one launch / in two on packed rows:
+//   d 64   42 x (21, 43, 34), depths 2 and 2   half to full 114/110, a quarter 78.5/76.4;   63 x (31, 21, 10), 4 and 3   187/165, 170/144
+//          14 x (59, 16, 57), 4 and 3 (one wave)   84.1/110, 76.2/93.8
+//   d 32   34 x (11, 60, 75), 2 and 1          52.3/47.1, 46.9/40.1;                            17 x (9, 152, 208), 3 and 2  85.3/86.5, 50.9/58.7
 // At d 128 an encoder's other choice is packed rows, whose second half then mostly fits one wave: there two thirds of the lengths must fit
-// one wave here (25 x (30, 26, 146), three layers in the stack's intra encoder, 148.6/124.9, 93.0/101.5).  A layer by itself takes up to
-// three waves (32 x (50, 52, 52) half to full 33.9/36.3, few 23.3/27.6).
+// one wave here (25 x (30, 26, 146), three layers in the stack's intra encoder, 124/111, 76.9/89.4).  A layer by itself takes up to
+// three waves (32 x (50, 52, 52) half to full 33.3/35.0, few 23.4/26.7).
 // Longest walk with valid_len: eight key tiles.  d 64, intra, 1.2 waves, us, one launch / two, by key tiles (lengths full, half to full,
 // 0.05 - 0.4):
 //   tiles     4          6          8          9          10         11         13         14
-//   full  23.5/21.0  27.2/23.9  30.5/26.5  33.1/28.5  34.9/29.8  37.8/31.1  41.8/34.2  44.6/35.3
-//   half  16.3/21.1  18.1/23.3  18.9/26.0  20.3/27.5  20.8/28.4  22.2/30.0  24.3/32.2  26.5/33.3
-//   few   13.2/16.8  13.4/16.9  13.6/17.7  13.9/18.4  13.7/17.9  14.2/18.6  14.9/19.2  15.3/19.2
-// What padding gains stays at a quarter from four tiles on; what a batch whose lengths are full after all loses grows from 12 % at four
-// and 15 % at eight to 26 % at fourteen.  The line lies where one still clearly outweighs the other.
+//   full  22.7/20.5  25.8/23.1  29.2/25.8  31.5/27.5  32.9/28.2  35.6/30.0  39.4/32.4  42.0/33.9
+//   half  16.9/21.0  18.3/23.2  18.9/25.5  20.0/27.3  22.4/28.4  24.4/29.8  25.8/32.6  27.9/34.2
+//   few   13.3/17.1  13.6/17.9  14.1/18.0  14.7/18.8  14.2/17.8  14.9/19.0  13.1/16.7  13.0/16.9
+// What padding gains is a quarter from four tiles on, a fifth from ten; what a batch whose lengths are full after all loses grows from 11 % at four
+// and 13 % at eight to 24 % at fourteen.  The line lies where one still clearly outweighs the other.
 bool layer_tail_preferred(const Geometry& g, const uint32_t* allowed, int n, bool in_encoder) {
   int n_sm = 0;
   if (sm_count_and_smem_once(nullptr, 0, &n_sm) != cudaSuccess) return false;

@@ -166,9 +166,9 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const int t0 = PAIR ? blockIdx.x >> 1 : blockIdx.x, dt = PAIR ? gridDim.x >> 1 : gridDim.x;
   // What is done with tile t, the i-th of this CTA: multiplied, zeroed (padding only) or left alone.  Which of the first two needs the lengths and
   // divisions, the better part of a thousand clocks, and the MMA warp stood still for them at every tile (a tile's products at K 512
-  // take 4256): all threads together look the first tiles up ahead.  With this and warp-uniform control flow a layer of 128 x
-  // (128, 1024, 1024), d 512, a quarter of the samples at half length, 2985 -> 2784 us (attention part of it 679 -> 637), the projection of 32
-  // x (39, 55, 400) at d 128 with its attention 23.9 -> 22.3.
+  // take 4256): all threads together look the first tiles up ahead.  The four products of a layer of 128 x (128, 1024, 1024), d 512, a
+  // quarter of the samples at half length, one by one: 385, 250, 533, 493 -> 344, 234, 466, 467 us, the second figures with warp-uniform control
+  // flow as well; the projection of 32 x (39, 55, 400) at d 128 with its attention 23.9 -> 22.3.
   enum { MULTIPLY = 0, PADDING = 1, OUTSIDE = 2 };
   auto look_up = [&](int t) -> int {
     const int m0 = (t / p.tiles_n) * GM * CTAS;
