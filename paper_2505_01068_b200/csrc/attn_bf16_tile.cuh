@@ -156,14 +156,20 @@ __device__ __forceinline__ void init_walk(uint32_t base, int tid) {
 // Walks the keys of tile t (t.T > 0), by all threads of the CTA: the heads of column slices first_slice .. + SL - 1, whose columns start at
 // xq, xk, xv in the three maps.  Leaves the normalised rows as bf16 where Q was (swizzled rows of CW columns, slice by slice) and ends
 // with a barrier; lse (with the heads of the whole problem) may be null.  meanwhile(): what every thread does once Q is there.
-template <typename C, int CTA_WARPS, typename F>
+// UNIFORM: what is the same in a whole warp is made known as such (ptx.cuh), which nearly every kernel is faster for.
+template <typename C, int CTA_WARPS, bool UNIFORM = true, typename F>
 __device__ __forceinline__ void attend_tile(const Geometry& g, const Tile& t_, const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                                             const int xq, const int xk, const int xv, const int first_slice, const float sl2, float* __restrict__ lse,
                                             const uint32_t base, F meanwhile) {
   constexpr int HD = C::HD, CW = C::CW, G = C::G, R = C::R, PITCH = C::PITCH, SWZ = C::SWZ,
                 KSTEP = C::KSTEP, NT = C::NT, KSQ = C::KSQ, NTO = C::NTO, SL = C::SL, STAGES = C::STAGES;
+  auto same = [](int v) { return UNIFORM ? uniform(v) : v; };
+  auto wait = [&](uint32_t bar, uint32_t parity) {
+    if constexpr (UNIFORM) mbar_wait_warp(g, bar, parity);
+    else mbar_wait(g, bar, parity);
+  };
   constexpr bool HOIST = (R > 1);  // several query slabs per warp reuse the K/V fragments of a step
-  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
+  const int tid = threadIdx.x, warp = same(tid >> 5), lane = tid & 31;
   const int head = warp % (G * SL), sg = warp / (G * SL), slice = head / G, head_in_slice = head % G;
   // Known at compile time where every warp of the CTA attends: a walk behind a branch takes longer (14 key tiles of one 16-row slab at head_dim 8:
   // 13.75 us, 13.50 without the branch; one sample of (50, 500, 500) 8.96 and 8.80).  Not with four slabs per warp, which then spill
@@ -176,7 +182,7 @@ __device__ __forceinline__ void attend_tile(const Geometry& g, const Tile& t_, c
   const uint32_t bar_empty = bar_full + 8 * STAGES;     // STAGES barriers: all attending warps are done with the stage
   const uint32_t bar_q = bar_empty + 8 * STAGES;
   const int cb = head_in_slice * (HD / 8);  // first 16-byte chunk of this warp's head inside a tile row
-  const int b = t_.b, s = t_.s, q0 = t_.q0, kn0 = t_.kn0, kn1 = t_.kn1, kn2 = t_.kn2, nk0 = t_.nk0, nk1 = t_.nk1, T = uniform(t_.T), q_real = uniform(t_.q_real);
+  const int b = t_.b, s = t_.s, q0 = t_.q0, kn0 = t_.kn0, kn1 = t_.kn1, kn2 = t_.kn2, nk0 = t_.nk0, nk1 = t_.nk1, T = same(t_.T), q_real = same(t_.q_real);
   const int kbase0 = t_.kbase0, kbase1 = t_.kbase1, kbase2 = t_.kbase2;
   const int64_t grow0 = t_.grow0;
 
@@ -224,7 +230,7 @@ __device__ __forceinline__ void attend_tile(const Geometry& g, const Tile& t_, c
   // ---- query fragments, kept in registers for the whole key walk ----
   uint32_t QF[R][KSQ][4];
   if (active) {
-    mbar_wait_warp(g, bar_q, 0);
+    wait(bar_q, 0);
 #pragma unroll
     for (int r_ = 0; r_ < R; ++r_) {
       const int row0 = (sg * R + r_) * 16;
@@ -446,10 +452,10 @@ __device__ __forceinline__ void attend_tile(const Geometry& g, const Tile& t_, c
         }
       }
       __syncwarp();
-      mbar_wait_warp(g, bar_full + 8 * st, (i / STAGES) & 1);
+      wait(bar_full + 8 * st, (i / STAGES) & 1);
       int krem, yrow;
       locate(i - from, krem, yrow);
-      krem = uniform(krem);
+      krem = same(krem);
       const bool first = i == from;
       const uint32_t sKs = sK + (st * SL + slice) * C::KV_BYTES, sVs = sV + (st * SL + slice) * C::KV_BYTES;
       if (krem >= KT) {
