@@ -96,7 +96,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(const WaitCtx& w, uint32_t bar
 // registers, and branches on it need nothing to bring the lanes together again.  The compiler takes a warp index, a tile's number of real rows or
 // the answer of a barrier for values that differ between lanes otherwise, and of the 37 M warp instructions of a head_dim 16 attention 10 M were
 // then the bookkeeping of reconvergence, against 13 M of arithmetic; 145 KB of text of the head_dim 8 kernel 113 KB with it.
-// us without / with this and mbar_wait_warp below, B200: 64 x (50, 500, 500), 8 heads of 16 intra 71.2/66.1, cross 51.5/47.8, of 4 heads of 32
+// us without / with this and mbar_wait_warp above, B200: 64 x (50, 500, 500), 8 heads of 16 intra 71.2/66.1, cross 51.5/47.8, of 4 heads of 32
 // intra 45.2/42.7; 128 x (128, 1024, 1024), 8 of 64 cross 468/439, intra 679/637; 64 x (50, 500, 500), 8 of 8 cross 43.0/41.9.
 __device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 
